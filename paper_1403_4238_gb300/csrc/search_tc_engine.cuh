@@ -41,8 +41,8 @@
 // the smallest (SSD << 32 | idx) key.  The read-back works in FP32:
 // fl(fl(S - 2X) + A2) is exact whenever the SSD is below 2^24 (then |S - 2X|
 // < 2^24 too, as A2 < 2^24) and at least 2^24 otherwise (rounding is
-// monotone), so a best value below 2^24 is the exact minimum; a thread
-// whose best is not repeats its candidates in integers.
+// monotone), so a best value below 2^24 is the exact minimum; a warp with a
+// thread whose best is not repeats its candidates in integers.
 #pragma once
 #include "inpaint_engine.h"
 #include "ptx.cuh"
@@ -299,12 +299,14 @@ __device__ __forceinline__ unsigned long long tc_epilogue(const ImgState& s, uin
       }
     }
   }
-  if (!any) return best;
-  if (bv < 16777216.0f) {  // exact
-    const unsigned long long key = ((unsigned long long)(uint32_t)bv << 32) | (unsigned)bi;
+  // tcgen05.ld is a whole warp's instruction, so the warp decides together: it
+  // takes the integer pass when any of its threads has no candidate below 2^24
+  if (!__any_sync(0xffffffffu, any && !(bv < 16777216.0f))) {
+    if (!any) return best;
+    const unsigned long long key = ((unsigned long long)(uint32_t)bv << 32) | (unsigned)bi;  // exact
     return key < best ? key : best;
   }
-  // no candidate below 2^24: the exact integer pass over the same accumulators
+  // the exact integer pass over the same accumulators
   for (int h = 0; h < cols; h += 16) {
     uint32_t X[16], S[16];
     tc_ld16(ta + (uint32_t)h, X);

@@ -160,3 +160,23 @@ def test_tc_rejects_unsupported(api):
     for loop in ("engine", "graph"):
         with pytest.raises(api.InpaintError):
             api.Inpainter(case.rgb, case.mask, 9, form="tc", loop=loop)
+
+
+@pytest.mark.parametrize("loop", LOOPS)
+@pytest.mark.parametrize("split", [38, 41, 43])
+def test_tc_ssd_above_two_to_24_in_part_of_a_warp(api, loop, split):
+    # 17x17 patches, dark rows above `split`, bright ones below: the SSD of a
+    # dark target passes 2^24 within a few candidate rows, so threads of one
+    # warp differ in whether their best needs the integer read-back
+    g = np.random.Generator(np.random.PCG64(split))
+    rgb = g.integers(0, 12, (96, 72, 3)).astype(np.uint8)
+    rgb[split:] = 255 - rgb[split:]
+    mask = np.zeros((96, 72), np.uint8)
+    mask[2:9, 30:39] = 1
+    mask[88:92, 10:16] = 1
+    case = synth.Case("two_tones", rgb, mask, 8)
+    ora = oracle.run(case.rgb, case.mask, case.r)
+    rc, n, tr, out, info = run_tc(api, case, loop)
+    assert rc == 0 and n == ora.iters
+    assert_trace_equal(tr, ora.trace)
+    assert np.array_equal(out, ora.rgb)
