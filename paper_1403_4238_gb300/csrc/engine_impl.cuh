@@ -30,6 +30,18 @@
 
 namespace inp {
 
+// The CTA's dynamic shared memory.  Every function names it itself instead of
+// taking a pointer to it, so that the compiler sees shared addresses: through
+// a pointer kept in memory each access of the leader's phases was a generic
+// load or store with 64-bit address arithmetic.
+__device__ __forceinline__ uint8_t* eng_smem() {
+  extern __shared__ __align__(128) uint8_t eng_smem_raw[];
+  return eng_smem_raw;
+}
+__device__ __forceinline__ const uint32_t* smem_words(int offset) {
+  return reinterpret_cast<const uint32_t*>(eng_smem() + offset);
+}
+
 // ---------------------------------------------------------------- search batch
 
 // A search batch is 32 candidate rows x BWC candidate columns.  Lane l of
@@ -188,15 +200,18 @@ __device__ __forceinline__ void unit_ssd(const uint32_t* __restrict__ strip,
 
 // The compute of a search round, outside the engine body so that its
 // registers hold only the row strips, the target row and the accumulators
-// (the engine body keeps the leader's state live across the search).
+// (the engine body keeps the leader's state live across the search).  These
+// functions take byte offsets into the CTA's shared memory, not pointers: a
+// pointer argument is a generic address, whose every access is a generic
+// load with 64-bit address arithmetic.
 
 // Smallest key (SSD << 32 | idx) of this lane's candidates in one unit:
 // `bits` marks the valid ones, idx0 is the linear index of the first.
 template <int R, int SRW>
-__device__ __noinline__ unsigned long long unit_best(const uint32_t* strip, const uint32_t* tgt,
-                                                     const uint32_t* rowd, uint32_t bits, unsigned idx0) {
+__device__ __noinline__ unsigned long long unit_best(int strip, int tgt, uint32_t bits, unsigned idx0) {
   uint32_t acc[4 * SRW];
-  unit_ssd<R, SRW>(strip, tgt, rowd, acc);
+  unit_ssd<R, SRW>(smem_words(strip), smem_words(tgt), smem_words(tgt) + EngGeom<R, SRW>::P * EngGeom<R, SRW>::TP,
+                   acc);
   unsigned long long best = ~0ull;
 #pragma unroll
   for (int k = 0; k < 4 * SRW; ++k) {
@@ -292,10 +307,10 @@ __device__ __forceinline__ void unit16_ssd(const uint32_t* __restrict__ strip, i
 // Smallest key (SSD << 32 | idx) of this lane's 16 candidates of one unit:
 // `vb` marks the valid ones, idx0 is the linear index of the first.
 template <int R>
-__device__ __noinline__ unsigned long long unit16_best(const uint32_t* strip, int pitch, const uint32_t* tgt,
-                                                       const uint32_t* rowd, uint32_t vb, unsigned idx0) {
+__device__ __noinline__ unsigned long long unit16_best(int strip, int pitch, int tgt, uint32_t vb,
+                                                       unsigned idx0) {
   uint32_t acc[kResCols];
-  unit16_ssd<R>(strip, pitch, tgt, rowd, acc);
+  unit16_ssd<R>(smem_words(strip), pitch, smem_words(tgt), smem_words(tgt) + ResGeom<R>::P * ResGeom<R>::TP, acc);
   unsigned long long best = ~0ull;
 #pragma unroll
   for (int k = 0; k < kResCols; ++k) {
@@ -308,21 +323,19 @@ __device__ __noinline__ unsigned long long unit16_best(const uint32_t* strip, in
 // All units of this CTA for the current target, warp w taking its local
 // units w, w + 16, ...; returns the lane's smallest key.
 template <int R>
-__device__ __noinline__ unsigned long long resident_units16(const ResPlan* pl, const uint8_t* tiles, int xb,
-                                                            int cy0, int W, const uint32_t* tgt,
-                                                            const uint32_t* rowd) {
+__device__ __noinline__ unsigned long long resident_units16(int plan, int tiles, int xb, int cy0, int W, int tgt) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const ResPlan* pl = reinterpret_cast<const ResPlan*>(smem_words(plan));
   const int u0 = pl->u0, n = pl->u1 - pl->u0, ncu = pl->ncu, b0 = pl->seg[0].band;
-  const uint16_t* bits = reinterpret_cast<const uint16_t*>(tiles + pl->bits_off);
+  const uint16_t* bits = reinterpret_cast<const uint16_t*>(smem_words(tiles + pl->bits_off));
   unsigned long long best = ~0ull;
 #pragma unroll 1
   for (int j = warp; j < n; j += kEngWarps) {
     const int u = u0 + j, band = u / ncu, col = u - band * ncu;
     const ResSeg& sg = pl->seg[band - b0];
-    const uint32_t* strip = reinterpret_cast<const uint32_t*>(tiles + sg.off) + lane * sg.pitch +
-                            (col - sg.c_lo) * kResCols;
+    const int strip = tiles + sg.off + 4 * (lane * sg.pitch + (col - sg.c_lo) * kResCols);
     const unsigned idx0 = (unsigned)((cy0 + band * kResRows + lane) * W + xb + col * kResCols);
-    const unsigned long long k = unit16_best<R>(strip, sg.pitch, tgt, rowd, bits[j * 32 + lane], idx0);
+    const unsigned long long k = unit16_best<R>(strip, sg.pitch, tgt, bits[j * 32 + lane], idx0);
     best = k < best ? k : best;
   }
   return best;
@@ -384,8 +397,9 @@ struct EngSmemTail {
 
 static_assert(offsetof(EngSmemTail, bars) == 0, "the kernel initialises the barriers at the start of shared memory");
 
+constexpr int kTgtOff = (int)((sizeof(EngSmemTail) + 15) & ~size_t(15));
 constexpr int kTgtWords = 17 * 20 + 17 + 3;  // padded target rows + row masks (R <= 8)
-constexpr size_t kHeadBytes = ((((sizeof(EngSmemTail) + 15) & ~size_t(15)) + kTgtWords * 4 + 127) / 128) * 128;
+constexpr size_t kHeadBytes = ((kTgtOff + kTgtWords * 4 + 127) / 128) * 128;
 
 // Shared memory of an engine CTA: head | (the leader only) update state and
 // update cache | two count tiles | tile slots.  The slots hold the source
@@ -525,11 +539,7 @@ __device__ inline bool gather_keys(const unsigned long long* slots, int n, unsig
         }
       }
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, o);
-      best = ob < best ? ob : best;
-    }
+    best = warp_min_u64(best);
     late = __any_sync(0xffffffffu, late);
     if (lane == 0) {
       red[0] = late ? 1ull : 0ull;
@@ -572,7 +582,7 @@ __device__ __noinline__ void run_tc_search(const EngineArgs& ea, EngCtx& x, cons
   // the context lives in the kernel's local memory, which misses L1 (shared
   // memory takes nearly all of it) and is re-read after every barrier or
   // fence: keep working copies in registers, write them back at the end
-  uint8_t* const smem = x.smem;
+  uint8_t* const smem = eng_smem();
   const uint32_t tmem = x.tmem;
   uint32_t tc_rows = x.tc_rows, tc_tiles = x.tc_tiles;
   int tc_pref = x.tc_pref, tc_nb = x.tc_nb;
@@ -652,8 +662,7 @@ __device__ __noinline__ void run_tc_search(const EngineArgs& ea, EngCtx& x, cons
         tp[2 * P * GT::TW] = (uint16_t)bf16_of_int(d2);
         tp[3 * P * GT::TW] = (uint16_t)bf16_of_int(known ? 1 : 0);
       }
-#pragma unroll
-      for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+      sq = __reduce_add_sync(0xffffffffu, sq);
       if (lane == 0) tl.a2row[dy] = sq;
     }
     __syncthreads();
@@ -772,9 +781,9 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
   using G = EngGeom<R, SRW>;
   using RG = ResGeom<R>;
   constexpr int P = G::P, B = G::B;
-  uint8_t* smem = x.smem;
+  uint8_t* const smem = eng_smem();
   EngSmemTail& tl = *reinterpret_cast<EngSmemTail*>(smem);
-  uint32_t* tgt = reinterpret_cast<uint32_t*>(smem + ((sizeof(EngSmemTail) + 15) & ~size_t(15)));
+  uint32_t* tgt = reinterpret_cast<uint32_t*>(smem + kTgtOff);
   uint32_t* rowd = tgt + P * G::TP;  // row descriptors of the target
   uint8_t* upd_base = smem + kHeadBytes;
   UpdSmem<R>& usm = *reinterpret_cast<UpdSmem<R>*>(upd_base);
@@ -820,7 +829,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
   if (s.planes && ea.tc_cols >= 2 * tt.N && tsize >= 2 && tc_ntiles > 0) {
     const int nsq = min(tsize - 1, tc_ntiles);
     const int ntl = (tc_ntiles + nsq - 1) / nsq;
-    const long long avail = (long long)(x.smem_end - (smem + kHeadBytes));
+    const long long avail = (long long)x.smem_bytes - (long long)kHeadBytes;
     const int slot = tc_slot(tt.N, R);
     const long long fixed =
         TcEngGeom<R>::A_BYTES + TcEngGeom<R>::TPAD_BYTES + (long long)ntl * tc_bit_words(tt.N) * 4;
@@ -869,7 +878,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     const long long U = (long long)ncu * nbands;
     const long long m = ns > 0 ? (U + ns - 1) / ns : 0;  // most units of one CTA
     const long long avail =
-        (long long)(x.smem_end - (smem + kHeadBytes)) -
+        (long long)x.smem_bytes - (long long)kHeadBytes -
         (lead_searches ? ((long long)(upd_smem_bytes<R>() + 127) / 128) * 128 : 0);
     // two tiles (a range may straddle a band boundary) plus the bits; more
     // than one band of units per CTA streams instead
@@ -914,8 +923,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     };
     const bool first = round == 0;
     if (!resident && tid == 0 && b0 < nbatch) issue(b0, slot_pix(0), cnt_t[0], &tl.bars.full[0]);
-    const uint8_t* tiles = area;
-    if (resident && first) {
+        if (resident && first) {
       // the source windows of every band segment (plain 16-byte loads;
       // outside the image: zero), then the validity bits of every unit
       for (int g = 0; g < pl.nseg; ++g) {
@@ -1003,7 +1011,8 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     unsigned long long best = ~0ull;
     bool ok = true;
     if (resident) {
-      if (pl.u1 > pl.u0) best = resident_units16<R>(&pl, tiles, xb, s.cy0, s.W, tgt, rowd);
+      if (pl.u1 > pl.u0)
+        best = resident_units16<R>((int)offsetof(EngSmemTail, plan), (int)(area - smem), xb, s.cy0, s.W, kTgtOff);
     } else {
       int cur = 0;
       for (int b = b0; b < nbatch; b += ns) {
@@ -1023,8 +1032,9 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
           const int qx = qx0 + k;
           if (qx >= s.cx0 && qx <= s.cx1 && qy <= s.cy1 && cw[G::COFF + k] == 0) bits |= 1u << k;
         }
-        const unsigned long long kb = unit_best<R, SRW>(slot_pix(cur) + lane * G::BW + G::NCL * warp, tgt, rowd,
-                                                        bits, (unsigned)(qy * s.W + qx0));
+        const unsigned long long kb = unit_best<R, SRW>(
+            (int)(slots - smem) + cur * G::SLOT_BYTES + 4 * (lane * G::BW + G::NCL * warp), kTgtOff, bits,
+            (unsigned)(qy * s.W + qx0));
         best = kb < best ? kb : best;
         if (__syncthreads_or(!got)) {  // a bounded wait gave up: stop uniformly
           ok = false;

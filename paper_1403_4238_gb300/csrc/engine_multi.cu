@@ -33,10 +33,7 @@ __device__ inline void run_by_radius(const EngineArgs& ea, int j, EngCtx& x) {
 __global__ void __launch_bounds__(kEngThreads, 1) k_engine(EngineArgs ea) {
   extern __shared__ __align__(128) uint8_t smem_raw[];
   EngCtx x;
-  x.smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
-  uint32_t dyn;
-  asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
-  x.smem_end = smem_raw + dyn;
+  asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(x.smem_bytes));
   const int team = ea.cta_team[blockIdx.x];
   const int first = ea.team_first[team];
   x.rank = blockIdx.x - first;
@@ -44,7 +41,7 @@ __global__ void __launch_bounds__(kEngThreads, 1) k_engine(EngineArgs ea) {
   x.tc = &ea.teams[team];
   x.tpart = ea.partials + first;
   // the barriers sit at the start of shared memory
-  EngBars* bars = reinterpret_cast<EngBars*>(x.smem);
+  EngBars* bars = reinterpret_cast<EngBars*>(smem_raw);
   if (threadIdx.x == 0) {
     mbar_init(&bars->full[0], 1);
     mbar_init(&bars->full[1], 1);

@@ -111,8 +111,7 @@ struct EngBars {
 
 // Per-CTA engine state carried from one image of a team's list to the next.
 struct EngCtx {
-  uint8_t* smem;                // dynamic shared memory, 128-byte aligned
-  uint8_t* smem_end;            // end of the dynamic shared memory
+  uint32_t smem_bytes;          // dynamic shared memory of the CTA
   int rank, tsize;              // this CTA's rank in its team, team size
   TeamCtl* tc;
   unsigned long long* tpart;    // partial keys of the team's CTAs

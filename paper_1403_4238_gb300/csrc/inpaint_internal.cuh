@@ -219,26 +219,31 @@ __device__ __forceinline__ void prio_take(unsigned long long& k, int& i, unsigne
   i = b ? ii : i;
 }
 
+// Warp reductions by redux.sync on 32-bit halves (high halves first, then the
+// low halves of the lanes that tie, then their indices): a 64-bit butterfly of
+// (key, index) pairs is 15 shuffles and about 60 instructions, this is three
+// reductions, and the leader's loop is bound by instruction fetch as much as
+// by latency.  All 32 lanes.
 __device__ inline unsigned long long warp_min_u64(unsigned long long v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long t = __shfl_xor_sync(0xffffffffu, v, o);
-    v = t < v ? t : v;
-  }
-  return v;
+  const unsigned hi = (unsigned)(v >> 32), lo = (unsigned)v;
+  const unsigned mh = __reduce_min_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_min_sync(0xffffffffu, hi == mh ? lo : 0xffffffffu);
+  return ((unsigned long long)mh << 32) | ml;
 }
 
+// (indices are never negative)
 __device__ inline void warp_best_prio(unsigned long long& k, int& i) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    unsigned long long tk = __shfl_xor_sync(0xffffffffu, k, o);
-    int ti = __shfl_xor_sync(0xffffffffu, i, o);
-    prio_take(k, i, tk, ti);
-  }
+  const unsigned hi = (unsigned)(k >> 32), lo = (unsigned)k;
+  const unsigned mh = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, hi == mh ? lo : 0u);
+  i = (int)__reduce_min_sync(0xffffffffu, hi == mh && lo == ml ? (unsigned)i : 0x7fffffffu);
+  k = ((unsigned long long)mh << 32) | ml;
 }
 
-// Block-wide best (key, idx); every thread gets the result.  scratch holds
-// one entry per warp; blockDim.x must be a multiple of 32.
+// Block reductions: one value per warp in scratch, then every warp reduces
+// those itself (no lone warp between two barriers).  The leading barrier
+// keeps the previous call's readers ahead of this call's writers; scratch
+// holds one entry per warp; blockDim.x must be a multiple of 32.
 __device__ inline void block_best_prio(unsigned long long& k, int& i, PrioBest* scratch) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   warp_best_prio(k, i);
@@ -248,23 +253,11 @@ __device__ inline void block_best_prio(unsigned long long& k, int& i, PrioBest* 
     scratch[wid].idx = i;
   }
   __syncthreads();
-  if (wid == 0) {
-    unsigned long long kk = lane < nw ? scratch[lane].key : 0ull;
-    int ii = lane < nw ? scratch[lane].idx : 0x7fffffff;
-    warp_best_prio(kk, ii);
-    if (lane == 0) {
-      scratch[0].key = kk;
-      scratch[0].idx = ii;
-    }
-  }
-  __syncthreads();
-  k = scratch[0].key;
-  i = scratch[0].idx;
+  k = lane < nw ? scratch[lane].key : 0ull;
+  i = lane < nw ? scratch[lane].idx : 0x7fffffff;
+  warp_best_prio(k, i);
 }
 
-// Block reductions: one value per warp in scratch, then every warp reduces
-// those itself (no lone warp between two barriers).  The leading barrier
-// keeps the previous call's readers ahead of this call's writers.
 __device__ inline unsigned long long block_min_u64(unsigned long long v, unsigned long long* scratch) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   v = warp_min_u64(v);
@@ -276,15 +269,11 @@ __device__ inline unsigned long long block_min_u64(unsigned long long v, unsigne
 
 __device__ inline int block_sum_int(int v, int* scratch) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  v = __reduce_add_sync(0xffffffffu, v);
   __syncthreads();
   if (lane == 0) scratch[wid] = v;
   __syncthreads();
-  int t = lane < nw ? scratch[lane] : 0;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  return t;
+  return __reduce_add_sync(0xffffffffu, lane < nw ? scratch[lane] : 0);
 }
 
 // ---- priority tiles: two-level argmax structure over the prio keys ----
@@ -349,6 +338,7 @@ __device__ inline void warp_global_best(const ImgState& s, unsigned long long& k
   k = 0ull;
   idx = 0x7fffffff;
   const int n = s.t1x * s.t1y;
+#pragma unroll 1
   for (int j = lane; j < n; j += 32) {
     const unsigned long long bk = __ldcg(&s.tiles1[j].key);
     const int bi = __ldcg(&s.tiles1[j].idx);

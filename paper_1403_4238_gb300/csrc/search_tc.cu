@@ -97,8 +97,7 @@ __global__ void __launch_bounds__(kEngThreads, 1) k_search_tc(ImgState s, int nb
       tp[2 * P * GT::TW] = (uint16_t)bf16_of_int(d2);
       tp[3 * P * GT::TW] = (uint16_t)bf16_of_int(known ? 1 : 0);
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    sq = __reduce_add_sync(0xffffffffu, sq);
     if (lane == 0) h.a2row[dy] = sq;
   }
   __syncthreads();

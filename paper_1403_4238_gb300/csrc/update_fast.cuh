@@ -229,6 +229,7 @@ __device__ inline void stage_nbhd(const ImgState& s, int cx, int cy, UpdSmem<R>&
   constexpr int RB = G::RB, NS = G::NS;
   constexpr int U = 4;  // entries per thread with their loads in flight together
   const int step = blockDim.x;
+#pragma unroll 1
   for (int i0 = threadIdx.x; i0 < NS * NS; i0 += U * step) {
     uint8_t o[U], g[U];
     double cf[U];
@@ -282,6 +283,7 @@ __device__ inline void isophote_at(UpdSmem<R>& sm, int lx, int ly) {
 template <int R>
 __device__ inline void stage_isophotes(UpdSmem<R>& sm) {
   constexpr int NS = UpdGeom<R>::NS;
+#pragma unroll 1
   for (int i = threadIdx.x; i < NS * NS; i += blockDim.x) isophote_at<R>(sm, i % NS, i / NS);
 }
 
@@ -297,6 +299,7 @@ __device__ inline void stage_isophotes_part(UpdSmem<R>& sm, int first, int last 
   constexpr int n = kRing ? NB * NB : NS * NS;
   if (last < 0) last = (int)blockDim.x;
   if ((int)threadIdx.x < first || (int)threadIdx.x >= last) return;
+#pragma unroll 1
   for (int k = (int)threadIdx.x - first; k < n; k += last - first) {
     if (kRing) {
       isophote_at<R>(sm, RB - RR + k % NB, RB - RR + k / NB);
@@ -346,6 +349,7 @@ __global__ void __launch_bounds__(256, 2) k_prio_init_fast(ImgState s) {
   __syncthreads();
   stage_isophotes<R>(sm);
   __syncthreads();
+#pragma unroll 1
   for (int i = threadIdx.x; i < NW * NW; i += blockDim.x) {
     const int wx = i % NW - R2, wy = i / NW - R2;
     const int lx = RB + wx, ly = RB + wy, l = ly * NS + lx;
@@ -383,6 +387,7 @@ __device__ void update_prefetch(const ImgState& s, UpdCache<R>& ca, int first, i
   if ((int)threadIdx.x < first) return;
   // every load is an asynchronous copy into the cache, all in flight at once
   const int step = (int)blockDim.x - first, t0 = (int)threadIdx.x - first;
+#pragma unroll 1
   for (int j = t0; j < NC * NC; j += step) {
     const int x = px + j % NC - 2 * R, y = py + j / NC - 2 * R;
     const bool ok = x >= 0 && x < W && y >= 0 && y < H;
@@ -390,6 +395,7 @@ __device__ void update_prefetch(const ImgState& s, UpdCache<R>& ca, int first, i
   }
   {
     const int n = ntx * nty * kT0 * kT0;
+#pragma unroll 1
     for (int e = t0; e < n; e += step) {
       const int t = e / (kT0 * kT0), j = e % (kT0 * kT0);
       const int x = (tx0 + t % ntx) * kT0 + (j & (kT0 - 1)), y = (ty0 + t / ntx) * kT0 + j / kT0;
@@ -399,6 +405,7 @@ __device__ void update_prefetch(const ImgState& s, UpdCache<R>& ca, int first, i
   }
   {
     const int n = nux * nuy * kT1 * kT1;
+#pragma unroll 1
     for (int e = t0; e < n; e += step) {
       const int u = e / (kT1 * kT1), j = e % (kT1 * kT1);
       const int tx = (ux0 + u % nux) * kT1 + (j & (kT1 - 1)), ty = (uy0 + u / nux) * kT1 + j / kT1;
@@ -412,6 +419,7 @@ __device__ void update_prefetch(const ImgState& s, UpdCache<R>& ca, int first, i
     }
   }
   if (n1 <= kT1Cache)
+#pragma unroll 1
     for (int e = t0; e < n1; e += step) cp_async16(&ca.t1c[e], &s.tiles1[e]);
   cp_async_wait_all();
   if ((int)threadIdx.x == first) {
@@ -433,20 +441,25 @@ template <int R>
 __device__ inline void warp_fsat(UpdSmem<R>& sm) {
   constexpr int P = UpdGeom<R>::P, P1 = P + 1;
   const int lane = threadIdx.x & 31;
+#pragma unroll 1
   for (int v = lane; v <= P; v += 32) {
     sm.fsat[v] = 0;
     sm.fsat[v * P1] = 0;
   }
   __syncwarp();
+#pragma unroll 1
   for (int v = lane; v < P; v += 32) {
     int run = 0;
+#pragma unroll 1
     for (int u = 0; u < P; ++u) {
       run += sm.filled[v * P + u];
       sm.fsat[(v + 1) * P1 + u + 1] = run;
     }
   }
   __syncwarp();
+#pragma unroll 1
   for (int u = lane + 1; u <= P; u += 32)
+#pragma unroll 1
     for (int v = 2; v <= P; ++v) sm.fsat[v * P1 + u] += sm.fsat[(v - 1) * P1 + u];
 }
 
@@ -483,45 +496,10 @@ __device__ void stage_next(const ImgState& s, int npx, int npy, UpdSmem<R>& sm, 
 // does not touch, level-0 tiles it does not touch inside the level-1 tiles
 // it does, and the pixels outside it inside the level-0 tiles it touches.
 // Those priorities are the ones the fill of this iteration leaves alone.
-// Whole block.
-template <int R>
-__device__ void best_outside_window(const ImgState& s, UpdSmem<R>& sm, const UpdCache<R>& ca, int px,
-                                    int py) {
-  constexpr int R2 = UpdGeom<R>::R2;
-  const int W = s.W;
-  unsigned long long k = 0ull;
-  int idx = 0x7fffffff;
-  const int n1 = s.t1x * s.t1y;
-  for (int e = threadIdx.x; e < n1; e += blockDim.x) {
-    const int ux = e % s.t1x, uy = e / s.t1x;
-    if (ux >= ca.ux0 && ux < ca.ux0 + ca.nux && uy >= ca.uy0 && uy < ca.uy0 + ca.nuy) continue;
-    if (ca.t1n) prio_take(k, idx, ca.t1c[e].key, ca.t1c[e].idx);
-    else prio_take(k, idx, __ldcg(&s.tiles1[e].key), __ldcg(&s.tiles1[e].idx));
-  }
-  for (int e = threadIdx.x; e < ca.nux * ca.nuy * kT1 * kT1; e += blockDim.x) {
-    const int u = e / (kT1 * kT1), j = e % (kT1 * kT1);
-    const int tx = (ca.ux0 + u % ca.nux) * kT1 + (j & (kT1 - 1)), ty = (ca.uy0 + u / ca.nux) * kT1 + j / kT1;
-    if (tx >= ca.tx0 && tx < ca.tx0 + ca.ntx && ty >= ca.ty0 && ty < ca.ty0 + ca.nty) continue;
-    prio_take(k, idx, ca.t0c[e].key, ca.t0c[e].idx);
-  }
-  for (int e = threadIdx.x; e < ca.ntx * ca.nty * kT0 * kT0; e += blockDim.x) {
-    const int t = e / (kT0 * kT0), j = e % (kT0 * kT0);
-    const int x = (ca.tx0 + t % ca.ntx) * kT0 + (j & (kT0 - 1)), y = (ca.ty0 + t / ca.ntx) * kT0 + j / kT0;
-    if (x >= W || y >= s.H || (abs(x - px) <= R2 && abs(y - py) <= R2)) continue;
-    prio_take(k, idx, ca.tp[e], y * W + x);
-  }
-  block_best_prio(k, idx, sm.red_pb);  // ends with a __syncthreads
-  if (threadIdx.x == 0) {
-    sm.out_key = k;
-    sm.out_idx = idx;
-  }
-}
-
-// best_outside_window for the threads [g0, blockDim.x) only (g0 a multiple
-// of 32, the group synchronised by named barrier 1): the speculative
-// phase's spare warps run it while the other warps' FP64 chains go on.
-// Writes sm.out_key / sm.out_idx; a block barrier must follow before they
-// are read.
+// Threads [g0, blockDim.x) (g0 a multiple of 32; the group is synchronised
+// by named barrier 1): the speculative phase's spare warps run it while the
+// other warps' FP64 chains go on.  Writes sm.out_key / sm.out_idx; a block
+// barrier must follow before they are read.
 template <int R>
 __device__ void best_outside_window_group(const ImgState& s, UpdSmem<R>& sm, const UpdCache<R>& ca, int px,
                                           int py, int g0) {
@@ -533,18 +511,21 @@ __device__ void best_outside_window_group(const ImgState& s, UpdSmem<R>& sm, con
   unsigned long long k = 0ull;
   int idx = 0x7fffffff;
   const int n1 = s.t1x * s.t1y;
+#pragma unroll 1
   for (int e = t0; e < n1; e += nt) {
     const int ux = e % s.t1x, uy = e / s.t1x;
     if (ux >= ca.ux0 && ux < ca.ux0 + ca.nux && uy >= ca.uy0 && uy < ca.uy0 + ca.nuy) continue;
     if (ca.t1n) prio_take(k, idx, ca.t1c[e].key, ca.t1c[e].idx);
     else prio_take(k, idx, __ldcg(&s.tiles1[e].key), __ldcg(&s.tiles1[e].idx));
   }
+#pragma unroll 1
   for (int e = t0; e < ca.nux * ca.nuy * kT1 * kT1; e += nt) {
     const int u = e / (kT1 * kT1), j = e % (kT1 * kT1);
     const int tx = (ca.ux0 + u % ca.nux) * kT1 + (j & (kT1 - 1)), ty = (ca.uy0 + u / ca.nux) * kT1 + j / kT1;
     if (tx >= ca.tx0 && tx < ca.tx0 + ca.ntx && ty >= ca.ty0 && ty < ca.ty0 + ca.nty) continue;
     prio_take(k, idx, ca.t0c[e].key, ca.t0c[e].idx);
   }
+#pragma unroll 1
   for (int e = t0; e < ca.ntx * ca.nty * kT0 * kT0; e += nt) {
     const int t = e / (kT0 * kT0), j = e % (kT0 * kT0);
     const int x = (ca.tx0 + t % ca.ntx) * kT0 + (j & (kT0 - 1)), y = (ca.ty0 + t / ca.ntx) * kT0 + j / kT0;
@@ -592,6 +573,7 @@ __device__ void update_tiles(const ImgState& s, UpdSmem<R>& sm, UpdCache<R>& ca,
       asm volatile("bar.sync 2, %0;" ::"r"(nt) : "memory");
   };
   const int lane = t0 & 31, wid = t0 >> 5, nw = nt >> 5;
+#pragma unroll 1
   for (int t = wid; t < ca.ntx * ca.nty; t += nw) {
     const int tx = ca.tx0 + t % ca.ntx, ty = ca.ty0 + t / ca.ntx;
     unsigned long long k = 0ull;
@@ -613,6 +595,7 @@ __device__ void update_tiles(const ImgState& s, UpdSmem<R>& sm, UpdCache<R>& ca,
     }
   }
   gsync();
+#pragma unroll 1
   for (int u = wid; u < ca.nux * ca.nuy; u += nw) {
     const int ux = ca.ux0 + u % ca.nux, uy = ca.uy0 + u / ca.nux;
     unsigned long long k = 0ull;
@@ -637,6 +620,7 @@ __device__ void update_tiles(const ImgState& s, UpdSmem<R>& sm, UpdCache<R>& ca,
     unsigned long long k = 0ull;
     int idx = 0x7fffffff;
     if (ca.t1n) {
+#pragma unroll 1
       for (int j = lane; j < ca.t1n; j += 32) prio_take(k, idx, ca.t1c[j].key, ca.t1c[j].idx);
       warp_best_prio(k, idx);
     } else {
@@ -675,6 +659,7 @@ __device__ void spec_phase(const ImgState& s, UpdSmem<R>& sm, UpdCache<R>& ca, b
     sm.iso_next = 0;
   }
   int my = 0;
+#pragma unroll 1
   for (int i = threadIdx.x; i < P * P; i += blockDim.x) {
     const int l = (RB + i / P - R) * NS + RB + i % P - R;
     uint8_t f = 0;
@@ -688,6 +673,7 @@ __device__ void spec_phase(const ImgState& s, UpdSmem<R>& sm, UpdCache<R>& ca, b
   }
   const int filled = block_sum_int(my, sm.red32);  // includes __syncthreads
   // post-fill front of the window, compacted
+#pragma unroll 1
   for (int i = threadIdx.x; i < NW * NW; i += blockDim.x) {
     const int l = (RB + i / NW - R2) * NS + RB + i % NW - R2;
     int nrm = kSpecOutside;
@@ -704,46 +690,31 @@ __device__ void spec_phase(const ImgState& s, UpdSmem<R>& sm, UpdCache<R>& ca, b
   // cannot change; the other warps (the spare group) bring the tiles up to
   // date, load the update phase's cache and find the best priority outside
   // the fill's window
-  const int nt = (int)blockDim.x;
-  const bool spare = nt >= 256;
-  if (spare) {
-    constexpr int g0 = 160;
-    // one dependent row-major chain per front pixel, packed into as few
-    // warps as the front needs: up to three warps of chains still run at the
-    // 64 cycles of one dependent add, four at 76 (the unit takes a warp
-    // instruction about every 19 cycles whatever the active lanes)
-    const int cw = nfront <= 96 ? (nfront + 31) >> 5 : 4;
-    if ((int)threadIdx.x < 32 * cw) {
-      for (int k = threadIdx.x; k < nfront; k += 32 * cw) {
-        const int i = sm.list[k];
-        const int wx = i % NW - R2, wy = i / NW - R2;
-        const int lx = RB + wx, ly = RB + wy, x = px + wx, y = py + wy;
-        sm.sC[i] = conf_local<R>(sm, s, lx, ly, x, y);
-        sm.snrm[i] = normal_local<R>(sm, s, lx, ly, x, y);
-      }
-    } else if ((int)(threadIdx.x >> 5) == 4) {
-      warp_fsat<R>(sm);
-    }
-    if ((int)threadIdx.x >= g0) {
-      if (want_outside && sm.tiles_pending) update_tiles<R>(s, sm, ca, g0);
-      update_prefetch<R>(s, ca, g0, px, py);
-      if (want_outside) best_outside_window_group<R>(s, sm, ca, px, py, g0);
-    } else {
-      // the warps without chains at once, the chain warps when done
-      stage_isophotes_dyn<R>(sm);
-    }
-  } else {
-    for (int k = threadIdx.x; k < nfront; k += nt) {
+  constexpr int g0 = 160;
+  // one dependent row-major chain per front pixel, packed into as few
+  // warps as the front needs: up to three warps of chains still run at the
+  // 64 cycles of one dependent add, four at 76 (the unit takes a warp
+  // instruction about every 19 cycles whatever the active lanes)
+  const int cw = nfront <= 96 ? (nfront + 31) >> 5 : 4;
+  if ((int)threadIdx.x < 32 * cw) {
+#pragma unroll 1
+    for (int k = threadIdx.x; k < nfront; k += 32 * cw) {
       const int i = sm.list[k];
       const int wx = i % NW - R2, wy = i / NW - R2;
       const int lx = RB + wx, ly = RB + wy, x = px + wx, y = py + wy;
       sm.sC[i] = conf_local<R>(sm, s, lx, ly, x, y);
       sm.snrm[i] = normal_local<R>(sm, s, lx, ly, x, y);
     }
-    if (threadIdx.x < 32) warp_fsat<R>(sm);
-    if (want_outside && sm.tiles_pending) update_tiles<R>(s, sm, ca, 0);
-    update_prefetch<R>(s, ca, 0, px, py);
-    stage_isophotes_part<R, false>(sm, 0);
+  } else if ((int)(threadIdx.x >> 5) == 4) {
+    warp_fsat<R>(sm);
+  }
+  if ((int)threadIdx.x >= g0) {
+    if (want_outside && sm.tiles_pending) update_tiles<R>(s, sm, ca, g0);
+    update_prefetch<R>(s, ca, g0, px, py);
+    if (want_outside) best_outside_window_group<R>(s, sm, ca, px, py, g0);
+  } else {
+    // the warps without chains at once, the chain warps when done
+    stage_isophotes_dyn<R>(sm);
   }
   if (threadIdx.x == 0) {
     sm.nfront = nfront;
@@ -751,10 +722,6 @@ __device__ void spec_phase(const ImgState& s, UpdSmem<R>& sm, UpdCache<R>& ca, b
     sm.spec_filled = filled;
   }
   __syncthreads();
-  if (want_outside && !spare) {
-    best_outside_window<R>(s, sm, ca, px, py);
-    __syncthreads();
-  }
 }
 
 // Early selection (persistent engine, resident mode): the next target is
@@ -802,6 +769,7 @@ __device__ bool update_phase(const ImgState& s, const unsigned long long* partia
   if (best_in) {
     best = *best_in;
   } else {
+#pragma unroll 1
     for (int i = tid; i < n_partial; i += nt) {
       const unsigned long long v = __ldcg(&partial[i]);
       best = v < best ? v : best;
@@ -861,6 +829,7 @@ __device__ bool update_phase(const ImgState& s, const unsigned long long* partia
     const int px = sm.px, py = sm.py, qx = sm.qx, qy = sm.qy, W = s.W, H = s.H;
     const double cp = sm.cp;
     int newly = 0;
+#pragma unroll 1
     for (int t = tid; t < P * P + NC * NC + NW * NW; t += nt) {
       if (t < P * P) {
         const int i = t;
@@ -932,6 +901,7 @@ __device__ bool update_phase(const ImgState& s, const unsigned long long* partia
   static_assert(sizeof(sm.cf) >= sizeof(uint32_t) * HR * NW, "key scratch");
   static_assert(NS * NS <= 4096, "local index fits in 12 bits");
   const int nhk = nt >= 512 ? nt - 32 : nt;  // the last warp (the fence thread's) sits out
+#pragma unroll 1
   for (int i = tid; i < HR * NW && tid < nhk; i += nhk) {
     const int ly = RB - R2 - R + i / NW, lx = RB - R2 + i % NW;
     uint32_t best = 0u;
@@ -953,6 +923,7 @@ __device__ bool update_phase(const ImgState& s, const unsigned long long* partia
   {
     const int px = sm.px, py = sm.py, W = s.W, nfront = sm.nfront;
     const int nlist = (nfront + 127) & ~127;
+#pragma unroll 1
     for (int t = tid; t < nlist; t += nt) {
       const int k = list_entry(t);
       if (k >= nfront) continue;
@@ -1023,6 +994,7 @@ __device__ bool update_phase(const ImgState& s, const unsigned long long* partia
 
   // level-0 tiles from the cached keys, then level-1, then the best
   const int lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
+#pragma unroll 1
   for (int t = wid; t < ca.ntx * ca.nty; t += nw) {
     const int tx = ca.tx0 + t % ca.ntx, ty = ca.ty0 + t / ca.ntx;
     unsigned long long k = 0ull;
@@ -1046,6 +1018,7 @@ __device__ bool update_phase(const ImgState& s, const unsigned long long* partia
     }
   }
   __syncthreads();
+#pragma unroll 1
   for (int u = wid; u < ca.nux * ca.nuy; u += nw) {
     const int ux = ca.ux0 + u % ca.nux, uy = ca.uy0 + u / ca.nux;
     unsigned long long k = 0ull;
@@ -1073,6 +1046,7 @@ __device__ bool update_phase(const ImgState& s, const unsigned long long* partia
     int idx = 0x7fffffff;
     if (sm.remaining > 0) {
       if (ca.t1n) {
+#pragma unroll 1
         for (int j = lane; j < ca.t1n; j += 32) prio_take(k, idx, ca.t1c[j].key, ca.t1c[j].idx);
         warp_best_prio(k, idx);
       } else {
