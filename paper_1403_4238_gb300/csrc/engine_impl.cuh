@@ -381,16 +381,11 @@ struct EngSmemTail {
   ImgState img;      // the image's state block (a leader that does not search reads it here)
   unsigned long long red64[32];
   int red32[32];
-  unsigned long long key;  // best key of the round (leader)
-  int flag;
-  int allow;  // leader: no iteration limit, status or error stops the loop after this iteration
   int stop;
   int px, py;
   int a2row[17];  // tensor-core search: per target row, sum of the known pixels' squared shifted values
   int tc_pref;  // tensor-core search: slots the producer prefetched for the next round
-  CtrlSnap snap;  // leader: the control fields its update reads (kept by the leader itself)
   int lim, status, err;  // leader: iteration limit, status and error word (the stop decision)
-  EarlySel es;           // leader: the early selection's inputs and outcome
   uint8_t known[2][17 * 17];  // known flags of the last two targets (by round parity)
   ResPlan plan;               // resident mode: this CTA's units and tiles
 };
@@ -410,7 +405,7 @@ constexpr size_t kHeadBytes = ((kTgtOff + kTgtWords * 4 + 127) / 128) * 128;
 // takes as many slots as fit.
 template <int R>
 __host__ __device__ constexpr size_t upd_smem_bytes() {
-  return ((sizeof(UpdSmem<R>) + 127) / 128) * 128 + sizeof(UpdCache<R>);
+  return ((sizeof(UpdSmem<R>) + 127) / 128) * 128;
 }
 
 // The least shared memory an engine CTA needs: a searching leader with two
@@ -424,11 +419,6 @@ __host__ __device__ constexpr size_t eng_smem_bytes() {
 
 static_assert(eng_smem_bytes<8, 2>() <= 227 * 1024, "engine CTA must fit in shared memory");
 static_assert(eng_smem_bytes<7, 2>() <= 227 * 1024, "engine CTA must fit in shared memory");
-
-template <int R>
-__device__ inline UpdCache<R>& upd_cache_of(uint8_t* upd_base) {
-  return *reinterpret_cast<UpdCache<R>*>(upd_base + ((sizeof(UpdSmem<R>) + 127) / 128) * 128);
-}
 
 // Team publication word: epoch (bits 0-31), next target px (32-46), py
 // (47-61), stop flag (62).  One acquire load gives a waiting CTA everything
@@ -458,12 +448,10 @@ __device__ inline unsigned long long ld_relaxed64(const unsigned long long* p) {
   return v;
 }
 
-// The leader's publishing thread: the last one.  It is the update phase's
-// fence thread: its warp has no isophote or row-maximum work there, so the
-// fence it issues after the copy waits off the path, and the same fence
-// makes its later publication of the next round a release.
+// The leader's publishing thread: the last one, which is also update_work's
+// fence thread, so the fence it issues after the copy makes its later
+// publication of the next round a release.
 constexpr int kPubThread = kEngThreads - 1;
-
 
 // Bounded wait (thread 0) for a publication with an epoch other than `epoch`;
 // returns it, or a stop word after setting *err on timeout.
@@ -499,59 +487,47 @@ __device__ inline unsigned long long key_untag(unsigned long long t) {
   return (ssd << 32) | idx;
 }
 
-// Leader: the best key of the round over the tagged slots [0, n), each
-// polled (bounded) by one thread until it carries the round's tag; the
-// untagged minimum lands in *out.  Returns false (every thread) when a
-// slot did not arrive in time.  Whole block; ends with a __syncthreads.
-__device__ inline bool gather_keys(const unsigned long long* slots, int n, unsigned epoch, int* err,
-                                   unsigned long long limit, unsigned long long* red,
-                                   unsigned long long* out) {
-  // a key is a message of its own (the leader reads nothing else the
-  // searchers write), so relaxed loads suffice; warp 0 polls up to eight
-  // slots per lane at a time and reduces them, the other warps wait at the
-  // one barrier
-  if (threadIdx.x < 32) {
-    constexpr int U = 8;
-    const int lane = threadIdx.x;
-    const unsigned tag = epoch & 0x7fu;
-    unsigned long long best = ~0ull;
-    bool late = false;
-    const unsigned long long t0 = globaltimer();
-    for (int b = 0; b < n && !late; b += 32 * U) {
-      unsigned pending = 0u;
+// The best key of the round over the tagged slots [0, n) (one warp), each
+// polled, bounded, until it carries the round's tag; *late when one did not
+// arrive in time.  A key is a message of its own (the leader reads nothing
+// else the searchers write), so relaxed loads suffice; a lane polls up to
+// five slots at a time (160 slots: every CTA of the chip in one pass).
+__device__ inline unsigned long long gather_keys(const unsigned long long* slots, int n, unsigned epoch, int* err,
+                                                 unsigned long long limit, bool* late_out) {
+  constexpr int U = 5;
+  const int lane = threadIdx.x & 31;
+  const unsigned tag = epoch & 0x7fu;
+  unsigned long long best = ~0ull;
+  bool late = false;
+  const unsigned long long t0 = globaltimer();
+#pragma unroll 1
+  for (int b = 0; b < n && !late; b += 32 * U) {
+    unsigned pending = 0u;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (b + lane + 32 * u < n) pending |= 1u << u;
+#pragma unroll 1
+    while (pending) {
+      unsigned long long v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) v[u] = (pending >> u) & 1u ? ld_relaxed64(&slots[b + lane + 32 * u]) : 0ull;
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (b + lane + 32 * u < n) pending |= 1u << u;
-      while (pending) {
-        unsigned long long v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) v[u] = (pending >> u) & 1u ? ld_relaxed64(&slots[b + lane + 32 * u]) : 0ull;
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (((pending >> u) & 1u) && (v[u] & 0xffu) == tag) {
-            const unsigned long long k = key_untag(v[u]);
-            best = k < best ? k : best;
-            pending &= ~(1u << u);
-          }
-        if (pending && globaltimer() - t0 > limit) {
-          late = true;
-          break;
+        if (((pending >> u) & 1u) && (v[u] & 0xffu) == tag) {
+          best = v[u] < best ? v[u] : best;  // one tag: tagged values order like their keys
+          pending &= ~(1u << u);
         }
+      if (pending && globaltimer() - t0 > limit) {
+        late = true;
+        break;
       }
     }
-    best = warp_min_u64(best);
-    late = __any_sync(0xffffffffu, late);
-    if (lane == 0) {
-      red[0] = late ? 1ull : 0ull;
-      *out = best;
-    }
   }
-  __syncthreads();
-  if (red[0] != 0ull) {
-    if (threadIdx.x == 0) atomicExch(err, INPAINT_ERR_TIMEOUT);
-    return false;
-  }
-  return true;
+  late = __any_sync(0xffffffffu, late);
+  best = warp_min_u64(best);
+  if (late && lane == 0) atomicExch(err, INPAINT_ERR_TIMEOUT);
+  *late_out = late;
+  return best == ~0ull ? best : key_untag(best);
 }
 
 __device__ inline bool ctrl_active(const Ctrl* c) {
@@ -787,11 +763,10 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
   uint32_t* rowd = tgt + P * G::TP;  // row descriptors of the target
   uint8_t* upd_base = smem + kHeadBytes;
   UpdSmem<R>& usm = *reinterpret_cast<UpdSmem<R>*>(upd_base);
-  UpdCache<R>& uca = upd_cache_of<R>(upd_base);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = x.rank, tsize = x.tsize;
-  TeamCtl* tc = x.tc;
-  unsigned long long* tpart = x.tpart;
+  TeamCtl* const tc = x.tc;
+  unsigned long long* const tpart = x.tpart;
   const unsigned long long t_start = x.t_start;  // (the context is in local memory)
   const unsigned long long limit = ea.wait_limit_ns;
   uint32_t ph0 = x.ph0, ph1 = x.ph1;
@@ -888,9 +863,6 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     // mode spread the search over more warps
     resident = !tcmode && m >= kEngWarps / 2 && m <= ncu && need <= avail;
   }
-  // large images: the leader publishes the next target as soon as the
-  // window's priorities are known and updates its tile maxima afterwards
-  const bool early_sel = (resident || tcmode) && !lead_searches;
   ResPlan& pl = tl.plan;
   if (resident && searcher) {
     if (tid == 0) res_plan<R>(pl, ncu, nbands, rank, ns);
@@ -904,7 +876,6 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
   __syncthreads();
   int prev_px = -1000000, prev_py = -1000000;
   int round = 0;        // search rounds of this image in this launch
-  bool staged = false;  // leader: neighbourhood of the next p^ already in shared memory
 
   // One search round for target (px, py): this CTA's batches; returns its
   // best key.  Whole block.
@@ -1052,90 +1023,73 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     return block_min_u64(best, tl.red64);
   };
 
-  // One iteration of the leader for target (px, py): speculative phase (and
-  // its own search share when it searches), the searchers' keys, update,
-  // publication of the next round, bookkeeping.  Whole block.
-  auto lead_round = [&](int px, int py, bool searches) {
-    const unsigned long long t_a = globaltimer();
-    spec_phase<R>(s, usm, uca, staged, early_sel);
-    if (tid == 32) {
-      // the stop decision's inputs that other CTAs may change, read by a
-      // thread outside the warp that gathers the keys; everything the update
-      // reads stays in shared memory (no local-memory state: it would miss
-      // L1, which the shared memory leaves nearly empty)
-      tl.status = __ldcg(&c->status);
-      tl.err = __ldcg(ea.err);
-      tl.allow = usm.spec_iter + 1 < tl.lim && tl.status == 0 && tl.err == 0;
-      tl.es.pub = early_sel ? &tc->pub : nullptr;
-      tl.es.epoch = epoch;
-      tl.es.allow = tl.allow != 0;
-      tl.es.tick_ns = ea.tick_ns;
-      tl.es.t_start = t_start;
-      tl.es.expired = &tc->expired;
-      tl.es.pub_thread = kPubThread;
-      tl.es.published = false;
+  // One iteration of the leader on the staged target (and its own search
+  // share when it searches), up to the publication of the next round and the
+  // staging of its target.  Whole block.
+  auto lead_round = [&](bool searches) {
+    const int px = usm.nx_px, py = usm.nx_py;
+    spec_front<R>(usm);
+    if (tid < kChainThreads) {
+      spec_chains<R>(s, usm);
+    } else if (tid < kRecThread) {
+      spec_rest<R>(s, usm);
+    } else {
+      if (tid == kRecThread + 1) {
+        // the stop decision's inputs that other CTAs may change
+        tl.status = __ldcg(&c->status);
+        tl.err = __ldcg(ea.err);
+      }
+      spec_record<R>(s, usm, false);
+      __syncwarp();
     }
     if constexpr (!kLeadOnly) {
       if (searches) {
+        __syncthreads();
         const unsigned long long best = search_round(px, py);
         if (tid == 0) st_relaxed64(&tpart[rank], key_tag(best, epoch));
       }
     }
-    tl.flag = gather_keys(tpart, ns, epoch, ea.err, limit, tl.red64, &tl.key);
-    bool stop = true, ok = false;
-    int npx = 0, npy = 0;
-    unsigned long long t_b = 0ull;
-    if (tl.flag) {
-      t_b = globaltimer();
-      ok = update_phase<R>(s, nullptr, 0, usm, uca, kPubThread, false, &tl.key, &tl.es,
-                           tcmode ? &tc->copied : nullptr, epoch + 1u, &tl.snap);  // ends with a __syncthreads
-      if (ok && tl.es.published) {
-        // the next round (or the stop) went out inside the update phase
-        if (tid == 0) tl.stop = usm.early_stop;
-        npx = usm.next_idx % s.W;
-        npy = usm.next_idx / s.W;
-      } else if (ok) {
-        // the next target is known: publish it before the bookkeeping.
-        // Thread 0 decides (the inputs are global and may change under
-        // other threads' feet) and the barrier below shares the decision.
-        if (tid == 0) {
-          bool st = usm.remaining <= 0 || usm.next_key == 0ull || usm.it + 1 >= tl.lim || tl.status != 0 ||
-                    tl.err != 0;
-          if (!st && ea.tick_ns && globaltimer() - t_start > ea.tick_ns) {
-            st = true;  // the launch's time budget is spent: resume in the next launch
-            tc->expired = 1u;
-          }
-          tl.stop = st;
+    if (tid >= kChainThreads) {
+      if (tid >= kRecThread) {
+        bool late;
+        const unsigned long long best = gather_keys(tpart, ns, epoch, ea.err, limit, &late);
+        if (lane == 0) {
+          usm.t_keys = globaltimer();
+          set_source<R>(s, usm, best, late);
         }
-        npx = usm.next_idx % s.W;
-        npy = usm.next_idx / s.W;
+        __syncwarp();
       }
+      work_sync();
+      if (usm.ok) update_work<R>(s, usm, true, tcmode ? &tc->copied : nullptr, epoch + 1u);
     }
     __syncthreads();
-    stop = ok ? tl.stop != 0 : true;
-    // publication: the update phase's fence (same thread) already ordered
-    // every write the searchers read before this store; without an update
-    // (timeout or error) the store carries its own release
-    if (tid == kPubThread && !(ok && tl.es.published)) {
-      if (ok)
-        st_relaxed64(&tc->pub, pub_pack(epoch + 1u, npx, npy, stop));
-      else
-        st_release64(&tc->pub, pub_pack(epoch + 1u, npx, npy, stop));
-    }
-    if (tid == 0) {
-      tl.stop = stop;
-      tl.px = npx;
-      tl.py = npy;
-    }
-    staged = ok && !stop;
-    if (staged) stage_next<R>(s, npx, npy, usm, &tl.snap.conf);  // next speculative phase's input
+    const bool ok = usm.ok != 0;
+    bool stop = true;
+    unsigned long long wk = 0ull;
+    int wi = 0, ny = 0;
     if (ok) {
-      update_finish<R>(s, usm, staged, false, &tl.snap);  // and the next round's snapshot
-      if (tid == 0) {
-        atomicAdd(&c->t_search, t_b - t_a);
-        atomicAdd(&c->t_update, globaltimer() - t_b);
-        atomicAdd(&c->timed_iters, 1);
+      update_prio<R>(s, usm, wk, wi, ny);
+      stop = usm.remaining <= 0 || wk == 0ull || usm.it + 1 >= tl.lim || tl.status != 0 || tl.err != 0;
+    }
+    if (tid == kPubThread) {
+      // the next round (or the stop) goes out before the bookkeeping; after
+      // an update, this thread's fence in update_work ordered every write
+      // the searchers read before this store, else the store is a release
+      const bool spent = ok && !stop && ea.tick_ns && globaltimer() - t_start > ea.tick_ns;
+      if (spent) {
+        stop = true;  // the launch's time budget is spent: resume in the next launch
+        tc->expired = 1u;
       }
+      const unsigned long long v = pub_pack(epoch + 1u, stop ? 0 : wi - ny * s.W, stop ? 0 : ny, stop);
+      if (ok && !spent)
+        st_relaxed64(&tc->pub, v);
+      else
+        st_release64(&tc->pub, v);
+      tl.stop = stop;
+    }
+    if (ok) {
+      update_store<R>(s, usm, wk, wi);
+      if (!stop) stage_next<R>(s, wk, wi, ny, usm);  // (the time budget is known to the publishing thread only)
     }
     ++epoch;
     prev_px = px;
@@ -1144,32 +1098,26 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     if (lane == 0) asm volatile("fence.proxy.async.global;" ::: "memory");
   };
 
-  if (leader) stage_dterm<R>(usm);  // (the first speculative phase's barriers publish it)
-  if (leader && tid == 0) {
-    // the leader's snapshot of the control block; update_finish keeps it
-    // current from here on
-    tl.snap.px = __ldcg(&c->px);
-    tl.snap.py = __ldcg(&c->py);
-    tl.snap.conf = __ldcg(&c->conf);
-    tl.snap.prio = __ldcg(&c->prio);
-    tl.snap.n_cand = __ldcg(&c->n_valid);
-    tl.snap.it = __ldcg(&c->iter);
-    tl.snap.remaining = __ldcg(&c->remaining);
-    tl.lim = __ldcg(&c->iter_limit);
+  if (leader && !tl.stop) {
+    stage_first<R>(s, usm, false);
+    if (tid == 0) tl.lim = __ldcg(&c->iter_limit);
+    __syncthreads();
   }
   if constexpr (kLeadOnly) {
-    if (tid == 0) usm.tiles_pending = 0;
-    __syncthreads();
-    while (!tl.stop) lead_round(tl.px, tl.py, false);
-    // the last update's tile maxima, deferred by the early selection
-    if (usm.tiles_pending) update_tiles<R>(s, usm, uca, 0);
+    if (!tl.stop) {
+      do lead_round(false);
+      while (!tl.stop);
+      if (tid == kRecThread) update_times<R>(s, usm);
+      update_drain<R>(s, usm, false);
+    }
     x.epoch = epoch;
     return;
   }
+  const bool led = leader && !tl.stop;
   while (!tl.stop) {
     const int px = tl.px, py = tl.py;
     if (leader) {
-      lead_round(px, py, true);
+      lead_round(true);
       continue;
     }
     if (searcher) {
@@ -1188,6 +1136,10 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     prev_py = py;
     __syncthreads();
     if (lane == 0) asm volatile("fence.proxy.async.global;" ::: "memory");
+  }
+  if (led) {
+    if (tid == kRecThread) update_times<R>(s, usm);
+    update_drain<R>(s, usm, false);
   }
   x.ph0 = ph0;
   x.ph1 = ph1;
@@ -1212,15 +1164,47 @@ __global__ void __launch_bounds__(kEngThreads) k_update_fast(ImgState s, cudaGra
                                                             int use_cond) {
   extern __shared__ __align__(128) uint8_t sm_raw[];
   UpdSmem<R>& usm = *reinterpret_cast<UpdSmem<R>*>(sm_raw);
-  UpdCache<R>& uca = upd_cache_of<R>(sm_raw);
   if (!loop_active(s.ctrl)) {
     if (use_cond && threadIdx.x == 0) cudaGraphSetConditional(cond, 0);
     return;
   }
-  stage_dterm<R>(usm);  // (spec_phase's barriers publish it)
-  spec_phase<R>(s, usm, uca, false);
-  const bool ok = update_phase<R>(s, s.partial, s.n_partial, usm, uca, -1, s.overlap != 0);
-  if (ok) update_finish<R>(s, usm, false, s.overlap != 0);
+  stage_first<R>(s, usm, s.overlap != 0);
+  __syncthreads();
+  spec_front<R>(usm);
+  if (threadIdx.x < kChainThreads) {
+    spec_chains<R>(s, usm);
+  } else {
+    if (threadIdx.x < kRecThread) {
+      spec_rest<R>(s, usm);
+    } else {
+      const int lane = threadIdx.x & 31;
+      spec_record<R>(s, usm, false);
+      __syncwarp();
+      unsigned long long best = ~0ull;
+#pragma unroll 4
+      for (int i = lane; i < s.n_partial; i += 32) {
+        const unsigned long long v = __ldcg(&s.partial[i]);
+        best = v < best ? v : best;
+      }
+      __syncwarp();
+      best = warp_min_u64(best);
+      if (lane == 0) set_source<R>(s, usm, best, false);
+      __syncwarp();
+    }
+    work_sync();
+    if (usm.ok) update_work<R>(s, usm, false, nullptr, 0u);
+  }
+  __syncthreads();
+  const bool ok = usm.ok != 0;
+  if (ok) {
+    unsigned long long wk;
+    int wi, ny;
+    update_prio<R>(s, usm, wk, wi, ny);
+    update_store<R>(s, usm, wk, wi);
+    __syncthreads();
+    update_drain<R>(s, usm, s.overlap != 0);
+    __syncthreads();
+  }
   if (use_cond && threadIdx.x == 0) cudaGraphSetConditional(cond, ok && loop_active(s.ctrl) ? 1u : 0u);
 }
 

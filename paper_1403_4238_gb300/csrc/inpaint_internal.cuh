@@ -188,8 +188,8 @@ __device__ inline void plane_store_at(const ImgState& s, int tx, int y, int o, u
 __device__ inline void plane_store(const ImgState& s, int x, int y, uint32_t w) {
   const int xl = x - s.tc_xs0;
   if (xl < 0) return;  // left of every tile's source columns
-  int tx = xl / s.tc_w;
-  if (tx >= s.tc_ntx) tx = s.tc_ntx - 1;
+  int tx = 0;  // (a few tile columns: cheaper than a division)
+  while (tx + 1 < s.tc_ntx && xl >= (tx + 1) * s.tc_w) ++tx;
   for (; tx >= 0 && xl - tx * s.tc_w < s.tc_len; --tx) plane_store_at(s, tx, y, xl - tx * s.tc_w, w);
 }
 

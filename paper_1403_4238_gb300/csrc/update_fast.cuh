@@ -6,20 +6,31 @@
 // before the next target is selected.  Everything involved lies within 3R+2
 // pixels of p^, so that neighbourhood is staged in shared memory.
 //
-// The work is split in two phases.  Which pixels are filled (Psi_p^ ∩ Omega)
-// and the confidence they receive (C(p^)) are known as soon as p^ is
-// selected; only their colours depend on the search result q~.  So the
-// *speculative phase* (spec_phase) runs while the search is still going: it
-// builds the post-fill mask and confidences, finds the post-fill front pixels
-// within 2R+1 of p^, and evaluates their confidence terms C(p) -- the
-// sequential FP64 sums, in row-major patch order (the part with the longest
-// dependency chain) -- and their front normals.  The *update phase*
-// (update_phase) then only copies the pixels, recomputes the isophotes from
-// the new grey levels, and combines them into the data terms D(p) and the
-// priorities.  The data term D = (|dot| / sqrt(nn)) / 510 takes one of a
-// finite set of values (nn = |n|^2 <= 32, |dot| <= 2040); the library
-// evaluates that set once with the same IEEE operations and reads it back
-// here, which gives the same bits as evaluating the expression.
+// Which pixels are filled (Psi_p^ n Omega) and the confidence they receive
+// (C(p^)) are known as soon as p^ is selected; only their colours depend on
+// the search result q~.  So an iteration is cut into pieces by what they wait
+// for, and by which warps run them (kEngThreads threads, one CTA):
+//   all warps      spec_front: post-fill mask, filled set, post-fill front
+//                  pixels within 2R+1 of p^ (from the staged neighbourhood);
+//   warps 0-3      spec_chains: the confidence terms C(p) of those pixels,
+//                  sequential FP64 sums in row-major patch order.  A dependent
+//                  FP64 add takes 64 cycles here, so this is the longest piece
+//                  (5.2k cycles at R = 4, 10.8k at R = 6, 18.5k at R = 8) and
+//                  nothing but the priorities waits for it;
+//   warps 4-14     meanwhile spec_rest (tile maxima of the last iteration, the
+//                  best priority the fill cannot change, new validity counts,
+//                  normals, isophotes the fill cannot change), then, once the
+//                  search's key is there, update_work (copy, validity counts,
+//                  isophotes of the new pixels, the strongest one of every
+//                  front patch);
+//   warp 15        meanwhile the last iteration's record, the search's keys
+//                  (so that their polling waits for nothing else), and after
+//                  the copy the fence that the publication needs;
+//   all warps      update_prio: data terms, priorities, and the next target,
+//                  which is the better of the window's best and the best
+//                  outside it; then update_store and stage_next.
+// Before this split the chains, the key gathering and the update ran one
+// after another on all warps: 12.6 us an iteration at 512x384, R = 4.
 #pragma once
 #include "inpaint_internal.cuh"
 #include "ptx.cuh"
@@ -37,72 +48,81 @@ struct UpdGeom {
   // level-0 / level-1 priority tiles an NW x NW window can touch (per axis)
   static constexpr int KT0 = (NW + kT0 - 2) / kT0 + 1;
   static constexpr int KT1 = 2;
+  static_assert(KT0 * KT0 + KT1 * KT1 + 1 <= 32, "one lane per segment");
 };
 
-constexpr int kT1Cache = 512;  // level-1 entries kept in shared memory (images up to 2^25 px)
-
-// State the update phase reads that the search does not change, loaded
-// while the search runs (update_prefetch): validity counts of the count
-// window, the priority keys of the level-0 tiles the priority window
-// touches, the level-0 entries of the level-1 tiles over them, and the
-// level-1 entries of the whole image.
+// The level-0 and level-1 tiles that the window of (px, py) touches.
+struct TouchedTiles {
+  int tx0, ty0, ntx, nty, ux0, uy0, nux, nuy;
+};
 template <int R>
-struct __align__(16) UpdCache {
-  using G = UpdGeom<R>;
-  unsigned long long tp[G::KT0 * G::KT0 * kT0 * kT0];
-  PrioBest t0c[G::KT1 * G::KT1 * kT1 * kT1];
-  PrioBest t1c[kT1Cache];
-  int cnt[G::NC * G::NC];
-  int tx0, ty0, ntx, nty;  // level-0 tiles [tx0, tx0 + ntx) x [ty0, ty0 + nty)
-  int ux0, uy0, nux, nuy;  // level-1 tiles
-  int t1n;                 // level-1 entries cached (0: read them from global memory)
-};
+__device__ __forceinline__ TouchedTiles touched_tiles(const ImgState& s, int px, int py) {
+  static_assert(kT0 == 16 && kT1 == 16, "tile shifts");
+  constexpr int R2 = UpdGeom<R>::R2;
+  TouchedTiles t;
+  t.tx0 = max(0, px - R2) >> 4;
+  t.ty0 = max(0, py - R2) >> 4;
+  const int tx1 = min(s.W - 1, px + R2) >> 4, ty1 = min(s.H - 1, py + R2) >> 4;
+  t.ntx = tx1 - t.tx0 + 1;
+  t.nty = ty1 - t.ty0 + 1;
+  t.ux0 = t.tx0 >> 4;
+  t.uy0 = t.ty0 >> 4;
+  t.nux = (tx1 >> 4) - t.ux0 + 1;
+  t.nuy = (ty1 >> 4) - t.uy0 + 1;
+  return t;
+}
+
+constexpr int kChainThreads = 128;  // warps 0-3: the FP64 chains, then the priorities
+constexpr int kMidThreads = 352;    // warps 4-14
+constexpr int kMidWarps = kMidThreads / 32;
+constexpr int kRecThread = kEngThreads - 32;  // first thread of warp 15
+
+// Named barriers: of warps 4-14, and of those with warp 15 (the chains join
+// neither).
+__device__ __forceinline__ void mid_sync() { asm volatile("barrier.sync 1, 352;" ::: "memory"); }
+__device__ __forceinline__ void work_sync() { asm volatile("barrier.sync 2, 384;" ::: "memory"); }
 
 template <int R>
 struct __align__(16) UpdSmem {
   using G = UpdGeom<R>;
-  double cf[G::NS * G::NS];
-  double sC[G::NW * G::NW];  // post-fill C(p) of the window (from the speculative phase)
-  int snrm[G::NW * G::NW];   // packed normal, or kSpecNotFront / kSpecOutside
-  int mag[G::NS * G::NS];    // isophote |grad|^2 at a local pixel, -1 if not eligible
-  int gxy[G::NS * G::NS];    // (gx + 512) << 16 | (gy + 512)
+  double cf[G::NS * G::NS];   // C of the known pixels, +0.0 elsewhere
+  double sC[2][G::NW * G::NW];   // (by iteration parity) post-fill C(p) of the front pixels
+                                 // (window index), then the bits of their priority keys
+  int snrm[G::NW * G::NW];    // packed normal, or kSpecNotFront / kSpecOutside
+  uint32_t ikey[G::NS * G::NS];  // isophote key at a local pixel (isophote_key), 0 if not eligible
+  uint32_t dotc[G::NW * G::NW];  // k-th front pixel: |isophote . normal| | normal length code << 12
+  int cnt[G::NC * G::NC];        // validity counts after the fill, -1: not changed by it
   int fsat[(G::P + 1) * (G::P + 1)];
   uint8_t om[G::NS * G::NS];  // 0 known, 1 Omega, 2 outside the image
   uint8_t gr[G::NS * G::NS];
   uint8_t filled[G::P * G::P];
-  uint16_t list[G::NW * G::NW];
-  int nlist;
-  unsigned long long red64[32];
-  int red32[32];
-  int spec_iter, spec_filled, nfront;  // speculative phase outcome
-  // the next target as staged by stage_next: centre, iteration, C(p^)
+  uint16_t list[2][G::NW * G::NW];  // (by parity) front pixels (window index)
+  int nlist[2], nfilled;
+  // the staged target: centre, iteration, C(p^), priority key
   int nx_px, nx_py, nx_it;
   double nx_cp;
-  // outcome of update_phase, consumed by update_finish
-  unsigned long long next_key;  // priority key of the next target (0: none)
-  int next_idx;
-  int it, remaining, n_filled, n_known, n_cand, newly, qx, qy;
+  unsigned long long nx_key;
+  // the iteration being applied, and its record
+  int px, py, it, qx, qy, n_filled, n_known, n_cand, newly, remaining;
   uint32_t ssd;
-  int px, py;
   double pp, cp;
+  int ok;           // the key is a source patch and the state is consistent
+  int rec_pending;  // the record is not written yet
   // the best front pixel whose priority this iteration's fill cannot change
-  // (outside the NW x NW window), found by spec_phase when asked
-  unsigned long long out_key;
-  int out_idx;
-  int early_stop;  // early selection: the loop stops after this iteration
-  int upd_ok;      // update_phase: the speculation matches the iteration
-  int iso_next;    // spec_phase: next chunk of the isophotes the fill cannot change
+  // (outside the NW x NW window), and the selected next target
+  unsigned long long out_key, next_key;
+  int out_idx, out_y, next_idx;
+  // per segment of spec_rest (touched level-0 tiles, touched level-1 tiles,
+  // the rest) the best priority that the iteration leaves alone; the touched
+  // tiles' new maxima are these and the new keys (update_tiles), and are due
+  // while tiles_pending
+  PrioBest seg[32];
+  int tiles_pending, tile_px, tile_py, tile_par;  // the iteration they belong to
+  unsigned long long t_start, t_keys;  // global timer: round start, keys gathered
+  PrioBest red_pb[4];
   // the data term's divisors: s = sqrt(nn) for the 14 normal lengths, their
   // reciprocals and that of 510 (stage_dterm, once per launch)
-  double dsq[kDTabRows], dinv[kDTabRows], dinv510;
-  // early selection: the tile maxima of the last update and the check of
-  // its selection are pending (run by the next speculative phase's spare
-  // warps, or by the leader before it leaves the image)
-  int tiles_pending;
-  unsigned long long pend_key;  // the published next target's key, index
-  int pend_idx;
-  int pend_rem;  // |Omega| after that update
-  PrioBest red_pb[32];
+  double dsq[kDTabRows], dinv[kDTabRows], dinv510, dinvP;  // dinvP: of P^2
 };
 
 // a / b rounded to nearest for a divisor known in advance, from y = RN(1/b):
@@ -128,21 +148,23 @@ __device__ inline void stage_dterm(UpdSmem<R>& sm) {
     sm.dinv[t] = __ddiv_rn(1.0, s);
   } else if (t == kDTabRows) {
     sm.dinv510 = __ddiv_rn(1.0, 510.0);
+    sm.dinvP = __ddiv_rn(1.0, (double)(UpdGeom<R>::P * UpdGeom<R>::P));
   }
 }
 
-// D of Eq. 2, the same bits as data_term_direct: fl(fl(dot / s) / 510), both
+// D of Eq. 2 for a normal of length code c, the same bits as
+// data_term_direct: fl(fl(dot / s) / 510) (0 for a zero normal, whose dot is
+// 0, under any code), both
 // quotients by div_known with the staged divisors (no global load on the
 // update's path).
 template <int R>
-__device__ inline double data_term_known(const UpdSmem<R>& sm, int dot, int nn) {
-  if (nn == 0) return 0.0;
-  const int c = dtab_code(nn);
+__device__ inline double data_term_known(const UpdSmem<R>& sm, int dot, int c) {
   return div_known(div_known((double)dot, sm.dsq[c], sm.dinv[c]), 510.0, sm.dinv510);
 }
 
 // Sobel normal of the Omega indicator at local (lx, ly) = image (x, y),
-// replicated image borders, packed as (nx + 8) << 8 | (ny + 8).
+// replicated image borders, packed as the length code << 16 | (nx + 8) << 8 |
+// (ny + 8).
 template <int R>
 __device__ inline int normal_local(const UpdSmem<R>& sm, const ImgState& s, int lx, int ly, int x,
                                    int y) {
@@ -155,62 +177,56 @@ __device__ inline int normal_local(const UpdSmem<R>& sm, const ImgState& s, int 
   const int m_ld = M(xl, yd), m_cd = M(0, yd), m_rd = M(xr, yd);
   const int nx = (m_ru + 2 * m_rc + m_rd) - (m_lu + 2 * m_lc + m_ld);
   const int ny = (m_ld + 2 * m_cd + m_rd) - (m_lu + 2 * m_cu + m_ru);
-  return ((nx + 8) << 8) | (ny + 8);
+  return (dtab_code(nx * nx + ny * ny) << 16) | ((nx + 8) << 8) | (ny + 8);
 }
 
-// C(p) of Eq. 2: the known part of Psi_p summed in row-major order (dy
-// outer, dx inner, one addition at a time), over the in-image area.
+// The sum of C(p) in Eq. 2: the known part of Psi_p in row-major order (dy
+// outer, dx inner, one addition at a time).
 // Unknown and out-of-image entries hold +0.0 in sm.cf, and adding +0.0 to a
 // non-negative double leaves it unchanged, so summing every entry gives
 // exactly the sum over the known pixels.
+// The next row's entries are loaded, into registers of their own, while a row
+// is summed: the chain then runs at the FP64 unit's 64 cycles an addition
+// (loading each entry over the one just added: 90).
 template <int R>
-__device__ inline double conf_local(const UpdSmem<R>& sm, const ImgState& s, int lx, int ly, int x,
-                                    int y) {
-  constexpr int NS = UpdGeom<R>::NS;
-  double sum = 0.0;
-#pragma unroll 1
-  for (int dy = -R; dy <= R; ++dy) {
+__device__ inline double conf_local(const UpdSmem<R>& sm, int lx, int ly) {
+  constexpr int NS = UpdGeom<R>::NS, P = UpdGeom<R>::P;
+  const double* row = &sm.cf[(ly - R) * NS + lx - R];
+  double a[P], b[P], sum = 0.0;
 #pragma unroll
-    for (int dx = -R; dx <= R; ++dx) sum = __dadd_rn(sum, sm.cf[(ly + dy) * NS + lx + dx]);
+  for (int i = 0; i < P; ++i) a[i] = row[i];
+#pragma unroll 1
+  for (int dy = 0; dy < R; ++dy) {  // rows 2 dy and 2 dy + 1
+    row += NS;
+#pragma unroll
+    for (int i = 0; i < P; ++i) b[i] = row[i];
+#pragma unroll
+    for (int i = 0; i < P; ++i) sum = __dadd_rn(sum, a[i]);
+    row += NS;
+#pragma unroll
+    for (int i = 0; i < P; ++i) a[i] = row[i];
+#pragma unroll
+    for (int i = 0; i < P; ++i) sum = __dadd_rn(sum, b[i]);
   }
-  const int n_in = (min(x + R, s.W - 1) - max(x - R, 0) + 1) * (min(y + R, s.H - 1) - max(y - R, 0) + 1);
-  return __ddiv_rn(sum, (double)n_in);
+#pragma unroll
+  for (int i = 0; i < P; ++i) sum = __dadd_rn(sum, a[i]);
+  return sum;
 }
 
-// Strongest precomputed isophote in Psi_p, first in row-major order.
+// In-image pixels of the patch at (x, y).
 template <int R>
-__device__ inline void isophote_local(const UpdSmem<R>& sm, int lx, int ly, int* gx, int* gy) {
-  constexpr int NS = UpdGeom<R>::NS;
-  int best = -1, bl = 0;
-#pragma unroll 1
-  for (int dy = -R; dy <= R; ++dy) {
-#pragma unroll
-    for (int dx = -R; dx <= R; ++dx) {
-      const int l = (ly + dy) * NS + lx + dx;
-      const int m = sm.mag[l];
-      if (m > best) {
-        best = m;
-        bl = l;
-      }
-    }
-  }
-  *gx = 0;
-  *gy = 0;
-  if (best >= 0) {
-    const int g = sm.gxy[bl];
-    *gx = (g >> 16) - 512;
-    *gy = (g & 0xffff) - 512;
-  }
+__device__ inline int patch_area(const ImgState& s, int x, int y) {
+  return (min(x + R, s.W - 1) - max(x - R, 0) + 1) * (min(y + R, s.H - 1) - max(y - R, 0) + 1);
 }
 
 __device__ inline int dot_abs(int gx, int gy, int nrm) {
-  const int nx = (nrm >> 8) - 8, ny = (nrm & 0xff) - 8;
+  const int nx = ((nrm >> 8) & 0xff) - 8, ny = (nrm & 0xff) - 8;
   const int d = (-gy) * nx + gx * ny;
   return d < 0 ? -d : d;
 }
 
 __device__ inline int nn_of(int nrm) {
-  const int nx = (nrm >> 8) - 8, ny = (nrm & 0xff) - 8;
+  const int nx = ((nrm >> 8) & 0xff) - 8, ny = (nrm & 0xff) - 8;
   return nx * nx + ny * ny;
 }
 
@@ -222,112 +238,66 @@ __device__ inline double data_term_direct(int dot, int nn) {
 
 
 // Stages the NS x NS neighbourhood of (cx, cy): mask (2 outside the image),
-// optionally grey levels and confidences (+0.0 under Omega and outside).
-template <int R, bool GRAY, bool CONF>
+// grey levels and confidences (+0.0 under Omega and outside).  NT threads;
+// each has up to U entries' loads in flight together.
+template <int R, int NT>
 __device__ inline void stage_nbhd(const ImgState& s, int cx, int cy, UpdSmem<R>& sm) {
   using G = UpdGeom<R>;
   constexpr int RB = G::RB, NS = G::NS;
-  constexpr int U = 4;  // entries per thread with their loads in flight together
-  const int step = blockDim.x;
+  constexpr int U = (NS * NS + NT - 1) / NT < 6 ? (NS * NS + NT - 1) / NT : 6;
 #pragma unroll 1
-  for (int i0 = threadIdx.x; i0 < NS * NS; i0 += U * step) {
+  for (int i0 = threadIdx.x; i0 < NS * NS; i0 += U * NT) {
     uint8_t o[U], g[U];
     double cf[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = i0 + u * step;
+      const int i = i0 + u * NT;
       const int x = cx - RB + i % NS, y = cy - RB + i / NS;
       o[u] = 2;
       g[u] = 0;
       cf[u] = 0.0;
       if (i < NS * NS && x >= 0 && x < s.W && y >= 0 && y < s.H) {
-        const size_t q = (size_t)y * s.W + x;
+        const int q = y * s.W + x;
         o[u] = __ldcg(&s.omega[q]);
-        if (GRAY) g[u] = __ldcg(&s.gray[q]);
-        if (CONF) cf[u] = __ldcg(&s.conf[q]);  // read unconditionally, kept for known pixels
+        g[u] = __ldcg(&s.gray[q]);
+        cf[u] = __ldcg(&s.conf[q]);  // read unconditionally, kept for known pixels
       }
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = i0 + u * step;
+      const int i = i0 + u * NT;
       if (i >= NS * NS) break;
       sm.om[i] = o[u];
-      if (GRAY) sm.gr[i] = g[u];
-      if (CONF) sm.cf[i] = o[u] ? 0.0 : cf[u];
+      sm.gr[i] = g[u];
+      sm.cf[i] = o[u] ? 0.0 : cf[u];
     }
   }
 }
 
 // Isophote candidate at local pixel (lx, ly): eligible when it and its four
-// neighbours are known, with its central-difference grey gradient.
+// neighbours are known.  The key orders candidates by |grad|^2 of the
+// central-difference grey gradient, then by the lowest local index (the first
+// in row-major order of any patch): (|grad|^2 + 1) << 12 | (4095 - index).
 template <int R>
-__device__ inline void isophote_at(UpdSmem<R>& sm, int lx, int ly) {
+__device__ inline uint32_t isophote_key(const UpdSmem<R>& sm, int lx, int ly) {
   constexpr int NS = UpdGeom<R>::NS;
+  static_assert(NS * NS <= 4096, "local index fits in 12 bits");
   const int i = ly * NS + lx;
-  int m = -1, g = 0;
-  if (lx >= 1 && lx < NS - 1 && ly >= 1 && ly < NS - 1) {
-    // all nine reads issued together (no short-circuit chain of loads)
-    const int o = sm.om[i] | sm.om[i - 1] | sm.om[i + 1] | sm.om[i - NS] | sm.om[i + NS];
-    const int gx = (int)sm.gr[i + 1] - (int)sm.gr[i - 1];
-    const int gy = (int)sm.gr[i + NS] - (int)sm.gr[i - NS];
-    if (o == 0) {
-      m = gx * gx + gy * gy;
-      g = ((gx + 512) << 16) | (gy + 512);
-    }
-  }
-  sm.mag[i] = m;
-  sm.gxy[i] = g;
+  if (lx < 1 || lx >= NS - 1 || ly < 1 || ly >= NS - 1) return 0u;
+  // all nine reads issued together (no short-circuit chain of loads)
+  const int o = sm.om[i] | sm.om[i - 1] | sm.om[i + 1] | sm.om[i - NS] | sm.om[i + NS];
+  const int gx = (int)sm.gr[i + 1] - (int)sm.gr[i - 1];
+  const int gy = (int)sm.gr[i + NS] - (int)sm.gr[i - NS];
+  return o == 0 ? ((uint32_t)(gx * gx + gy * gy + 1) << 12) | (uint32_t)(4095 - i) : 0u;
 }
 
-// Isophote candidates of the whole staged neighbourhood.
+// |grad . normal| (the data term's numerator) of the isophote with key `ik`.
 template <int R>
-__device__ inline void stage_isophotes(UpdSmem<R>& sm) {
+__device__ inline int isophote_dot(const UpdSmem<R>& sm, uint32_t ik, int nrm) {
   constexpr int NS = UpdGeom<R>::NS;
-#pragma unroll 1
-  for (int i = threadIdx.x; i < NS * NS; i += blockDim.x) isophote_at<R>(sm, i % NS, i / NS);
-}
-
-// Isophote candidates of part of the neighbourhood of p^.  The fill of the
-// iteration changes grey levels and the mask only inside Psi_p^, so a
-// candidate can change only within one pixel of it: in the box of
-// Chebyshev radius R + 1 around p^.  kRing false: every candidate outside
-// that box (the speculative phase, before the search ends, threads
-// [first, blockDim.x)); kRing true: the box itself, from the copied pixels.
-template <int R, bool kRing>
-__device__ inline void stage_isophotes_part(UpdSmem<R>& sm, int first, int last = -1) {
-  constexpr int NS = UpdGeom<R>::NS, RB = UpdGeom<R>::RB, RR = R + 1, NB = 2 * RR + 1;
-  constexpr int n = kRing ? NB * NB : NS * NS;
-  if (last < 0) last = (int)blockDim.x;
-  if ((int)threadIdx.x < first || (int)threadIdx.x >= last) return;
-#pragma unroll 1
-  for (int k = (int)threadIdx.x - first; k < n; k += last - first) {
-    if (kRing) {
-      isophote_at<R>(sm, RB - RR + k % NB, RB - RR + k / NB);
-    } else {
-      const int lx = k % NS, ly = k / NS;
-      if (abs(lx - RB) > RR || abs(ly - RB) > RR) isophote_at<R>(sm, lx, ly);
-    }
-  }
-}
-
-// stage_isophotes_part<R, false> with the work handed out in chunks of 32
-// positions from sm.iso_next (0 on entry): a warp that starts late takes
-// fewer.  Whole warps.  No barrier.
-template <int R>
-__device__ inline void stage_isophotes_dyn(UpdSmem<R>& sm) {
-  constexpr int NS = UpdGeom<R>::NS, RB = UpdGeom<R>::RB, RR = R + 1;
-  const int lane = threadIdx.x & 31;
-  while (true) {
-    int base = 0;
-    if (lane == 0) base = atomicAdd(&sm.iso_next, 32);
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (base >= NS * NS) break;
-    const int k = base + lane;
-    if (k < NS * NS) {
-      const int lx = k % NS, ly = k / NS;
-      if (abs(lx - RB) > RR || abs(ly - RB) > RR) isophote_at<R>(sm, lx, ly);
-    }
-  }
+  if (ik == 0u) return 0;
+  const int l = 4095 - (int)(ik & 4095u);
+  return dot_abs((int)sm.gr[l + 1] - (int)sm.gr[l - 1], (int)sm.gr[l + NS] - (int)sm.gr[l - NS], nrm);
 }
 
 __device__ inline bool front_local(const uint8_t* om, int l, int NS) {
@@ -342,15 +312,16 @@ template <int R>
 __global__ void __launch_bounds__(256, 2) k_prio_init_fast(ImgState s) {
   using G = UpdGeom<R>;
   constexpr int RB = G::RB, NS = G::NS, R2 = G::R2, NW = G::NW;
-  extern __shared__ __align__(16) uint8_t sm_raw[];
+  extern __shared__ __align__(128) uint8_t sm_raw[];
   UpdSmem<R>& sm = *reinterpret_cast<UpdSmem<R>*>(sm_raw);
   const int cx = R2 + blockIdx.x * NW, cy = R2 + blockIdx.y * NW;
-  stage_nbhd<R, true, true>(s, cx, cy, sm);
-  __syncthreads();
-  stage_isophotes<R>(sm);
+  stage_nbhd<R, 256>(s, cx, cy, sm);
   __syncthreads();
 #pragma unroll 1
-  for (int i = threadIdx.x; i < NW * NW; i += blockDim.x) {
+  for (int i = threadIdx.x; i < NS * NS; i += 256) sm.ikey[i] = isophote_key<R>(sm, i % NS, i / NS);
+  __syncthreads();
+#pragma unroll 1
+  for (int i = threadIdx.x; i < NW * NW; i += 256) {
     const int wx = i % NW - R2, wy = i / NW - R2;
     const int lx = RB + wx, ly = RB + wy, l = ly * NS + lx;
     if (sm.om[l] == 2) continue;
@@ -358,11 +329,15 @@ __global__ void __launch_bounds__(256, 2) k_prio_init_fast(ImgState s) {
     unsigned long long key = 0ull;
     double c = 0.0;
     if (front_local(sm.om, l, NS)) {
-      c = conf_local<R>(sm, s, lx, ly, x, y);
+      c = __ddiv_rn(conf_local<R>(sm, lx, ly), (double)patch_area<R>(s, x, y));
       const int nrm = normal_local<R>(sm, s, lx, ly, x, y);
-      int gx, gy;
-      isophote_local<R>(sm, lx, ly, &gx, &gy);
-      const double d = data_term_direct(dot_abs(gx, gy, nrm), nn_of(nrm));
+      uint32_t ik = 0u;
+#pragma unroll 1
+      for (int dy = -R; dy <= R; ++dy) {
+#pragma unroll
+        for (int dx = -R; dx <= R; ++dx) ik = max(ik, sm.ikey[l + dy * NS + dx]);
+      }
+      const double d = data_term_direct(isophote_dot<R>(sm, ik, nrm), nn_of(nrm));
       key = (unsigned long long)__double_as_longlong(__dmul_rn(c, d)) + 1ull;
     }
     const size_t p = (size_t)y * s.W + x;
@@ -371,67 +346,116 @@ __global__ void __launch_bounds__(256, 2) k_prio_init_fast(ImgState s) {
   }
 }
 
-// Loads what the update phase of target (px, py) reads but the search does
-// not change (see UpdCache), with threads [first, blockDim.x).  No barrier.
+// The iteration state from the control block and the neighbourhood of its
+// target, for the first iteration of a launch.  Whole block; the caller's
+// barrier makes it visible.  `overlap_counts`: the partial-overlap search
+// counted its admissible candidates in ctrl->n_adm.
 template <int R>
-__device__ void update_prefetch(const ImgState& s, UpdCache<R>& ca, int first, int px, int py) {
+__device__ inline void stage_first(const ImgState& s, UpdSmem<R>& sm, bool overlap_counts) {
+  const Ctrl* c = s.ctrl;
+  const int px = __ldcg(&c->px), py = __ldcg(&c->py);
+  stage_dterm<R>(sm);
+  if (threadIdx.x == kEngThreads - 1) {
+    sm.nx_px = px;
+    sm.nx_py = py;
+    sm.nx_it = __ldcg(&c->iter);
+    sm.nx_cp = __ldcg(&c->conf);
+    sm.nx_key = (unsigned long long)__double_as_longlong(__ldcg(&c->prio)) + 1ull;
+    sm.n_cand = overlap_counts ? __ldcg(&c->n_adm) : __ldcg(&c->n_valid);
+    sm.remaining = __ldcg(&c->remaining);
+    sm.newly = 0;
+    sm.nlist[0] = sm.nlist[1] = 0;
+    sm.rec_pending = 0;
+    sm.tiles_pending = 0;
+  }
+  stage_nbhd<R, kEngThreads>(s, px, py, sm);
+}
+
+// The next iteration's input, once the next target idx (in row npy) has been selected: its
+// neighbourhood, and in sm.nx_* its centre, iteration number and confidence.
+// Whole block; the caller's barrier makes it visible.
+template <int R>
+__device__ inline void stage_next(const ImgState& s, unsigned long long key, int idx, int npy, UpdSmem<R>& sm) {
+  const int npx = idx - npy * s.W;
+  const bool mine = threadIdx.x == kEngThreads - 1;  // a thread with the fewest staging entries
+  double ncp = 0.0;
+  if (mine) ncp = __ldcg(&s.pconf[idx]);
+  stage_nbhd<R, kEngThreads>(s, npx, npy, sm);
+  if (mine) {
+    sm.nx_px = npx;
+    sm.nx_py = npy;
+    sm.nx_it = sm.it + 1;
+    sm.nx_cp = ncp;
+    sm.nx_key = key;
+    sm.nlist[(sm.it + 1) & 1] = 0;
+  }
+}
+
+// Post-fill mask and confidences of the staged neighbourhood, the filled set,
+// and the post-fill front of the window.  Whole block; ends with a
+// __syncthreads.
+template <int R>
+__device__ inline void spec_front(UpdSmem<R>& sm) {
   using G = UpdGeom<R>;
-  constexpr int R2 = G::R2, NC = G::NC;
-  const int W = s.W, H = s.H;
-  const int tx0 = max(0, px - R2) / kT0, tx1 = min(W - 1, px + R2) / kT0;
-  const int ty0 = max(0, py - R2) / kT0, ty1 = min(H - 1, py + R2) / kT0;
-  const int ntx = tx1 - tx0 + 1, nty = ty1 - ty0 + 1;
-  const int ux0 = tx0 / kT1, ux1 = tx1 / kT1, uy0 = ty0 / kT1, uy1 = ty1 / kT1;
-  const int nux = ux1 - ux0 + 1, nuy = uy1 - uy0 + 1;
-  const int n1 = s.t1x * s.t1y;
-  if ((int)threadIdx.x < first) return;
-  // every load is an asynchronous copy into the cache, all in flight at once
-  const int step = (int)blockDim.x - first, t0 = (int)threadIdx.x - first;
-#pragma unroll 1
-  for (int j = t0; j < NC * NC; j += step) {
-    const int x = px + j % NC - 2 * R, y = py + j / NC - 2 * R;
-    const bool ok = x >= 0 && x < W && y >= 0 && y < H;
-    cp_async4(&ca.cnt[j], ok ? &s.count[(size_t)y * s.pitch + x] : s.count, ok);
+  constexpr int P = G::P, RB = G::RB, NS = G::NS, R2 = G::R2, NW = G::NW;
+  static_assert(P * P <= kEngThreads, "one thread per patch pixel");
+  const int tid = threadIdx.x, lane = tid & 31, par = sm.nx_it & 1;
+  bool f = false;
+  if (tid < P * P) {
+    const int l = (RB + tid / P - R) * NS + RB + tid % P - R;
+    f = sm.om[l] == 1;
+    if (f) {
+      sm.om[l] = 0;
+      sm.cf[l] = sm.nx_cp;
+    }
+    sm.filled[tid] = f;
   }
-  {
-    const int n = ntx * nty * kT0 * kT0;
+  const int filled = __syncthreads_count(f);
 #pragma unroll 1
-    for (int e = t0; e < n; e += step) {
-      const int t = e / (kT0 * kT0), j = e % (kT0 * kT0);
-      const int x = (tx0 + t % ntx) * kT0 + (j & (kT0 - 1)), y = (ty0 + t / ntx) * kT0 + j / kT0;
-      const bool ok = x < W && y < H;
-      cp_async8(&ca.tp[e], ok ? &s.prio[(size_t)y * W + x] : s.prio, ok);
+  for (int i0 = 0; i0 < NW * NW; i0 += kEngThreads) {
+    const int i = i0 + tid;
+    bool fr = false;
+    if (i < NW * NW) {
+      const int l = (RB + i / NW - R2) * NS + RB + i % NW - R2;
+      fr = front_local(sm.om, l, NS);
+      sm.snrm[i] = sm.om[l] != 2 ? kSpecNotFront : kSpecOutside;  // front pixels: overwritten by spec_rest
+    }
+    const unsigned bal = __ballot_sync(0xffffffffu, fr);
+    if (bal != 0u) {
+      int base = 0;
+      if (lane == 0) base = atomicAdd(&sm.nlist[par], __popc(bal));
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if (fr) sm.list[par][base + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)i;
     }
   }
-  {
-    const int n = nux * nuy * kT1 * kT1;
+  if (tid == 0) sm.nfilled = filled;
+  __syncthreads();
+}
+
+// Confidence terms of the front pixels (warps 0-3): one dependent row-major
+// chain per pixel, packed into as few warps as the front needs: up to three
+// warps of chains still run at the 64 cycles of one dependent add, four at 76
+// (the unit takes a warp instruction about every 19 cycles whatever the
+// active lanes).
+__device__ __forceinline__ int chain_threads(int nfront) { return nfront <= 96 ? (nfront + 31) & ~31 : kChainThreads; }
+
+template <int R>
+__device__ inline void spec_chains(const ImgState& s, UpdSmem<R>& sm) {
+  using G = UpdGeom<R>;
+  constexpr int RB = G::RB, R2 = G::R2, NW = G::NW, P2 = G::P * G::P;
+  const int par = sm.nx_it & 1, nfront = sm.nlist[par], nt = chain_threads(nfront);
+  if ((int)threadIdx.x >= nt) return;
 #pragma unroll 1
-    for (int e = t0; e < n; e += step) {
-      const int u = e / (kT1 * kT1), j = e % (kT1 * kT1);
-      const int tx = (ux0 + u % nux) * kT1 + (j & (kT1 - 1)), ty = (uy0 + u / nux) * kT1 + j / kT1;
-      if (tx < s.t0x && ty < s.t0y) {
-        cp_async16(&ca.t0c[e], &s.tiles0[ty * s.t0x + tx]);
-      } else {
-        ca.t0c[e].key = 0ull;
-        ca.t0c[e].idx = 0x7fffffff;
-        ca.t0c[e].pad = 0;
-      }
-    }
-  }
-  if (n1 <= kT1Cache)
-#pragma unroll 1
-    for (int e = t0; e < n1; e += step) cp_async16(&ca.t1c[e], &s.tiles1[e]);
-  cp_async_wait_all();
-  if ((int)threadIdx.x == first) {
-    ca.tx0 = tx0;
-    ca.ty0 = ty0;
-    ca.ntx = ntx;
-    ca.nty = nty;
-    ca.ux0 = ux0;
-    ca.uy0 = uy0;
-    ca.nux = nux;
-    ca.nuy = nuy;
-    ca.t1n = n1 <= kT1Cache ? n1 : 0;
+  for (int k = threadIdx.x; k < nfront; k += nt) {
+    const int i = sm.list[par][k];
+    const int wx = i % NW - R2, wy = i / NW - R2;
+    const int n_in = patch_area<R>(s, sm.nx_px + wx, sm.nx_py + wy);
+    const double sum = conf_local<R>(sm, RB + wx, RB + wy), q = div_known(sum, (double)P2, sm.dinvP);
+    // a second correction by the same reciprocal: after the first the
+    // quotient is within an ulp, so this one rounds it correctly (Markstein),
+    // unless the remainder underflows: tiny sums and clipped patches divide
+    const double c = __fma_rn(__fma_rn(-q, (double)P2, sum), sm.dinvP, q);
+    sm.sC[par][i] = n_in == P2 && sum > 1e-250 ? c : __ddiv_rn(sum, (double)n_in);
   }
 }
 
@@ -441,690 +465,464 @@ template <int R>
 __device__ inline void warp_fsat(UpdSmem<R>& sm) {
   constexpr int P = UpdGeom<R>::P, P1 = P + 1;
   const int lane = threadIdx.x & 31;
-#pragma unroll 1
-  for (int v = lane; v <= P; v += 32) {
-    sm.fsat[v] = 0;
-    sm.fsat[v * P1] = 0;
+  if (lane <= P) {
+    sm.fsat[lane] = 0;
+    sm.fsat[lane * P1] = 0;
   }
   __syncwarp();
-#pragma unroll 1
-  for (int v = lane; v < P; v += 32) {
+  if (lane < P) {
     int run = 0;
 #pragma unroll 1
     for (int u = 0; u < P; ++u) {
-      run += sm.filled[v * P + u];
-      sm.fsat[(v + 1) * P1 + u + 1] = run;
+      run += sm.filled[lane * P + u];
+      sm.fsat[(lane + 1) * P1 + u + 1] = run;
     }
   }
   __syncwarp();
+  if (lane < P) {
+    int run = 0;
 #pragma unroll 1
-  for (int u = lane + 1; u <= P; u += 32)
-#pragma unroll 1
-    for (int v = 2; v <= P; ++v) sm.fsat[v * P1 + u] += sm.fsat[(v - 1) * P1 + u];
-}
-
-// The next iteration's input, once update_phase has selected the next
-// target (npx, npy): its neighbourhood, and in sm.nx_* its centre,
-// iteration number and confidence C(p^), so that spec_phase(staged = true)
-// reads no global control state.  The thread that reads C(p^) also installs
-// it in the control block.  Whole block; the caller's barrier makes it
-// visible.
-template <int R>
-__device__ void stage_next(const ImgState& s, int npx, int npy, UpdSmem<R>& sm, double* conf_out = nullptr) {
-  const int t_cp = (int)blockDim.x - 1;  // a thread with the fewest staging entries
-  double ncp = 0.0;
-  if ((int)threadIdx.x == t_cp) ncp = __ldcg(&s.pconf[sm.next_idx]);
-  stage_nbhd<R, true, true>(s, npx, npy, sm);
-  if ((int)threadIdx.x == t_cp) {
-    sm.nx_px = npx;
-    sm.nx_py = npy;
-    sm.nx_it = sm.it + 1;
-    sm.nx_cp = ncp;
-    s.ctrl->conf = ncp;
-    if (conf_out) *conf_out = ncp;
-  }
-}
-
-// Speculative phase: post-fill mask, grey levels and confidences of the
-// neighbourhood of p^, the filled set and its integral image, the post-fill
-// front of the window with its normals and confidence terms.  Everything
-// stays in shared memory for update_phase.  Whole block.
-// `staged`: the neighbourhood of p^ is already in shared memory (the engine
-// stages it while it records the previous iteration).
-// Best (key, idx) of the priorities outside the NW x NW window around
-// (px, py), from the caches update_prefetch filled: level-1 tiles the window
-// does not touch, level-0 tiles it does not touch inside the level-1 tiles
-// it does, and the pixels outside it inside the level-0 tiles it touches.
-// Those priorities are the ones the fill of this iteration leaves alone.
-// Threads [g0, blockDim.x) (g0 a multiple of 32; the group is synchronised
-// by named barrier 1): the speculative phase's spare warps run it while the
-// other warps' FP64 chains go on.  Writes sm.out_key / sm.out_idx; a block
-// barrier must follow before they are read.
-template <int R>
-__device__ void best_outside_window_group(const ImgState& s, UpdSmem<R>& sm, const UpdCache<R>& ca, int px,
-                                          int py, int g0) {
-  constexpr int R2 = UpdGeom<R>::R2;
-  const int W = s.W;
-  const int nt = (int)blockDim.x - g0, t0 = (int)threadIdx.x - g0;
-  // the group's cache loads (update_prefetch) are complete and visible
-  asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
-  unsigned long long k = 0ull;
-  int idx = 0x7fffffff;
-  const int n1 = s.t1x * s.t1y;
-#pragma unroll 1
-  for (int e = t0; e < n1; e += nt) {
-    const int ux = e % s.t1x, uy = e / s.t1x;
-    if (ux >= ca.ux0 && ux < ca.ux0 + ca.nux && uy >= ca.uy0 && uy < ca.uy0 + ca.nuy) continue;
-    if (ca.t1n) prio_take(k, idx, ca.t1c[e].key, ca.t1c[e].idx);
-    else prio_take(k, idx, __ldcg(&s.tiles1[e].key), __ldcg(&s.tiles1[e].idx));
-  }
-#pragma unroll 1
-  for (int e = t0; e < ca.nux * ca.nuy * kT1 * kT1; e += nt) {
-    const int u = e / (kT1 * kT1), j = e % (kT1 * kT1);
-    const int tx = (ca.ux0 + u % ca.nux) * kT1 + (j & (kT1 - 1)), ty = (ca.uy0 + u / ca.nux) * kT1 + j / kT1;
-    if (tx >= ca.tx0 && tx < ca.tx0 + ca.ntx && ty >= ca.ty0 && ty < ca.ty0 + ca.nty) continue;
-    prio_take(k, idx, ca.t0c[e].key, ca.t0c[e].idx);
-  }
-#pragma unroll 1
-  for (int e = t0; e < ca.ntx * ca.nty * kT0 * kT0; e += nt) {
-    const int t = e / (kT0 * kT0), j = e % (kT0 * kT0);
-    const int x = (ca.tx0 + t % ca.ntx) * kT0 + (j & (kT0 - 1)), y = (ca.ty0 + t / ca.ntx) * kT0 + j / kT0;
-    if (x >= W || y >= s.H || (abs(x - px) <= R2 && abs(y - py) <= R2)) continue;
-    prio_take(k, idx, ca.tp[e], y * W + x);
-  }
-  warp_best_prio(k, idx);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, w0 = g0 >> 5, nw = (int)(blockDim.x >> 5);
-  if (lane == 0) {
-    sm.red_pb[wid].key = k;
-    sm.red_pb[wid].idx = idx;
-  }
-  asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
-  if (wid == w0) {
-    unsigned long long kk = w0 + lane < nw ? sm.red_pb[w0 + lane].key : 0ull;
-    int ii = w0 + lane < nw ? sm.red_pb[w0 + lane].idx : 0x7fffffff;
-    warp_best_prio(kk, ii);
-    if (lane == 0) {
-      sm.out_key = kk;
-      sm.out_idx = ii;
+    for (int v = 1; v <= P; ++v) {
+      run += sm.fsat[v * P1 + lane + 1];
+      sm.fsat[v * P1 + lane + 1] = run;
     }
   }
 }
 
-// The control-block fields the update phase reads, taken early by a caller
-// that knows nothing writes them before the update (the engine's leader
-// reads them at the start of its round, so their latency is hidden).
-struct CtrlSnap {
-  int px, py, n_cand, it, remaining;
-  double conf, prio;
-};
-
-// The tile maxima of the last update (level-0 tiles of its priority window
-// from the cached keys, then their level-1 tiles, in global memory and the
-// caches) and the check that the best of the tiles is the target the early
-// selection published.  Threads [g0, blockDim.x) (g0 a multiple of 32; named
-// barrier 2 when g0 > 0).  Runs before update_prefetch replaces the caches.
+// The engine's phase clocks of the iteration applied last (round start to
+// keys, keys to the next round's start), by the thread that also writes the
+// records.
 template <int R>
-__device__ void update_tiles(const ImgState& s, UpdSmem<R>& sm, UpdCache<R>& ca, int g0) {
-  const int W = s.W, nt = (int)blockDim.x - g0, t0 = (int)threadIdx.x - g0;
-  auto gsync = [&]() {
-    if (g0 == 0)
-      __syncthreads();
-    else
-      asm volatile("bar.sync 2, %0;" ::"r"(nt) : "memory");
-  };
-  const int lane = t0 & 31, wid = t0 >> 5, nw = nt >> 5;
+__device__ inline void update_times(const ImgState& s, UpdSmem<R>& sm) {
+  const unsigned long long now = globaltimer();
+  if (sm.rec_pending) {
+    atomicAdd(&s.ctrl->t_search, sm.t_keys - sm.t_start);
+    atomicAdd(&s.ctrl->t_update, now - sm.t_keys);
+    atomicAdd(&s.ctrl->timed_iters, 1);
+  }
+  sm.t_start = now;
+}
+
+// Writes the record of the iteration applied last (trace, counters) and the
+// next target in the control block; one thread.  Nothing else reads these
+// while a launch runs, so the persistent engine writes them during the next
+// iteration's search.
+template <int R>
+__device__ inline void write_record(const ImgState& s, UpdSmem<R>& sm, bool overlap_counts) {
+  Ctrl* c = s.ctrl;
+  inpaint_step_info e;
+  e.iter = sm.it;
+  e.px = sm.px;
+  e.py = sm.py;
+  e.qx = sm.qx;
+  e.qy = sm.qy;
+  e.ssd = sm.ssd;
+  e.priority = sm.pp;
+  e.confidence = sm.cp;
+  e.filled = sm.n_filled;
+  e.remaining = sm.remaining;
+  e.n_known = sm.n_known;
+  e.n_cand = sm.n_cand;
+  c->last = e;
+  if (sm.it < s.trace_cap) s.trace[sm.it] = e;
+  c->remaining = sm.remaining;
+  c->iter = sm.it + 1;
+  atomicAdd(&c->evals, (unsigned long long)sm.n_cand * (unsigned long long)sm.n_known);
+  sm.n_cand += sm.newly;
+  sm.newly = 0;
+  c->n_valid = sm.n_cand;
+  if (overlap_counts) c->n_adm = 0;  // the next search counts afresh
+  if (sm.remaining > 0 && sm.next_key != 0ull) {
+    c->px = sm.next_idx % s.W;
+    c->py = sm.next_idx / s.W;
+    c->prio = __longlong_as_double((long long)(sm.next_key - 1ull));
+    c->conf = __ldcg(&s.pconf[sm.next_idx]);
+  } else {
+    c->px = -1;
+    c->py = -1;
+    if (sm.remaining > 0) c->status = INPAINT_ERR_INTERNAL;  // Omega non-empty but no front
+  }
+  sm.rec_pending = 0;
+}
+
+// The tile maxima of the last update: for a level-0 tile its window touched,
+// the best of the pixels outside the window (seg, kept from spec_rest) and of
+// the new keys; for a level-1 tile, the best of its other level-0 tiles (seg)
+// and of those.  Warps 4-14; a barrier of theirs follows the writes.
+template <int R>
+__device__ inline void update_tiles(const ImgState& s, UpdSmem<R>& sm) {
+  constexpr int R2 = UpdGeom<R>::R2, NW = UpdGeom<R>::NW;
+  const int lane = threadIdx.x & 31, wid = ((int)threadIdx.x - kChainThreads) >> 5;
+  const int par = sm.tile_par, x0 = sm.tile_px - R2, y0 = sm.tile_py - R2, W = s.W;
+  const TouchedTiles g = touched_tiles<R>(s, sm.tile_px, sm.tile_py);
+  const int n0 = g.ntx * g.nty, nfront = sm.nlist[par];
 #pragma unroll 1
-  for (int t = wid; t < ca.ntx * ca.nty; t += nw) {
-    const int tx = ca.tx0 + t % ca.ntx, ty = ca.ty0 + t / ca.ntx;
-    unsigned long long k = 0ull;
-    int idx = 0x7fffffff;
-#pragma unroll
-    for (int r8 = 0; r8 < kT0 * kT0 / 32; ++r8) {
-      const int j = lane + 32 * r8;
-      const int x = tx * kT0 + (j & (kT0 - 1)), y = ty * kT0 + j / kT0;
-      prio_take(k, idx, ca.tp[t * (kT0 * kT0) + j], y * W + x);
+  for (int t = wid; t < n0; t += kMidWarps) {
+    const int v = t / g.ntx, tx = g.tx0 + t - v * g.ntx, ty = g.ty0 + v;
+    unsigned long long k = sm.seg[t].key;
+    int idx = sm.seg[t].idx;
+#pragma unroll 1
+    for (int e = lane; e < nfront; e += 32) {
+      const int i = sm.list[par][e], x = x0 + i % NW, y = y0 + i / NW;
+      if ((x >> 4) == tx && (y >> 4) == ty)
+        prio_take(k, idx, (unsigned long long)__double_as_longlong(sm.sC[par][i]), y * W + x);
     }
+    __syncwarp();
     warp_best_prio(k, idx);
     if (lane == 0) {
-      s.tiles0[ty * s.t0x + tx].key = k;
-      s.tiles0[ty * s.t0x + tx].idx = idx;
-      const int u = (ty / kT1 - ca.uy0) * ca.nux + (tx / kT1 - ca.ux0);
-      PrioBest& e = ca.t0c[u * (kT1 * kT1) + (ty & (kT1 - 1)) * kT1 + (tx & (kT1 - 1))];
-      e.key = k;
-      e.idx = idx;
+      PrioBest& e = s.tiles0[ty * s.t0x + tx];
+      sm.seg[t].key = e.key = k;
+      sm.seg[t].idx = e.idx = idx;
     }
   }
-  gsync();
+  mid_sync();
+  if (wid == 0 && lane < g.nux * g.nuy) {
+    const int v = lane >= g.nux ? 1 : 0, ux = g.ux0 + lane - v * g.nux, uy = g.uy0 + v;
+    unsigned long long k = sm.seg[n0 + lane].key;
+    int idx = sm.seg[n0 + lane].idx, tx = g.tx0, ty = g.ty0;
 #pragma unroll 1
-  for (int u = wid; u < ca.nux * ca.nuy; u += nw) {
-    const int ux = ca.ux0 + u % ca.nux, uy = ca.uy0 + u / ca.nux;
-    unsigned long long k = 0ull;
-    int idx = 0x7fffffff;
-#pragma unroll
-    for (int r8 = 0; r8 < kT1 * kT1 / 32; ++r8) {
-      const PrioBest& e = ca.t0c[u * (kT1 * kT1) + lane + 32 * r8];
-      prio_take(k, idx, e.key, e.idx);
-    }
-    warp_best_prio(k, idx);
-    if (lane == 0) {
-      s.tiles1[uy * s.t1x + ux].key = k;
-      s.tiles1[uy * s.t1x + ux].idx = idx;
-      if (ca.t1n) {
-        ca.t1c[uy * s.t1x + ux].key = k;
-        ca.t1c[uy * s.t1x + ux].idx = idx;
+    for (int t = 0; t < n0; ++t) {
+      if ((tx >> 4) == ux && (ty >> 4) == uy) prio_take(k, idx, sm.seg[t].key, sm.seg[t].idx);
+      if (++tx == g.tx0 + g.ntx) {
+        tx = g.tx0;
+        ++ty;
       }
     }
+    s.tiles1[uy * s.t1x + ux].key = k;
+    s.tiles1[uy * s.t1x + ux].idx = idx;
   }
-  gsync();
-  if (wid == 0 && sm.pend_rem > 0) {
+  __syncwarp();
+  mid_sync();
+}
+
+// The best priority that the fill of (px, py) leaves alone, by segments: the
+// pixels outside the window of each level-0 tile it touches, the untouched
+// level-0 tiles of each level-1 tile it touches, and the untouched level-1
+// tiles; one warp per segment.  Warps 4-14.
+template <int R>
+__device__ inline void scan_segments(const ImgState& s, UpdSmem<R>& sm, const TouchedTiles& g, int px, int py) {
+  constexpr int R2 = UpdGeom<R>::R2;
+  const int lane = threadIdx.x & 31, W = s.W, H = s.H;
+  const int n0 = g.ntx * g.nty, nseg = n0 + g.nux * g.nuy + 1;
+#pragma unroll 1
+  for (int e = ((int)threadIdx.x - kChainThreads) >> 5; e < nseg; e += kMidWarps) {
     unsigned long long k = 0ull;
     int idx = 0x7fffffff;
-    if (ca.t1n) {
-#pragma unroll 1
-      for (int j = lane; j < ca.t1n; j += 32) prio_take(k, idx, ca.t1c[j].key, ca.t1c[j].idx);
-      warp_best_prio(k, idx);
+    if (e < n0) {
+      const int v = e / g.ntx, xt = (g.tx0 + e - v * g.ntx) * kT0 + (lane & 15), yt = (g.ty0 + v) * kT0 + (lane >> 4);
+      unsigned long long kk[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int y = yt + 2 * j;
+        const bool use = xt < W && y < H && (abs(xt - px) > R2 || abs(y - py) > R2);
+        kk[j] = use ? __ldcg(&s.prio[y * W + xt]) : 0ull;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) prio_take(k, idx, kk[j], (yt + 2 * j) * W + xt);
+    } else if (e < nseg - 1) {
+      const int u = e - n0, v = u >= g.nux ? 1 : 0;
+      const int tx = (g.ux0 + u - v * g.nux) * kT1 + (lane & 15);
+      const int ty = (g.uy0 + v) * kT1 + (lane >> 4);
+      const bool in_x = tx >= g.tx0 && tx < g.tx0 + g.ntx;
+      uint4 b[8];  // all eight loads in flight (one after the other: 4.3k cycles)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const int yy = ty + 2 * j;
+        const bool touched = in_x && yy >= g.ty0 && yy < g.ty0 + g.nty;
+        b[j] = tx < s.t0x && yy < s.t0y && !touched
+                   ? __ldcg(reinterpret_cast<const uint4*>(&s.tiles0[yy * s.t0x + tx]))
+                   : make_uint4(0u, 0u, 0x7fffffffu, 0u);
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        prio_take(k, idx, ((unsigned long long)b[j].y << 32) | b[j].x, (int)b[j].z);
     } else {
-      warp_global_best(s, k, idx);
+      const int n1 = s.t1x * s.t1y;
+#pragma unroll 1
+      for (int j = lane; j < n1; j += 32) {
+        const int uy = j / s.t1x, ux = j - uy * s.t1x;
+        if (ux >= g.ux0 && ux < g.ux0 + g.nux && uy >= g.uy0 && uy < g.uy0 + g.nuy) continue;
+        prio_take(k, idx, __ldcg(&s.tiles1[j].key), __ldcg(&s.tiles1[j].idx));
+      }
     }
-    if (lane == 0 && (k != sm.pend_key || (k != 0ull && idx != sm.pend_idx)))
-      s.ctrl->status = INPAINT_ERR_INTERNAL;  // the tiles and the early selection disagree
+    __syncwarp();
+    warp_best_prio(k, idx);
+    if (lane == 0) {
+      sm.seg[e].key = k;
+      sm.seg[e].idx = idx;
+    }
   }
-  gsync();  // every read of the caches is done before they are replaced
-  if (t0 == 0) sm.tiles_pending = 0;
 }
 
+// What warps 4-14 do while the search and the chains run.
 template <int R>
-__device__ void spec_phase(const ImgState& s, UpdSmem<R>& sm, UpdCache<R>& ca, bool staged,
-                           bool want_outside = false) {
+__device__ inline void spec_rest(const ImgState& s, UpdSmem<R>& sm) {
   using G = UpdGeom<R>;
-  constexpr int P = G::P, RB = G::RB, NS = G::NS, R2 = G::R2, NW = G::NW;
-  const Ctrl* c = s.ctrl;
-  int px, py, it;
-  double cp;
-  if (staged) {
-    px = sm.nx_px;
-    py = sm.nx_py;
-    it = sm.nx_it;
-    cp = sm.nx_cp;
-  } else {
-    px = __ldcg(&c->px);
-    py = __ldcg(&c->py);
-    it = __ldcg(&c->iter);
-    cp = __ldcg(&c->conf);
-    stage_nbhd<R, true, true>(s, px, py, sm);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    sm.nlist = 0;
-    sm.iso_next = 0;
-  }
-  int my = 0;
+  constexpr int P = G::P, RB = G::RB, NS = G::NS, R2 = G::R2, NW = G::NW, NC = G::NC, RR = R + 1, P1 = P + 1;
+  const int px = sm.nx_px, py = sm.nx_py, t0 = (int)threadIdx.x - kChainThreads, W = s.W, H = s.H;
 #pragma unroll 1
-  for (int i = threadIdx.x; i < P * P; i += blockDim.x) {
-    const int l = (RB + i / P - R) * NS + RB + i % P - R;
-    uint8_t f = 0;
-    if (sm.om[l] == 1) {
-      sm.om[l] = 0;
-      sm.cf[l] = cp;
-      f = 1;
-      ++my;
-    }
-    sm.filled[i] = f;
+  for (int j = t0; j < NC * NC; j += kMidThreads) {
+    const int x = px + j % NC - 2 * R, y = py + j / NC - 2 * R;
+    const bool ok = x >= 0 && x < W && y >= 0 && y < H;
+    cp_async4(&sm.cnt[j], ok ? &s.count[y * s.pitch + x] : s.count, ok);
   }
-  const int filled = block_sum_int(my, sm.red32);  // includes __syncthreads
-  // post-fill front of the window, compacted
+  if (t0 >= kMidThreads - 32) warp_fsat<R>(sm);
+  // (every thread reads the flag before update_tiles' barriers, which precede its reset)
+  if (sm.tiles_pending) update_tiles<R>(s, sm);
+  const TouchedTiles g = touched_tiles<R>(s, px, py);
+  scan_segments<R>(s, sm, g, px, py);
+  // normals of the front pixels, and the isophotes the fill cannot change: it
+  // changes grey levels and the mask only inside Psi_p^, so a candidate can
+  // change only in the box of Chebyshev radius R + 1 around p^
+  const int par = sm.nx_it & 1, nfront = sm.nlist[par];
 #pragma unroll 1
-  for (int i = threadIdx.x; i < NW * NW; i += blockDim.x) {
-    const int l = (RB + i / NW - R2) * NS + RB + i % NW - R2;
-    int nrm = kSpecOutside;
-    if (sm.om[l] != 2) {
-      nrm = kSpecNotFront;
-      if (front_local(sm.om, l, NS)) sm.list[atomicAdd(&sm.nlist, 1)] = (uint16_t)i;
-    }
-    sm.snrm[i] = nrm;  // front entries are overwritten below
+  for (int k = t0; k < nfront; k += kMidThreads) {
+    const int i = sm.list[par][k];
+    const int wx = i % NW - R2, wy = i / NW - R2;
+    sm.snrm[i] = normal_local<R>(sm, s, RB + wx, RB + wy, px + wx, py + wy);
   }
-  __syncthreads();
-  const int nfront = sm.nlist;
-  // FP64 confidence sums (Eq. 2) by the first warps, warp 4 builds the
-  // filled-flag integral image, and warps 0-4 share the isophotes the fill
-  // cannot change; the other warps (the spare group) bring the tiles up to
-  // date, load the update phase's cache and find the best priority outside
-  // the fill's window
-  constexpr int g0 = 160;
-  // one dependent row-major chain per front pixel, packed into as few
-  // warps as the front needs: up to three warps of chains still run at the
-  // 64 cycles of one dependent add, four at 76 (the unit takes a warp
-  // instruction about every 19 cycles whatever the active lanes)
-  const int cw = nfront <= 96 ? (nfront + 31) >> 5 : 4;
-  if ((int)threadIdx.x < 32 * cw) {
 #pragma unroll 1
-    for (int k = threadIdx.x; k < nfront; k += 32 * cw) {
-      const int i = sm.list[k];
-      const int wx = i % NW - R2, wy = i / NW - R2;
-      const int lx = RB + wx, ly = RB + wy, x = px + wx, y = py + wy;
-      sm.sC[i] = conf_local<R>(sm, s, lx, ly, x, y);
-      sm.snrm[i] = normal_local<R>(sm, s, lx, ly, x, y);
+  for (int i = t0; i < NS * NS; i += kMidThreads) {
+    const int lx = i % NS, ly = i / NS;
+    if (abs(lx - RB) > RR || abs(ly - RB) > RR) sm.ikey[i] = isophote_key<R>(sm, lx, ly);
+  }
+  cp_async_wait_all();
+  mid_sync();
+  if (t0 < 32) {
+    const int nseg = g.ntx * g.nty + g.nux * g.nuy + 1;
+    unsigned long long k = t0 < nseg ? sm.seg[t0].key : 0ull;
+    int idx = t0 < nseg ? sm.seg[t0].idx : 0x7fffffff;
+    warp_best_prio(k, idx);
+    if (t0 == 0) {
+      sm.out_key = k;
+      sm.out_idx = idx;
+      sm.out_y = idx / W;
+      sm.tiles_pending = 0;
     }
-  } else if ((int)(threadIdx.x >> 5) == 4) {
-    warp_fsat<R>(sm);
   }
-  if ((int)threadIdx.x >= g0) {
-    if (want_outside && sm.tiles_pending) update_tiles<R>(s, sm, ca, g0);
-    update_prefetch<R>(s, ca, g0, px, py);
-    if (want_outside) best_outside_window_group<R>(s, sm, ca, px, py, g0);
-  } else {
-    // the warps without chains at once, the chain warps when done
-    stage_isophotes_dyn<R>(sm);
+  // validity counts after the fill: the centre at (wx, wy) from p^ loses the
+  // filled pixels of its patch
+#pragma unroll 1
+  for (int j = t0; j < NC * NC; j += kMidThreads) {
+    const int jy = j / NC, wy = jy - 2 * R, wx = j - jy * NC - 2 * R;
+    const int u0 = max(0, wx), u1 = min(P, wx + 2 * R + 1), v0 = max(0, wy), v1 = min(P, wy + 2 * R + 1);
+    const int dec = sm.fsat[v1 * P1 + u1] - sm.fsat[v0 * P1 + u1] - sm.fsat[v1 * P1 + u0] + sm.fsat[v0 * P1 + u0];
+    const int x = px + wx, y = py + wy;
+    sm.cnt[j] = dec != 0 && x >= 0 && x < W && y >= 0 && y < H ? sm.cnt[j] - dec : -1;
   }
-  if (threadIdx.x == 0) {
-    sm.nfront = nfront;
-    sm.spec_iter = it;
-    sm.spec_filled = filled;
-  }
-  __syncthreads();
 }
 
-// Early selection (persistent engine, resident mode): the next target is
-// the better of the best new priority in the window and the best one
-// outside it (found by spec_phase), so it is published as soon as the
-// window's priorities are known; the tile maxima are brought up to date
-// after the publication, off the searchers' path.
-struct EarlySel {
-  unsigned long long* pub;  // the team's publication word; nullptr: select through the tiles first
-  unsigned epoch;           // epoch of the round being applied
-  bool allow;               // no iteration limit, status or error stops the loop after this one
-  unsigned long long tick_ns, t_start;  // the launch's time budget (0: none) and start
-  unsigned* expired;        // set when the time budget stops the loop
-  int pub_thread;
-  bool published;           // out (every thread): the next round (or the stop) went out
-};
-
-__device__ inline unsigned long long pub_word(unsigned epoch, int px, int py, bool stop) {
-  return (unsigned long long)epoch | ((unsigned long long)(px & 0x7fff) << 32) |
-         ((unsigned long long)(py & 0x7fff) << 47) | ((unsigned long long)(stop ? 1 : 0) << 62);
-}
-
-// Update phase: applies the iteration whose best source key is *best_in, or
-// the minimum of partial[0..n_partial), on the state prepared by spec_phase and
-// update_prefetch.  Returns false (status written) when there is no source
-// patch or the state is inconsistent.  Whole block; ends with a __syncthreads.
-// Thread `fence_thread` (if any) issues a gpu-scope fence once the pixel,
-// mask and count writes of the iteration are issued (see the engine's
-// publication).  `overlap_counts`: the search was the partial-overlap variant,
-// whose admissible candidates it counted in ctrl->n_adm.
+// The scalars of the iteration on the staged target, after the last one's
+// record (thread kRecThread).
 template <int R>
-__device__ bool update_phase(const ImgState& s, const unsigned long long* partial, int n_partial,
-                             UpdSmem<R>& sm, UpdCache<R>& ca, int fence_thread = -1,
-                             bool overlap_counts = false, const unsigned long long* best_in = nullptr,
-                             EarlySel* es = nullptr, unsigned* copied = nullptr, unsigned copied_val = 0u,
-                             const CtrlSnap* snap = nullptr) {
+__device__ inline void spec_record(const ImgState& s, UpdSmem<R>& sm, bool overlap_counts) {
+  if (threadIdx.x != kRecThread) return;
+  update_times<R>(s, sm);
+  if (sm.rec_pending) write_record<R>(s, sm, overlap_counts);
+  const int filled = sm.nfilled, W = s.W, H = s.H, px = sm.nx_px, py = sm.nx_py;
+  sm.px = px;
+  sm.py = py;
+  sm.it = sm.nx_it;
+  sm.cp = sm.nx_cp;
+  sm.pp = __longlong_as_double((long long)(sm.nx_key - 1ull));
+  sm.n_filled = filled;
+  sm.remaining -= filled;
+  sm.n_known = (min(px + R, W - 1) - max(px - R, 0) + 1) * (min(py + R, H - 1) - max(py - R, 0) + 1) - filled;
+}
+
+// The search's result (one thread): q~ and its SSD, or why there is none.
+template <int R>
+__device__ inline void set_source(const ImgState& s, UpdSmem<R>& sm, unsigned long long best, bool late) {
+  int ok = 0;
+  if (!late) {
+    if (best == ~0ull) {
+      s.ctrl->status = INPAINT_ERR_NO_SOURCE;
+    } else if (sm.n_filled == 0) {
+      s.ctrl->status = INPAINT_ERR_INTERNAL;  // p^ not in Omega
+    } else {
+      const int q = (int)(best & 0xffffffffull);
+      sm.qy = q / s.W;
+      sm.qx = q - sm.qy * s.W;
+      sm.ssd = (uint32_t)(best >> 32);
+      ok = 1;
+    }
+  }
+  sm.ok = ok;
+}
+
+// Applies the iteration whose source set_source has stored (warps 4-15, after
+// a barrier of theirs): the copy of the unknown in-image part of Psi_p^ from
+// Psi_q~, the validity counts of the candidates it touches, the isophotes of
+// the new grey levels and, for every front pixel, the strongest isophote of
+// its patch and its product with the normal.  The block's barrier must follow.
+// The last thread issues a gpu-scope fence once the writes the next search
+// reads (pixels, planes, mask, counts) are issued, and then, if `copied` is
+// given, tells the searchers so; its warp has no later work, so the fence
+// waits off the path, and the same fence makes its later publication of the
+// next round a release.
+template <int R>
+__device__ inline void update_work(const ImgState& s, UpdSmem<R>& sm, bool fence, unsigned* copied,
+                                   unsigned copied_val) {
   using G = UpdGeom<R>;
   constexpr int P = G::P, RB = G::RB, NS = G::NS, R2 = G::R2, NW = G::NW, NC = G::NC;
-  Ctrl* c = s.ctrl;
-  const int tid = threadIdx.x, nt = blockDim.x;
-
-  // best source key: given (already reduced, in shared memory), or the
-  // minimum of the partial keys in global memory
-  unsigned long long best = ~0ull;
-  if (best_in) {
-    best = *best_in;
-  } else {
-#pragma unroll 1
-    for (int i = tid; i < n_partial; i += nt) {
-      const unsigned long long v = __ldcg(&partial[i]);
-      best = v < best ? v : best;
+  static_assert(P * P <= kMidThreads, "one thread per patch pixel");
+  const int t0 = (int)threadIdx.x - kChainThreads, lane = threadIdx.x & 31;
+  if (t0 >= kMidThreads) {
+    work_sync();
+    if (fence && lane == 31) {
+      asm volatile("fence.acq_rel.gpu;" ::: "memory");
+      if (copied) asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(copied), "r"(copied_val) : "memory");
     }
-    best = block_min_u64(best, sm.red64);
+    return;
   }
-  if (best == ~0ull) {
-    if (tid == 0) c->status = INPAINT_ERR_NO_SOURCE;
-    __syncthreads();
-    return false;
-  }
-  // The iteration's scalars go to shared memory once (they are also the
-  // record update_finish writes): each phase below reads the ones it needs,
-  // so that none stays in a register across the phases.  A spilled one
-  // would come back from L2, since local memory misses the L1 that the
-  // shared memory leaves nearly empty.  Candidates of this iteration's
-  // search: the validity-count total, or the admissible ones the
-  // partial-overlap search counted.
-  if (tid == 0) {
-    const int px = snap ? snap->px : __ldcg(&c->px), py = snap ? snap->py : __ldcg(&c->py);
-    const int it = snap ? snap->it : __ldcg(&c->iter);
-    const int filled = sm.spec_filled, q = (int)(best & 0xffffffffull), W = s.W, H = s.H;
-    sm.px = px;
-    sm.py = py;
-    sm.cp = snap ? snap->conf : __ldcg(&c->conf);
-    sm.pp = snap ? snap->prio : __ldcg(&c->prio);
-    sm.n_cand = snap ? snap->n_cand : overlap_counts ? __ldcg(&c->n_adm) : __ldcg(&c->n_valid);
-    sm.it = it;
-    sm.n_filled = filled;
-    sm.remaining = (snap ? snap->remaining : __ldcg(&c->remaining)) - filled;
-    sm.qx = q % W;
-    sm.qy = q / W;
-    sm.ssd = (uint32_t)(best >> 32);
-    sm.n_known = (min(px + R, W - 1) - max(px - R, 0) + 1) * (min(py + R, H - 1) - max(py - R, 0) + 1) - filled;
-    sm.newly = 0;
-    sm.upd_ok = filled != 0 && sm.spec_iter == it;
-  }
-  __syncthreads();
-  if (!sm.upd_ok) {
-    if (tid == 0) c->status = INPAINT_ERR_INTERNAL;  // p^ not in Omega, or stale speculation
-    __syncthreads();
-    return false;
-  }
-  // the window's keys before this update (every key of the cached level-0
-  // tiles, from update_prefetch); a front pixel's key is never 0
-  auto cache_key = [&](int x, int y) -> unsigned long long& {
-    const int t = (y / kT0 - ca.ty0) * ca.ntx + (x / kT0 - ca.tx0);
-    return ca.tp[t * (kT0 * kT0) + (y & (kT0 - 1)) * kT0 + (x & (kT0 - 1))];
-  };
-
-  // one pass over: the copy of the unknown in-image part of Psi_p^ from
-  // Psi_q~ (first, so that its loads go out at once), the validity counts of
-  // the candidates the fill touches (they depend on the filled pixels only),
-  // and key 0 for the window's pixels off the new front; everything the next
-  // search reads is written here, before the fence below
+  const int px = sm.px, py = sm.py, W = s.W;
   {
-    const int px = sm.px, py = sm.py, qx = sm.qx, qy = sm.qy, W = s.W, H = s.H;
-    const double cp = sm.cp;
+    const bool mine = t0 < P * P && sm.filled[t0 < P * P ? t0 : 0];
+    const int dy = t0 / P - R, dx = t0 % P - R;
+    uint32_t w = 0u;
+    if (mine) w = __ldcg(&s.img[(sm.qy + dy) * s.pitch + sm.qx + dx]);  // in flight during the counts
     int newly = 0;
 #pragma unroll 1
-    for (int t = tid; t < P * P + NC * NC + NW * NW; t += nt) {
-      if (t < P * P) {
-        const int i = t;
-        if (!sm.filled[i]) continue;
-        const int dy = i / P - R, dx = i % P - R;
-        const int l = (RB + dy) * NS + RB + dx;
-        const int tx = px + dx, ty = py + dy;
-        const uint32_t w = __ldcg(&s.img[(size_t)(qy + dy) * s.pitch + qx + dx]);
-        const uint8_t g = (uint8_t)luma_word(w);
-        const size_t q = (size_t)ty * W + tx;
-        s.img[(size_t)ty * s.pitch + tx] = w;
-        if (s.planes) plane_store(s, tx, ty, w);  // the tensor-core search's operands
-        s.gray[q] = g;
-        s.conf[q] = cp;
-        s.omega[q] = 0;
-        sm.gr[l] = g;
-      } else if (t < P * P + NC * NC) {
-        const int j = t - P * P;
-        const int wy = j / NC - 2 * R, wx = j % NC - 2 * R;
-        const int x = px + wx, y = py + wy;
-        if (x < 0 || x >= W || y < 0 || y >= H) continue;
-        const int u0 = max(0, wx), u1 = min(P - 1, wx + 2 * R);
-        const int v0 = max(0, wy), v1 = min(P - 1, wy + 2 * R);
-        constexpr int P1 = P + 1;
-        const int dec = sm.fsat[(v1 + 1) * P1 + u1 + 1] - sm.fsat[v0 * P1 + u1 + 1] -
-                        sm.fsat[(v1 + 1) * P1 + u0] + sm.fsat[v0 * P1 + u0];
-        if (dec) {
-          const int nv = ca.cnt[j] - dec;
-          s.count[(size_t)y * s.pitch + x] = nv;
-          if (nv == 0 && x >= s.cx0 && x <= s.cx1 && y >= s.cy0 && y <= s.cy1) ++newly;
-        }
-      } else {
-        const int i = t - P * P - NC * NC;
-        if (sm.snrm[i] != kSpecNotFront) continue;  // outside, or a front pixel
-        const int x = px + i % NW - R2, y = py + i / NW - R2;
-        unsigned long long& ck = cache_key(x, y);
-        if (ck == 0ull) continue;  // not on the old front: key and C are 0 already
-        const size_t p = (size_t)y * W + x;
-        s.prio[p] = 0ull;
-        s.pconf[p] = 0.0;
-        ck = 0ull;
-      }
+    for (int j = t0; j < NC * NC; j += kMidThreads) {
+      const int nv = sm.cnt[j];
+      if (nv < 0) continue;
+      const int jy = j / NC, y = py + jy - 2 * R, x = px + j - jy * NC - 2 * R;
+      s.count[y * s.pitch + x] = nv;
+      if (nv == 0 && x >= s.cx0 && x <= s.cx1 && y >= s.cy0 && y <= s.cy1) ++newly;
+    }
+    if (mine) {
+      const int tx = px + dx, ty = py + dy, q = ty * W + tx;
+      const uint8_t g = (uint8_t)luma_word(w);
+      s.img[ty * s.pitch + tx] = w;
+      if (s.planes) plane_store(s, tx, ty, w);  // the tensor-core search's operands
+      s.gray[q] = g;
+      s.conf[q] = sm.cp;
+      s.omega[q] = 0;
+      sm.gr[(RB + dy) * NS + RB + dx] = g;
     }
     if (newly) atomicAdd(&sm.newly, newly);
   }
-  __syncthreads();
-  const int fthread = fence_thread >= 0 ? fence_thread : copied ? 0 : -1;
-  if (tid == fthread) {
-    // every write the next search reads (pixels, planes, mask, counts) is
-    // issued; the barrier above orders the other threads' ones before this
-    // fence, which also serves the thread's later publication of the next
-    // round.  The fence thread has no isophote or row-maximum work below, so
-    // its wait overlaps them.  Then the searchers may prefetch the next
-    // round's first source rows.
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
-    if (copied) asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(copied), "r"(copied_val) : "memory");
-  }
-
-  // isophotes of the new grey levels (the ones the fill cannot change were
-  // computed by the speculative phase), then for every front pixel the
-  // strongest one of its patch (first in row-major order on ties) as a
-  // separable windowed maximum of keys (|grad|^2 + 1) << 12 | (4095 - l) over
-  // local indices l: rows here, columns in the priority loop below; the
-  // confidence array is free here and holds the row maxima
-  stage_isophotes_part<R, true>(sm, 0);
-  __syncthreads();
-  constexpr int HR = NW + 2 * R;  // rows of the horizontal pass
-  uint32_t* hkey = reinterpret_cast<uint32_t*>(sm.cf);
-  static_assert(sizeof(sm.cf) >= sizeof(uint32_t) * HR * NW, "key scratch");
-  static_assert(NS * NS <= 4096, "local index fits in 12 bits");
-  const int nhk = nt >= 512 ? nt - 32 : nt;  // the last warp (the fence thread's) sits out
+  __syncwarp();
+  work_sync();
+  constexpr int NB = 2 * (R + 1) + 1;  // the box the fill can change
 #pragma unroll 1
-  for (int i = tid; i < HR * NW && tid < nhk; i += nhk) {
-    const int ly = RB - R2 - R + i / NW, lx = RB - R2 + i % NW;
-    uint32_t best = 0u;
+  for (int j = t0; j < NB * NB; j += kMidThreads) {
+    const int lx = RB - R - 1 + j % NB, ly = RB - R - 1 + j / NB;
+    sm.ikey[ly * NS + lx] = isophote_key<R>(sm, lx, ly);
+  }
+  // strongest isophote of a front pixel's patch: one warp per pixel, each
+  // lane with a fixed set of patch offsets (a separable windowed maximum over
+  // the whole window took 1.8k + 0.5k cycles at R = 6)
+  constexpr int NL = (P * P + 31) / 32;
+  int off[NL];
 #pragma unroll
-    for (int dx = -R; dx <= R; ++dx) {
-      const int l = ly * NS + lx + dx;
-      const int m = sm.mag[l];
-      const uint32_t key = m >= 0 ? ((uint32_t)(m + 1) << 12) | (uint32_t)(4095 - l) : 0u;
-      best = key > best ? key : best;
-    }
-    hkey[i] = best;
+  for (int j = 0; j < NL; ++j) {
+    const int e = lane + 32 * j;
+    off[j] = e < P * P ? (e / P - R) * NS + e % P - R : 0;  // past the end: the centre once more
   }
-  __syncthreads();
-
-  // priorities of the new front (from the compact list, spread over the
-  // sub-partitions); the new keys also go to the cached level-0 tiles
-  unsigned long long wk = 0ull;  // best new key of the window (early selection)
-  int wi = 0x7fffffff;
-  {
-    const int px = sm.px, py = sm.py, W = s.W, nfront = sm.nfront;
-    const int nlist = (nfront + 127) & ~127;
+  const int par = sm.it & 1, nfront = sm.nlist[par];
+  __syncwarp();
+  mid_sync();
 #pragma unroll 1
-    for (int t = tid; t < nlist; t += nt) {
-      const int k = list_entry(t);
-      if (k >= nfront) continue;
-      const int i = sm.list[k];
-      const int wx = i % NW - R2, wy = i / NW - R2;
-      int gx, gy;
-      uint32_t ik = 0u;  // column maximum of the row maxima
-  #pragma unroll
-      for (int dy = 0; dy <= 2 * R; ++dy) {
-        const uint32_t key = hkey[(i / NW + dy) * NW + i % NW];
-        ik = key > ik ? key : ik;
-      }
-      gx = 0;
-      gy = 0;
-      if (ik) {
-        const int g = sm.gxy[4095 - (int)(ik & 4095u)];
-        gx = (g >> 16) - 512;
-        gy = (g & 0xffff) - 512;
-      }
-      const double cc = sm.sC[i];
-      const int nrm = sm.snrm[i];
-      const double d = data_term_known(sm, dot_abs(gx, gy, nrm), nn_of(nrm));
-      const int x = px + wx, y = py + wy;
-      const size_t p = (size_t)y * W + x;
-      const unsigned long long key = (unsigned long long)__double_as_longlong(__dmul_rn(cc, d)) + 1ull;
-      s.prio[p] = key;
-      s.pconf[p] = cc;
-      cache_key(x, y) = key;
-      prio_take(wk, wi, key, (int)p);
-    }
-  }
-  const bool early = es && es->pub;
-  if (early) {
-    // the next target: the better of the window's best and the best outside
-    // it; published now unless the loop stops, in which case the stop goes
-    // out (the publishing thread is the fence thread: its fence after the
-    // copy makes this store a release of everything the search reads)
-    block_best_prio(wk, wi, sm.red_pb);  // every thread gets the window's best
-    prio_take(wk, wi, sm.out_key, sm.out_idx);
-    if ((int)threadIdx.x == es->pub_thread) {
-      bool st = sm.remaining <= 0 || wk == 0ull || !es->allow;
-      if (!st && es->tick_ns && globaltimer() - es->t_start > es->tick_ns) {
-        st = true;  // the launch's time budget is spent: resume in the next launch
-        *es->expired = 1u;
-      }
-      const int W = s.W;
-      asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(es->pub),
-                   "l"(pub_word(es->epoch + 1u, st ? 0 : wi % W, st ? 0 : wi / W, st))
-                   : "memory");
-      sm.early_stop = st;
-    }
-    es->published = true;
-    // the outcome is known: the tile maxima and the check of this selection
-    // are left to the next speculative phase's spare warps
-    if (tid == 0) {
-      const int rem = sm.remaining;
-      sm.next_key = rem > 0 ? wk : 0ull;
-      sm.next_idx = wi;
-      sm.pend_key = wk;
-      sm.pend_idx = wi;
-      sm.pend_rem = rem;
-      sm.tiles_pending = 1;
-    }
-    __syncthreads();
-    return true;
-  }
-  __syncthreads();  // the priority loop's cache writes before the tiles read them
-
-  // level-0 tiles from the cached keys, then level-1, then the best
-  const int lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
+  for (int b = t0 >> 5; b < nfront; b += 32 * kMidWarps) {
+    uint32_t mine = 0u;  // lane j: the key of the warp's j-th pixel
+    int j = 0;
 #pragma unroll 1
-  for (int t = wid; t < ca.ntx * ca.nty; t += nw) {
-    const int tx = ca.tx0 + t % ca.ntx, ty = ca.ty0 + t / ca.ntx;
-    unsigned long long k = 0ull;
-    int idx = 0x7fffffff;
+    for (int k = b; k < nfront && j < 32; k += kMidWarps, ++j) {
+      const int i = sm.list[par][k], l = (RB + i / NW - R2) * NS + RB + i % NW - R2;
+      uint32_t best = 0u;
 #pragma unroll
-    for (int r8 = 0; r8 < kT0 * kT0 / 32; ++r8) {
-      const int j = lane + 32 * r8;
-      const int x = tx * kT0 + (j & (kT0 - 1)), y = ty * kT0 + j / kT0;
-      const unsigned long long kk = ca.tp[t * (kT0 * kT0) + j];
-      const int ii = y * s.W + x;
-      prio_take(k, idx, kk, ii);
+      for (int q = 0; q < NL; ++q) best = max(best, sm.ikey[l + off[q]]);
+      best = __reduce_max_sync(0xffffffffu, best);
+      if (lane == j) mine = best;
     }
-    warp_best_prio(k, idx);
-    if (lane == 0) {
-      s.tiles0[ty * s.t0x + tx].key = k;
-      s.tiles0[ty * s.t0x + tx].idx = idx;
-      const int u = (ty / kT1 - ca.uy0) * ca.nux + (tx / kT1 - ca.ux0);
-      PrioBest& e = ca.t0c[u * (kT1 * kT1) + (ty & (kT1 - 1)) * kT1 + (tx & (kT1 - 1))];
-      e.key = k;
-      e.idx = idx;
+    if (lane < j) {
+      const int k = b + kMidWarps * lane, nrm = sm.snrm[sm.list[par][k]];
+      sm.dotc[k] = (uint32_t)isophote_dot<R>(sm, mine, nrm) | ((uint32_t)(nrm >> 16) << 12);
     }
   }
-  __syncthreads();
-#pragma unroll 1
-  for (int u = wid; u < ca.nux * ca.nuy; u += nw) {
-    const int ux = ca.ux0 + u % ca.nux, uy = ca.uy0 + u / ca.nux;
-    unsigned long long k = 0ull;
-    int idx = 0x7fffffff;
-#pragma unroll
-    for (int r8 = 0; r8 < kT1 * kT1 / 32; ++r8) {
-      const PrioBest& e = ca.t0c[u * (kT1 * kT1) + lane + 32 * r8];
-      prio_take(k, idx, e.key, e.idx);
-    }
-    warp_best_prio(k, idx);
-    if (lane == 0) {
-      s.tiles1[uy * s.t1x + ux].key = k;
-      s.tiles1[uy * s.t1x + ux].idx = idx;
-      if (ca.t1n) {
-        ca.t1c[uy * s.t1x + ux].key = k;
-        ca.t1c[uy * s.t1x + ux].idx = idx;
-      }
-    }
-  }
-  __syncthreads();
-  {
-    // every warp takes the same decision: a lone warp running while the
-    // others wait at the barrier was several times slower here
-    unsigned long long k = 0ull;
-    int idx = 0x7fffffff;
-    if (sm.remaining > 0) {
-      if (ca.t1n) {
-#pragma unroll 1
-        for (int j = lane; j < ca.t1n; j += 32) prio_take(k, idx, ca.t1c[j].key, ca.t1c[j].idx);
-        warp_best_prio(k, idx);
-      } else {
-        warp_global_best(s, k, idx);
-      }
-    }
-    if (tid == 0) {
-      sm.next_key = k;
-      sm.next_idx = idx;
-    }
-  }
-  __syncthreads();
-  return true;
 }
 
-// Records the iteration applied by update_phase (trace, counters) and
-// installs the next target p^ with its priority and confidence in the
-// control block (stage_next has installed the confidence when
-// `cp_staged`).  Neither the image state nor the tiles change here, so the
-// persistent engine publishes the next target to its searchers first.
-// Whole block; ends with a __syncthreads.
+// Priorities of the new front (warps 0-3) and the next target: the better of
+// the window's best and the best outside it.  Whole block, after a barrier;
+// has one barrier, after which every thread holds the target (key 0: none).
+// (*ny: its row, found where a division by W is off the path.)
 template <int R>
-__device__ void update_finish(const ImgState& s, const UpdSmem<R>& sm, bool cp_staged,
-                              bool overlap_counts = false, CtrlSnap* next_snap = nullptr) {
-  Ctrl* c = s.ctrl;
-  const bool next = sm.remaining > 0 && sm.next_key != 0ull;
-  if (threadIdx.x == 0) {
-    // the record is built in registers: no global read-backs on the
-    // leader's critical path
-    inpaint_step_info e;
-    e.iter = sm.it;
-    e.px = sm.px;
-    e.py = sm.py;
-    e.qx = sm.qx;
-    e.qy = sm.qy;
-    e.ssd = sm.ssd;
-    e.priority = sm.pp;
-    e.confidence = sm.cp;
-    e.filled = sm.n_filled;
-    e.remaining = sm.remaining;
-    e.n_known = sm.n_known;
-    e.n_cand = sm.n_cand;
-    c->last = e;
-    if (sm.it < s.trace_cap) s.trace[sm.it] = e;
-    c->remaining = sm.remaining;
-    c->iter = sm.it + 1;
-    c->n_valid = sm.n_cand + sm.newly;
-    if (next_snap) {
-      next_snap->remaining = sm.remaining;
-      next_snap->it = sm.it + 1;
-      next_snap->n_cand = sm.n_cand + sm.newly;
+__device__ inline void update_prio(const ImgState& s, UpdSmem<R>& sm, unsigned long long& wk, int& wi, int& ny) {
+  using G = UpdGeom<R>;
+  constexpr int R2 = G::R2, NW = G::NW;
+  const int tid = threadIdx.x;
+  wk = 0ull;
+  wi = 0x7fffffff;
+  if (tid < kChainThreads) {
+    int mine_i = 0x7fffffff, mine_y = 0;
+    const int par = sm.it & 1, nfront = sm.nlist[par], nt = chain_threads(nfront), W = s.W;
+    if (tid < nt) {
+#pragma unroll 1
+      for (int k = tid; k < nfront; k += nt) {
+        const int i = sm.list[par][k];
+        const uint32_t dc = sm.dotc[k];
+        const double cc = sm.sC[par][i];
+        const double d = data_term_known(sm, (int)(dc & 0xfffu), (int)(dc >> 12));
+        const int py = sm.py + i / NW - R2, p = py * W + sm.px + i % NW - R2;
+        const unsigned long long key = (unsigned long long)__double_as_longlong(__dmul_rn(cc, d)) + 1ull;
+        s.prio[p] = key;
+        s.pconf[p] = cc;
+        sm.sC[par][i] = __longlong_as_double((long long)key);
+        if (prio_better(key, p, wk, mine_i)) {
+          wk = key;
+          mine_i = p;
+          mine_y = py;
+        }
+      }
     }
-    if (overlap_counts) c->n_adm = 0;  // the next search counts afresh
-    atomicAdd(&c->evals, (unsigned long long)sm.n_cand * (unsigned long long)sm.n_known);
-    if (!next) {
-      c->px = -1;
-      c->py = -1;
-      if (sm.remaining > 0) c->status = INPAINT_ERR_INTERNAL;  // Omega non-empty but no front
-    }
-  }
-  if (next && (int)threadIdx.x == (blockDim.x > 32 ? 32 : 0)) {
-    // the next target, from another warp (its confidence is a global read)
-    const double prio = __longlong_as_double((long long)(sm.next_key - 1ull));
-    c->px = sm.next_idx % s.W;
-    c->py = sm.next_idx / s.W;
-    c->prio = prio;
-    if (!cp_staged) {
-      const double conf = __ldcg(&s.pconf[sm.next_idx]);
-      c->conf = conf;
-      if (next_snap) next_snap->conf = conf;  // (staged: stage_next wrote it)
-    }
-    if (next_snap) {
-      next_snap->px = sm.next_idx % s.W;
-      next_snap->py = sm.next_idx / s.W;
-      next_snap->prio = prio;
-    }
+    __syncwarp();
+    wi = mine_i;
+    warp_best_prio(wk, wi);
+    if (wk != 0ull && mine_i == wi) sm.red_pb[tid >> 5] = PrioBest{wk, wi, mine_y};
+    else if ((tid & 31) == 0 && wk == 0ull) sm.red_pb[tid >> 5] = PrioBest{0ull, 0x7fffffff, 0};
   }
   __syncthreads();
+  wk = sm.out_key;
+  wi = sm.out_idx;
+  ny = sm.out_y;
+#pragma unroll
+  for (int w = 0; w < kChainThreads / 32; ++w) {
+    const PrioBest b = sm.red_pb[w];
+    const bool t = prio_better(b.key, b.idx, wk, wi);
+    wk = t ? b.key : wk;
+    wi = t ? b.idx : wi;
+    ny = t ? b.pad : ny;
+  }
+}
+
+// After the selection (whole block, no barrier inside): key 0 for the
+// window's pixels that are not on the front, and the state of the deferred
+// record and tile maxima.
+template <int R>
+__device__ inline void update_store(const ImgState& s, UpdSmem<R>& sm, unsigned long long wk, int wi) {
+  using G = UpdGeom<R>;
+  constexpr int R2 = G::R2, NW = G::NW;
+#pragma unroll 1
+  for (int i = threadIdx.x; i < NW * NW; i += kEngThreads)
+    if (sm.snrm[i] == kSpecNotFront) s.prio[(sm.py + i / NW - R2) * s.W + sm.px + i % NW - R2] = 0ull;
+  if (threadIdx.x == 0) {
+    sm.next_key = sm.remaining > 0 ? wk : 0ull;
+    sm.next_idx = wi;
+    sm.tile_px = sm.px;
+    sm.tile_py = sm.py;
+    sm.tile_par = sm.it & 1;
+    sm.tiles_pending = 1;
+    sm.rec_pending = 1;
+  }
+}
+
+// The deferred record and tile maxima of the last iteration, before a launch
+// leaves the image.  Whole block, after a barrier.
+template <int R>
+__device__ inline void update_drain(const ImgState& s, UpdSmem<R>& sm, bool overlap_counts) {
+  if (threadIdx.x == kRecThread && sm.rec_pending) write_record<R>(s, sm, overlap_counts);
+  if ((int)threadIdx.x >= kChainThreads && (int)threadIdx.x < kRecThread && sm.tiles_pending) update_tiles<R>(s, sm);
 }
 
 }  // namespace inp
