@@ -21,23 +21,81 @@
 
 namespace inp {
 
-__device__ inline unsigned long long cand_key(const ImgState& s, uint32_t ssd, int qx, int qy) {
-  if (qx > s.cx1 || qy > s.cy1) return ~0ull;
-  const int idx = qy * s.W + qx;
-  if (s.count[(size_t)qy * s.pitch + qx] != 0) return ~0ull;
-  return ((unsigned long long)ssd << 32) | (unsigned)idx;
+// The unknown counts of a thread's S candidates, requested before the SSD work
+// that hides them; 1 (not a candidate) outside the search rectangle.
+template <int S>
+__device__ inline void load_counts(const ImgState& s, int qx0, int qy, int (&cnt)[S]) {
+#pragma unroll
+  for (int k = 0; k < S; ++k)
+    cnt[k] = qx0 + k <= s.cx1 && qy <= s.cy1 ? s.count[(size_t)qy * s.pitch + qx0 + k] : 1;
 }
 
-// Stage a rows x pitch window of image words whose top-left is (x0, y0);
-// out-of-image words read as 0 (never used by a valid candidate).
-__device__ inline void stage_tile(const ImgState& s, uint32_t* dst, int x0, int y0, int rows,
-                                  int pitch) {
-  const int n = rows * pitch;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const int yy = y0 + i / pitch, xx = x0 + i % pitch;
+// Smallest key over a thread's S candidates.
+template <int S>
+__device__ inline unsigned long long best_key(const ImgState& s, const uint32_t (&ssd)[S], const int (&cnt)[S],
+                                              int qx0, int qy) {
+  unsigned long long best = ~0ull;
+#pragma unroll
+  for (int k = 0; k < S; ++k) {
+    const unsigned long long key = ((unsigned long long)ssd[k] << 32) | (unsigned)(qy * s.W + qx0 + k);
+    if (cnt[k] == 0 && key < best) best = key;
+  }
+  return best;
+}
+
+// Stage a ROWS x PITCH window of image words whose top-left is (x0, y0), every
+// load of a thread in flight at once (one L2 round trip).  Out-of-image words
+// read as 0 (never used by a valid candidate); with AVAIL (partial-overlap
+// search) the alpha byte says whether the pixel may be used as a source (0:
+// known and in the image; 0xFF, with RGB bytes 0: unknown or outside).
+template <int ROWS, int PITCH, bool AVAIL>
+__device__ inline void stage_tile(const ImgState& s, uint32_t* dst, int x0, int y0) {
+  constexpr int n = ROWS * PITCH, U = (n + kSearchThreads - 1) / kSearchThreads;
+  constexpr uint32_t kNone = AVAIL ? 0xff000000u : 0u;
+  uint32_t w[U];
+  uint8_t o[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int i = threadIdx.x + u * kSearchThreads;
+    const int yy = y0 + i / PITCH, xx = x0 + i % PITCH;
+    const bool in = i < n && xx >= 0 && xx < s.W && yy >= 0 && yy < s.H;
+    w[u] = in ? s.img[(size_t)yy * s.pitch + xx] : kNone;
+    o[u] = AVAIL && in ? s.omega[(size_t)yy * s.W + xx] : 0;
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int i = threadIdx.x + u * kSearchThreads;
+    if (i < n) dst[i] = AVAIL && o[u] ? kNone : w[u];
+  }
+}
+
+// Target patch: known in-image pixels with their RGBA words (row pitch TP, 0
+// elsewhere) and one bit mask per row; unk (may be null): the unknown in-image
+// ones.  One warp per row, one lane per column, so the reads of a row are one
+// L2 round trip (a thread that walked its row took one per pixel).
+template <int P, int TP>
+__device__ inline void stage_target(const ImgState& s, int px, int py, uint32_t* tgt, uint32_t* rowmask,
+                                    uint32_t* unk) {
+  constexpr int R = P / 2;
+  static_assert(P <= 32, "one lane per column");
+  const int lane = threadIdx.x & 31;
+  for (int dy = threadIdx.x >> 5; dy < P; dy += kSearchThreads / 32) {
+    const int tx = px + lane - R, ty = py + dy - R;
+    const bool in = lane < P && tx >= 0 && tx < s.W && ty >= 0 && ty < s.H;
     uint32_t w = 0;
-    if (xx >= 0 && xx < s.W && yy >= 0 && yy < s.H) w = s.img[(size_t)yy * s.pitch + xx];
-    dst[i] = w;
+    bool known = false;
+    if (in) {
+      const uint8_t o = s.omega[(size_t)ty * s.W + tx];
+      const uint32_t v = s.img[(size_t)ty * s.pitch + tx];
+      known = o == 0;
+      w = known ? v : 0u;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, known), u = __ballot_sync(0xffffffffu, in && !known);
+    if (lane < TP) tgt[dy * TP + lane] = w;
+    if (lane == 0) {
+      rowmask[dy] = m;
+      if (unk) unk[dy] = u;
+    }
   }
 }
 
@@ -66,28 +124,13 @@ __global__ void __launch_bounds__(kSearchThreads) k_search_plain(ImgState s) {
   const int ox = s.cx0 + blockIdx.x * TW, oy = s.cy0 + blockIdx.y * TH;
   const int tid = threadIdx.x;
 
-  // Target patch: known in-image pixels with their RGBA words, one bit mask per row.
-  if (tid < P) {
-    const int ty = py + tid - R;
-    uint32_t m = 0;
-    for (int dx = 0; dx < P; ++dx) {
-      const int tx = px + dx - R;
-      uint32_t w = 0;
-      if (tx >= 0 && tx < s.W && ty >= 0 && ty < s.H) {
-        const size_t t = (size_t)ty * s.W + tx;
-        if (!s.omega[t]) {
-          w = s.img[(size_t)ty * s.pitch + tx];
-          m |= 1u << dx;
-        }
-      }
-      tgt[tid * P + dx] = w;
-    }
-    rowmask[tid] = m;
-  }
-  stage_tile(s, src, ox - R, oy - R, SH, SW);
+  const int lane = tid & 31, wr = tid >> 5;  // warp = one candidate row of the tile
+  int cnt[S];
+  load_counts<S>(s, ox + lane * S, oy + wr, cnt);
+  stage_target<P, P>(s, px, py, tgt, rowmask, nullptr);
+  stage_tile<SH, SW, false>(s, src, ox - R, oy - R);
   __syncthreads();
 
-  const int lane = tid & 31, wr = tid >> 5;  // warp = one candidate row of the tile
   uint32_t acc[S];
 #pragma unroll
   for (int k = 0; k < S; ++k) acc[k] = 0;
@@ -119,32 +162,7 @@ __global__ void __launch_bounds__(kSearchThreads) k_search_plain(ImgState s) {
     }
   }
 
-  unsigned long long best = ~0ull;
-  const int qy = oy + wr;
-#pragma unroll
-  for (int k = 0; k < S; ++k) {
-    const unsigned long long key = cand_key(s, acc[k], ox + lane * S + k, qy);
-    best = key < best ? key : best;
-  }
-  write_partial(s, best, red);
-}
-
-// Stage a rows x pitch window of image words for the partial-overlap search:
-// the alpha byte says whether the pixel may be used as a source (0: known and
-// in the image; 0xFF: unknown or outside the image, RGB bytes 0).
-__device__ inline void stage_tile_avail(const ImgState& s, uint32_t* dst, int x0, int y0, int rows,
-                                        int pitch) {
-  const int n = rows * pitch;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const int yy = y0 + i / pitch, xx = x0 + i % pitch;
-    uint32_t w = 0xff000000u;
-    if (xx >= 0 && xx < s.W && yy >= 0 && yy < s.H) {
-      const uint8_t o = s.omega[(size_t)yy * s.W + xx];
-      const uint32_t v = s.img[(size_t)yy * s.pitch + xx];
-      w = o ? 0xff000000u : v;
-    }
-    dst[i] = w;
-  }
+  write_partial(s, best_key<S>(s, acc, cnt, ox + lane * S, oy + wr), red);
 }
 
 // findBestPatch, partial-overlap variant (Algorithm 1 and Sec. 5.4): every
@@ -179,27 +197,8 @@ __global__ void __launch_bounds__(kSearchThreads) k_search_overlap(ImgState s) {
   const int ox = s.cx0 + blockIdx.x * TW, oy = s.cy0 + blockIdx.y * TH;
   const int tid = threadIdx.x;
 
-  // target patch: known pixels (words, bit masks per row) and unknown in-image pixels
-  if (tid < P) {
-    const int ty = py + tid - R;
-    uint32_t m = 0, u = 0;
-    for (int dx = 0; dx < P; ++dx) {
-      const int tx = px + dx - R;
-      uint32_t w = 0;
-      if (tx >= 0 && tx < s.W && ty >= 0 && ty < s.H) {
-        if (!s.omega[(size_t)ty * s.W + tx]) {
-          w = s.img[(size_t)ty * s.pitch + tx];
-          m |= 1u << dx;
-        } else {
-          u |= 1u << dx;
-        }
-      }
-      tgt[tid * P + dx] = w;
-    }
-    rowmask[tid] = m;
-    unkmask[tid] = u;
-  }
-  stage_tile_avail(s, src, ox - R, oy - R, SH, SW);
+  stage_target<P, P>(s, px, py, tgt, rowmask, unkmask);
+  stage_tile<SH, SW, true>(s, src, ox - R, oy - R);
   __syncthreads();
 
   const int lane = tid & 31, wr = tid >> 5;
@@ -258,80 +257,110 @@ __global__ void __launch_bounds__(kSearchThreads) k_search_overlap(ImgState s) {
   write_partial(s, best, red);
 }
 
-// Any radius up to kMaxRadius: the known target pixels are compacted into a
-// list in shared memory and each evaluation reads its source word from there.
-__global__ void __launch_bounds__(kGenThreads) k_search_generic(ImgState s) {
+// Any radius up to kMaxRadius, same tiles and threads.  A target row is taken
+// in chunks of eight columns: a chunk without a known pixel is skipped, one
+// that is all known runs without tests, another tests a bit per column; its
+// source words and target words arrive by five 128-bit shared loads for up to
+// 32 evaluations.  (A compacted list of known pixels, built by one thread and
+// read with one source load per evaluation, took 76 us a search at 512x384,
+// 25x25.)
+struct GenGeom {
+  int P, TP, SW, SH;
+  __host__ __device__ explicit GenGeom(int R)
+      : P(2 * R + 1), TP((2 * R + 1 + 7) & ~7), SW((kSearchTW + 2 * R + 15) & ~3), SH(kSearchTH + 2 * R) {}
+  __host__ __device__ size_t bytes() const { return (size_t)(SH * SW + P * TP + 3 * P) * sizeof(uint32_t); }
+};
+
+__global__ void __launch_bounds__(kSearchThreads) k_search_generic(ImgState s) {
   extern __shared__ __align__(16) uint32_t dyn[];
   __shared__ unsigned long long red[32];
-  __shared__ int nk_s;
   const Ctrl* c = s.ctrl;
   if (!loop_active(c)) return;
-  const int R = s.r, P = 2 * R + 1;
-  const int TW = kGenTW, TH = kGenTH, S = kGenS;
-  const int SW = TW + 2 * R, SH = TH + 2 * R;
-  uint32_t* src = dyn;                          // SH * SW
-  uint32_t* koff = dyn + SH * SW;               // P * P offsets into the tile
-  uint32_t* kval = koff + P * P;                // P * P target words
+  constexpr int S = kSearchS;
+  const int R = s.r;
+  const GenGeom g(R);
+  uint32_t* src = dyn;                  // SH x SW
+  uint32_t* tgt = src + g.SH * g.SW;    // P x TP, 0 where unknown
+  uint32_t* rmask = tgt + g.P * g.TP;   // P x 3: bits of the known columns
   const int px = c->px, py = c->py;
-  const int ox = s.cx0 + blockIdx.x * TW, oy = s.cy0 + blockIdx.y * TH;
-  const int tid = threadIdx.x;
-  if (tid == 0) {
-    int n = 0;
-    for (int dy = 0; dy < P; ++dy)
-      for (int dx = 0; dx < P; ++dx) {
-        const int tx = px + dx - R, ty = py + dy - R;
-        if (tx >= 0 && tx < s.W && ty >= 0 && ty < s.H) {
-          const size_t t = (size_t)ty * s.W + tx;
-          if (!s.omega[t]) {
-            koff[n] = dy * SW + dx;
-            kval[n] = s.img[(size_t)ty * s.pitch + tx];
-            ++n;
+  const int ox = s.cx0 + blockIdx.x * kSearchTW, oy = s.cy0 + blockIdx.y * kSearchTH;
+  const int tid = threadIdx.x, lane = tid & 31, wr = tid >> 5;
+  int cnt[S];
+  load_counts<S>(s, ox + lane * S, oy + wr, cnt);
+  for (int dy = wr; dy < g.P; dy += kSearchThreads / 32) {
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int dx = 32 * b + lane, tx = px + dx - R, ty = py + dy - R;
+      uint32_t w = 0;
+      bool known = false;
+      if (dx < g.P && tx >= 0 && tx < s.W && ty >= 0 && ty < s.H) {
+        const uint8_t o = s.omega[(size_t)ty * s.W + tx];
+        const uint32_t v = s.img[(size_t)ty * s.pitch + tx];
+        known = o == 0;
+        w = known ? v : 0u;
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, known);
+      if (dx < g.TP) tgt[dy * g.TP + dx] = w;
+      if (lane == 0) rmask[3 * dy + b] = m;
+    }
+  }
+  for (int yy = wr; yy < g.SH; yy += kSearchThreads / 32) {
+    const int y = oy - R + yy;
+#pragma unroll 4
+    for (int xx = lane; xx < g.SW; xx += 32) {
+      const int x = ox - R + xx;
+      src[yy * g.SW + xx] = x >= 0 && x < s.W && y >= 0 && y < s.H ? s.img[(size_t)y * s.pitch + x] : 0u;
+    }
+  }
+  __syncthreads();
+  uint32_t acc[S] = {0u, 0u, 0u, 0u};
+  for (int dy = 0; dy < g.P; ++dy) {
+    const uint32_t* srow = &src[(wr + dy) * g.SW + lane * S];
+    for (int ch = 0; ch < g.TP / 8; ++ch) {
+      const uint32_t m = (rmask[3 * dy + (ch >> 2)] >> (8 * (ch & 3))) & 0xffu;
+      if (m == 0u) continue;
+      uint32_t row[12], t[8];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) reinterpret_cast<uint4*>(row)[i] = reinterpret_cast<const uint4*>(srow + 8 * ch)[i];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        reinterpret_cast<uint4*>(t)[i] = reinterpret_cast<const uint4*>(&tgt[dy * g.TP + 8 * ch])[i];
+      if (m == 0xffu) {
+#pragma unroll
+        for (int dx = 0; dx < 8; ++dx) {
+#pragma unroll
+          for (int k = 0; k < S; ++k) {
+            const uint32_t d = __vabsdiffu4(t[dx], row[k + dx]);
+            acc[k] = __dp4a(d, d, acc[k]);
+          }
+        }
+      } else {
+#pragma unroll
+        for (int dx = 0; dx < 8; ++dx) {
+          if (m & (1u << dx)) {
+#pragma unroll
+            for (int k = 0; k < S; ++k) {
+              const uint32_t d = __vabsdiffu4(t[dx], row[k + dx]);
+              acc[k] = __dp4a(d, d, acc[k]);
+            }
           }
         }
       }
-    nk_s = n;
-  }
-  stage_tile(s, src, ox - R, oy - R, SH, SW);
-  __syncthreads();
-  const int nk = nk_s;
-  const int lane = tid & 31, wr = tid >> 5;
-  uint32_t acc[kGenS] = {0, 0};
-  const uint32_t* base = src + wr * SW + lane * S;
-  for (int k = 0; k < nk; ++k) {
-    const uint32_t a = kval[k];
-    const uint32_t* b = base + koff[k];
-#pragma unroll
-    for (int j = 0; j < S; ++j) {
-      const uint32_t d = __vabsdiffu4(a, b[j]);
-      acc[j] = __dp4a(d, d, acc[j]);
     }
   }
-  unsigned long long best = ~0ull;
-  const int qy = oy + wr;
-#pragma unroll
-  for (int j = 0; j < S; ++j) {
-    const unsigned long long key = cand_key(s, acc[j], ox + lane * S + j, qy);
-    best = key < best ? key : best;
-  }
-  write_partial(s, best, red);
-}
-
-static size_t generic_smem(int R) {
-  const int P = 2 * R + 1;
-  return (size_t)((kGenTH + 2 * R) * (kGenTW + 2 * R) + 2 * P * P) * sizeof(uint32_t);
+  write_partial(s, best_key<S>(s, acc, cnt, ox + lane * S, oy + wr), red);
 }
 
 cudaError_t prepare_search_plain(int r) {
   if (r <= 8) return cudaSuccess;
   return cudaFuncSetAttribute(k_search_generic, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)generic_smem(r));
+                              (int)GenGeom(r).bytes());
 }
 
 dim3 search_plain_grid(const ImgState& s) {
   const int cw = s.cx1 - s.cx0 + 1, ch = s.cy1 - s.cy0 + 1;
   if (cw <= 0 || ch <= 0) return dim3(0, 0, 1);
-  if (s.r <= 8) return dim3((cw + kSearchTW - 1) / kSearchTW, (ch + kSearchTH - 1) / kSearchTH, 1);
-  return dim3((cw + kGenTW - 1) / kGenTW, (ch + kGenTH - 1) / kGenTH, 1);
+  return dim3((cw + kSearchTW - 1) / kSearchTW, (ch + kSearchTH - 1) / kSearchTH, 1);
 }
 
 cudaError_t launch_search_plain(const ImgState& s, cudaStream_t st) {
@@ -361,7 +390,7 @@ cudaError_t launch_search_plain(const ImgState& s, cudaStream_t st) {
     case 7: k_search_plain<7><<<g, kSearchThreads, 0, st>>>(s); break;
     case 8: k_search_plain<8><<<g, kSearchThreads, 0, st>>>(s); break;
     default:
-      k_search_generic<<<g, kGenThreads, generic_smem(s.r), st>>>(s);
+      k_search_generic<<<g, kSearchThreads, GenGeom(s.r).bytes(), st>>>(s);
   }
   return cudaGetLastError();
 }
