@@ -41,9 +41,25 @@ __global__ void k_planes(ImgState s) {
     const int xl = (int)(e % s.tc_len);
     const size_t ry = e / s.tc_len;
     const int y = (int)(ry % s.prows), tx = (int)(ry / s.prows);
-    const int x = s.tc_xs0 + tx * s.tc_w + xl;
-    const uint32_t w = (x < s.W && y < s.H) ? __ldg(&s.img[(size_t)y * s.pitch + x]) : 0x00808080u;
+    const int f = s.tc_f > 1 ? min((xl >> 3) / s.tc_n1, s.tc_f) : 0;
+    const int x = s.tc_xs0 + 8 * (tx * s.tc_n - f * s.tc_n1) + xl, yi = y + f * s.tc_h;
+    const bool in = x < s.W && yi < s.H && (f == 0 || f < s.tc_f);
+    const uint32_t w = in ? __ldg(&s.img[(size_t)yi * s.pitch + x]) : 0x00808080u;
     plane_store_at(s, tx, y, xl, w);  // outside the image: 128 - 128 = 0 everywhere
+  }
+}
+
+// The validity bits from the counts; one warp per word.
+__global__ void k_vbits(ImgState s, int nwords) {
+  const int lane = threadIdx.x & 31, wpr = s.tc_n >> 2;
+  for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nwords; w += (gridDim.x * blockDim.x) >> 5) {
+    const int row = w / wpr, t = row >> 4, ty = t / s.tc_ntx, xt = (w - row * wpr) * 32 + lane;
+    const int f = s.tc_f > 1 ? min((xt >> 3) / s.tc_n1, s.tc_f) : 0;
+    const int x = s.tc_xs0 + 8 * ((t - ty * s.tc_ntx) * s.tc_n - f * s.tc_n1) + xt + s.r;
+    const int y = s.cy0 + ty * 16 + (row & 15) + f * s.tc_h;
+    const bool valid = f < s.tc_f && x >= s.cx0 && x <= s.cx1 && y <= s.cy1 && s.count[(size_t)y * s.pitch + x] == 0;
+    const unsigned bal = __ballot_sync(0xffffffffu, valid);
+    if (lane == 0) s.vbits[w] = bal;
   }
 }
 
@@ -52,6 +68,8 @@ cudaError_t launch_planes(const ImgState& s, cudaStream_t st) {
   const size_t n = (size_t)s.tc_ntx * s.prows * s.tc_len;
   const int blocks = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
   k_planes<<<blocks, 256, 0, st>>>(s);
+  const int nwords = s.tc_ntx * s.tc_nty * kTcRows * (s.tc_n / 4);
+  k_vbits<<<(nwords + 7) / 8 < 2048 ? (nwords + 7) / 8 : 2048, 256, 0, st>>>(s, nwords);
   return cudaGetLastError();
 }
 

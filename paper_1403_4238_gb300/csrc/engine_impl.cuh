@@ -384,7 +384,7 @@ struct EngSmemTail {
   int stop;
   int px, py;
   int a2row[17];  // tensor-core search: per target row, sum of the known pixels' squared shifted values
-  int tc_pref;  // tensor-core search: slots the producer prefetched for the next round
+  int tc_pref;    // tensor-core search: slots the producer prefetched for the next round
   int lim, status, err;  // leader: iteration limit, status and error word (the stop decision)
   uint8_t known[2][17 * 17];  // known flags of the last two targets (by round parity)
   ResPlan plan;               // resident mode: this CTA's units and tiles
@@ -546,149 +546,198 @@ __device__ inline bool ctrl_active(const Ctrl* c) {
 template <int R, int SRW, bool kLeadOnly = false>
 __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x);
 
-// The loop of a searching CTA in the tensor-core form (the image's state
-// block, the stop flag and the first target are in shared memory), compiled
-// as a function of its own with every phase inlined: a call would save and
-// restore the caller's registers through local memory, which misses L1
-// while shared memory takes nearly all of it.
+// The state of a CTA's tensor-core search that outlives a round: source rows
+// through the ring and tiles through the accumulator buffers so far (their
+// barriers' phases).
+struct TcRun {
+  TcArea a;
+  uint32_t rows, tiles;
+};
+
+// Where the tensor-core search keeps its state, from byte `off` of the CTA's
+// shared memory.  A ring with another slot count than the last image's starts
+// its phases over (every slot of an earlier image was consumed, so no barrier
+// has a pending phase).  Whole block.
 template <int R>
-__device__ __noinline__ void run_tc_search(const EngineArgs& ea, EngCtx& x, const TcTiles tt, TcArea tca, int ns) {
+__device__ __forceinline__ void tc_setup(TcRun& t, EngCtx& x, EngBars& bars, int off, int nb, int slot) {
+  using GT = TcEngGeom<R>;
+  uint8_t* area = eng_smem() + off;
+  t.a.a = area;
+  t.a.tpad = reinterpret_cast<uint16_t*>(area + GT::A_BYTES);
+  t.a.ring = area + GT::A_BYTES + GT::TPAD_BYTES;
+  t.a.nb = nb;
+  t.a.slot = slot;
+  t.rows = x.tc_rows;
+  t.tiles = x.tc_tiles;
+  if (x.tc_nb != nb) {
+    if (x.tc_nb != 0 && threadIdx.x == 0) {
+      for (int i = 0; i < kTcRing; ++i) {
+        mbar_inval(&bars.tc_full[i]);
+        mbar_inval(&bars.tc_empty[i]);
+        mbar_init(&bars.tc_full[i], 1);
+        mbar_init(&bars.tc_empty[i], 2);
+      }
+    }
+    fence_mbar_init();
+    t.rows = 0;
+  }
+  // the padded target table's columns outside the patch stay zero
+  for (int e = threadIdx.x; e < 4 * GT::P * GT::TW; e += kEngThreads) t.a.tpad[e] = 0;
+  __syncthreads();
+  x.tc_nb = nb;
+}
+
+// The k-th tile of searching CTA `rank` of ns, or -1.  Tiles go round-robin;
+// when the leader (the last of them) searches too, its first turn is its
+// speculative phase, which takes about as long as a tile.
+__device__ __forceinline__ int tc_tile_of(int k, int rank, int ns, int ntiles, bool lead_searches) {
+  const int v = rank + k * ns, t = lead_searches && v >= ns - 1 ? v - 1 : v;
+  return (lead_searches && v == ns - 1) || t >= ntiles ? -1 : t;
+}
+
+// One round of a CTA's tensor-core search for target (px, py): its tiles k0,
+// k0 + 1, ...; `pref` ring slots of the first one are already requested.
+// Returns the thread's best key; *bad (of this thread) when a bounded wait
+// gave up.  Whole block.
+template <int R>
+__device__ __forceinline__ unsigned long long tc_round(const ImgState& s, const TcTiles& tt, TcRun& tr,
+                                                       EngSmemTail& tl, uint32_t tmem, int px, int py, bool first,
+                                                       int k0, int pref, int rank, int ns, bool lead_searches,
+                                                       unsigned long long limit, int* bad_out) {
   using GT = TcEngGeom<R>;
   constexpr int P = GT::P, NSL = GT::NSL;
-  // the context lives in the kernel's local memory, which misses L1 (shared
-  // memory takes nearly all of it) and is re-read after every barrier or
-  // fence: keep working copies in registers, write them back at the end
-  uint8_t* const smem = eng_smem();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ntiles = tt.ntx * tt.nty, npre = min(tr.a.nb, NSL);
+  int n = 0;  // tiles of this round
+  while (tc_tile_of(k0 + n, rank, ns, ntiles, lead_searches) >= 0) ++n;
+  auto tile = [&](int k, int& tx, int& y0) {
+    const int t = tc_tile_of(k0 + k, rank, ns, ntiles, lead_searches), ty = t / tt.ntx;
+    tx = t - ty * tt.ntx;
+    y0 = s.cy0 + kTcRows * ty;
+    return t;
+  };
+  int bad = 0, tx, y0;
+  // the producer starts the first tile's rows at once, unless it
+  // prefetched them while the leader was updating
+  if (n > 0 && pref == 0 && warp == kEngWarps - 1 && lane == 0) {
+    tile(0, tx, y0);
+    if (!tc_produce<R>(s, tr.a, tl.bars, tx, y0, tr.rows, 0, npre, limit)) bad = 1;
+  }
+  tc_stage_target<R>(s, tr.a.tpad, tl.a2row, px, py);
+  __syncthreads();
+  // every warp but the producer's (its copies are in flight) writes A
+  tc_build_a<R>(tr.a.a, tr.a.tpad, first, 32 * (kEngWarps - 1));
+  __syncthreads();
+  int a2 = 0;
+#pragma unroll
+  for (int dy = 0; dy < P; ++dy) a2 += tl.a2row[dy];
+  unsigned long long best = ~0ull;
+  auto bits_of = [&](int t) { return s.vbits + (size_t)t * kTcRows * (tt.N / 4); };
+  if (warp == kEngWarps - 1) {
+    for (int k = 0; k < n && !bad; ++k) {
+      tile(k, tx, y0);
+      if (lane == 0 && !tc_produce<R>(s, tr.a, tl.bars, tx, y0, tr.rows + (uint32_t)(k * NSL), k == 0 ? npre : 0, NSL, limit))
+        bad = 1;
+    }
+    __syncwarp();
+  } else if (warp == kEngWarps - 2 || warp == kEngWarps - 3) {
+    for (int k = 0; k < n && !bad; ++k) {
+      const uint32_t c = tr.tiles + (uint32_t)k, b = c & 1u, g0 = tr.rows + (uint32_t)(k * NSL);
+      // the buffer's previous tile has been read
+      if (c >= 2u && !__all_sync(0xffffffffu, mbar_wait(&tl.bars.tc_free[b], ((c >> 1) - 1u) & 1u, limit))) bad = 1;
+      tc_fence_after();
+      if (warp == kEngWarps - 2 ? !tc_issue<R, 0>(tr.a, tl.bars, tt.N, tmem + 256u * b, &tl.bars.tc_done[b], g0, limit)
+                                : !tc_issue<R, 1>(tr.a, tl.bars, tt.N, tmem + 256u * b, &tl.bars.tc_done[b], g0, limit))
+        bad = 1;
+    }
+    // the one warp that waits for the last tile's MMAs (the others sleep at
+    // the block barrier: spinning warps would take issue slots from the
+    // issuers)
+    if (warp == kEngWarps - 2 && n > 0) {
+      const uint32_t c = tr.tiles + (uint32_t)(n - 1);
+      if (!mbar_wait(&tl.bars.tc_done[c & 1u], (c >> 1) & 1u, limit)) bad = 1;
+    }
+  } else if (warp < kTcReaders) {
+    for (int k = 0; k + 1 < n && !bad; ++k) {
+      const int t = tile(k, tx, y0);
+      const uint32_t c = tr.tiles + (uint32_t)k, b = c & 1u;
+      const uint2 bits = tc_bits_load(bits_of(t), tt.N, kTcReaders / 4);
+      if (!__all_sync(0xffffffffu, mbar_wait(&tl.bars.tc_done[b], (c >> 1) & 1u, limit))) {
+        bad = 1;
+        break;
+      }
+      tc_fence_after();
+      best = tc_epilogue<R>(s, tmem + 256u * b, tt, kTcReaders / 4, a2, bits, y0, tx, best);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&tl.bars.tc_free[b]);
+    }
+  }
+  uint2 bits = make_uint2(0u, 0u);
+  const int ng = (tt.N & 31) ? 2 : 4;  // column groups of the last tile's read-back
+  if (n > 0) {
+    const int t = tile(n - 1, tx, y0);
+    if (warp < 4 * ng) bits = tc_bits_load(bits_of(t), tt.N, ng);
+  }
+  tc_fence_before();
+  if (__syncthreads_or(bad)) {
+    *bad_out = 1;
+    return ~0ull;
+  }
+  tc_fence_after();
+  if (n > 0) {
+    const uint32_t b = (tr.tiles + (uint32_t)(n - 1)) & 1u;
+    if (warp < 4 * ng) best = tc_epilogue<R>(s, tmem + 256u * b, tt, ng, a2, bits, y0, tx, best);
+    tc_fence_before();
+    __syncwarp();
+    // (all 16 warps read this tile; the block's reduction precedes the next
+    // tile's MMAs, so eight arrivals complete the phase)
+    if (warp < kTcReaders && lane == 0) mbar_arrive(&tl.bars.tc_free[b]);
+  }
+  tr.tiles += (uint32_t)n;
+  tr.rows += (uint32_t)(n * NSL);
+  *bad_out = 0;
+  return best;
+}
+
+// The loop of a CTA that only searches, in the tensor-core form (the image's
+// state block, the stop flag and the first target are in shared memory),
+// compiled as a function of its own with every phase inlined: a call would
+// save and restore the caller's registers through local memory, which misses
+// L1 while shared memory takes nearly all of it.
+template <int R>
+__device__ __noinline__ void run_tc_search(const EngineArgs& ea, EngCtx& x, const TcTiles tt, int nb, int slot, int ns,
+                                           bool lead_searches) {
+  using GT = TcEngGeom<R>;
+  // working copies of the context (it lives in the kernel's local memory)
   const uint32_t tmem = x.tmem;
-  uint32_t tc_rows = x.tc_rows, tc_tiles = x.tc_tiles;
-  int tc_pref = x.tc_pref, tc_nb = x.tc_nb;
   unsigned long long* const tpart = x.tpart;
-  EngSmemTail& tl = *reinterpret_cast<EngSmemTail*>(smem);
+  EngSmemTail& tl = *reinterpret_cast<EngSmemTail*>(eng_smem());
   const ImgState& s = tl.img;
-  Ctrl* c = s.ctrl;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int rank = x.rank;
   TeamCtl* tc = x.tc;
   const unsigned long long limit = ea.wait_limit_ns;
   unsigned epoch = x.epoch;
-  // A | padded target | ring | validity bits
-  uint8_t* area = smem + kHeadBytes;
-  tca.a = area;
-  tca.tpad = reinterpret_cast<uint16_t*>(area + GT::A_BYTES);
-  tca.ring = area + GT::A_BYTES + GT::TPAD_BYTES;
-  tca.bits = reinterpret_cast<uint32_t*>(tca.ring + (size_t)tca.nb * tca.slot);
-  if (tc_nb != tca.nb) {
-    // the ring's phases are counted from the slot sequence number modulo the
-    // slot count: a new slot count restarts them (every slot of an earlier
-    // image was consumed, so no barrier has a pending phase)
-    if (tc_nb != 0 && tid == 0) {
-      for (int i = 0; i < kTcRing; ++i) {
-        mbar_inval(&tl.bars.tc_full[i]);
-        mbar_inval(&tl.bars.tc_empty[i]);
-        mbar_init(&tl.bars.tc_full[i], 1);
-        mbar_init(&tl.bars.tc_empty[i], 2);
-      }
-    }
-    fence_mbar_init();
-    __syncthreads();
-    tc_nb = tca.nb;
-    tc_rows = 0;
-  }
-  const int ntiles = tt.ntx * tt.nty;
-  const int first_y = s.cy0 + kTcRows * (rank / tt.ntx), first_tx = rank % tt.ntx;  // this CTA's first tile
-  const int npre = min(tca.nb, NSL);
-  int prev_px = -1000000, prev_py = -1000000;
-  int round = 0;
+  TcRun tr;
+  tc_setup<R>(tr, x, tl.bars, (int)kHeadBytes, nb, slot);
+  const int ntiles = tt.ntx * tt.nty, t0 = tc_tile_of(0, rank, ns, ntiles, lead_searches);
+  const int first_y = s.cy0 + kTcRows * (t0 / tt.ntx), first_tx = t0 % tt.ntx;  // this CTA's first tile
+  const int npre = min(nb, GT::NSL);
+  int pref = 0;
+  bool first = true;
   while (!tl.stop) {
     const int px = tl.px, py = tl.py;
-    const bool first = round == 0;
-    int bad = 0;
-    // the producer starts the first tile's rows at once, unless it
-    // prefetched them while the leader was updating
-    if (tc_pref == 0 && warp == kEngWarps - 1 && lane == 0 &&
-        !tc_produce<R>(s, tca, tl.bars, first_tx, first_y, tc_rows, 0, npre, limit))
-      bad = 1;
-    if (first) {
-      tc_bits_init<R>(s, tt, tca.bits, tca.ntl, rank, ns);
-      // the padded target table's columns outside the patch stay zero
-      for (int e = tid; e < 4 * P * GT::TW; e += kEngThreads) tca.tpad[e] = 0;
-      __syncthreads();
-    }
-    // target patch: warp dy reads row dy (lane = dx) and writes its
-    // entries of the padded target table (R' G' B' and the known flag, zero
-    // where unknown) and the row's share of A2
-    for (int dy = warp; dy < P; dy += kEngWarps) {
-      const int tx = px + lane - R, ty = py + dy - R;
-      uint32_t w = 0;
-      bool known = false;
-      if (lane < P && tx >= 0 && tx < s.W && ty >= 0 && ty < s.H) {
-        const uint8_t o = __ldcg(&s.omega[(size_t)ty * s.W + tx]);
-        const uint32_t v = __ldcg(&s.img[(size_t)ty * s.pitch + tx]);
-        known = o == 0;
-        w = known ? v : 0u;
-      }
-      int sq = 0;
-      if (lane < P) {
-        const int d0 = known ? (int)(w & 255u) - 128 : 0, d1 = known ? (int)((w >> 8) & 255u) - 128 : 0,
-                  d2 = known ? (int)((w >> 16) & 255u) - 128 : 0;
-        sq = d0 * d0 + d1 * d1 + d2 * d2;
-        uint16_t* tp = tca.tpad + dy * GT::TW + 8 + lane;
-        tp[0] = (uint16_t)bf16_of_int(d0);
-        tp[P * GT::TW] = (uint16_t)bf16_of_int(d1);
-        tp[2 * P * GT::TW] = (uint16_t)bf16_of_int(d2);
-        tp[3 * P * GT::TW] = (uint16_t)bf16_of_int(known ? 1 : 0);
-      }
-      sq = __reduce_add_sync(0xffffffffu, sq);
-      if (lane == 0) tl.a2row[dy] = sq;
-    }
-    __syncthreads();
-    // every warp but the producer's (its copies are in flight) writes A
-    tc_build_a<R>(tca.a, tca.tpad, first, 32 * (kEngWarps - 1));
-    __syncthreads();
-    int a2 = 0;
-#pragma unroll
-    for (int dy = 0; dy < P; ++dy) a2 += tl.a2row[dy];
-    unsigned long long best = ~0ull;
-    for (int kt = 0; kt < tca.ntl; ++kt) {
-      const int t = rank + kt * ns;
-      if (t >= ntiles) break;  // uniform
-      const int y0 = s.cy0 + kTcRows * (t / tt.ntx), xs = tt.xs0 + 8 * tt.N * (t % tt.ntx);
-      const uint32_t g0 = tc_rows;
-      if (warp == kEngWarps - 1) {
-        if (lane == 0 && !tc_produce<R>(s, tca, tl.bars, t % tt.ntx, y0, g0, kt == 0 ? npre : 0, NSL, limit))
-          bad = 1;
-        __syncwarp();
-      } else if (warp == kEngWarps - 2) {
-        if (!(tt.N == 128 ? tc_issue<R, 0, 128>(tca, tl.bars, tmem, g0, limit)
-                          : tc_issue<R, 0, 64>(tca, tl.bars, tmem, g0, limit)))
-          bad = 1;
-        // the one warp that waits for the tile's MMAs (the others sleep at
-        // the block barrier: spinning warps would take issue slots from the
-        // issuers)
-        if (!mbar_wait(&tl.bars.tc_done, tc_tiles & 1u, limit)) bad = 1;
-      } else if (warp == kEngWarps - 3) {
-        if (!(tt.N == 128 ? tc_issue<R, 1, 128>(tca, tl.bars, tmem, g0, limit)
-                          : tc_issue<R, 1, 64>(tca, tl.bars, tmem, g0, limit)))
-          bad = 1;
-      } else if (kt == 0 && !first) {
-        // validity bits near the previous fill: needed only by the read-back
-        tc_bits_refresh<R>(s, tt, tca.bits, rank, ns, prev_px, prev_py, 32 * (kEngWarps - 3));
-      }
-      tc_fence_before();
-      if (__syncthreads_or(bad)) break;
-      tc_fence_after();
-      best = tc_epilogue<R>(s, tmem, tt.N, a2, tca.bits + kt * tc_bit_words(tt.N), y0, xs, best);
-      tc_fence_before();
-      ++tc_tiles;
-      tc_rows += NSL;
-      __syncthreads();  // the accumulators are read before the next tile's MMAs
-    }
-    tc_pref = 0;
+    int bad;
+    unsigned long long best = tc_round<R>(s, tt, tr, tl, tmem, px, py, first, 0, pref, rank, ns, lead_searches, limit, &bad);
+    first = false;
     best = block_min_u64(best, tl.red64);
-    ++round;
-    if (bad && tid == 0) atomicExch(ea.err, INPAINT_ERR_TIMEOUT);
-    if (tid == 0 && rank + 1 != ea.withhold) st_relaxed64(&tpart[rank], key_tag(best, epoch));
-    if (rank == 0 && tid == 0) atomicAdd(&c->tc_rounds, 1);
+    if (tid == 0) {
+      if (bad) atomicExch(ea.err, INPAINT_ERR_TIMEOUT);
+      if (rank + 1 != ea.withhold) st_relaxed64(&tpart[rank], key_tag(best, epoch));
+      if (rank == 0) atomicAdd(&s.ctrl->tc_rounds, 1);
+    }
+    if (bad) break;
     if (warp == kEngWarps - 1 && lane == 0) {
       // once the leader has written this round's fill, the next round's
       // first source rows are final: request them now, while the leader
@@ -699,7 +748,7 @@ __device__ __noinline__ void run_tc_search(const EngineArgs& ea, EngCtx& x, cons
         if ((int)(ld_acquire(&tc->copied) - (epoch + 1u)) >= 0) {
           asm volatile("fence.proxy.async.global;" ::: "memory");
           n = npre;
-          if (!tc_produce<R>(s, tca, tl.bars, first_tx, first_y, tc_rows, 0, n, limit))
+          if (!tc_produce<R>(s, tr.a, tl.bars, first_tx, first_y, tr.rows, 0, n, limit))
             atomicExch(ea.err, INPAINT_ERR_TIMEOUT);
           break;
         }
@@ -715,33 +764,59 @@ __device__ __noinline__ void run_tc_search(const EngineArgs& ea, EngCtx& x, cons
       tl.py = (int)((v >> 47) & 0x7fff);
     }
     ++epoch;
-    prev_px = px;
-    prev_py = py;
     __syncthreads();
-    tc_pref = tl.tc_pref;
+    pref = tl.tc_pref;
     if (lane == 0) asm volatile("fence.proxy.async.global;" ::: "memory");
   }
-  if (tc_pref > 0) {
+  if (pref > 0) {
     // the loop stopped with a prefetch in flight: let it land and release
     // its slots (two arrivals stand for the two issuers' commits)
     if (warp == kEngWarps - 1 && lane == 0) {
-      for (int h = 0; h < tc_pref; ++h) {
-        const uint32_t g = tc_rows + (uint32_t)h;
-        const int slot = (int)(g % (uint32_t)tca.nb);
-        if (!mbar_wait(&tl.bars.tc_full[slot], (g / tca.nb) & 1u, limit)) atomicExch(ea.err, INPAINT_ERR_TIMEOUT);
-        mbar_arrive(&tl.bars.tc_empty[slot]);
-        mbar_arrive(&tl.bars.tc_empty[slot]);
+      for (int h = 0; h < pref; ++h) {
+        const uint32_t g = tr.rows + (uint32_t)h;
+        const int sl = (int)(g % (uint32_t)nb);
+        if (!mbar_wait(&tl.bars.tc_full[sl], (g / (uint32_t)nb) & 1u, limit)) atomicExch(ea.err, INPAINT_ERR_TIMEOUT);
+        mbar_arrive(&tl.bars.tc_empty[sl]);
+        mbar_arrive(&tl.bars.tc_empty[sl]);
       }
     }
-    tc_rows += (uint32_t)tc_pref;
-    tc_pref = 0;
+    tr.rows += (uint32_t)pref;
     __syncthreads();
   }
   x.epoch = epoch;
-  x.tc_rows = tc_rows;
-  x.tc_tiles = tc_tiles;
-  x.tc_pref = tc_pref;
-  x.tc_nb = tc_nb;
+  x.tc_rows = tr.rows;
+  x.tc_tiles = tr.tiles;
+}
+
+// A searching leader's share of one tensor-core round (its state at byte `off`
+// of shared memory); the block's best key.
+template <int R>
+__device__ __noinline__ unsigned long long tc_lead_share(const EngineArgs& ea, EngCtx& x, const TcTiles tt, int off,
+                                                         int nb, int slot, int ns, int px, int py, bool first) {
+  EngSmemTail& tl = *reinterpret_cast<EngSmemTail*>(eng_smem());
+  const ImgState& s = tl.img;
+  TcRun tr;
+  if (first) {
+    tc_setup<R>(tr, x, tl.bars, off, nb, slot);
+  } else {
+    uint8_t* area = eng_smem() + off;
+    tr.a.a = area;
+    tr.a.tpad = reinterpret_cast<uint16_t*>(area + TcEngGeom<R>::A_BYTES);
+    tr.a.ring = area + TcEngGeom<R>::A_BYTES + TcEngGeom<R>::TPAD_BYTES;
+    tr.a.nb = nb;
+    tr.a.slot = slot;
+    tr.rows = x.tc_rows;
+    tr.tiles = x.tc_tiles;
+  }
+  int bad;
+  unsigned long long best = tc_round<R>(s, tt, tr, tl, x.tmem, px, py, first, 1, 0, x.rank, ns, true, ea.wait_limit_ns, &bad);
+  if (bad && threadIdx.x == 0) {
+    atomicExch(ea.err, INPAINT_ERR_TIMEOUT);
+    tl.err = INPAINT_ERR_TIMEOUT;
+  }
+  x.tc_rows = tr.rows;
+  x.tc_tiles = tr.tiles;
+  return block_min_u64(best, tl.red64);
 }
 
 // The loop of a leader that does not search, compiled as a function of its
@@ -794,30 +869,30 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
   // searches its share after the speculative phase, which is short next to
   // a CTA's share of such a search.  A CTA that neither searches nor leads
   // idles until the image is done.
-  // Tensor-core form (an image given planes, a team of two or more): every
-  // CTA but the leader searches whole tiles, when its A strips, a ring of
-  // at least four source-row slots and the validity bits of its tiles fit.
-  const TcTiles tt = s.planes ? tc_tiles(s) : TcTiles{0, 0, 0, 0};
+  // Tensor-core form (an image given planes): whole tiles, round-robin, when
+  // the A strips and a ring of at least four source-row slots fit beside a
+  // searching leader's update state.  The leader searches too when every CTA
+  // has three tiles or more.  An image that leaves the choice of the form to
+  // the engine (tc_auto) takes the one with the lower estimate for this team.
+  const TcTiles tt = s.planes ? tc_tiles(s) : TcTiles{0, 0, 0, 0, 1, 0};
   const int tc_ntiles = tt.ntx * tt.nty;
-  TcArea tca{nullptr, nullptr, nullptr, nullptr, 0, 0, 0};
+  const int tc_slot_b = s.planes ? tc_slot(tt.N, R) : 1;
+  constexpr int kUpdB = (int)(((upd_smem_bytes<R>() + 127) / 128) * 128);
+  const bool tc_lead = tsize == 1 || tc_ntiles >= 3 * tsize;
+  const int tc_off = (int)kHeadBytes + (tc_lead && rank == tsize - 1 ? kUpdB : 0);
+  int tc_nb = 0;
   bool tcmode = false;
-  if (s.planes && ea.tc_cols >= 2 * tt.N && tsize >= 2 && tc_ntiles > 0) {
-    const int nsq = min(tsize - 1, tc_ntiles);
-    const int ntl = (tc_ntiles + nsq - 1) / nsq;
-    const long long avail = (long long)x.smem_bytes - (long long)kHeadBytes;
-    const int slot = tc_slot(tt.N, R);
-    const long long fixed =
-        TcEngGeom<R>::A_BYTES + TcEngGeom<R>::TPAD_BYTES + (long long)ntl * tc_bit_words(tt.N) * 4;
-    const long long nbl = (avail - fixed) / slot;
-    if (ntl <= 8 && nbl >= 4) {
-      tcmode = true;
-      tca.nb = nbl < kTcRing ? (int)nbl : kTcRing;
-      tca.ntl = ntl;
-      tca.slot = slot;
-    }
+  if (s.planes && ea.tc_cols >= kTcCols && tc_ntiles > 0) {
+    const int fixed = (int)kHeadBytes + TcEngGeom<R>::A_BYTES + TcEngGeom<R>::TPAD_BYTES;
+    const int tc_ns = tc_lead ? min(tsize, tc_ntiles) : min(tsize - 1, tc_ntiles);
+    tcmode = ((int)x.smem_bytes - fixed - (tc_lead ? kUpdB : 0)) / tc_slot_b >= 4 &&
+             (!s.tc_auto || tc_round_cycles(s, tc_ns) < plain_round_cycles(s, tsize));
+    tc_nb = min(kTcRing, ((int)x.smem_bytes - (tc_off - (int)kHeadBytes) - fixed) / tc_slot_b);
   }
-  const bool lead_searches = !tcmode && (tsize == 1 || nbatch >= 8 * tsize);
-  const int ns = tcmode ? min(tsize - 1, tc_ntiles) : lead_searches ? tsize : min(tsize - 1, nbatch);
+  const bool lead_searches = tcmode ? tc_lead : tsize == 1 || nbatch >= 8 * tsize;
+  const int ns = tcmode         ? (tc_lead ? min(tsize, tc_ntiles) : min(tsize - 1, tc_ntiles))
+                 : lead_searches ? tsize
+                                 : min(tsize - 1, nbatch);
   const bool leader = rank == tsize - 1;
   const bool searcher = rank < ns;
   if constexpr (!kLeadOnly) {
@@ -825,14 +900,14 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
       run_lead_only<R, SRW>(ea, j, x);
       return;
     }
-    if (tcmode && searcher) {
+    if (tcmode && searcher && !leader) {
       if (tid == 0) {
         tl.stop = !ctrl_active(c) || __ldcg(ea.err) != 0;
         tl.px = __ldcg(&c->px);
         tl.py = __ldcg(&c->py);
       }
       __syncthreads();
-      run_tc_search<R>(ea, x, tt, tca, ns);
+      run_tc_search<R>(ea, x, tt, tc_nb, tc_slot_b, ns, tc_lead);
       return;
     }
   }
@@ -893,6 +968,11 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
       tma_load_2d(ct, cmap, xb - G::COFF + G::BWC * gx, s.cy0 + B * gy, bar);
     };
     const bool first = round == 0;
+    if (tcmode) {
+      ++round;
+      if (tid == 0 && ns == 1) atomicAdd(&c->tc_rounds, 1);  // (else the team's first searcher counts)
+      return tc_lead_share<R>(ea, x, tt, tc_off, tc_nb, tc_slot_b, ns, px, py, first);
+    }
     if (!resident && tid == 0 && b0 < nbatch) issue(b0, slot_pix(0), cnt_t[0], &tl.bars.full[0]);
         if (resident && first) {
       // the source windows of every band segment (plain 16-byte loads;
@@ -1019,7 +1099,10 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
       }
     }
     ++round;
-    if (!ok && tid == 0) atomicExch(ea.err, INPAINT_ERR_TIMEOUT);
+    if (!ok && tid == 0) {
+      atomicExch(ea.err, INPAINT_ERR_TIMEOUT);
+      tl.err = INPAINT_ERR_TIMEOUT;  // (a searching leader: its key would be partial)
+    }
     return block_min_u64(best, tl.red64);
   };
 
@@ -1055,7 +1138,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
         const unsigned long long best = gather_keys(tpart, ns, epoch, ea.err, limit, &late);
         if (lane == 0) {
           usm.t_keys = globaltimer();
-          set_source<R>(s, usm, best, late);
+          set_source<R>(s, usm, best, late || tl.err != 0);
         }
         __syncwarp();
       }

@@ -50,7 +50,10 @@ __global__ void __launch_bounds__(kEngThreads, 1) k_engine(EngineArgs ea) {
         mbar_init(&bars->tc_full[i], 1);
         mbar_init(&bars->tc_empty[i], 2);  // one commit from each issuer
       }
-      mbar_init(&bars->tc_done, 2);
+      for (int b = 0; b < 2; ++b) {
+        mbar_init(&bars->tc_done[b], 2);
+        mbar_init(&bars->tc_free[b], kTcReaders);
+      }
     }
   }
   fence_mbar_init();

@@ -292,7 +292,7 @@ int setup_engine(inpaint_ctx* c) {
   ea.partials = c->d_epart;
   ea.err = c->d_err;
   ea.wait_limit_ns = 4000000000ull;  // 4 s: far beyond any iteration
-  ea.tc_cols = c->st.planes ? 256 : 0;  // X and S accumulators of N <= 128 columns each
+  ea.tc_cols = c->st.planes ? kTcCols : 0;
   c->eng_ready = true;
   return INPAINT_OK;
 }
@@ -347,7 +347,7 @@ int read_ctrl(const inpaint_ctx* c) {
 }
 
 int create_impl(const uint8_t* rgb, int W, int H, int rgb_stride, const uint8_t* mask,
-                int mask_stride, int r, const inpaint_options* opt, inpaint_ctx** out) {
+                int mask_stride, int r, const inpaint_options* opt, inpaint_ctx** out, bool tc_auto = false) {
   if (!out) return INPAINT_ERR_ARG;
   *out = nullptr;
   if (!rgb || !mask || rgb_stride < 3 * W || mask_stride < W) {
@@ -420,6 +420,16 @@ int create_impl(const uint8_t* rgb, int W, int H, int rgb_stride, const uint8_t*
   s.trace_cap = (int)n_omega + 1;
   const dim3 g = search_plain_grid(s);
   s.n_partial = (int)(g.x * g.y);
+  size_t plane_bytes = 0;
+  if (o.form == INPAINT_FORM_TC || tc_auto) {
+    // the tensor-core search reads five BF16 planes of the image
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return fail(INPAINT_ERR_CUDA);
+    s.tc_auto = tc_auto ? 1 : 0;
+    plane_bytes = tc_plane_layout(s, tc_auto ? 0 : sms - 1);
+  }
   if (o.form == INPAINT_FORM_TC) {
     if (prepare_search_tc(s, &c->tc) != cudaSuccess) {
       g_last_error = "tensor-core search set-up failed";
@@ -439,13 +449,13 @@ int create_impl(const uint8_t* rgb, int W, int H, int rgb_stride, const uint8_t*
     g_last_error = "device allocation failed";
     return fail(INPAINT_ERR_NOMEM);
   }
-  if (o.form == INPAINT_FORM_TC) {
-    // the tensor-core search reads five BF16 planes of the image
-    const size_t np = tc_plane_layout(s);
-    if (np > 0 && !alloc_n(c, s.planes, np)) {
+  if (plane_bytes > 0) {
+    uint8_t* planes = nullptr;
+    if (!alloc_n(c, planes, plane_bytes)) {
       g_last_error = "device allocation failed";
       return fail(INPAINT_ERR_NOMEM);
     }
+    tc_bind_planes(s, planes);
   }
   if (prepare_search_plain(r) != cudaSuccess) return fail(INPAINT_ERR_CUDA);
   *out = c;
@@ -636,13 +646,18 @@ int inpaint_time_search(inpaint_ctx* c, int form, int reps, double* ms_per_searc
   TcPlan plan{};
   uint16_t* tmp_planes = nullptr;  // a plain-form context has no planes: build them for the timing
   if (form == INPAINT_FORM_TC) {
+    if (!s.planes) {
+      int dev = 0, sms = 0;
+      CK(cudaGetDevice(&dev));
+      CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+      const size_t bytes = tc_plane_layout(s, sms - 1);
+      if (bytes > 0) {
+        CK(cudaMalloc(&tmp_planes, bytes));
+        tc_bind_planes(s, tmp_planes);
+      }
+    }
     CK(prepare_search_tc(s, &plan));
     s.n_partial = plan.grid;
-    if (!s.planes && s.n_partial > 0) {
-      const size_t np = tc_plane_layout(s);
-      CK(cudaMalloc(&tmp_planes, np * sizeof(uint16_t)));
-      s.planes = tmp_planes;
-    }
     CK(launch_planes(s, c->stream));
   } else {
     CK(prepare_search_plain(s.r));
@@ -885,14 +900,28 @@ struct EngineSet {
 
 namespace {
 
-// Teams: with fewer images than CTAs every image gets its own team, sized in
-// proportion to its estimated work (|Omega| x valid candidates, i.e. the
-// exhaustive evaluation count up to the patch area), at least one CTA; with
-// more images than CTAs every CTA is a team and images are dealt longest
-// first to the least loaded team.
-void plan_teams(const std::vector<double>& work, int grid, std::vector<int>& team_size,
-                std::vector<int>& img_team, std::vector<std::vector<int>>& team_imgs) {
-  const int n = (int)work.size();
+// Estimated cycles that image s (n_omega pixels left) takes on a team of
+// `size` CTAs: about 2 |Omega| / P^2 iterations, each a search round of the
+// form the engine would choose and 16,000 cycles of leader work, which a
+// leader that also searches does before and after its share.
+double image_cycles(const ImgState& s, double n_omega, int size) {
+  const int P = 2 * s.r + 1;
+  const double iters = 2.0 * n_omega / (P * P) + 1.0;
+  const bool lead = size == 1 || s.tc_ntx * s.tc_nty >= 3 * size;
+  double round = plain_round_cycles(s, size);
+  if (s.planes) round = std::min(round, (double)tc_round_cycles(s, lead ? size : size - 1));
+  return iters * (round + 16000.0);
+}
+
+// Teams: with fewer images than CTAs every image gets its own team: one CTA
+// each, then every further CTA to the image that would end last; with more
+// images than CTAs every CTA is a team and images are dealt longest first to
+// the least loaded team.
+void plan_teams(const std::vector<const ImgState*>& st, const std::vector<double>& n_omega, int grid,
+                std::vector<int>& team_size, std::vector<int>& img_team, std::vector<std::vector<int>>& team_imgs) {
+  const int n = (int)st.size();
+  std::vector<double> work(n);
+  for (int i = 0; i < n; ++i) work[i] = image_cycles(*st[i], n_omega[i], 1);
   img_team.assign(n, 0);
   if (n >= grid) {
     team_size.assign(grid, 1);
@@ -909,8 +938,6 @@ void plan_teams(const std::vector<double>& work, int grid, std::vector<int>& tea
     }
     return;
   }
-  // one CTA per image, then each further CTA to the team whose work per CTA
-  // is largest (minimises the largest work per CTA, i.e. the batch's end)
   team_size.assign(n, 1);
   team_imgs.assign(n, {});
   std::priority_queue<std::pair<double, int>> pq;
@@ -919,7 +946,7 @@ void plan_teams(const std::vector<double>& work, int grid, std::vector<int>& tea
     const int i = pq.top().second;
     pq.pop();
     team_size[i] += 1;
-    pq.emplace(work[i] / team_size[i], i);
+    pq.emplace(image_cycles(*st[i], n_omega[i], team_size[i]), i);
   }
   for (int i = 0; i < n; ++i) {
     img_team[i] = i;
@@ -942,15 +969,17 @@ int grid_for(const std::vector<inpaint_ctx*>& cs, int* grid) {
   return INPAINT_OK;
 }
 
-// Plans the teams for the contexts (work estimates from their last control
-// block mirrors) and uploads everything the engine reads.
-int engine_set_prepare(EngineSet& es, const std::vector<inpaint_ctx*>& cs, const std::vector<double>& work,
+// Plans the teams for the contexts (n_omega: the pixels each has left, from
+// their last control block mirrors) and uploads everything the engine reads.
+int engine_set_prepare(EngineSet& es, const std::vector<inpaint_ctx*>& cs, const std::vector<double>& n_omega,
                        const inpaint_options& opt, DevAlloc& da, cudaStream_t st) {
   const int n = (int)cs.size();
   int rc = grid_for(cs, &es.grid);
   if (rc) return rc;
   std::vector<std::vector<int>> team_imgs;
-  plan_teams(work, es.grid, es.team_size, es.img_team, team_imgs);
+  std::vector<const ImgState*> states;
+  for (inpaint_ctx* c : cs) states.push_back(&c->st);
+  plan_teams(states, n_omega, es.grid, es.team_size, es.img_team, team_imgs);
   es.n_teams = (int)es.team_size.size();
   const int G = es.grid, T = es.n_teams;
   std::vector<ImgState> imgs(n);
@@ -1029,6 +1058,7 @@ int engine_set_prepare(EngineSet& es, const std::vector<inpaint_ctx*>& cs, const
   ea.partials = d_part;
   ea.err = es.d_err;
   ea.wait_limit_ns = 4000000000ull;
+  ea.tc_cols = kTcCols;
   return INPAINT_OK;
 }
 
@@ -1098,7 +1128,11 @@ int make_member(const inpaint_image& im, const inpaint_options& base, cudaStream
   o.loop_mode = INPAINT_LOOP_ENGINE;
   inpaint_ctx* c = nullptr;
   int rc = create_impl(im.rgb, im.width, im.height, im.rgb_stride_bytes, im.mask, im.mask_stride_bytes,
-                       im.patch_radius, &o, &c);
+                       im.patch_radius, &o, &c, true);
+  if (rc >= 0 && launch_planes(c->st, st) != cudaSuccess) {
+    inpaint_destroy(c);
+    return INPAINT_ERR_CUDA;
+  }
   if (rc < 0) {
     char buf[200];
     snprintf(buf, sizeof buf, "image %d: %s", index, g_last_error.c_str());
@@ -1119,9 +1153,7 @@ int make_member(const inpaint_image& im, const inpaint_options& base, cudaStream
   return INPAINT_OK;
 }
 
-double work_of(const Ctrl& h) {
-  return (double)std::max(1, h.remaining) * std::max(1, h.n_valid);
-}
+double left_of(const Ctrl& h) { return (double)std::max(1, h.remaining); }
 
 }  // namespace
 
@@ -1199,7 +1231,8 @@ void build_batch_graphs(inpaint_batch* b) {
     for (int i = 0; i < b->n; ++i) {
       inpaint_ctx* c = b->ctx[i];
       if (launch_init(c->st, c->orig_rgb, 3 * c->W, c->orig_mask, c->W, c->sat, nullptr,
-                      b->aux[i % inpaint_batch::kBatchAux]) != cudaSuccess)
+                      b->aux[i % inpaint_batch::kBatchAux]) != cudaSuccess ||
+          launch_planes(c->st, b->aux[i % inpaint_batch::kBatchAux]) != cudaSuccess)
         return false;
     }
     for (int k = 0; k < inpaint_batch::kBatchAux; ++k)
@@ -1258,7 +1291,7 @@ int batch_create_impl(const inpaint_image* images, int n, const inpaint_options*
     const int rc = make_member(images[i], b->opt, b->stream, i, &c);
     if (rc < 0) return fail(rc);
     b->ctx.push_back(c);
-    work[i] = work_of(*c->h_ctrl);
+    work[i] = left_of(*c->h_ctrl);
   }
   const int rc = engine_set_prepare(b->es, b->ctx, work, b->opt, b->da, b->stream);
   if (rc < 0) return fail(rc);
@@ -1288,8 +1321,10 @@ int inpaint_batch_reset(inpaint_batch* b) {
     CK(cudaStreamSynchronize(b->stream));
     return INPAINT_OK;
   }
-  for (inpaint_ctx* c : b->ctx)
+  for (inpaint_ctx* c : b->ctx) {
     CK(launch_init(c->st, c->orig_rgb, 3 * c->W, c->orig_mask, c->W, c->sat, nullptr, b->stream));
+    CK(launch_planes(c->st, b->stream));
+  }
   CK(cudaStreamSynchronize(b->stream));
   return INPAINT_OK;
 }
@@ -1395,9 +1430,17 @@ struct SrvReq {
 };
 
 // Upper estimate of a request's device memory (the buffers create_impl and
-// the batch member copy allocate, about 48 bytes per pixel plus the trace).
-size_t est_bytes(int W, int H, int n_omega) {
-  return (size_t)W * H * 48 + (size_t)(n_omega + 1) * sizeof(inpaint_step_info) + (1u << 20);
+// the batch member copy allocate: about 48 bytes per pixel, the tensor-core
+// search's planes, the trace).
+size_t est_bytes(int W, int H, int r, int n_omega) {
+  ImgState s{};
+  s.W = W;
+  s.H = H;
+  s.r = r;
+  s.cx0 = s.cy0 = r;
+  s.cx1 = W - 1 - r;
+  s.cy1 = H - 1 - r;
+  return (size_t)W * H * 48 + tc_plane_layout(s, 0) + (size_t)(n_omega + 1) * sizeof(inpaint_step_info) + (1u << 20);
 }
 
 }  // namespace
@@ -1405,7 +1448,7 @@ size_t est_bytes(int W, int H, int n_omega) {
 // Device time budget of one serving tick: long enough to amortise the
 // launch and the host's admission work, short enough to admit new requests
 // often.
-constexpr unsigned long long kServerTickNs = 20000000ull;
+constexpr unsigned long long kServerTickNs = 8000000ull;
 
 struct inpaint_server {
   size_t budget = 0, used = 0;
@@ -1455,7 +1498,7 @@ struct inpaint_server {
           SrvReq* q = queue.front();
           int n_omega = 0;
           for (uint8_t m : q->mask) n_omega += m != 0;
-          const size_t b = est_bytes(q->W, q->H, n_omega);
+          const size_t b = est_bytes(q->W, q->H, q->r, n_omega);
           if (used + b > budget && !(active.empty() && admit.empty())) break;
           queue.pop_front();
           q->bytes = b;
@@ -1505,7 +1548,7 @@ struct inpaint_server {
         std::vector<double> work;
         for (SrvReq* q : act) {
           cs.push_back(q->ctx);
-          work.push_back(work_of(*q->ctx->h_ctrl));
+          work.push_back(left_of(*q->ctx->h_ctrl));
         }
         int rc = engine_set_prepare(es, cs, work, opt, da, stream);
         if (rc >= 0) rc = engine_set_run(es, cs, iters_per_tick, stream, kServerTickNs);

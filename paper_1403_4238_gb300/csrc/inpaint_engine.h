@@ -27,46 +27,100 @@ __host__ __device__ constexpr int eng_count_width(int srw) { return eng_batch_co
 
 // Tensor-core search of the engine (Sec. 3, Eq. 3-4 as correlations; the
 // exact BF16 form of the tensor-core search).  A tile is kTcRows candidate
-// rows x 8N candidate columns (N = 64 or 128): the MMA's M = 128 rows are
-// 16 candidate rows x 8 column shifts, its N columns blocks of 8 candidate
-// columns.  Tiles are numbered row-major; searching CTA k of a team takes
-// tiles k, k + ns, ...
+// rows x 8N candidate columns (N a multiple of 16, at most 128): the MMA's
+// M = 128 rows are 16 candidate rows x 8 column shifts, its N columns blocks
+// of 8 candidate columns.  Tiles are numbered row-major; searching CTA k of a
+// team takes tiles k, k + ns, ...
 constexpr int kTcRows = 16;
 constexpr int kTcRing = 8;  // most slots of the shared-memory ring
 constexpr int kTcRps = 2;   // source rows per ring slot (one bulk copy)
+constexpr int kTcReaders = 8;  // warps that read a tile's accumulators beside the next tile's MMAs
+constexpr int kTcCols = 512;   // tensor-memory columns: two buffers of X and S, N <= 128 columns each
 struct TcTiles {
-  int N;         // MMA N: 8-column candidate blocks per tile (64 or 128)
+  int N;         // MMA N: 8-column candidate blocks per tile
   int ntx, nty;  // tiles per row / per column of the candidate rectangle
   int xs0;       // first source column of tile column 0 (a multiple of 8)
+  int n1, h;     // folds: block pitch and row distance of one (n1 = N without folds)
 };
 __host__ __device__ inline int tc_chunks(int r) { return (2 * r + 1 + 14) / 8; }  // 8-tap chunks of a row
 __host__ __device__ inline TcTiles tc_tiles(const ImgState& s) {
-  TcTiles t{0, 0, 0, 0};
-  if (s.cx1 < s.cx0 || s.cy1 < s.cy0) return t;
-  t.xs0 = (s.cx0 - s.r) & ~7;
-  const int wneed = s.cx1 - s.r - t.xs0 + 1;  // candidate columns from the first tile's column 0
-  t.ntx = (wneed + 1023) / 1024;
-  t.N = (wneed + 8 * t.ntx - 1) / (8 * t.ntx) <= 64 ? 64 : 128;
-  t.nty = (s.cy1 - s.cy0 + kTcRows) / kTcRows;
-  return t;
+  return TcTiles{s.tc_n, s.tc_ntx, s.tc_nty, s.tc_xs0, s.tc_n1, s.tc_h};
 }
-// Plane geometry of an image (fills the tc_* fields and prows of s): the
-// segment of tile column tx is columns [xs0 + 8N tx, + 8 (N + chunks - 1)),
-// the rows every tile reads (y0 - r .. y0 + 15 + r) all exist.  Returns the
-// plane elements to allocate (0: no tile).
-__host__ __device__ inline size_t tc_plane_layout(ImgState& s) {
-  const TcTiles t = tc_tiles(s);
-  if (t.ntx == 0) return 0;
-  s.tc_xs0 = t.xs0;
-  s.tc_w = 8 * t.N;
-  s.tc_len = 8 * (t.N + tc_chunks(s.r) - 1);
-  s.tc_ntx = t.ntx;
-  const int hr = s.cy0 + kTcRows * t.nty + s.r;
-  s.prows = hr > s.H ? hr : s.H;
-  return (size_t)t.ntx * s.prows * 5 * s.tc_len;
+// Measured cycles of one 128 x N x 16 MMA: 74 at N = 128, 59 at N = 64.
+__host__ __device__ inline float tc_mma_cycles(int N) { return 43.5f + 0.24f * (float)N; }
+
+// Tile and plane geometry of an image (the tc_* fields and prows of s); the
+// rows every tile reads (y0 - r .. y0 + 15 + r) all exist.  want > 0: the tiles
+// of one image spread over `want` CTAs, so the number of tile columns (narrower
+// tiles, cheaper MMAs) is what makes the round shortest; want 0: throughput of
+// small teams, so a narrow image is folded until its tiles are close to
+// N = 128 wide (an MMA costs 59 cycles at N = 64 and 74 at N = 128: half the
+// cycles per candidate for an image 500 wide).  Returns the bytes to allocate
+// for the planes and the validity bits behind them (0: no tile).
+inline size_t tc_plane_layout(ImgState& s, int want) {
+  s.tc_ntx = s.tc_nty = 0;
+  if (s.cx1 < s.cx0 || s.cy1 < s.cy0) return 0;
+  const int nc = tc_chunks(s.r), rows = s.cy1 - s.cy0 + 1;
+  s.tc_xs0 = (s.cx0 - s.r) & ~7;
+  const int wneed = s.cx1 - s.r - s.tc_xs0 + 1;  // candidate columns from the first tile's column 0
+  const int least = (wneed + 1023) / 1024;
+  auto n_of = [&](int ntx) { return ((wneed + 8 * ntx - 1) / (8 * ntx) + 15) & ~15; };
+  int ntx = least, folds = 1;
+  const int nty1 = (rows + kTcRows - 1) / kTcRows;
+  if (want > 0) {
+    float best = 0.f;
+    for (int t = least; t <= least + 4 && n_of(t) >= 32; ++t) {
+      const float c = tc_mma_cycles(n_of(t)) * (float)((t * nty1 + want - 1) / want);
+      if (t == least || c < best) {
+        best = c;
+        ntx = t;
+      }
+    }
+  } else if (least == 1) {
+    const int n1 = (wneed + 7) / 8 + nc - 1;
+    folds = n1 <= 64 ? 128 / n1 : 1;
+    folds = folds < nty1 ? folds : nty1;
+  }
+  s.tc_f = folds;
+  s.tc_ntx = ntx;
+  if (folds > 1) {
+    s.tc_n1 = (wneed + 7) / 8 + nc - 1;
+    s.tc_n = (folds * s.tc_n1 + 15) & ~15;
+    s.tc_nty = (nty1 + folds - 1) / folds;
+  } else {
+    s.tc_n1 = s.tc_n = n_of(ntx);
+    s.tc_nty = nty1;
+  }
+  s.tc_h = kTcRows * s.tc_nty;
+  s.tc_len = 8 * (s.tc_n + nc - 1);
+  const int hr = s.cy0 + s.tc_h + s.r;
+  s.prows = folds == 1 && hr < s.H ? s.H : hr;
+  return (size_t)s.tc_ntx * s.prows * 5 * s.tc_len * 2 + (size_t)s.tc_ntx * s.tc_nty * kTcRows * s.tc_n;
 }
-// The five planes of the image's current pixels (run before every engine
-// launch of an image in the tensor-core form).
+// The planes and the bits in a buffer of that size.
+inline void tc_bind_planes(ImgState& s, void* p) {
+  s.planes = static_cast<uint16_t*>(p);
+  s.vbits = reinterpret_cast<uint32_t*>(s.planes + (size_t)s.tc_ntx * s.prows * 5 * s.tc_len);
+}
+
+// Estimated cycles of one search round on ns searching CTAs, for the choice
+// between the forms and for the batch plan.  Tensor-core form: a tile is
+// (rows) x (MMAs a row), after about 4,500 cycles of target staging, A strips
+// and read-back.  Plain form: about 0.6 of the patch known, 24 evaluations a
+// cycle and CTA (the streaming mode of one- and two-CTA teams measured 20-28 of
+// the 64 its two instructions allow), after 2,500 cycles.
+__host__ __device__ inline float tc_round_cycles(const ImgState& s, int ns) {
+  const int P = 2 * s.r + 1, nc = tc_chunks(s.r), tiles = s.tc_ntx * s.tc_nty;
+  const float tile = (float)((kTcRows + P - 1) * ((3 * nc + 1) / 2 + nc)) * tc_mma_cycles(s.tc_n) + 300.f;
+  return 4500.f + (float)((tiles + ns - 1) / ns) * tile;
+}
+__host__ __device__ inline float plain_round_cycles(const ImgState& s, int ns) {
+  const float P2 = (float)((2 * s.r + 1) * (2 * s.r + 1));
+  return 2500.f + (float)(s.cx1 - s.cx0 + 1) * (float)(s.cy1 - s.cy0 + 1) * 0.6f * P2 / (24.f * (float)ns);
+}
+
+// The five planes of the image's current pixels and the validity bits (run
+// before every engine launch of an image in the tensor-core form).
 cudaError_t launch_planes(const ImgState& s, cudaStream_t st);
 
 // Per-team synchronisation words (global memory).
@@ -104,7 +158,8 @@ struct EngBars {
   uint64_t full[2];               // TMA completion of the two streaming stages
   uint64_t tc_full[kTcRing];      // tensor-core search: source rows landed in ring slot
   uint64_t tc_empty[kTcRing];     // their MMAs (both issuers) completed: the slot is free
-  uint64_t tc_done;               // a tile's MMAs (both issuers) completed
+  uint64_t tc_done[2];            // a tile's MMAs (both issuers) completed, per accumulator buffer
+  uint64_t tc_free[2];            // the buffer's accumulators have been read (kTcReaders warps)
   uint32_t tmem;                  // tensor-memory base written by tcgen05.alloc
   uint32_t pad;
 };

@@ -44,12 +44,6 @@ constexpr int kSearchTW = 128;
 constexpr int kSearchTH = 8;
 constexpr int kSearchS = 4;
 constexpr int kSearchThreads = (kSearchTW / kSearchS) * kSearchTH;  // 256
-// Generic (large-radius) search tile.
-constexpr int kGenTW = 64;
-constexpr int kGenTH = 8;
-constexpr int kGenS = 2;
-constexpr int kGenThreads = (kGenTW / kGenS) * kGenTH;  // 256
-
 constexpr int kUpdThreads = 512;
 
 struct PrioBest {
@@ -151,14 +145,20 @@ struct ImgState {
   Ctrl* ctrl;
   inpaint_step_info* trace;
   unsigned long long* partial;  // per-CTA best search key of the iteration
-  // tensor-core form in the persistent engine (null otherwise): five BF16
-  // planes of the image, R' G' B' (byte - 128) and the square sum
-  // sq = sum_c (byte_c - 128)^2 as 256 hi and lo (sq = 256 hi + lo), stored per tile column tx
-  // of the search (columns [tc_xs0 + tx * tc_w, + tc_len)) as
-  // [tx][row y < prows][plane][tc_len], zero outside W x H, so that two
-  // source rows of a tile are one contiguous copy
+  // tensor-core form (null otherwise): five BF16 planes of the image, R' G' B'
+  // (byte - 128) and the square sum sq = sum_c (byte_c - 128)^2 as 256 hi and
+  // lo (sq = 256 hi + lo), stored per tile column tx of the search (columns
+  // [tc_xs0 + tx * 8 tc_n, + tc_len)) as [tx][row y < prows][plane][tc_len],
+  // zero outside W x H, so that two source rows of a tile are one contiguous
+  // copy.  A narrow image can be folded: fold f < tc_f holds the rows from
+  // f * tc_h on, 8 tc_n1 columns to the right of fold f - 1 (tc_ntx is 1 then).
   uint16_t* planes;
-  int prows, tc_xs0, tc_w, tc_len, tc_ntx;
+  int prows, tc_xs0, tc_len, tc_ntx, tc_nty, tc_n, tc_n1, tc_f, tc_h;
+  // with the planes: one validity bit per candidate of every search tile,
+  // [tile][16 rows][8 tc_n bits] (set iff the centre lies in the search
+  // rectangle and count is 0)
+  uint32_t* vbits;
+  int tc_auto;  // 1: the engine chooses per launch between this form and the plain one
 };
 
 // BF16 bits of an integer with at most 8 significant bits (|v| <= 256, or
@@ -184,13 +184,36 @@ __device__ inline void plane_store_at(const ImgState& s, int tx, int y, int o, u
 }
 
 // Pixel (x, y) changed to w: its copies in the (at most two) tile columns
-// whose segments hold column x.
+// whose segments hold column x, or in the (at most two) folds that hold row y.
 __device__ inline void plane_store(const ImgState& s, int x, int y, uint32_t w) {
   const int xl = x - s.tc_xs0;
   if (xl < 0) return;  // left of every tile's source columns
+  if (s.tc_f > 1) {
+    if (xl >= 8 * s.tc_n1) return;
+    for (int f = 0, yf = y; f < s.tc_f && yf >= 0; ++f, yf -= s.tc_h)
+      if (yf < s.prows) plane_store_at(s, 0, yf, xl + 8 * f * s.tc_n1, w);
+    return;
+  }
   int tx = 0;  // (a few tile columns: cheaper than a division)
-  while (tx + 1 < s.tc_ntx && xl >= (tx + 1) * s.tc_w) ++tx;
-  for (; tx >= 0 && xl - tx * s.tc_w < s.tc_len; --tx) plane_store_at(s, tx, y, xl - tx * s.tc_w, w);
+  while (tx + 1 < s.tc_ntx && xl >= (tx + 1) * 8 * s.tc_n) ++tx;
+  for (; tx >= 0 && xl - tx * 8 * s.tc_n < s.tc_len; --tx) plane_store_at(s, tx, y, xl - tx * 8 * s.tc_n, w);
+}
+
+// Candidate centre (x, y) of the search rectangle became valid: its bit.
+__device__ inline void vbit_set(const ImgState& s, int x, int y) {
+  int xt = x - s.r - s.tc_xs0, yl = y - s.cy0, tx = 0;
+  if (s.tc_f > 1) {
+    while (yl >= s.tc_h) {
+      yl -= s.tc_h;
+      xt += 8 * s.tc_n1;
+    }
+  } else {
+    while (tx + 1 < s.tc_ntx && xt >= 8 * s.tc_n) {
+      xt -= 8 * s.tc_n;
+      ++tx;
+    }
+  }
+  atomicOr(&s.vbits[(((yl >> 4) * s.tc_ntx + tx) * 16 + (yl & 15)) * (s.tc_n >> 2) + (xt >> 5)], 1u << (xt & 31));
 }
 
 __host__ __device__ inline uint32_t pack_rgb(uint32_t r, uint32_t g, uint32_t b) {

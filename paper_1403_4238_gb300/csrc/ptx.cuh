@@ -102,34 +102,19 @@ __device__ inline uint64_t tc_desc(uint32_t addr, uint32_t lbo, uint32_t sbo) {
          ((uint64_t)(sbo >> 4) << 32) | (1ull << 46);
 }
 
-// Same MMA with the descriptors given as 32-bit halves (the high halves of
-// every A and every B descriptor are the same constants), so a fully
-// unrolled issue loop only adds immediates to the low halves; ACC = 0
-// overwrites the accumulator.
-template <int ACC>
-__device__ inline void tc_mma_lo(uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                 uint32_t idesc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-      "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
-      "setp.ne.b32 p, %6, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}" ::"r"(d),
-      "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "n"(ACC)
-      : "memory");
-}
-
-// The same MMA issued by one elected lane of a converged warp (the whole
-// warp runs the issue loop, so the descriptor arithmetic stays warp-uniform).
-template <int ACC>
+// An MMA with the descriptors given as 32-bit halves (the high halves of every
+// A and every B descriptor are the same constants), issued by one elected lane
+// of a converged warp (the whole warp runs the issue loop, so the descriptor
+// arithmetic stays warp-uniform); acc false overwrites the accumulator.
 __device__ inline void tc_mma_lo_elect(uint32_t d, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                       uint32_t idesc) {
+                                       uint32_t idesc, bool acc) {
   asm volatile(
       "{\n\t.reg .pred p, e;\n\t.reg .b64 da, db;\n\t"
       "elect.sync _|e, 0xffffffff;\n\t"
       "mov.b64 da, {%1, %2};\n\tmov.b64 db, {%3, %4};\n\t"
       "setp.ne.b32 p, %6, 0;\n\t"
       "@e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}" ::"r"(d),
-      "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "n"(ACC)
+      "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"((uint32_t)acc)
       : "memory");
 }
 

@@ -30,7 +30,8 @@ constexpr int kTcHeadBytes = (int)((sizeof(TcHead) + 127) / 128 * 128);
 
 template <int R>
 __host__ __device__ inline int tc_fixed_bytes(int N) {
-  return kTcHeadBytes + TcEngGeom<R>::A_BYTES + TcEngGeom<R>::TPAD_BYTES + tc_bit_words(N) * 4;
+  (void)N;
+  return kTcHeadBytes + TcEngGeom<R>::A_BYTES + TcEngGeom<R>::TPAD_BYTES;
 }
 
 template <int R>
@@ -43,23 +44,21 @@ __global__ void __launch_bounds__(kEngThreads, 1) k_search_tc(ImgState s, int nb
   const Ctrl* c = s.ctrl;
   if (!loop_active(c)) return;
   const TcTiles tt = tc_tiles(s);
-  const int t = blockIdx.x, ntiles = tt.ntx * tt.nty;
-  const int tx = t % tt.ntx, y0 = s.cy0 + kTcRows * (t / tt.ntx), xs = tt.xs0 + 8 * tt.N * tx;
+  const int t = blockIdx.x;
+  const int tx = t % tt.ntx, y0 = s.cy0 + kTcRows * (t / tt.ntx);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   TcArea ta;
   ta.a = sm + kTcHeadBytes;
   ta.tpad = reinterpret_cast<uint16_t*>(ta.a + GT::A_BYTES);
   ta.ring = ta.a + GT::A_BYTES + GT::TPAD_BYTES;
-  ta.bits = reinterpret_cast<uint32_t*>(ta.ring + (size_t)nb * slot);
   ta.nb = nb;
-  ta.ntl = 1;
   ta.slot = slot;
   if (tid == 0) {
     for (int i = 0; i < nb; ++i) {
       mbar_init(&h.bars.tc_full[i], 1);
       mbar_init(&h.bars.tc_empty[i], 2);  // one commit from each issuer
     }
-    mbar_init(&h.bars.tc_done, 2);
+    mbar_init(&h.bars.tc_done[0], 2);
   }
   fence_mbar_init();
   if (warp == 0) tc_alloc(&h.bars.tmem, 256);
@@ -72,34 +71,9 @@ __global__ void __launch_bounds__(kEngThreads, 1) k_search_tc(ImgState s, int nb
   int bad = 0;
   // the producer starts the tile's first rows at once
   if (warp == kEngWarps - 1 && lane == 0 && !tc_produce<R>(s, ta, h.bars, tx, y0, 0u, 0, npre, kTcWaitNs)) bad = 1;
-  tc_bits_init<R>(s, tt, ta.bits, 1, t, ntiles);
   for (int e = tid; e < 4 * P * GT::TW; e += kEngThreads) ta.tpad[e] = 0;
   __syncthreads();
-  // target patch: warp dy reads row dy (lane = dx) into the padded table
-  for (int dy = warp; dy < P; dy += kEngWarps) {
-    const int qx = px + lane - R, qy = py + dy - R;
-    uint32_t w = 0;
-    bool known = false;
-    if (lane < P && qx >= 0 && qx < s.W && qy >= 0 && qy < s.H) {
-      const uint8_t o = __ldcg(&s.omega[(size_t)qy * s.W + qx]);
-      const uint32_t v = __ldcg(&s.img[(size_t)qy * s.pitch + qx]);
-      known = o == 0;
-      w = known ? v : 0u;
-    }
-    int sq = 0;
-    if (lane < P) {
-      const int d0 = known ? (int)(w & 255u) - 128 : 0, d1 = known ? (int)((w >> 8) & 255u) - 128 : 0,
-                d2 = known ? (int)((w >> 16) & 255u) - 128 : 0;
-      sq = d0 * d0 + d1 * d1 + d2 * d2;
-      uint16_t* tp = ta.tpad + dy * GT::TW + 8 + lane;
-      tp[0] = (uint16_t)bf16_of_int(d0);
-      tp[P * GT::TW] = (uint16_t)bf16_of_int(d1);
-      tp[2 * P * GT::TW] = (uint16_t)bf16_of_int(d2);
-      tp[3 * P * GT::TW] = (uint16_t)bf16_of_int(known ? 1 : 0);
-    }
-    sq = __reduce_add_sync(0xffffffffu, sq);
-    if (lane == 0) h.a2row[dy] = sq;
-  }
+  tc_stage_target<R>(s, ta.tpad, h.a2row, px, py);
   __syncthreads();
   // every warp but the producer's (its copies are in flight) writes A
   tc_build_a<R>(ta.a, ta.tpad, true, 32 * (kEngWarps - 1));
@@ -111,20 +85,18 @@ __global__ void __launch_bounds__(kEngThreads, 1) k_search_tc(ImgState s, int nb
     if (lane == 0 && !tc_produce<R>(s, ta, h.bars, tx, y0, 0u, npre, NSL, kTcWaitNs)) bad = 1;
     __syncwarp();
   } else if (warp == kEngWarps - 2) {
-    if (!(tt.N == 128 ? tc_issue<R, 0, 128>(ta, h.bars, tmem, 0u, kTcWaitNs)
-                      : tc_issue<R, 0, 64>(ta, h.bars, tmem, 0u, kTcWaitNs)))
-      bad = 1;
-    if (!mbar_wait(&h.bars.tc_done, 0u, kTcWaitNs)) bad = 1;  // the tile's MMAs
+    if (!tc_issue<R, 0>(ta, h.bars, tt.N, tmem, &h.bars.tc_done[0], 0u, kTcWaitNs)) bad = 1;
+    if (!mbar_wait(&h.bars.tc_done[0], 0u, kTcWaitNs)) bad = 1;  // the tile's MMAs
   } else if (warp == kEngWarps - 3) {
-    if (!(tt.N == 128 ? tc_issue<R, 1, 128>(ta, h.bars, tmem, 0u, kTcWaitNs)
-                      : tc_issue<R, 1, 64>(ta, h.bars, tmem, 0u, kTcWaitNs)))
-      bad = 1;
+    if (!tc_issue<R, 1>(ta, h.bars, tt.N, tmem, &h.bars.tc_done[0], 0u, kTcWaitNs)) bad = 1;
   }
+  const int ng = (tt.N & 31) ? 2 : 4;  // column groups of eight columns at a time
+  const uint2 bits = warp < 4 * ng ? tc_bits_load(s.vbits + (size_t)t * kTcRows * (tt.N / 4), tt.N, ng) : make_uint2(0u, 0u);
   tc_fence_before();
   const bool failed = __syncthreads_or(bad) != 0;
   tc_fence_after();
   unsigned long long best = ~0ull;
-  if (!failed) best = tc_epilogue<R>(s, tmem, tt.N, a2, ta.bits, y0, xs, best);
+  if (!failed && warp < 4 * ng) best = tc_epilogue<R>(s, tmem, tt, ng, a2, bits, y0, tx, best);
   best = block_min_u64(best, h.red64);
   if (tid == 0) {
     s.partial[t] = best;

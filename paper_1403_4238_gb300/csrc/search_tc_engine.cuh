@@ -11,7 +11,7 @@
 // (|X| <= 17^2 * 3 * 128^2, S <= 17^2 * 49152), so the FP32 accumulation is
 // exact and the SSD equals the CUDA-core form's bit for bit.
 //
-// One MMA (M = 128, N = 64 or 128, K = 16, BF16 operands in shared memory,
+// One MMA (M = 128, N = 16 .. 128, K = 16, BF16 operands in shared memory,
 // FP32 accumulators in tensor memory) takes one source row y of a tile
 // whose candidate rows are y0 .. y0 + 15 and whose candidate columns start
 // at xs + R:
@@ -32,13 +32,15 @@
 //    planes) or S (256 hi and lo of one chunk against the same mask strip:
 //    a leading byte offset of 0 in A); lane m, column n is candidate
 //    (y0 + m / 8, xs + 8 n + m % 8 + R).
-// Per tile one producer thread copies the tile's source rows into a ring of
+// One producer thread copies the tiles' source rows into a ring of
 // shared-memory slots (one bulk copy of two rows, five plane segments each,
-// from the planes' tiled layout), two issuer threads issue the X and the S
-// MMAs of a slot's rows once they have landed and free the slot with
-// tcgen05.commit, and then all 16 warps read the accumulators back
-// (tcgen05.ld), test validity against bits kept in shared memory and keep
-// the smallest (SSD << 32 | idx) key.  The read-back works in FP32:
+// from the planes' tiled layout), two issuer warps issue the X and the S MMAs
+// of a slot's rows once they have landed and free the slot with
+// tcgen05.commit.  Accumulators are read back (tcgen05.ld), tested against the
+// tile's validity bits and reduced to the smallest (SSD << 32 | idx) key: by
+// eight warps beside the next tile's MMAs, which fill the other of two
+// accumulator buffers, and by all 16 warps after a CTA's last tile.  The
+// read-back works in FP32:
 // fl(fl(S - 2X) + A2) is exact whenever the SSD is below 2^24 (then |S - 2X|
 // < 2^24 too, as A2 < 2^24) and at least 2^24 otherwise (rounding is
 // monotone), so a best value below 2^24 is the exact minimum; a warp with a
@@ -73,10 +75,8 @@ struct TcEngGeom {
 // of five segments).
 __host__ __device__ inline int tc_lrow(int N, int r) { return 16 * (N + tc_chunks(r) - 1); }
 __host__ __device__ inline int tc_slot(int N, int r) { return (kTcRps * 5 * tc_lrow(N, r) + 16 + 127) & ~127; }
-// Validity-bit words of one tile: kTcRows rows of 8N bits.
-__host__ __device__ inline int tc_bit_words(int N) { return kTcRows * N / 4; }
 
-// Where a tensor-core search keeps its state: A | padded target | ring | bits.
+// Where a tensor-core search keeps its state: A | padded target | ring.
 // The padded target table (written by the searcher's target staging):
 // tpad[(p * P + k) * TW + 8 + jj] = w_p(k, jj) for p < 4 (R' G' B', the
 // known flag) and jj in [-8, 24), zero outside the patch or where unknown.
@@ -84,57 +84,40 @@ struct TcArea {
   uint8_t* a;
   uint16_t* tpad;
   uint8_t* ring;
-  uint32_t* bits;
   int nb;    // ring slots
-  int ntl;   // tiles of this CTA
   int slot;  // bytes per slot
 };
 
-// Validity bits of this CTA's tiles from the counts (whole block).
+// The target patch at (px, py) into the padded table, and per target row its
+// share of A2 (whole block; a barrier must follow).  Warp dy reads row dy.
 template <int R>
-__device__ __forceinline__ void tc_bits_init(const ImgState& s, const TcTiles& tt, uint32_t* bits, int ntl, int rank,
-                                          int ns) {
-  const int bw = tt.N / 4, ntiles = tt.ntx * tt.nty;
-  for (int e = threadIdx.x; e < ntl * kTcRows * bw; e += blockDim.x) {
-    const int kt = e / (kTcRows * bw), i = (e / bw) % kTcRows, w = e % bw;
-    const int t = rank + kt * ns;
-    uint32_t v = 0;
-    if (t < ntiles) {
-      const int qy = s.cy0 + kTcRows * (t / tt.ntx) + i;
-      const int qx0 = tt.xs0 + 8 * tt.N * (t % tt.ntx) + 32 * w + R;
-      if (qy <= s.cy1) {
-        // all 32 loads in flight together (one L2 round trip)
-        const int32_t* row = s.count + (size_t)qy * s.pitch;
-        int cnt[32];
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          const int qx = qx0 + k;
-          cnt[k] = (qx >= s.cx0 && qx <= s.cx1) ? __ldcg(&row[qx]) : 1;
-        }
-#pragma unroll
-        for (int k = 0; k < 32; ++k) v |= (cnt[k] == 0 ? 1u : 0u) << k;
-      }
+__device__ __forceinline__ void tc_stage_target(const ImgState& s, uint16_t* tpad, int* a2row, int px, int py) {
+  using G = TcEngGeom<R>;
+  constexpr int P = G::P;
+  const int lane = threadIdx.x & 31;
+  for (int dy = threadIdx.x >> 5; dy < P; dy += kEngWarps) {
+    const int tx = px + lane - R, ty = py + dy - R;
+    uint32_t w = 0;
+    bool known = false;
+    if (lane < P && tx >= 0 && tx < s.W && ty >= 0 && ty < s.H) {
+      const uint8_t o = __ldcg(&s.omega[(size_t)ty * s.W + tx]);
+      const uint32_t v = __ldcg(&s.img[(size_t)ty * s.pitch + tx]);
+      known = o == 0;
+      w = known ? v : 0u;
     }
-    bits[e] = v;
-  }
-}
-
-// Candidates within 2R of the previous target may have become valid (the
-// fill only makes pixels known): set their bits (threads [0, nthr)).
-template <int R>
-__device__ __forceinline__ void tc_bits_refresh(const ImgState& s, const TcTiles& tt, uint32_t* bits, int rank, int ns,
-                                             int ppx, int ppy, int nthr) {
-  constexpr int NCW = 4 * R + 1;
-  const int bw = tt.N / 4;
-  for (int e = threadIdx.x; e < NCW * NCW; e += nthr) {
-    const int qx = ppx + e % NCW - 2 * R, qy = ppy + e / NCW - 2 * R;
-    if (qx < s.cx0 || qx > s.cx1 || qy < s.cy0 || qy > s.cy1) continue;
-    const int xl = qx - R - tt.xs0;
-    const int t = ((qy - s.cy0) / kTcRows) * tt.ntx + xl / (8 * tt.N);
-    if (t % ns != rank) continue;
-    if (__ldcg(&s.count[(size_t)qy * s.pitch + qx]) != 0) continue;
-    const int kt = t / ns, i = (qy - s.cy0) % kTcRows, x = xl % (8 * tt.N);
-    atomicOr(&bits[(kt * kTcRows + i) * bw + (x >> 5)], 1u << (x & 31));
+    int sq = 0;
+    if (lane < P) {
+      const int d0 = known ? (int)(w & 255u) - 128 : 0, d1 = known ? (int)((w >> 8) & 255u) - 128 : 0,
+                d2 = known ? (int)((w >> 16) & 255u) - 128 : 0;
+      sq = d0 * d0 + d1 * d1 + d2 * d2;
+      uint16_t* tp = tpad + dy * G::TW + 8 + lane;
+      tp[0] = (uint16_t)bf16_of_int(d0);
+      tp[P * G::TW] = (uint16_t)bf16_of_int(d1);
+      tp[2 * P * G::TW] = (uint16_t)bf16_of_int(d2);
+      tp[3 * P * G::TW] = (uint16_t)bf16_of_int(known ? 1 : 0);
+    }
+    sq = __reduce_add_sync(0xffffffffu, sq);
+    if (lane == 0) a2row[dy] = sq;
   }
 }
 
@@ -187,22 +170,31 @@ __device__ __forceinline__ bool tc_produce(const ImgState& s, const TcArea& ta, 
 }
 
 // Issuer of the X MMAs (KIND 0) or the S MMAs (KIND 1) of a tile's NRS source
-// rows, then a commit to the tile's done barrier.  One whole warp (the
-// descriptor arithmetic is warp-uniform; one elected lane issues).  N is a
-// template parameter so that every descriptor is a base plus an immediate.
-template <int R, int KIND, int N>
-__device__ __forceinline__ bool tc_issue(const TcArea& ta, EngBars& bars, uint32_t tmem, uint32_t g0,
-                                      unsigned long long limit) {
+// rows into the accumulators at `tmem` (X: columns [0, N), S: [128, 128 + N)),
+// then a commit to `done`.  One whole warp (the descriptor arithmetic is
+// warp-uniform; one elected lane issues).  The parts of a descriptor that
+// depend on N are a few registers, the rest are immediates.
+template <int R, int KIND>
+__device__ __forceinline__ bool tc_issue(const TcArea& ta, EngBars& bars, int N, uint32_t tmem, uint64_t* done,
+                                         uint32_t g0, unsigned long long limit) {
   using G = TcEngGeom<R>;
   constexpr int P = G::P, NC = G::NC, NM = KIND == 0 ? G::NXP : NC;
-  constexpr int LROW = 16 * (N + NC - 1);  // bytes of a plane-row segment
-  constexpr uint32_t IDESC =
-      (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+  const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
   const uint32_t hi = (128u >> 4) | (1u << 14);  // stride byte offset 128, descriptor version 1
-  const uint32_t d = tmem + (KIND == 0 ? 0u : (uint32_t)N);
+  const uint32_t d = tmem + (KIND == 0 ? 0u : 128u);
   const uint32_t a_lo0 = smem_addr(ta.a) >> 4, r_lo0 = smem_addr(ta.ring) >> 4;
   const int nb = ta.nb;
   const uint32_t slot_units = (uint32_t)ta.slot >> 4;
+  const uint32_t L = (uint32_t)(N + NC - 1);  // 16-byte units of a plane-row segment
+  uint32_t boff[NM];                          // B: first item's offset | leading byte offset to the second
+#pragma unroll
+  for (int q = 0; q < NM; ++q) {
+    const int i1 = KIND == 0 ? 2 * q : 3 * NC + q, i2 = KIND == 0 ? 2 * q + 1 : 4 * NC + q;
+    const uint32_t o1 = (uint32_t)(i1 / NC) * L + (uint32_t)(i1 % NC);
+    // (zero weights take any finite data)
+    const uint32_t o2 = KIND == 1 || i2 < G::NX ? (uint32_t)(i2 / NC) * L + (uint32_t)(i2 % NC) : o1 + 1u;
+    boff[q] = o1 + ((o2 - o1) << 16);
+  }
   int slot = (int)(g0 % (uint32_t)nb);
   uint32_t par = (g0 / (uint32_t)nb) & 1u;
   bool ok = true;
@@ -218,11 +210,12 @@ __device__ __forceinline__ bool tc_issue(const TcArea& ta, EngBars& bars, uint32
     for (int rr = 0; rr < kTcRps; ++rr) {
       const int j = kTcRps * h + rr;
       const uint32_t a_row = a_lo0 + (uint32_t)(P - 1 - j) * 8u;
+      const uint32_t b_row = b_slot + (rr ? 5u * L : 0u);
 #pragma unroll
       for (int q = 0; q < NM; ++q) {
         // A: first item's core matrix for row j, leading byte offset to the second
         // (offsets relative to row j's A base a_lo0 + (P - 1 - j) * 8)
-        int a1, a2, o1, o2;
+        int a1, a2;
         uint32_t zl = 0u;  // row-dependent part of a leading byte offset
         if (KIND == 0) {
           const int i1 = 2 * q, i2 = 2 * q + 1;
@@ -233,21 +226,15 @@ __device__ __forceinline__ bool tc_issue(const TcArea& ta, EngBars& bars, uint32
             a2 = G::ZERO - (P - 1);
             zl = (uint32_t)(j * 8) << 16;
           }
-          o1 = (i1 / NC) * LROW + 16 * (i1 % NC);
-          o2 = i2 < G::NX ? (i2 / NC) * LROW + 16 * (i2 % NC) : o1 + 16;  // zero weights: any finite data
         } else {
           a1 = a2 = G::sg(3 * NC + q);  // both K halves: the mask strip
-          o1 = 3 * LROW + 16 * q;
-          o2 = o1 + LROW;
         }
-        o1 += rr * 5 * LROW;
-        o2 += rr * 5 * LROW;
         const uint32_t alo = a_row + (uint32_t)(a1 * 8 + ((a2 - a1) * 8 << 16)) + zl;
-        const uint32_t blo = b_slot + (uint32_t)((o1 >> 4) + (((o2 - o1) >> 4) << 16));
-        if (j == 0 && q == 0)
-          tc_mma_lo_elect<0>(d, alo, hi, blo, hi, IDESC);
+        const uint32_t blo = b_row + boff[q];
+        if (q == 0)
+          tc_mma_lo_elect(d, alo, hi, blo, hi, idesc, j != 0);
         else
-          tc_mma_lo_elect<1>(d, alo, hi, blo, hi, IDESC);
+          tc_mma_lo_elect(d, alo, hi, blo, hi, idesc, true);
       }
     }
     tc_commit_elect(&bars.tc_empty[slot]);
@@ -256,46 +243,63 @@ __device__ __forceinline__ bool tc_issue(const TcArea& ta, EngBars& bars, uint32
       par ^= 1u;
     }
   }
-  tc_commit_elect(&bars.tc_done);  // also when a wait gave up: the MMAs issued so far
+  tc_commit_elect(done);  // also when a wait gave up: the MMAs issued so far
   return ok;
 }
 
-// Accumulators of tile (y0, xs) -> this thread's best key over its 16 or 32
-// candidates (whole block, after the tile's done barrier): warp w reads the
-// tensor-memory lanes of its quarter w % 4 and columns [w / 4 * N / 4, + N / 4),
-// 16 at a time.
-template <int R>
-__device__ __forceinline__ unsigned long long tc_epilogue(const ImgState& s, uint32_t tmem, int N, int a2,
-                                                       const uint32_t* tbits, int y0, int xs,
-                                                       unsigned long long best) {
+// The validity bits a warp's read-back needs (its four candidate rows, the
+// columns of its group): lane l holds the words of row l / (cols / 8), columns
+// 8 (l % (cols / 8)) .. + 7.  One load, issued before the wait for the MMAs.
+__device__ __forceinline__ uint2 tc_bits_load(const uint32_t* tbits, int N, int ngroups) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int q = warp & 3, cg = warp >> 2;
+  const int steps = N / ngroups / 8, r4 = lane / steps;
+  if (r4 >= 4) return make_uint2(0u, 0u);
+  return __ldcg(reinterpret_cast<const uint2*>(tbits + (4 * (warp & 3) + r4) * (N / 4)) + (warp >> 2) * steps +
+                lane - r4 * steps);
+}
+
+// Accumulators at `tmem` of tile (y0, xs) -> this thread's best key, after the
+// tile's done barrier.  ngroups = warps / 4 column groups: warp w reads the
+// tensor-memory lanes of its quarter w % 4 and the columns of group w / 4,
+// eight at a time.  bits: tc_bits_load of the tile.
+template <int R>
+__device__ __forceinline__ unsigned long long tc_epilogue(const ImgState& s, uint32_t tmem, const TcTiles& tt,
+                                                          int ngroups, int a2, uint2 bits, int y0, int tx,
+                                                          unsigned long long best) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int q = warp & 3;
   const int m = 32 * q + lane, i = m >> 3, b = m & 7;
-  const int cols = N / 4;
-  const int c0 = cg * cols;
-  const uint32_t* brow = tbits + i * (N / 4) + c0 / 4;
-  const int idx0 = (y0 + i) * s.W + xs + b + R + 8 * c0;  // candidate of this warp's first column
+  const int cols = tt.N / ngroups, c0 = (warp >> 2) * cols;
+  const int src0 = (lane >> 3) * (cols / 8);  // the lane that holds this row's first words
+  // candidate of accumulator column n: n / n1 folds down, 8 (n % n1) columns right
+  const int idx0 = (y0 + i) * s.W + tt.xs0 + 8 * tt.N * tx + b + R;
+  auto idx_of = [&](int n) {
+    const int f = n / tt.n1;
+    return idx0 + f * tt.h * s.W + 8 * (n - f * tt.n1);
+  };
   const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0;
   const float a2f = (float)a2;  // exact: a2 < 2^24
   float bv = __int_as_float(0x7f800000);  // +inf
   int bi = 0;
   bool any = false;
-  for (int h = 0; h < cols; h += 16) {
-    uint32_t X[16], S[16];
-    tc_ld16(ta + (uint32_t)h, X);
-    tc_ld16(ta + (uint32_t)(N + h), S);
-    const uint4 w = *reinterpret_cast<const uint4*>(brow + h / 4);
+#pragma unroll 1
+  for (int h = 0; h < cols; h += 8) {
+    uint32_t X[8], S[8];
+    tc_ld8(ta + (uint32_t)h, X);
+    tc_ld8(ta + (uint32_t)(128 + h), S);
+    const uint2 w = make_uint2(__shfl_sync(0xffffffffu, bits.x, src0 + h / 8),
+                               __shfl_sync(0xffffffffu, bits.y, src0 + h / 8));
     tc_wait_ld();
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      // candidates in increasing index order: the strict test keeps the first of equals
+    for (int k = 0; k < 8; ++k) {
+      // candidates in increasing index order (a fold's rows lie below the
+      // previous one's): the strict test keeps the first of equals
       const float v = __fadd_rn(__fmaf_rn(-2.0f, __uint_as_float(X[k]), __uint_as_float(S[k])), a2f);
-      const uint32_t word = k < 4 ? w.x : k < 8 ? w.y : k < 12 ? w.z : w.w;
-      const bool valid = (word >> (8 * (k & 3) + b)) & 1u;
+      const bool valid = ((k < 4 ? w.x : w.y) >> (8 * (k & 3) + b)) & 1u;
       any |= valid;
       if (valid && v < bv) {
         bv = v;
-        bi = idx0 + 8 * (h + k);
+        bi = c0 + h + k;
       }
     }
   }
@@ -303,24 +307,25 @@ __device__ __forceinline__ unsigned long long tc_epilogue(const ImgState& s, uin
   // takes the integer pass when any of its threads has no candidate below 2^24
   if (!__any_sync(0xffffffffu, any && !(bv < 16777216.0f))) {
     if (!any) return best;
-    const unsigned long long key = ((unsigned long long)(uint32_t)bv << 32) | (unsigned)bi;  // exact
+    const unsigned long long key = ((unsigned long long)(uint32_t)bv << 32) | (unsigned)idx_of(bi);  // exact
     return key < best ? key : best;
   }
   // the exact integer pass over the same accumulators
-  for (int h = 0; h < cols; h += 16) {
-    uint32_t X[16], S[16];
-    tc_ld16(ta + (uint32_t)h, X);
-    tc_ld16(ta + (uint32_t)(N + h), S);
-    const uint4 w = *reinterpret_cast<const uint4*>(brow + h / 4);
+#pragma unroll 1
+  for (int h = 0; h < cols; h += 8) {
+    uint32_t X[8], S[8];
+    tc_ld8(ta + (uint32_t)h, X);
+    tc_ld8(ta + (uint32_t)(128 + h), S);
+    const uint2 w = make_uint2(__shfl_sync(0xffffffffu, bits.x, src0 + h / 8),
+                               __shfl_sync(0xffffffffu, bits.y, src0 + h / 8));
     tc_wait_ld();
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const uint32_t word = k < 4 ? w.x : k < 8 ? w.y : k < 12 ? w.z : w.w;
-      if ((word >> (8 * (k & 3) + b)) & 1u) {
+    for (int k = 0; k < 8; ++k) {
+      if (((k < 4 ? w.x : w.y) >> (8 * (k & 3) + b)) & 1u) {
         const int xv = __float2int_rz(__uint_as_float(X[k]));
         const int sv = __float2int_rz(__uint_as_float(S[k]));
         const uint32_t ssd = (uint32_t)(a2 - 2 * xv + sv);
-        const unsigned long long key = ((unsigned long long)ssd << 32) | (unsigned)(idx0 + 8 * (h + k));
+        const unsigned long long key = ((unsigned long long)ssd << 32) | (unsigned)idx_of(c0 + h + k);
         best = key < best ? key : best;
       }
     }

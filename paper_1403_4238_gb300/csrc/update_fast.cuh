@@ -756,7 +756,7 @@ __device__ inline void set_source(const ImgState& s, UpdSmem<R>& sm, unsigned lo
 // the new grey levels and, for every front pixel, the strongest isophote of
 // its patch and its product with the normal.  The block's barrier must follow.
 // The last thread issues a gpu-scope fence once the writes the next search
-// reads (pixels, planes, mask, counts) are issued, and then, if `copied` is
+// reads (pixels, planes, mask, counts, validity bits) are issued, and then, if `copied` is
 // given, tells the searchers so; its warp has no later work, so the fence
 // waits off the path, and the same fence makes its later publication of the
 // next round a release.
@@ -788,7 +788,10 @@ __device__ inline void update_work(const ImgState& s, UpdSmem<R>& sm, bool fence
       if (nv < 0) continue;
       const int jy = j / NC, y = py + jy - 2 * R, x = px + j - jy * NC - 2 * R;
       s.count[y * s.pitch + x] = nv;
-      if (nv == 0 && x >= s.cx0 && x <= s.cx1 && y >= s.cy0 && y <= s.cy1) ++newly;
+      if (nv == 0 && x >= s.cx0 && x <= s.cx1 && y >= s.cy0 && y <= s.cy1) {
+        ++newly;
+        if (s.planes) vbit_set(s, x, y);
+      }
     }
     if (mine) {
       const int tx = px + dx, ty = py + dy, q = ty * W + tx;
