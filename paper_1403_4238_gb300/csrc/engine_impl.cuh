@@ -376,6 +376,16 @@ __host__ __device__ inline long long res_plan(ResPlan& pl, int ncu, int nbands, 
 
 // ---------------------------------------------------------------- kernel
 
+// The state of a CTA's tensor-core search that outlives a round: source rows
+// through the ring and tiles through the accumulator buffers so far (their
+// barriers' phases).
+struct TcRun {
+  TcArea a;
+  uint32_t rows, tiles;
+  int k0, n;    // this CTA's turns that are tiles: k0 .. k0 + n - 1 (tc_tile_of)
+  int tx0, y0;  // the first one's tile column and candidate row
+};
+
 struct EngSmemTail {
   EngBars bars;      // mbarriers (streaming stages, tensor-core ring), tensor-memory base
   ImgState img;      // the image's state block (a leader that does not search reads it here)
@@ -385,6 +395,7 @@ struct EngSmemTail {
   int px, py;
   int a2row[17];  // tensor-core search: per target row, sum of the known pixels' squared shifted values
   int tc_pref;    // tensor-core search: slots the producer prefetched for the next round
+  TcRun tc_run;   // a searching leader's tensor-core search between its rounds
   int lim, status, err;  // leader: iteration limit, status and error word (the stop decision)
   uint8_t known[2][17 * 17];  // known flags of the last two targets (by round parity)
   ResPlan plan;               // resident mode: this CTA's units and tiles
@@ -546,20 +557,21 @@ __device__ inline bool ctrl_active(const Ctrl* c) {
 template <int R, int SRW, bool kLeadOnly = false>
 __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x);
 
-// The state of a CTA's tensor-core search that outlives a round: source rows
-// through the ring and tiles through the accumulator buffers so far (their
-// barriers' phases).
-struct TcRun {
-  TcArea a;
-  uint32_t rows, tiles;
-};
+// The k-th tile of searching CTA `rank` of ns, or -1.  Tiles go round-robin;
+// when the leader (the last of them) searches too, its first turn is its
+// speculative phase, which takes about as long as a tile.
+__device__ __forceinline__ int tc_tile_of(int k, int rank, int ns, int ntiles, bool lead_searches) {
+  const int v = rank + k * ns, t = lead_searches && v >= ns - 1 ? v - 1 : v;
+  return (lead_searches && v == ns - 1) || t >= ntiles ? -1 : t;
+}
 
 // Where the tensor-core search keeps its state, from byte `off` of the CTA's
 // shared memory.  A ring with another slot count than the last image's starts
 // its phases over (every slot of an earlier image was consumed, so no barrier
 // has a pending phase).  Whole block.
 template <int R>
-__device__ __forceinline__ void tc_setup(TcRun& t, EngCtx& x, EngBars& bars, int off, int nb, int slot) {
+__device__ __forceinline__ void tc_setup(TcRun& t, EngCtx& x, EngBars& bars, const ImgState& s, const TcTiles& tt,
+                                         int k0, int ns, bool lead_searches, int off, int nb, int slot) {
   using GT = TcEngGeom<R>;
   uint8_t* area = eng_smem() + off;
   t.a.a = area;
@@ -569,6 +581,12 @@ __device__ __forceinline__ void tc_setup(TcRun& t, EngCtx& x, EngBars& bars, int
   t.a.slot = slot;
   t.rows = x.tc_rows;
   t.tiles = x.tc_tiles;
+  t.k0 = k0;
+  t.n = 0;
+  while (tc_tile_of(k0 + t.n, x.rank, ns, tt.ntx * tt.nty, lead_searches) >= 0) ++t.n;
+  const int t0 = max(0, tc_tile_of(k0, x.rank, ns, tt.ntx * tt.nty, lead_searches)), ty = t0 / tt.ntx;
+  t.tx0 = t0 - ty * tt.ntx;
+  t.y0 = s.cy0 + kTcRows * ty;
   if (x.tc_nb != nb) {
     if (x.tc_nb != 0 && threadIdx.x == 0) {
       for (int i = 0; i < kTcRing; ++i) {
@@ -587,31 +605,26 @@ __device__ __forceinline__ void tc_setup(TcRun& t, EngCtx& x, EngBars& bars, int
   x.tc_nb = nb;
 }
 
-// The k-th tile of searching CTA `rank` of ns, or -1.  Tiles go round-robin;
-// when the leader (the last of them) searches too, its first turn is its
-// speculative phase, which takes about as long as a tile.
-__device__ __forceinline__ int tc_tile_of(int k, int rank, int ns, int ntiles, bool lead_searches) {
-  const int v = rank + k * ns, t = lead_searches && v >= ns - 1 ? v - 1 : v;
-  return (lead_searches && v == ns - 1) || t >= ntiles ? -1 : t;
-}
-
-// One round of a CTA's tensor-core search for target (px, py): its tiles k0,
-// k0 + 1, ...; `pref` ring slots of the first one are already requested.
+// One round of a CTA's tensor-core search for target (px, py): its tiles;
+// `pref` ring slots of the first one are already requested.
 // Returns the thread's best key; *bad (of this thread) when a bounded wait
 // gave up.  Whole block.
 template <int R>
 __device__ __forceinline__ unsigned long long tc_round(const ImgState& s, const TcTiles& tt, TcRun& tr,
                                                        EngSmemTail& tl, uint32_t tmem, int px, int py, bool first,
-                                                       int k0, int pref, int rank, int ns, bool lead_searches,
+                                                       int pref, int rank, int ns, bool lead_searches,
                                                        unsigned long long limit, int* bad_out) {
   using GT = TcEngGeom<R>;
   constexpr int P = GT::P, NSL = GT::NSL;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int ntiles = tt.ntx * tt.nty, npre = min(tr.a.nb, NSL);
-  int n = 0;  // tiles of this round
-  while (tc_tile_of(k0 + n, rank, ns, ntiles, lead_searches) >= 0) ++n;
+  const int npre = min(tr.a.nb, NSL), n = tr.n;
   auto tile = [&](int k, int& tx, int& y0) {
-    const int t = tc_tile_of(k0 + k, rank, ns, ntiles, lead_searches), ty = t / tt.ntx;
+    if (k == 0) {
+      tx = tr.tx0;
+      y0 = tr.y0;
+      return ((y0 - s.cy0) / kTcRows) * tt.ntx + tx;
+    }
+    const int t = tc_tile_of(tr.k0 + k, rank, ns, tt.ntx * tt.nty, lead_searches), ty = t / tt.ntx;
     tx = t - ty * tt.ntx;
     y0 = s.cy0 + kTcRows * ty;
     return t;
@@ -623,16 +636,26 @@ __device__ __forceinline__ unsigned long long tc_round(const ImgState& s, const 
     tile(0, tx, y0);
     if (!tc_produce<R>(s, tr.a, tl.bars, tx, y0, tr.rows, 0, npre, limit)) bad = 1;
   }
+  // the last tile's validity bits, requested before a warp's role: by the
+  // producer's and the issuers' warps while the others write A (13 warps need
+  // as many passes for it as 15), by those when they are done
+  const int ng = (tt.N & 31) ? 2 : 4;  // column groups of that tile's read-back
+  uint2 bits_last = make_uint2(0u, 0u);
+  auto bits_of = [&](int t) { return s.vbits + (size_t)t * kTcRows * (tt.N / 4); };
+  auto load_last = [&]() {
+    int tx_, y0_;
+    if (n > 0 && warp < 4 * ng) bits_last = tc_bits_load(bits_of(tile(n - 1, tx_, y0_)), tt.N, ng);
+  };
   tc_stage_target<R>(s, tr.a.tpad, tl.a2row, px, py);
   __syncthreads();
-  // every warp but the producer's (its copies are in flight) writes A
-  tc_build_a<R>(tr.a.a, tr.a.tpad, first, 32 * (kEngWarps - 1));
+  if (warp >= kEngWarps - 3) load_last();
+  else tc_build_a<R>(tr.a.a, tr.a.tpad, first, 32 * (kEngWarps - 3));
   __syncthreads();
+  if (warp < kEngWarps - 3) load_last();
   int a2 = 0;
 #pragma unroll
   for (int dy = 0; dy < P; ++dy) a2 += tl.a2row[dy];
   unsigned long long best = ~0ull;
-  auto bits_of = [&](int t) { return s.vbits + (size_t)t * kTcRows * (tt.N / 4); };
   if (warp == kEngWarps - 1) {
     for (int k = 0; k < n && !bad; ++k) {
       tile(k, tx, y0);
@@ -673,12 +696,6 @@ __device__ __forceinline__ unsigned long long tc_round(const ImgState& s, const 
       if (lane == 0) mbar_arrive(&tl.bars.tc_free[b]);
     }
   }
-  uint2 bits = make_uint2(0u, 0u);
-  const int ng = (tt.N & 31) ? 2 : 4;  // column groups of the last tile's read-back
-  if (n > 0) {
-    const int t = tile(n - 1, tx, y0);
-    if (warp < 4 * ng) bits = tc_bits_load(bits_of(t), tt.N, ng);
-  }
   tc_fence_before();
   if (__syncthreads_or(bad)) {
     *bad_out = 1;
@@ -687,7 +704,8 @@ __device__ __forceinline__ unsigned long long tc_round(const ImgState& s, const 
   tc_fence_after();
   if (n > 0) {
     const uint32_t b = (tr.tiles + (uint32_t)(n - 1)) & 1u;
-    if (warp < 4 * ng) best = tc_epilogue<R>(s, tmem + 256u * b, tt, ng, a2, bits, y0, tx, best);
+    tile(n - 1, tx, y0);
+    if (warp < 4 * ng) best = tc_epilogue<R>(s, tmem + 256u * b, tt, ng, a2, bits_last, y0, tx, best);
     tc_fence_before();
     __syncwarp();
     // (all 16 warps read this tile; the block's reduction precedes the next
@@ -718,23 +736,23 @@ __device__ __noinline__ void run_tc_search(const EngineArgs& ea, EngCtx& x, cons
   const int rank = x.rank;
   TeamCtl* tc = x.tc;
   const unsigned long long limit = ea.wait_limit_ns;
+  const bool withheld = rank + 1 == ea.withhold;  // (the arguments lie in local memory)
+  int* const err = ea.err;
   unsigned epoch = x.epoch;
   TcRun tr;
-  tc_setup<R>(tr, x, tl.bars, (int)kHeadBytes, nb, slot);
-  const int ntiles = tt.ntx * tt.nty, t0 = tc_tile_of(0, rank, ns, ntiles, lead_searches);
-  const int first_y = s.cy0 + kTcRows * (t0 / tt.ntx), first_tx = t0 % tt.ntx;  // this CTA's first tile
+  tc_setup<R>(tr, x, tl.bars, s, tt, 0, ns, lead_searches, (int)kHeadBytes, nb, slot);
   const int npre = min(nb, GT::NSL);
   int pref = 0;
   bool first = true;
   while (!tl.stop) {
     const int px = tl.px, py = tl.py;
     int bad;
-    unsigned long long best = tc_round<R>(s, tt, tr, tl, tmem, px, py, first, 0, pref, rank, ns, lead_searches, limit, &bad);
+    unsigned long long best = tc_round<R>(s, tt, tr, tl, tmem, px, py, first, pref, rank, ns, lead_searches, limit, &bad);
     first = false;
     best = block_min_u64(best, tl.red64);
     if (tid == 0) {
-      if (bad) atomicExch(ea.err, INPAINT_ERR_TIMEOUT);
-      if (rank + 1 != ea.withhold) st_relaxed64(&tpart[rank], key_tag(best, epoch));
+      if (!withheld) st_relaxed64(&tpart[rank], key_tag(best, epoch));
+      if (bad) atomicExch(err, INPAINT_ERR_TIMEOUT);
       if (rank == 0) atomicAdd(&s.ctrl->tc_rounds, 1);
     }
     if (bad) break;
@@ -748,8 +766,8 @@ __device__ __noinline__ void run_tc_search(const EngineArgs& ea, EngCtx& x, cons
         if ((int)(ld_acquire(&tc->copied) - (epoch + 1u)) >= 0) {
           asm volatile("fence.proxy.async.global;" ::: "memory");
           n = npre;
-          if (!tc_produce<R>(s, tr.a, tl.bars, first_tx, first_y, tr.rows, 0, n, limit))
-            atomicExch(ea.err, INPAINT_ERR_TIMEOUT);
+          if (!tc_produce<R>(s, tr.a, tl.bars, tr.tx0, tr.y0, tr.rows, 0, n, limit))
+            atomicExch(err, INPAINT_ERR_TIMEOUT);
           break;
         }
         if ((unsigned)ld_acquire64(&tc->pub) != epoch || globaltimer() - t0 > limit) break;
@@ -758,7 +776,7 @@ __device__ __noinline__ void run_tc_search(const EngineArgs& ea, EngCtx& x, cons
     }
     // wait for the next round
     if (tid == 0) {
-      const unsigned long long v = wait_pub(tc, epoch, ea.err, limit);
+      const unsigned long long v = wait_pub(tc, epoch, err, limit);
       tl.stop = ((v >> 62) & 1ull) != 0;
       tl.px = (int)((v >> 32) & 0x7fff);
       tl.py = (int)((v >> 47) & 0x7fff);
@@ -795,28 +813,21 @@ __device__ __noinline__ unsigned long long tc_lead_share(const EngineArgs& ea, E
                                                          int nb, int slot, int ns, int px, int py, bool first) {
   EngSmemTail& tl = *reinterpret_cast<EngSmemTail*>(eng_smem());
   const ImgState& s = tl.img;
+  // the run's state stays in shared memory between the rounds (tl.tc_run)
   TcRun tr;
-  if (first) {
-    tc_setup<R>(tr, x, tl.bars, off, nb, slot);
-  } else {
-    uint8_t* area = eng_smem() + off;
-    tr.a.a = area;
-    tr.a.tpad = reinterpret_cast<uint16_t*>(area + TcEngGeom<R>::A_BYTES);
-    tr.a.ring = area + TcEngGeom<R>::A_BYTES + TcEngGeom<R>::TPAD_BYTES;
-    tr.a.nb = nb;
-    tr.a.slot = slot;
-    tr.rows = x.tc_rows;
-    tr.tiles = x.tc_tiles;
-  }
+  if (first) tc_setup<R>(tr, x, tl.bars, s, tt, 1, ns, true, off, nb, slot);
+  else tr = tl.tc_run;
   int bad;
-  unsigned long long best = tc_round<R>(s, tt, tr, tl, x.tmem, px, py, first, 1, 0, x.rank, ns, true, ea.wait_limit_ns, &bad);
+  unsigned long long best = tc_round<R>(s, tt, tr, tl, x.tmem, px, py, first, 0, x.rank, ns, true, ea.wait_limit_ns, &bad);
   if (bad && threadIdx.x == 0) {
     atomicExch(ea.err, INPAINT_ERR_TIMEOUT);
     tl.err = INPAINT_ERR_TIMEOUT;
   }
   x.tc_rows = tr.rows;
   x.tc_tiles = tr.tiles;
-  return block_min_u64(best, tl.red64);
+  best = block_min_u64(best, tl.red64);  // (its barriers: every thread has read tl.tc_run)
+  if (threadIdx.x == 0) tl.tc_run = tr;
+  return best;
 }
 
 // The loop of a leader that does not search, compiled as a function of its
@@ -844,6 +855,9 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
   unsigned long long* const tpart = x.tpart;
   const unsigned long long t_start = x.t_start;  // (the context is in local memory)
   const unsigned long long limit = ea.wait_limit_ns;
+  int* const err = ea.err;
+  const unsigned long long tick_ns = ea.tick_ns;
+  const bool withheld = rank + 1 == ea.withhold;
   uint32_t ph0 = x.ph0, ph1 = x.ph1;
   unsigned epoch = x.epoch;
 
@@ -902,7 +916,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     }
     if (tcmode && searcher && !leader) {
       if (tid == 0) {
-        tl.stop = !ctrl_active(c) || __ldcg(ea.err) != 0;
+        tl.stop = !ctrl_active(c) || __ldcg(err) != 0;
         tl.px = __ldcg(&c->px);
         tl.py = __ldcg(&c->py);
       }
@@ -944,7 +958,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     __syncthreads();
   }
   if (tid == 0) {
-    tl.stop = !ctrl_active(c) || __ldcg(ea.err) != 0;
+    tl.stop = !ctrl_active(c) || __ldcg(err) != 0;
     tl.px = __ldcg(&c->px);
     tl.py = __ldcg(&c->py);
   }
@@ -1100,7 +1114,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     }
     ++round;
     if (!ok && tid == 0) {
-      atomicExch(ea.err, INPAINT_ERR_TIMEOUT);
+      atomicExch(err, INPAINT_ERR_TIMEOUT);
       tl.err = INPAINT_ERR_TIMEOUT;  // (a searching leader: its key would be partial)
     }
     return block_min_u64(best, tl.red64);
@@ -1120,7 +1134,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
       if (tid == kRecThread + 1) {
         // the stop decision's inputs that other CTAs may change
         tl.status = __ldcg(&c->status);
-        tl.err = __ldcg(ea.err);
+        tl.err = __ldcg(err);
       }
       spec_record<R>(s, usm, false);
       __syncwarp();
@@ -1135,7 +1149,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     if (tid >= kChainThreads) {
       if (tid >= kRecThread) {
         bool late;
-        const unsigned long long best = gather_keys(tpart, ns, epoch, ea.err, limit, &late);
+        const unsigned long long best = gather_keys(tpart, ns, epoch, err, limit, &late);
         if (lane == 0) {
           usm.t_keys = globaltimer();
           set_source<R>(s, usm, best, late || tl.err != 0);
@@ -1158,7 +1172,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
       // the next round (or the stop) goes out before the bookkeeping; after
       // an update, this thread's fence in update_work ordered every write
       // the searchers read before this store, else the store is a release
-      const bool spent = ok && !stop && ea.tick_ns && globaltimer() - t_start > ea.tick_ns;
+      const bool spent = ok && !stop && tick_ns && globaltimer() - t_start > tick_ns;
       if (spent) {
         stop = true;  // the launch's time budget is spent: resume in the next launch
         tc->expired = 1u;
@@ -1205,11 +1219,11 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     }
     if (searcher) {
       const unsigned long long best = search_round(px, py);
-      if (tid == 0 && rank + 1 != ea.withhold) st_relaxed64(&tpart[rank], key_tag(best, epoch));
+      if (tid == 0 && !withheld) st_relaxed64(&tpart[rank], key_tag(best, epoch));
     }
     // searchers and idle CTAs: wait for the next round
     if (tid == 0) {
-      const unsigned long long v = wait_pub(tc, epoch, ea.err, limit);
+      const unsigned long long v = wait_pub(tc, epoch, err, limit);
       tl.stop = ((v >> 62) & 1ull) != 0;
       tl.px = (int)((v >> 32) & 0x7fff);
       tl.py = (int)((v >> 47) & 0x7fff);

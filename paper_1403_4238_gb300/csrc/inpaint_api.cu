@@ -191,7 +191,7 @@ int launch_iteration(inpaint_ctx* c, int use_cond) {
   if (c->r <= 8)
     CK(launch_update_fast(c->st, c->cond, use_cond, c->stream));
   else
-    CK(launch_update(c->st, 1, c->cond, use_cond, c->stream));
+    CK(launch_update(c->st, c->cond, use_cond, c->stream));
   if (c->opt.debug_checks) CK(launch_verify_count(c->st, c->stream));
   return INPAINT_OK;
 }
@@ -440,7 +440,7 @@ int create_impl(const uint8_t* rgb, int W, int H, int rgb_stride, const uint8_t*
   const size_t n = (size_t)W * H;
   if (!alloc_n(c, s.img, (size_t)s.pitch * H) || !alloc_n(c, s.omega, n) || !alloc_n(c, s.gray, n) ||
       !alloc_n(c, s.conf, n) || !alloc_n(c, s.count, (size_t)s.pitch * H) || !alloc_n(c, s.prio, n) ||
-      !alloc_n(c, s.pconf, n) || !alloc_n(c, s.tiles0, (size_t)s.t0x * s.t0y) ||
+      !alloc_n(c, s.pconf, n) || (r > 8 && !alloc_n(c, s.front, n)) || !alloc_n(c, s.tiles0, (size_t)s.t0x * s.t0y) ||
       !alloc_n(c, s.tiles1, (size_t)s.t1x * s.t1y) ||
       !alloc_n(c, s.ctrl, 1) || !alloc_n(c, s.trace, (size_t)s.trace_cap) ||
       !alloc_n(c, s.partial, (size_t)(s.n_partial > 0 ? s.n_partial : 1)) ||
@@ -772,7 +772,7 @@ int inpaint_apply_key(inpaint_ctx* c, unsigned long long key, inpaint_step_info*
   if (c->r <= 8)
     CK(launch_update_fast(s, c->cond, 0, c->stream));
   else
-    CK(launch_update(s, 1, c->cond, 0, c->stream));
+    CK(launch_update(s, c->cond, 0, c->stream));
   if (c->opt.debug_checks) CK(launch_verify_count(c->st, c->stream));
   if ((rc = read_ctrl(c))) return rc;
   if (c->h_ctrl->status != 0) return c->h_ctrl->status;

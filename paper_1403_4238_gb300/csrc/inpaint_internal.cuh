@@ -69,6 +69,8 @@ struct Ctrl {
   unsigned long long t_search, t_update, t_last;
   int timed_iters;
   int tc_rounds;   // engine search rounds run in the tensor-core form
+  int n_front;     // patch radius > 8: front pixels in ImgState::front whose priorities
+                   // are to be evaluated; -1: the last update applied nothing
 };
 
 // Window codes of the speculative phase (update_fast.cuh): a pixel of the
@@ -145,6 +147,7 @@ struct ImgState {
   Ctrl* ctrl;
   inpaint_step_info* trace;
   unsigned long long* partial;  // per-CTA best search key of the iteration
+  int* front;              // patch radius > 8: linear indices of the pixels to evaluate
   // tensor-core form (null otherwise): five BF16 planes of the image, R' G' B'
   // (byte - 128) and the square sum sq = sum_c (byte_c - 128)^2 as 256 hi and
   // lo (sq = 256 hi + lo), stored per tile column tx of the search (columns
@@ -424,8 +427,8 @@ struct TcPlan {
 // Geometry and launch shape (needs the search rectangle, not the buffers).
 cudaError_t prepare_search_tc(const ImgState& s, TcPlan* plan);
 cudaError_t launch_search_tc(const ImgState& s, const TcPlan& plan, cudaStream_t st);
-cudaError_t launch_update(const ImgState& s, int do_fill, unsigned long long cond_handle,
-                          int use_cond, cudaStream_t st);
+cudaError_t launch_update(const ImgState& s, unsigned long long cond_handle, int use_cond,
+                          cudaStream_t st);  // patch radius > 8
 cudaError_t launch_verify_count(const ImgState& s, cudaStream_t st);
 cudaError_t launch_export(const ImgState& s, uint8_t* rgb_dense, cudaStream_t st);
 

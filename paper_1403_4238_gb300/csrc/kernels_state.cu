@@ -36,7 +36,22 @@ __device__ inline bool on_front(const ImgState& s, int x, int y) {
          known_px(s, x, y + 1);
 }
 
-// P(p) of Eq. 1 with C(p), D(p) of Eq. 2; writes C(p) to *c_out.
+// D(p) of Eq. 2 from the isophote's gradient; normal to the front: Sobel of
+// the Omega indicator (replicated borders).
+__device__ inline double data_term_at(const ImgState& s, int x, int y, int gx, int gy) {
+  const int m_lu = omega_clamped(s, x - 1, y - 1), m_cu = omega_clamped(s, x, y - 1);
+  const int m_ru = omega_clamped(s, x + 1, y - 1), m_lc = omega_clamped(s, x - 1, y);
+  const int m_rc = omega_clamped(s, x + 1, y), m_ld = omega_clamped(s, x - 1, y + 1);
+  const int m_cd = omega_clamped(s, x, y + 1), m_rd = omega_clamped(s, x + 1, y + 1);
+  const int nx = (m_ru + 2 * m_rc + m_rd) - (m_lu + 2 * m_lc + m_ld);
+  const int ny = (m_ld + 2 * m_cd + m_rd) - (m_lu + 2 * m_cu + m_ru);
+  int dot = (-gy) * nx + gx * ny;
+  dot = dot < 0 ? -dot : dot;
+  const int nn = nx * nx + ny * ny;
+  return nn != 0 ? __ddiv_rn(__ddiv_rn((double)dot, __dsqrt_rn((double)nn)), 510.0) : 0.0;
+}
+
+// P(p) of Eq. 1 with C(p), D(p) of Eq. 2; writes C(p) to *c_out (debug check).
 __device__ double priority_at(const ImgState& s, int x, int y, double* c_out) {
   const int W = s.W, H = s.H, r = s.r;
   // Confidence term: known part of Psi_p over its in-image area, summed in
@@ -55,14 +70,6 @@ __device__ double priority_at(const ImgState& s, int x, int y, double* c_out) {
     }
   }
   const double c = __ddiv_rn(sum, (double)n_in);
-
-  // Normal to the front: Sobel of the Omega indicator (replicated borders).
-  const int m_lu = omega_clamped(s, x - 1, y - 1), m_cu = omega_clamped(s, x, y - 1);
-  const int m_ru = omega_clamped(s, x + 1, y - 1), m_lc = omega_clamped(s, x - 1, y);
-  const int m_rc = omega_clamped(s, x + 1, y), m_ld = omega_clamped(s, x - 1, y + 1);
-  const int m_cd = omega_clamped(s, x, y + 1), m_rd = omega_clamped(s, x + 1, y + 1);
-  const int nx = (m_ru + 2 * m_rc + m_rd) - (m_lu + 2 * m_lc + m_ld);
-  const int ny = (m_ld + 2 * m_cd + m_rd) - (m_lu + 2 * m_cu + m_ru);
 
   // Isophote: strongest central-difference grey gradient among pixels of
   // Psi_p whose four neighbours are known (first in row-major order on ties).
@@ -85,26 +92,108 @@ __device__ double priority_at(const ImgState& s, int x, int y, double* c_out) {
       }
     }
   }
-  int dot = (-gy) * nx + gx * ny;
-  dot = dot < 0 ? -dot : dot;
-  const int nn = nx * nx + ny * ny;
-  double d = 0.0;
-  if (nn != 0) d = __ddiv_rn(__ddiv_rn((double)dot, __dsqrt_rn((double)nn)), 510.0);
+  const double d = data_term_at(s, x, y, gx, gy);
   *c_out = c;
   return __dmul_rn(c, d);
 }
 
-__device__ inline void eval_pixel(const ImgState& s, int x, int y) {
-  const size_t i = (size_t)y * s.W + x;
-  unsigned long long key = 0ull;
-  double c = 0.0;
-  if (on_front(s, x, y)) {
-    const double p = priority_at(s, x, y, &c);
-    key = (unsigned long long)__double_as_longlong(p) + 1ull;
-  }
-  s.prio[i] = key;
-  s.pconf[i] = c;
+// Appends pixel i to the list of front pixels to evaluate when `mine`; whole
+// warps (one counter update per warp).
+__device__ inline void append_front(const ImgState& s, bool mine, int i) {
+  const unsigned bal = __ballot_sync(0xffffffffu, mine);
+  if (bal == 0u) return;
+  const int lane = threadIdx.x & 31;
+  int base = 0;
+  if (lane == 0) base = atomicAdd(&s.ctrl->n_front, __popc(bal));
+  base = __shfl_sync(0xffffffffu, base, 0);
+  if (mine) s.front[base + __popc(bal & ((1u << lane) - 1u))] = i;
 }
+
+// Priorities of the listed front pixels for patch radii above the engine's:
+// one CTA of two warps per pixel.  Warp 0 sums the confidences: its lanes load
+// a patch row coalesced (the next row while this one is summed) and the known
+// entries are added one by one in row-major order; unknown ones are skipped,
+// which changes nothing (adding +0.0 to a non-negative sum) and halves the
+// chain of dependent FP64 additions (69 cycles each).  Warp 1 meanwhile finds
+// the strongest isophote.  (One thread per pixel reading the patch from global
+// memory, in the update's one CTA, took 390 us an iteration at 512x384, 25x25.)
+__global__ void __launch_bounds__(64) k_prio_list(ImgState s) {
+  __shared__ unsigned long long iso_s;
+  const int n = s.ctrl->n_front;
+  const int W = s.W, H = s.H, r = s.r, P = 2 * r + 1;
+  const int lane = threadIdx.x & 31;
+  for (int k = blockIdx.x; k < n; k += gridDim.x) {
+    const int p = s.front[k], y = p / W, x = p - y * W;
+    const int x0 = max(x - r, 0), x1 = min(x + r, W - 1), y0 = max(y - r, 0), y1 = min(y + r, H - 1);
+    double sum = 0.0;
+    if (threadIdx.x < 32) {
+      constexpr int NB = (2 * kMaxRadius + 1 + 31) / 32;
+      double c[NB], nc[NB];
+      bool kn[NB], nkn[NB];
+      auto load_row = [&](int yy, double (&cv)[NB], bool (&kv)[NB]) {
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+          const int xx = x0 + 32 * b + lane;
+          const bool in = 32 * b < P && xx <= x1;
+          cv[b] = in ? s.conf[(size_t)yy * W + xx] : 0.0;
+          kv[b] = in && s.omega[(size_t)yy * W + xx] == 0;
+        }
+      };
+      load_row(y0, c, kn);
+      for (int yy = y0; yy <= y1; ++yy) {
+        if (yy < y1) load_row(yy + 1, nc, nkn);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+          if (32 * b >= P) break;
+          for (unsigned m = __ballot_sync(0xffffffffu, kn[b]); m; m &= m - 1)
+            sum = __dadd_rn(sum, __shfl_sync(0xffffffffu, c[b], __ffs(m) - 1));
+        }
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+          c[b] = nc[b];
+          kn[b] = nkn[b];
+        }
+      }
+    } else {
+      // key: (|grad|^2 + 1) << 32 | ~(row-major index in the patch), 0: none
+      unsigned long long best = 0ull;
+      const int ya = max(y - r, 1), yb = min(y + r, H - 2), xa = max(x - r, 1), xb = min(x + r, W - 2);
+      for (int xx = xa + lane; xx <= xb; xx += 32) {
+#pragma unroll 4
+        for (int yy = ya; yy <= yb; ++yy) {
+          const size_t q = (size_t)yy * W + xx;
+          const int o = s.omega[q] | s.omega[q - 1] | s.omega[q + 1] | s.omega[q - W] | s.omega[q + W];
+          const int gx = (int)s.gray[q + 1] - (int)s.gray[q - 1], gy = (int)s.gray[q + W] - (int)s.gray[q - W];
+          const unsigned long long key = ((unsigned long long)(gx * gx + gy * gy + 1) << 32) |
+                                         (0xffffffffu - (unsigned)((yy - ya) * P + xx - xa));
+          if (o == 0 && key > best) best = key;
+        }
+      }
+      __syncwarp();
+      const unsigned mh = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32));
+      const unsigned ml = __reduce_max_sync(0xffffffffu, (unsigned)(best >> 32) == mh ? (unsigned)best : 0u);
+      if (lane == 0) iso_s = ((unsigned long long)mh << 32) | ml;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      const double cc = __ddiv_rn(sum, (double)((x1 - x0 + 1) * (y1 - y0 + 1)));
+      const unsigned long long iso = iso_s;
+      int gx = 0, gy = 0;
+      if (iso >> 32) {
+        const int l = (int)(0xffffffffu - (unsigned)iso);
+        const size_t q = (size_t)(max(y - r, 1) + l / P) * W + max(x - r, 1) + l % P;
+        gx = (int)s.gray[q + 1] - (int)s.gray[q - 1];
+        gy = (int)s.gray[q + W] - (int)s.gray[q - W];
+      }
+      s.prio[p] = (unsigned long long)__double_as_longlong(__dmul_rn(cc, data_term_at(s, x, y, gx, gy))) + 1ull;
+      s.pconf[p] = cc;
+    }
+    __syncthreads();
+  }
+}
+
+// CTAs of k_prio_list (a grid-stride loop): a window's front is 100-200 pixels.
+constexpr int kPrioCtas = 608;
 
 // ---------------------------------------------------------------- init
 
@@ -125,6 +214,7 @@ __global__ void k_ctrl_init(Ctrl* c) {
   c->t_last = 0ull;
   c->timed_iters = 0;
   c->tc_rounds = 0;
+  c->n_front = 0;
 }
 
 // RGB (or RGBA words) + mask -> packed state; counts |Omega|.
@@ -243,10 +333,18 @@ __global__ void k_count(ImgState s, const int32_t* sat) {
   if (threadIdx.x == 0 && tot) atomicAdd(&s.ctrl->n_valid, tot);
 }
 
-__global__ void k_prio_all(ImgState s) {
+// Key 0 everywhere and the list of the front pixels (patch radius > 8).
+__global__ void k_front_all(ImgState s) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y;
-  if (x < s.W) eval_pixel(s, x, y);
+  bool fr = false;
+  if (x < s.W) {
+    const size_t i = (size_t)y * s.W + x;
+    s.prio[i] = 0ull;
+    s.pconf[i] = 0.0;
+    fr = on_front(s, x, y);
+  }
+  append_front(s, fr, y * s.W + x);
 }
 
 // Level-0 tiles from the pixel keys, then level-1 tiles: one warp per tile.
@@ -265,26 +363,23 @@ __global__ void k_tiles1_all(ImgState s) {
 struct UpdSmem {
   uint8_t filled[(2 * kMaxRadius + 1) * (2 * kMaxRadius + 1)];
   int32_t fsat[(2 * kMaxRadius + 2) * (2 * kMaxRadius + 2)];
-  PrioBest pb[32];
   unsigned long long u64s[32];
   int ints[32];
 };
 
-// One iteration's copy/update and the selection of the next target patch.
-// Single CTA.  With do_fill == 0 only the selection runs (initialisation).
-__global__ void __launch_bounds__(kUpdThreads) k_update(ImgState s, int do_fill,
-                                                       cudaGraphConditionalHandle cond,
-                                                       int use_cond) {
+// One iteration's copy and validity update for patch radii above the
+// engine's, up to the list of front pixels whose priorities it changes.
+// Single CTA; k_prio_list and k_select_big follow.
+__global__ void __launch_bounds__(kUpdThreads) k_fill_big(ImgState s) {
   __shared__ UpdSmem sm;
   Ctrl* c = s.ctrl;
   const int tid = threadIdx.x, nt = blockDim.x;
   const int W = s.W, H = s.H, r = s.r, P = 2 * r + 1;
   if (!loop_active(c)) {
-    if (use_cond && tid == 0) cudaGraphSetConditional(cond, 0);
+    if (tid == 0) c->n_front = -1;
     return;
   }
-  int remaining = c->remaining;
-  if (do_fill) {
+  {
     // findBestPatch result: lowest (SSD << 32 | idx) over all search CTAs.
     unsigned long long best = ~0ull;
     for (int i = tid; i < s.n_partial; i += nt) {
@@ -295,7 +390,7 @@ __global__ void __launch_bounds__(kUpdThreads) k_update(ImgState s, int do_fill,
     if (best == ~0ull) {  // no fully-known source patch: leave the state as is
       if (tid == 0) {
         c->status = INPAINT_ERR_NO_SOURCE;
-        if (use_cond) cudaGraphSetConditional(cond, 0);
+        c->n_front = -1;
       }
       return;
     }
@@ -375,57 +470,79 @@ __global__ void __launch_bounds__(kUpdThreads) k_update(ImgState s, int do_fill,
     }
     newly = block_sum_int(newly, sm.ints);  // also orders the global writes above
 
+    if (tid == 0) c->n_front = 0;
+    __syncthreads();
     // Priorities that can change: front pixels within 2r+1 of p^.
     const int R2 = 2 * r + 1, side2 = 2 * R2 + 1;
-    for (int j = tid; j < side2 * side2; j += nt) {
+    for (int j0 = 0; j0 < side2 * side2; j0 += nt) {
+      const int j = j0 + tid;
       const int x = px - R2 + j % side2, y = py - R2 + j / side2;
-      if (x >= 0 && x < W && y >= 0 && y < H) eval_pixel(s, x, y);
+      bool fr = false;
+      if (j < side2 * side2 && x >= 0 && x < W && y >= 0 && y < H) {
+        fr = on_front(s, x, y);
+        if (!fr) {
+          s.prio[(size_t)y * W + x] = 0ull;
+          s.pconf[(size_t)y * W + x] = 0.0;
+        }
+      }
+      append_front(s, fr, y * W + x);
     }
     __syncthreads();
-    block_refresh_tiles(s, max(0, px - R2), min(W - 1, px + R2), max(0, py - R2),
-                        min(H - 1, py + R2));
-
-    remaining -= filled;
-    if (filled == 0) {  // p^ must lie in Omega; stop rather than loop without progress
-      if (tid == 0) {
-        c->status = INPAINT_ERR_INTERNAL;
-        if (use_cond) cudaGraphSetConditional(cond, 0);
-      }
-      return;
-    }
     if (tid == 0) {
-      const int it = c->iter;
-      {
-        inpaint_step_info* e = &c->last;
-        e->iter = it;
-        e->px = px;
-        e->py = py;
-        e->qx = qx;
-        e->qy = qy;
-        e->ssd = ssd;
-        e->priority = pp;
-        e->confidence = cp;
-        e->filled = filled;
-        e->remaining = remaining;
-        e->n_known = n_known;
-        e->n_cand = n_cand;
-        if (it < s.trace_cap) s.trace[it] = *e;
+      if (filled == 0) {  // p^ must lie in Omega; stop rather than loop without progress
+        c->status = INPAINT_ERR_INTERNAL;
+        c->n_front = -1;
+        return;
       }
+      const int it = c->iter, remaining = c->remaining - filled;
+      inpaint_step_info e;
+      e.iter = it;
+      e.px = px;
+      e.py = py;
+      e.qx = qx;
+      e.qy = qy;
+      e.ssd = ssd;
+      e.priority = pp;
+      e.confidence = cp;
+      e.filled = filled;
+      e.remaining = remaining;
+      e.n_known = n_known;
+      e.n_cand = n_cand;
+      c->last = e;
+      if (it < s.trace_cap) s.trace[it] = e;
       c->remaining = remaining;
       c->iter = it + 1;
       c->n_valid = n_cand + newly;
       c->evals += (unsigned long long)n_cand * (unsigned long long)n_known;
-      c->px = -1;
-      c->py = -1;
+    }
+  }
+}
+
+// After k_prio_list: the tiles over the window of the target just filled and
+// the selection of the next one.  Single CTA.
+__global__ void __launch_bounds__(kUpdThreads) k_select_big(ImgState s, cudaGraphConditionalHandle cond,
+                                                            int use_cond) {
+  Ctrl* c = s.ctrl;
+  const int tid = threadIdx.x;
+  if (c->n_front >= 0) {
+    const int px = c->px, py = c->py, R2 = 2 * s.r + 1;
+    block_refresh_tiles(s, max(0, px - R2), min(s.W - 1, px + R2), max(0, py - R2), min(s.H - 1, py + R2));
+    if (tid < 32) {
+      if (c->remaining > 0) {
+        warp_select(s);
+      } else if (tid == 0) {
+        c->px = -1;
+        c->py = -1;
+      }
     }
     __syncthreads();
   }
+  if (use_cond && tid == 0) cudaGraphSetConditional(cond, c->n_front >= 0 && loop_active(c) ? 1u : 0u);
+}
 
-  // Selection of the next target: highest priority on the front, lowest
-  // index on ties, from the level-1 tile maxima.
-  if (remaining > 0 && tid < 32) warp_select(s);
-  __syncthreads();
-  if (use_cond && tid == 0) cudaGraphSetConditional(cond, loop_active(c) ? 1u : 0u);
+// Selection of the first target (initialisation).  One warp.
+__global__ void k_select_first(ImgState s) {
+  if (loop_active(s.ctrl) && s.ctrl->remaining > 0) warp_select(s);
 }
 
 // Debug self-check: recount every candidate's unknown pixels and re-evaluate
@@ -481,11 +598,12 @@ static cudaError_t init_tail(const ImgState& s, int32_t* sat, cudaStream_t st) {
     const cudaError_t e = launch_prio_init_fast(s, st);
     if (e != cudaSuccess) return e;
   } else {
-    k_prio_all<<<rows, 256, 0, st>>>(s);
+    k_front_all<<<rows, 256, 0, st>>>(s);
+    k_prio_list<<<kPrioCtas, 64, 0, st>>>(s);
   }
   k_tiles0_all<<<(s.t0x * s.t0y + 7) / 8, 256, 0, st>>>(s);
   k_tiles1_all<<<(s.t1x * s.t1y + 7) / 8, 256, 0, st>>>(s);
-  k_update<<<1, kUpdThreads, 0, st>>>(s, 0, 0ull, 0);
+  k_select_first<<<1, 32, 0, st>>>(s);
   return cudaGetLastError();
 }
 
@@ -504,10 +622,10 @@ cudaError_t launch_import(const ImgState& s, const uint8_t* rgb, const uint8_t* 
   return init_tail(s, sat, st);
 }
 
-cudaError_t launch_update(const ImgState& s, int do_fill, unsigned long long cond_handle,
-                          int use_cond, cudaStream_t st) {
-  k_update<<<1, kUpdThreads, 0, st>>>(s, do_fill, (cudaGraphConditionalHandle)cond_handle,
-                                      use_cond);
+cudaError_t launch_update(const ImgState& s, unsigned long long cond_handle, int use_cond, cudaStream_t st) {
+  k_fill_big<<<1, kUpdThreads, 0, st>>>(s);
+  k_prio_list<<<kPrioCtas, 64, 0, st>>>(s);
+  k_select_big<<<1, kUpdThreads, 0, st>>>(s, (cudaGraphConditionalHandle)cond_handle, use_cond);
   return cudaGetLastError();
 }
 

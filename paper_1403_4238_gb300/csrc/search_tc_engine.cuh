@@ -260,8 +260,8 @@ __device__ __forceinline__ uint2 tc_bits_load(const uint32_t* tbits, int N, int 
 
 // Accumulators at `tmem` of tile (y0, xs) -> this thread's best key, after the
 // tile's done barrier.  ngroups = warps / 4 column groups: warp w reads the
-// tensor-memory lanes of its quarter w % 4 and the columns of group w / 4,
-// eight at a time.  bits: tc_bits_load of the tile.
+// tensor-memory lanes of its quarter w % 4 and the columns of group w / 4, 16
+// (8 at the end) at a time.  bits: tc_bits_load of the tile.
 template <int R>
 __device__ __forceinline__ unsigned long long tc_epilogue(const ImgState& s, uint32_t tmem, const TcTiles& tt,
                                                           int ngroups, int a2, uint2 bits, int y0, int tx,
@@ -274,7 +274,7 @@ __device__ __forceinline__ unsigned long long tc_epilogue(const ImgState& s, uin
   // candidate of accumulator column n: n / n1 folds down, 8 (n % n1) columns right
   const int idx0 = (y0 + i) * s.W + tt.xs0 + 8 * tt.N * tx + b + R;
   auto idx_of = [&](int n) {
-    const int f = n / tt.n1;
+    const int f = tt.n1 == tt.N ? 0 : n / tt.n1;
     return idx0 + f * tt.h * s.W + 8 * (n - f * tt.n1);
   };
   const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0;
@@ -282,26 +282,52 @@ __device__ __forceinline__ unsigned long long tc_epilogue(const ImgState& s, uin
   float bv = __int_as_float(0x7f800000);  // +inf
   int bi = 0;
   bool any = false;
+  // eight columns from h: the smallest valid value and its column, kept in a
+  // chain of their own (the two halves of a step overlap); candidates in
+  // increasing index order (a fold's rows lie below the previous one's), so
+  // the strict tests keep the first of equals
+  auto test = [&](const uint32_t* X, const uint32_t* S, int h, float& v0, int& n0) {
+    const uint32_t wx = __shfl_sync(0xffffffffu, bits.x, src0 + h / 8) >> b;
+    const uint32_t wy = __shfl_sync(0xffffffffu, bits.y, src0 + h / 8) >> b;
+    any |= ((wx | wy) & 0x01010101u) != 0u;
+    v0 = __int_as_float(0x7f800000);
+    n0 = 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float v = __fadd_rn(__fmaf_rn(-2.0f, __uint_as_float(X[k]), __uint_as_float(S[k])), a2f);
+      if (((k < 4 ? wx : wy) & (1u << (8 * (k & 3)))) && v < v0) {
+        v0 = v;
+        n0 = c0 + h + k;
+      }
+    }
+  };
+  auto keep = [&](float v, int n) {
+    if (v < bv) {
+      bv = v;
+      bi = n;
+    }
+  };
+  float v0, v1;
+  int n0, n1;
+  int h = 0;
 #pragma unroll 1
-  for (int h = 0; h < cols; h += 8) {
+  for (; h + 16 <= cols; h += 16) {
+    uint32_t X[16], S[16];
+    tc_ld16(ta + (uint32_t)h, X);
+    tc_ld16(ta + (uint32_t)(128 + h), S);
+    tc_wait_ld();
+    test(X, S, h, v0, n0);
+    test(X + 8, S + 8, h + 8, v1, n1);
+    keep(v0, n0);
+    keep(v1, n1);
+  }
+  if (h < cols) {
     uint32_t X[8], S[8];
     tc_ld8(ta + (uint32_t)h, X);
     tc_ld8(ta + (uint32_t)(128 + h), S);
-    const uint2 w = make_uint2(__shfl_sync(0xffffffffu, bits.x, src0 + h / 8),
-                               __shfl_sync(0xffffffffu, bits.y, src0 + h / 8));
     tc_wait_ld();
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      // candidates in increasing index order (a fold's rows lie below the
-      // previous one's): the strict test keeps the first of equals
-      const float v = __fadd_rn(__fmaf_rn(-2.0f, __uint_as_float(X[k]), __uint_as_float(S[k])), a2f);
-      const bool valid = ((k < 4 ? w.x : w.y) >> (8 * (k & 3) + b)) & 1u;
-      any |= valid;
-      if (valid && v < bv) {
-        bv = v;
-        bi = c0 + h + k;
-      }
-    }
+    test(X, S, h, v0, n0);
+    keep(v0, n0);
   }
   // tcgen05.ld is a whole warp's instruction, so the warp decides together: it
   // takes the integer pass when any of its threads has no candidate below 2^24

@@ -777,8 +777,14 @@ __device__ inline void update_work(const ImgState& s, UpdSmem<R>& sm, bool fence
   }
   const int px = sm.px, py = sm.py, W = s.W;
   {
-    const bool mine = t0 < P * P && sm.filled[t0 < P * P ? t0 : 0];
-    const int dy = t0 / P - R, dx = t0 % P - R;
+    // one thread copies a pixel; the tensor-core search's planes of it are
+    // another thread's when there are two per pixel (the planes take as long
+    // as all the rest)
+    constexpr bool kTwo = 2 * P * P <= kMidThreads;
+    const bool second = kTwo && t0 >= P * P;
+    const int tp = second ? t0 - P * P : t0;
+    const bool mine = tp < P * P && (!second || s.planes) && sm.filled[tp < P * P ? tp : 0];
+    const int dy = tp / P - R, dx = tp % P - R;
     uint32_t w = 0u;
     if (mine) w = __ldcg(&s.img[(sm.qy + dy) * s.pitch + sm.qx + dx]);  // in flight during the counts
     int newly = 0;
@@ -795,13 +801,15 @@ __device__ inline void update_work(const ImgState& s, UpdSmem<R>& sm, bool fence
     }
     if (mine) {
       const int tx = px + dx, ty = py + dy, q = ty * W + tx;
-      const uint8_t g = (uint8_t)luma_word(w);
-      s.img[ty * s.pitch + tx] = w;
-      if (s.planes) plane_store(s, tx, ty, w);  // the tensor-core search's operands
-      s.gray[q] = g;
-      s.conf[q] = sm.cp;
-      s.omega[q] = 0;
-      sm.gr[(RB + dy) * NS + RB + dx] = g;
+      if (!second) {
+        const uint8_t g = (uint8_t)luma_word(w);
+        s.img[ty * s.pitch + tx] = w;
+        s.gray[q] = g;
+        s.conf[q] = sm.cp;
+        s.omega[q] = 0;
+        sm.gr[(RB + dy) * NS + RB + dx] = g;
+      }
+      if (second || (!kTwo && s.planes)) plane_store(s, tx, ty, w);
     }
     if (newly) atomicAdd(&sm.newly, newly);
   }
@@ -886,17 +894,16 @@ __device__ inline void update_prio(const ImgState& s, UpdSmem<R>& sm, unsigned l
     else if ((tid & 31) == 0 && wk == 0ull) sm.red_pb[tid >> 5] = PrioBest{0ull, 0x7fffffff, 0};
   }
   __syncthreads();
-  wk = sm.out_key;
-  wi = sm.out_idx;
-  ny = sm.out_y;
-#pragma unroll
-  for (int w = 0; w < kChainThreads / 32; ++w) {
-    const PrioBest b = sm.red_pb[w];
-    const bool t = prio_better(b.key, b.idx, wk, wi);
-    wk = t ? b.key : wk;
-    wi = t ? b.idx : wi;
-    ny = t ? b.pad : ny;
-  }
+  // every warp reduces the five candidates (lanes 0-3: the warps', 4: outside)
+  const int lane = tid & 31;
+  PrioBest b = {0ull, 0x7fffffff, 0};
+  if (lane < kChainThreads / 32) b = sm.red_pb[lane];
+  else if (lane == kChainThreads / 32) b = PrioBest{sm.out_key, sm.out_idx, sm.out_y};
+  wk = b.key;
+  wi = b.idx;
+  warp_best_prio(wk, wi);
+  const unsigned at = __ballot_sync(0xffffffffu, b.key == wk && b.idx == wi);
+  ny = __shfl_sync(0xffffffffu, b.pad, __ffs(at) - 1);
 }
 
 // After the selection (whole block, no barrier inside): key 0 for the
