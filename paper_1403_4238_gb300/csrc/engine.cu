@@ -45,7 +45,7 @@ __global__ void k_planes(ImgState s) {
     const int x = s.tc_xs0 + 8 * (tx * s.tc_n - f * s.tc_n1) + xl, yi = y + f * s.tc_h;
     const bool in = x < s.W && yi < s.H && (f == 0 || f < s.tc_f);
     const uint32_t w = in ? __ldg(&s.img[(size_t)yi * s.pitch + x]) : 0x00808080u;
-    plane_store_at(s, tx, y, xl, w);  // outside the image: 128 - 128 = 0 everywhere
+    plane_write(s.planes + ((size_t)tx * s.prows + y) * 5 * s.tc_len + xl, s.tc_len, w);  // outside the image: 128 - 128 = 0 everywhere
   }
 }
 

@@ -104,88 +104,45 @@ __device__ __forceinline__ uint32_t row_desc(uint32_t m, int P) {
   return kRowMask | m;
 }
 
-// SSD terms of target column DX for the lane's NCL candidates.
-#define INP_SSD_COL(DX)                                                   \
-  if constexpr ((DX) < P) {                                               \
-    _Pragma("unroll") for (int k = 0; k < NCL; ++k) {                     \
-      const uint32_t d_ = __vabsdiffu4(t[(DX)], r[k + (DX)]);             \
-      acc[k] = __dp4a(d_, d_, acc[k]);                                    \
-    }                                                                     \
-  }
-
 // SSD of this lane's NCL candidates against the staged target (Eq. 4): for
 // every known target pixel one byte-SIMD absolute difference and one 4-way
 // byte dot product per candidate (|a-b| per channel, squares summed; alpha
-// is 0 on both sides).  `strip` points at the lane's row strip in the tile
-// (row = lane, column = warp * NCL); `rowd` holds one row descriptor per
-// target row.  A run of known columns [s, P) enters an ascending sequence of
-// columns at s, a run [0, e) a descending one at e - 1 (one warp-uniform
-// indirect jump per row); other rows test a bit per column.
-template <int R, int SRW>
-__device__ __forceinline__ void unit_ssd(const uint32_t* __restrict__ strip,
-                                         const uint32_t* __restrict__ tgt,
-                                         const uint32_t* __restrict__ rowd,
-                                         uint32_t (&acc)[4 * SRW]) {
-  using G = EngGeom<R, SRW>;
-  constexpr int P = G::P, NS = G::NS, NCL = G::NCL, BW = G::BW, TP = G::TP;
-  static_assert(P <= 17, "column sequences are written out for P <= 17");
+// is 0 on both sides).  `strip` points at the lane's row strip in its tile
+// (row pitch `pitch` words), over the target rows [r0, r1); `rowd` holds one
+// row descriptor per target row:
+// per row one indexed jump into the sequences of ssd_rows.cuh (a run of known
+// columns [s, P) enters an ascending sequence at s, a run [0, e) a descending
+// one at e - 1); other row shapes test a bit per column.
+template <int R, int NCL>
+__device__ __forceinline__ void unit_ssd(const uint32_t* __restrict__ strip, int pitch,
+                                         const uint32_t* __restrict__ tgt, const uint32_t* __restrict__ rowd,
+                                         int r0, int r1, uint32_t (&acc)[NCL]) {
+  constexpr int P = 2 * R + 1, NS = (NCL + P - 1 + 3) & ~3, TP = (P + 3) & ~3;
 #pragma unroll
   for (int k = 0; k < NCL; ++k) acc[k] = 0;
 #pragma unroll 1
-  for (int dy = 0; dy < P; ++dy) {
+  for (int dy = r0; dy < r1; ++dy) {
     const uint32_t desc = rowd[dy];
     if (desc == kRowSkip) continue;
     uint32_t r[NS], t[TP];
-    lds_words(r, strip + dy * BW);
+    lds_words(r, strip + dy * pitch);
     lds_words(t, tgt + dy * TP);
-    const uint32_t kind = desc & (3u << 30), arg = desc & 0xffffu;
-    if (kind == kRowFrom) {
-      switch (arg) {
-        case 0: INP_SSD_COL(0) [[fallthrough]];
-        case 1: INP_SSD_COL(1) [[fallthrough]];
-        case 2: INP_SSD_COL(2) [[fallthrough]];
-        case 3: INP_SSD_COL(3) [[fallthrough]];
-        case 4: INP_SSD_COL(4) [[fallthrough]];
-        case 5: INP_SSD_COL(5) [[fallthrough]];
-        case 6: INP_SSD_COL(6) [[fallthrough]];
-        case 7: INP_SSD_COL(7) [[fallthrough]];
-        case 8: INP_SSD_COL(8) [[fallthrough]];
-        case 9: INP_SSD_COL(9) [[fallthrough]];
-        case 10: INP_SSD_COL(10) [[fallthrough]];
-        case 11: INP_SSD_COL(11) [[fallthrough]];
-        case 12: INP_SSD_COL(12) [[fallthrough]];
-        case 13: INP_SSD_COL(13) [[fallthrough]];
-        case 14: INP_SSD_COL(14) [[fallthrough]];
-        case 15: INP_SSD_COL(15) [[fallthrough]];
-        case 16: INP_SSD_COL(16) [[fallthrough]];
-        default: break;
-      }
-    } else if (kind == kRowUpTo) {
-      switch (arg) {
-        case 17: INP_SSD_COL(16) [[fallthrough]];
-        case 16: INP_SSD_COL(15) [[fallthrough]];
-        case 15: INP_SSD_COL(14) [[fallthrough]];
-        case 14: INP_SSD_COL(13) [[fallthrough]];
-        case 13: INP_SSD_COL(12) [[fallthrough]];
-        case 12: INP_SSD_COL(11) [[fallthrough]];
-        case 11: INP_SSD_COL(10) [[fallthrough]];
-        case 10: INP_SSD_COL(9) [[fallthrough]];
-        case 9: INP_SSD_COL(8) [[fallthrough]];
-        case 8: INP_SSD_COL(7) [[fallthrough]];
-        case 7: INP_SSD_COL(6) [[fallthrough]];
-        case 6: INP_SSD_COL(5) [[fallthrough]];
-        case 5: INP_SSD_COL(4) [[fallthrough]];
-        case 4: INP_SSD_COL(3) [[fallthrough]];
-        case 3: INP_SSD_COL(2) [[fallthrough]];
-        case 2: INP_SSD_COL(1) [[fallthrough]];
-        case 1: INP_SSD_COL(0) [[fallthrough]];
-        default: break;
-      }
+    const uint32_t kind = desc & (3u << 30);
+    if (kind != kRowMask) {
+      const uint32_t arg = desc & 0xffffu;
+      // entry of the jump table: [0, P) ascending from column s, [P, 2P)
+      // descending from column e - 1; clamped so that it stays in the table
+      const uint32_t idx = min(kind == kRowFrom ? arg : (uint32_t)P + arg - 1u, (uint32_t)(2 * P - 1));
+#define INP_ROW(N, PP) \
+  if constexpr (NCL == N && P == PP) INP_SSD_ROW##N##_P##PP(acc, r, t, idx);
+#define INP_ROWS(PP) INP_ROW(4, PP) INP_ROW(8, PP) INP_ROW(16, PP)
+      INP_ROWS(3) INP_ROWS(5) INP_ROWS(7) INP_ROWS(9) INP_ROWS(11) INP_ROWS(13) INP_ROWS(15) INP_ROWS(17)
+#undef INP_ROWS
+#undef INP_ROW
     } else {
-      const uint32_t m = desc;  // kRowMask: bits of the known columns (P <= 17 < 30)
 #pragma unroll
       for (int dx = 0; dx < P; ++dx) {
-        if (m & (1u << dx)) {
+        if (desc & (1u << dx)) {
 #pragma unroll
           for (int k = 0; k < NCL; ++k) {
             const uint32_t d = __vabsdiffu4(t[dx], r[k + dx]);
@@ -196,25 +153,24 @@ __device__ __forceinline__ void unit_ssd(const uint32_t* __restrict__ strip,
     }
   }
 }
-#undef INP_SSD_COL
 
-// The compute of a search round, outside the engine body so that its
+// The compute of a streaming search round, outside the engine body so that its
 // registers hold only the row strips, the target row and the accumulators
 // (the engine body keeps the leader's state live across the search).  These
 // functions take byte offsets into the CTA's shared memory, not pointers: a
 // pointer argument is a generic address, whose every access is a generic
 // load with 64-bit address arithmetic.
 
-// Smallest key (SSD << 32 | idx) of this lane's candidates in one unit:
+// Smallest key (SSD << 32 | idx) of this lane's NCL candidates in one unit:
 // `bits` marks the valid ones, idx0 is the linear index of the first.
-template <int R, int SRW>
-__device__ __noinline__ unsigned long long unit_best(int strip, int tgt, uint32_t bits, unsigned idx0) {
-  uint32_t acc[4 * SRW];
-  unit_ssd<R, SRW>(smem_words(strip), smem_words(tgt), smem_words(tgt) + EngGeom<R, SRW>::P * EngGeom<R, SRW>::TP,
-                   acc);
+template <int R, int NCL>
+__device__ __noinline__ unsigned long long unit_best(int strip, int pitch, int tgt, uint32_t bits, unsigned idx0) {
+  constexpr int P = 2 * R + 1, TP = (P + 3) & ~3;
+  uint32_t acc[NCL];
+  unit_ssd<R, NCL>(smem_words(strip), pitch, smem_words(tgt), smem_words(tgt) + P * TP, 0, P, acc);
   unsigned long long best = ~0ull;
 #pragma unroll
-  for (int k = 0; k < 4 * SRW; ++k) {
+  for (int k = 0; k < NCL; ++k) {
     const unsigned long long key = ((unsigned long long)acc[k] << 32) | (idx0 + (unsigned)k);
     if ((bits & (1u << k)) && key < best) best = key;
   }
@@ -224,13 +180,18 @@ __device__ __noinline__ unsigned long long unit_best(int strip, int tgt, uint32_
 // ---------------------------------------------------------------- resident search
 
 // Resident mode: the candidate rectangle is cut into units of 32 candidate
-// rows (one per lane) x 16 candidate columns (one lane's candidates); the
+// rows (one per lane) x KC candidate columns (one lane's candidates); the
 // units, in band-major order, are split into contiguous ranges of equal
 // size, one per searching CTA.  A CTA keeps the source window of its units
 // in shared memory for the whole removal (one tile per 32-row band its range
-// touches) and after each publication only patches the pixels the previous
-// iteration filled and the validity of the candidates near them.
-constexpr int kResCols = 16;   // candidates per lane
+// touches) and after each iteration's copy only patches the pixels it filled
+// and the validity of the candidates near them.  KC is 16 when that gives a
+// CTA 12 units or more (most of its warps one), else 4, with the target rows of the
+// CTA's units dealt to its warps in equal shares and the partial SSDs summed
+// in shared memory: a small image has few units per CTA (512x384 over 151
+// CTAs: 3 of 16 columns, 10 of 4), and a warp alone on its scheduler takes
+// about 500 cycles a row, most of it latency.  Only CTAs that do not lead
+// search this way (a leader that searches too has a small team and streams).
 constexpr int kResRows = 32;   // candidate rows per unit (one per lane)
 constexpr int kResMaxSeg = 4;  // bands one CTA's tiles may span
 
@@ -249,104 +210,11 @@ struct ResPlan {
   ResSeg seg[kResMaxSeg];
 };
 
-template <int R>
-struct ResGeom {
-  static constexpr int P = 2 * R + 1;
-  static constexpr int NS = (kResCols + P - 1 + 3) & ~3;  // strip words per lane
-  static constexpr int TP = (P + 3) & ~3;
-  static constexpr int TH = kResRows + 2 * R;             // tile rows
-};
-
-// SSD of this lane's 16 candidates (Eq. 4) for one unit: per target row one
-// indexed jump into the row sequences of ssd_rows.cuh (known run [s, P) or
-// [0, e)); other row shapes test a bit per column.
-template <int R>
-__device__ __forceinline__ void unit16_ssd(const uint32_t* __restrict__ strip, int pitch,
-                                           const uint32_t* __restrict__ tgt,
-                                           const uint32_t* __restrict__ rowd, uint32_t (&acc)[kResCols]) {
-  using G = ResGeom<R>;
-  constexpr int P = G::P, NS = G::NS, TP = G::TP;
-#pragma unroll
-  for (int k = 0; k < kResCols; ++k) acc[k] = 0;
-#pragma unroll 1
-  for (int dy = 0; dy < P; ++dy) {
-    const uint32_t desc = rowd[dy];
-    if (desc == kRowSkip) continue;
-    uint32_t r[NS], t[TP];
-    lds_words(r, strip + dy * pitch);
-    lds_words(t, tgt + dy * G::TP);
-    const uint32_t kind = desc & (3u << 30);
-    if (kind != kRowMask) {
-      const uint32_t arg = desc & 0xffffu;
-      // entry of the jump table: [0, P) ascending from column s, [P, 2P)
-      // descending from column e - 1; clamped so that it stays in the table
-      const uint32_t idx = min(kind == kRowFrom ? arg : (uint32_t)P + arg - 1u, (uint32_t)(2 * P - 1));
-      if constexpr (P == 3) INP_SSD_ROW16_P3(acc, r, t, idx);
-      if constexpr (P == 5) INP_SSD_ROW16_P5(acc, r, t, idx);
-      if constexpr (P == 7) INP_SSD_ROW16_P7(acc, r, t, idx);
-      if constexpr (P == 9) INP_SSD_ROW16_P9(acc, r, t, idx);
-      if constexpr (P == 11) INP_SSD_ROW16_P11(acc, r, t, idx);
-      if constexpr (P == 13) INP_SSD_ROW16_P13(acc, r, t, idx);
-      if constexpr (P == 15) INP_SSD_ROW16_P15(acc, r, t, idx);
-      if constexpr (P == 17) INP_SSD_ROW16_P17(acc, r, t, idx);
-    } else {
-#pragma unroll
-      for (int dx = 0; dx < P; ++dx) {
-        if (desc & (1u << dx)) {
-#pragma unroll
-          for (int k = 0; k < kResCols; ++k) {
-            const uint32_t d = __vabsdiffu4(t[dx], r[k + dx]);
-            acc[k] = __dp4a(d, d, acc[k]);
-          }
-        }
-      }
-    }
-  }
-}
-
-// Smallest key (SSD << 32 | idx) of this lane's 16 candidates of one unit:
-// `vb` marks the valid ones, idx0 is the linear index of the first.
-template <int R>
-__device__ __noinline__ unsigned long long unit16_best(int strip, int pitch, int tgt, uint32_t vb,
-                                                       unsigned idx0) {
-  uint32_t acc[kResCols];
-  unit16_ssd<R>(smem_words(strip), pitch, smem_words(tgt), smem_words(tgt) + ResGeom<R>::P * ResGeom<R>::TP, acc);
-  unsigned long long best = ~0ull;
-#pragma unroll
-  for (int k = 0; k < kResCols; ++k) {
-    const unsigned long long key = ((unsigned long long)acc[k] << 32) | (idx0 + (unsigned)k);
-    if ((vb & (1u << k)) && key < best) best = key;
-  }
-  return best;
-}
-
-// All units of this CTA for the current target, warp w taking its local
-// units w, w + 16, ...; returns the lane's smallest key.
-template <int R>
-__device__ __noinline__ unsigned long long resident_units16(int plan, int tiles, int xb, int cy0, int W, int tgt) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const ResPlan* pl = reinterpret_cast<const ResPlan*>(smem_words(plan));
-  const int u0 = pl->u0, n = pl->u1 - pl->u0, ncu = pl->ncu, b0 = pl->seg[0].band;
-  const uint16_t* bits = reinterpret_cast<const uint16_t*>(smem_words(tiles + pl->bits_off));
-  unsigned long long best = ~0ull;
-#pragma unroll 1
-  for (int j = warp; j < n; j += kEngWarps) {
-    const int u = u0 + j, band = u / ncu, col = u - band * ncu;
-    const ResSeg& sg = pl->seg[band - b0];
-    const int strip = tiles + sg.off + 4 * (lane * sg.pitch + (col - sg.c_lo) * kResCols);
-    const unsigned idx0 = (unsigned)((cy0 + band * kResRows + lane) * W + xb + col * kResCols);
-    const unsigned long long k = unit16_best<R>(strip, sg.pitch, tgt, bits[j * 32 + lane], idx0);
-    best = k < best ? k : best;
-  }
-  return best;
-}
-
 // Plan of rank `rank`'s units: the tile of each band its range touches.
 // Returns the bytes of shared memory the plan needs (tiles + validity
 // bits), or -1 when the range spans more bands than kResMaxSeg.
 template <int R>
-__host__ __device__ inline long long res_plan(ResPlan& pl, int ncu, int nbands, int rank, int ns) {
-  using G = ResGeom<R>;
+__host__ __device__ inline long long res_plan(ResPlan& pl, int kc, int ncu, int nbands, int rank, int ns) {
   const long long U = (long long)ncu * nbands;
   pl.u0 = (int)(U * rank / ns);
   pl.u1 = (int)(U * (rank + 1) / ns);
@@ -365,9 +233,9 @@ __host__ __device__ inline long long res_plan(ResPlan& pl, int ncu, int nbands, 
     ResSeg& sg = pl.seg[pl.nseg++];
     sg.band = b;
     sg.c_lo = c_lo;
-    sg.pitch = width_odd16((c_hi - c_lo) * kResCols + 2 * R);
+    sg.pitch = width_odd16((c_hi - c_lo) * kc + 2 * R + 4);  // (+ the strips' rounding)
     sg.off = (int)off;
-    off += (((long long)sg.pitch * G::TH * 4) + 127) / 128 * 128;
+    off += (((long long)sg.pitch * (kResRows + 2 * R) * 4) + 127) / 128 * 128;
   }
   pl.bits_off = (int)off;
   off += (long long)(pl.u1 - pl.u0) * 32 * 2;
@@ -397,7 +265,7 @@ struct EngSmemTail {
   int tc_pref;    // tensor-core search: slots the producer prefetched for the next round
   TcRun tc_run;   // a searching leader's tensor-core search between its rounds
   int lim, status, err;  // leader: iteration limit, status and error word (the stop decision)
-  uint8_t known[2][17 * 17];  // known flags of the last two targets (by round parity)
+  uint8_t known[17 * 17];     // known flags of the round's target
   ResPlan plan;               // resident mode: this CTA's units and tiles
 };
 
@@ -830,6 +698,185 @@ __device__ __noinline__ unsigned long long tc_lead_share(const EngineArgs& ea, E
   return best;
 }
 
+// The loop of a CTA that searches in resident mode and does not lead (its plan,
+// the image's state block, the stop flag and the first target are in shared
+// memory), compiled as a function of its own with everything inlined: the
+// registers a call saves come back from L2, since L1 is nearly all shared
+// memory (two nested calls per unit took 2,000 cycles a round).
+template <int R, int KC>
+__device__ __noinline__ void run_res_search(const EngineArgs& ea, EngCtx& x, int xb, int ncu, int acc_off) {
+  constexpr int P = 2 * R + 1, TP = (P + 3) & ~3, TH = kResRows + 2 * R;
+  EngSmemTail& tl = *reinterpret_cast<EngSmemTail*>(eng_smem());
+  const ImgState& s = tl.img;
+  const ResPlan& pl = tl.plan;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rank = x.rank;
+  TeamCtl* const tc = x.tc;
+  unsigned long long* const tpart = x.tpart;
+  const unsigned long long limit = ea.wait_limit_ns;
+  const bool withheld = rank + 1 == ea.withhold;
+  int* const err = ea.err;
+  unsigned epoch = x.epoch;
+  uint8_t* const area = eng_smem() + kHeadBytes;
+  uint32_t* const tgt = reinterpret_cast<uint32_t*>(eng_smem() + kTgtOff);
+  uint32_t* const rowd = tgt + P * TP;
+  uint32_t* const part = reinterpret_cast<uint32_t*>(eng_smem() + acc_off);  // KC < 16: partial SSDs [unit][k][lane]
+  const int u0 = pl.u0, n = pl.u1 - pl.u0, b0 = pl.seg[0].band;
+  uint16_t* const bits = reinterpret_cast<uint16_t*>(area + pl.bits_off);
+  // the source windows of every band segment (plain 16-byte loads; outside
+  // the image: zero), then the validity bits of every unit
+  for (int g = 0; g < pl.nseg; ++g) {
+    const ResSeg sg = pl.seg[g];
+    const int x0 = xb - R + sg.c_lo * KC, y0 = s.cy0 + sg.band * kResRows - R;
+    const int nq = sg.pitch / 4;
+    uint4* dst = reinterpret_cast<uint4*>(area + sg.off);
+    for (int i = tid; i < TH * nq; i += kEngThreads) {
+      const int row = i / nq, q = i - row * nq, y = y0 + row, xw = x0 + 4 * q;
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
+      if (y >= 0 && y < s.H && xw + 3 < s.pitch)
+        v = __ldcg(reinterpret_cast<const uint4*>(s.img + (size_t)y * s.pitch + xw));
+      dst[i] = v;
+    }
+  }
+  for (int j = warp; j < n; j += kEngWarps) {
+    const int u = u0 + j, band = u / ncu, col = u - band * ncu;
+    const int qy = s.cy0 + band * kResRows + lane, qx0 = xb + col * KC;
+    uint32_t v = 0;
+    if (qy <= s.cy1) {
+#pragma unroll
+      for (int k = 0; k < KC; ++k) {
+        const int qx = qx0 + k;
+        if (qx >= s.cx0 && qx <= s.cx1 && __ldcg(&s.count[(size_t)qy * s.pitch + qx]) == 0) v |= 1u << k;
+      }
+    }
+    bits[j * 32 + lane] = (uint16_t)v;
+  }
+  while (!tl.stop) {
+    const int px = tl.px, py = tl.py;
+    // target patch: warp dy reads row dy (lane = dx); the ballot of the
+    // known flags gives the row descriptor
+    for (int dy = warp; dy < P; dy += kEngWarps) {
+      const int tx = px + lane - R, ty = py + dy - R;
+      uint32_t w = 0;
+      bool known = false;
+      if (lane < P && tx >= 0 && tx < s.W && ty >= 0 && ty < s.H) {
+        // both reads in flight together; the pixel is kept only if known
+        const uint8_t o = __ldcg(&s.omega[(size_t)ty * s.W + tx]);
+        const uint32_t v = __ldcg(&s.img[(size_t)ty * s.pitch + tx]);
+        known = o == 0;
+        w = known ? v : 0u;
+      }
+      const unsigned bal = __ballot_sync(0xffffffffu, known);
+      if (lane < P) {
+        tgt[dy * TP + lane] = w;
+        tl.known[dy * P + lane] = (uint8_t)known;
+      }
+      if (lane == 0) rowd[dy] = row_desc(bal & ((1u << P) - 1u), P);
+    }
+    if constexpr (KC < 16)
+      for (int i = tid; i < n * KC * 32; i += kEngThreads) part[i] = 0u;
+    __syncthreads();
+    unsigned long long best = ~0ull;
+    auto take = [&](int j, const uint32_t (&acc)[KC]) {
+      const int u = u0 + j, band = u / ncu, col = u - band * ncu;
+      const uint32_t vb = bits[j * 32 + lane];
+      const unsigned idx0 = (unsigned)((s.cy0 + band * kResRows + lane) * s.W + xb + col * KC);
+#pragma unroll
+      for (int k = 0; k < KC; ++k) {
+        const unsigned long long key = ((unsigned long long)acc[k] << 32) | (idx0 + (unsigned)k);
+        if ((vb & (1u << k)) && key < best) best = key;
+      }
+    };
+    // (KC 16: whole units, warp w takes w, w + 16, ...; else the rows
+    // [w T / 16, (w + 1) T / 16) of the T = n P unit rows)
+    int t = KC < 16 ? warp * n * P / kEngWarps : warp * P;
+    const int t1 = KC < 16 ? (warp + 1) * n * P / kEngWarps : n * P;
+#pragma unroll 1
+    while (t < t1) {
+      const int j = t / P, r0 = t - j * P, r1 = min(P, r0 + t1 - t);
+      const int u = u0 + j, band = u / ncu, col = u - band * ncu;
+      const ResSeg& sg = pl.seg[band - b0];
+      const uint32_t* strip = reinterpret_cast<const uint32_t*>(area + sg.off) + lane * sg.pitch + (col - sg.c_lo) * KC;
+      uint32_t acc[KC];
+      unit_ssd<R, KC>(strip, sg.pitch, tgt, rowd, r0, r1, acc);
+      if constexpr (KC < 16) {
+#pragma unroll
+        for (int k = 0; k < KC; ++k) atomicAdd(&part[(j * KC + k) * 32 + lane], acc[k]);
+        t += r1 - r0;
+      } else {
+        take(j, acc);
+        t += kEngWarps * P;
+      }
+    }
+    if constexpr (KC < 16) {
+      __syncthreads();
+#pragma unroll 1
+      for (int j = warp; j < n; j += kEngWarps) {
+        uint32_t acc[KC];
+#pragma unroll
+        for (int k = 0; k < KC; ++k) acc[k] = part[(j * KC + k) * 32 + lane];
+        take(j, acc);
+      }
+    }
+    best = block_min_u64(best, tl.red64);
+    if (tid == 0) {
+      if (!withheld) st_relaxed64(&tpart[rank], key_tag(best, epoch));
+      // the tiles are brought up to date as soon as the copy is done, while the
+      // leader still works on the priorities (after the publication, this and
+      // the target's reads were three L2 round trips one after another)
+      const unsigned long long t0 = globaltimer();
+      while ((int)(ld_acquire(&tc->copied) - (epoch + 1u)) < 0 && (unsigned)ld_acquire64(&tc->pub) == epoch &&
+             globaltimer() - t0 <= limit) {
+      }
+    }
+    __syncthreads();
+    {
+      // the iteration's filled pixels (the target patch's unknown in-image
+      // ones) into every tile that holds them, and the candidates within 2R of
+      // it that became valid; every load in flight before the first use
+      constexpr int NCW = 4 * R + 1, NV = (NCW * NCW + kEngThreads - 1) / kEngThreads;
+      const int tx = px + tid % P - R, ty = py + tid / P - R;
+      const bool filled = tid < P * P && tx >= 0 && tx < s.W && ty >= 0 && ty < s.H && !tl.known[tid < P * P ? tid : 0];
+      uint32_t w = 0u;
+      if (filled) w = __ldcg(&s.img[(size_t)ty * s.pitch + tx]);
+      int cnt[NV];
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        const int jj = tid + v * kEngThreads, qx = px + jj % NCW - 2 * R, qy = py + jj / NCW - 2 * R;
+        const bool in = jj < NCW * NCW && qx >= s.cx0 && qx <= s.cx1 && qy >= s.cy0 && qy <= s.cy1;
+        cnt[v] = in ? __ldcg(&s.count[(size_t)qy * s.pitch + qx]) : 1;
+      }
+      if (filled) {
+#pragma unroll 1
+        for (int g = 0; g < pl.nseg; ++g) {
+          const ResSeg& sg = pl.seg[g];
+          const int lx = tx - (xb - R + sg.c_lo * KC), ly = ty - (s.cy0 + sg.band * kResRows - R);
+          if (lx >= 0 && lx < sg.pitch && ly >= 0 && ly < TH)
+            reinterpret_cast<uint32_t*>(area + sg.off)[ly * sg.pitch + lx] = w;
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < NV; ++v) {
+        if (cnt[v] != 0) continue;
+        const int jj = tid + v * kEngThreads, qx = px + jj % NCW - 2 * R, qy = py + jj / NCW - 2 * R;
+        const int col = (qx - xb) / KC, j = (qy - s.cy0) / kResRows * ncu + col - u0;
+        if (j < 0 || j >= n) continue;
+        const int e = j * 32 + (qy - s.cy0) % kResRows;
+        atomicOr(reinterpret_cast<unsigned*>(bits) + (e >> 1), (1u << (qx - xb - col * KC)) << (16 * (e & 1)));
+      }
+    }
+    if (tid == 0) {
+      const unsigned long long v = wait_pub(tc, epoch, err, limit);
+      tl.stop = ((v >> 62) & 1ull) != 0;
+      tl.px = (int)((v >> 32) & 0x7fff);
+      tl.py = (int)((v >> 47) & 0x7fff);
+    }
+    ++epoch;
+    __syncthreads();
+  }
+  x.epoch = epoch;
+}
+
 // The loop of a leader that does not search, compiled as a function of its
 // own: none of the search state is live through its phases, so its
 // registers hold the update's working set.
@@ -841,7 +888,7 @@ __device__ __noinline__ void run_lead_only(const EngineArgs& ea, int j, EngCtx& 
 template <int R, int SRW, bool kLeadOnly>
 __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x) {
   using G = EngGeom<R, SRW>;
-  using RG = ResGeom<R>;
+  constexpr int TH = kResRows + 2 * R;  // rows of a resident tile
   constexpr int P = G::P, B = G::B;
   uint8_t* const smem = eng_smem();
   EngSmemTail& tl = *reinterpret_cast<EngSmemTail*>(smem);
@@ -904,9 +951,28 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     tc_nb = min(kTcRing, ((int)x.smem_bytes - (tc_off - (int)kHeadBytes) - fixed) / tc_slot_b);
   }
   const bool lead_searches = tcmode ? tc_lead : tsize == 1 || nbatch >= 8 * tsize;
-  const int ns = tcmode         ? (tc_lead ? min(tsize, tc_ntiles) : min(tsize - 1, tc_ntiles))
-                 : lead_searches ? tsize
-                                 : min(tsize - 1, nbatch);
+  const int nsmax = lead_searches ? tsize : tsize - 1;  // CTAs that may search
+  // Plain form, resident mode when the leader does not search and every
+  // searching CTA's tiles fit (the same decision in every CTA of the team: it
+  // depends only on the image and the team): two tiles (a range may straddle a
+  // band boundary), the validity bits and the partial SSDs; more than one band
+  // of units per CTA streams instead.
+  const int nbands = s.cy1 >= s.cy0 ? (s.cy1 - s.cy0 + kResRows) / kResRows : 0;
+  int kc = 16, ncu = 0, ns = 0;
+  bool resident = false;
+  if (tcmode) {
+    ns = min(nsmax, tc_ntiles);
+  } else {
+    for (; !lead_searches; kc = 4) {
+      ncu = s.cx1 >= s.cx0 ? (s.cx1 - xb + kc) / kc : 0;
+      ns = min(nsmax, ncu * nbands);
+      const int m = ns > 0 ? (ncu * nbands + ns - 1) / ns : 0;  // most units of one CTA
+      const int need = TH * 4 * (m * kc + 2 * (2 * R + 12)) + 640 + m * 64 + (kc < 16 ? m * kc * 128 : 0);
+      resident = m > 0 && m <= ncu && need <= (int)x.smem_bytes - (int)kHeadBytes;
+      if (m >= 3 * kEngWarps / 4 || kc == 4) break;
+    }
+    if (!resident) ns = min(nsmax, nbatch);
+  }
   const bool leader = rank == tsize - 1;
   const bool searcher = rank < ns;
   if constexpr (!kLeadOnly) {
@@ -914,14 +980,23 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
       run_lead_only<R, SRW>(ea, j, x);
       return;
     }
+  }
+  if (tid == 0) {
+    tl.stop = !ctrl_active(c) || __ldcg(err) != 0;
+    tl.px = __ldcg(&c->px);
+    tl.py = __ldcg(&c->py);
+    if (resident && searcher) res_plan<R>(tl.plan, kc, ncu, nbands, rank, ns);
+  }
+  __syncthreads();
+  if constexpr (!kLeadOnly) {
     if (tcmode && searcher && !leader) {
-      if (tid == 0) {
-        tl.stop = !ctrl_active(c) || __ldcg(err) != 0;
-        tl.px = __ldcg(&c->px);
-        tl.py = __ldcg(&c->py);
-      }
-      __syncthreads();
       run_tc_search<R>(ea, x, tt, tc_nb, tc_slot_b, ns, tc_lead);
+      return;
+    }
+    if (resident && searcher) {
+      const int acc_off = ((int)kHeadBytes + tl.plan.bits_off + (tl.plan.u1 - tl.plan.u0) * 64 + 127) & ~127;
+      if (kc == 16) run_res_search<R, 16>(ea, x, xb, ncu, acc_off);
+      else run_res_search<R, 4>(ea, x, xb, ncu, acc_off);
       return;
     }
   }
@@ -932,45 +1007,12 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
                         reinterpret_cast<uint32_t*>(area + G::CNT_BYTES)};
   uint8_t* slots = area + 2 * G::CNT_BYTES;
   auto slot_pix = [&](int i) { return reinterpret_cast<uint32_t*>(slots + (size_t)i * G::SLOT_BYTES); };
-  // resident mode when every searching CTA's tiles fit (the same decision
-  // in every CTA of the team: the bound below depends only on the image,
-  // the team and the smallest work area, a searching leader's)
-  const int ncu = s.cx1 >= s.cx0 ? (s.cx1 - xb + kResCols) / kResCols : 0;
-  const int nbands = s.cy1 >= s.cy0 ? (s.cy1 - s.cy0 + kResRows) / kResRows : 0;
-  bool resident = false;
-  {
-    const long long U = (long long)ncu * nbands;
-    const long long m = ns > 0 ? (U + ns - 1) / ns : 0;  // most units of one CTA
-    const long long avail =
-        (long long)x.smem_bytes - (long long)kHeadBytes -
-        (lead_searches ? ((long long)(upd_smem_bytes<R>() + 127) / 128) * 128 : 0);
-    // two tiles (a range may straddle a band boundary) plus the bits; more
-    // than one band of units per CTA streams instead
-    const long long need = (long long)(kResRows + 2 * R) * 4 *
-                               (m * kResCols + 2 * (2 * R + 8)) + 256 + m * 64;
-    // at least half a unit per warp, else the batches of the streaming
-    // mode spread the search over more warps
-    resident = !tcmode && m >= kEngWarps / 2 && m <= ncu && need <= avail;
-  }
-  ResPlan& pl = tl.plan;
-  if (resident && searcher) {
-    if (tid == 0) res_plan<R>(pl, ncu, nbands, rank, ns);
-    __syncthreads();
-  }
-  if (tid == 0) {
-    tl.stop = !ctrl_active(c) || __ldcg(err) != 0;
-    tl.px = __ldcg(&c->px);
-    tl.py = __ldcg(&c->py);
-  }
-  __syncthreads();
-  int prev_px = -1000000, prev_py = -1000000;
   int round = 0;        // search rounds of this image in this launch
 
   // One search round for target (px, py): this CTA's batches; returns its
   // best key.  Whole block.
   auto search_round = [&](int px, int py) -> unsigned long long {
     const int b0 = rank < ns ? rank : nbatch;
-    const int par = round & 1;
     // a batch's stage in streaming mode: its RGBA window and the validity
     // counts of its candidates, on one mbarrier
     auto issue = [&](int b, uint32_t* st, uint32_t* ct, uint64_t* bar) {
@@ -987,72 +1029,10 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
       if (tid == 0 && ns == 1) atomicAdd(&c->tc_rounds, 1);  // (else the team's first searcher counts)
       return tc_lead_share<R>(ea, x, tt, tc_off, tc_nb, tc_slot_b, ns, px, py, first);
     }
-    if (!resident && tid == 0 && b0 < nbatch) issue(b0, slot_pix(0), cnt_t[0], &tl.bars.full[0]);
-        if (resident && first) {
-      // the source windows of every band segment (plain 16-byte loads;
-      // outside the image: zero), then the validity bits of every unit
-      for (int g = 0; g < pl.nseg; ++g) {
-        const ResSeg sg = pl.seg[g];
-        const int x0 = xb - R + sg.c_lo * kResCols, y0 = s.cy0 + sg.band * kResRows - R;
-        const int nq = sg.pitch / 4;
-        uint4* dst = reinterpret_cast<uint4*>(area + sg.off);
-        for (int i = tid; i < RG::TH * nq; i += kEngThreads) {
-          const int row = i / nq, q = i - row * nq, y = y0 + row, xw = x0 + 4 * q;
-          uint4 v = make_uint4(0u, 0u, 0u, 0u);
-          if (y >= 0 && y < s.H && xw + 3 < s.pitch)
-            v = __ldcg(reinterpret_cast<const uint4*>(s.img + (size_t)y * s.pitch + xw));
-          dst[i] = v;
-        }
-      }
-      uint16_t* bits = reinterpret_cast<uint16_t*>(area + pl.bits_off);
-      for (int jj = warp; jj < pl.u1 - pl.u0; jj += kEngWarps) {
-        const int u = pl.u0 + jj, band = u / ncu, col = u - band * ncu;
-        const int qy = s.cy0 + band * kResRows + lane, qx0 = xb + col * kResCols;
-        uint32_t v = 0;
-        if (qy <= s.cy1) {
-#pragma unroll
-          for (int k = 0; k < kResCols; ++k) {
-            const int qx = qx0 + k;
-            if (qx >= s.cx0 && qx <= s.cx1 && __ldcg(&s.count[(size_t)qy * s.pitch + qx]) == 0) v |= 1u << k;
-          }
-        }
-        bits[jj * 32 + lane] = (uint16_t)v;
-      }
-    } else if (resident && pl.u1 > pl.u0) {
-      // the previous target's filled pixels (its unknown in-image pixels),
-      // copied by the leader before the publication, into every tile that
-      // holds them
-      const uint8_t* kprev = tl.known[par ^ 1];
-      if (tid < P * P) {
-        const int tx = prev_px + tid % P - R, ty = prev_py + tid / P - R;
-        if (tx >= 0 && tx < s.W && ty >= 0 && ty < s.H && !kprev[tid]) {
-          const uint32_t w = __ldcg(&s.img[(size_t)ty * s.pitch + tx]);
-          for (int g = 0; g < pl.nseg; ++g) {
-            const ResSeg& sg = pl.seg[g];
-            const int lx = tx - (xb - R + sg.c_lo * kResCols), ly = ty - (s.cy0 + sg.band * kResRows - R);
-            if (lx >= 0 && lx < sg.pitch && ly >= 0 && ly < RG::TH)
-              reinterpret_cast<uint32_t*>(area + sg.off)[ly * sg.pitch + lx] = w;
-          }
-        }
-      }
-      // candidates within 2R of the previous target may have become valid
-      constexpr int NCW = 4 * R + 1;
-      for (int jj = tid; jj < NCW * NCW; jj += kEngThreads) {
-        const int qx = prev_px + jj % NCW - 2 * R, qy = prev_py + jj / NCW - 2 * R;
-        if (qx < s.cx0 || qx > s.cx1 || qy < s.cy0 || qy > s.cy1) continue;
-        const int band = (qy - s.cy0) / kResRows, col = (qx - xb) / kResCols;
-        const int u = band * ncu + col;
-        if (u < pl.u0 || u >= pl.u1) continue;
-        if (__ldcg(&s.count[(size_t)qy * s.pitch + qx]) != 0) continue;
-        const int e = (u - pl.u0) * 32 + (qy - s.cy0) % kResRows;
-        atomicOr(reinterpret_cast<unsigned*>(area + pl.bits_off) + (e >> 1),
-                 (1u << ((qx - xb) % kResCols)) << (16 * (e & 1)));
-      }
-    }
+    if (tid == 0 && b0 < nbatch) issue(b0, slot_pix(0), cnt_t[0], &tl.bars.full[0]);
     // target patch: warp dy reads row dy (lane = dx); the ballot of the
     // known flags gives the row descriptor
     {
-      uint8_t* kn = tl.known[par];
       for (int dy = warp; dy < P; dy += kEngWarps) {
         const int tx = px + lane - R, ty = py + dy - R;
         uint32_t w = 0;
@@ -1067,7 +1047,6 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
         const unsigned bal = __ballot_sync(0xffffffffu, known);
         if (lane < P) {
           tgt[dy * G::TP + lane] = w;
-          kn[dy * P + lane] = (uint8_t)known;
         }
         if (lane == 0) rowd[dy] = row_desc(bal & G::FULL, P);
       }
@@ -1075,10 +1054,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     __syncthreads();
     unsigned long long best = ~0ull;
     bool ok = true;
-    if (resident) {
-      if (pl.u1 > pl.u0)
-        best = resident_units16<R>((int)offsetof(EngSmemTail, plan), (int)(area - smem), xb, s.cy0, s.W, kTgtOff);
-    } else {
+    {
       int cur = 0;
       for (int b = b0; b < nbatch; b += ns) {
         const int nb = b + ns;
@@ -1097,8 +1073,8 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
           const int qx = qx0 + k;
           if (qx >= s.cx0 && qx <= s.cx1 && qy <= s.cy1 && cw[G::COFF + k] == 0) bits |= 1u << k;
         }
-        const unsigned long long kb = unit_best<R, SRW>(
-            (int)(slots - smem) + cur * G::SLOT_BYTES + 4 * (lane * G::BW + G::NCL * warp), kTgtOff, bits,
+        const unsigned long long kb = unit_best<R, G::NCL>(
+            (int)(slots - smem) + cur * G::SLOT_BYTES + 4 * (lane * G::BW + G::NCL * warp), G::BW, kTgtOff, bits,
             (unsigned)(qy * s.W + qx0));
         best = kb < best ? kb : best;
         if (__syncthreads_or(!got)) {  // a bounded wait gave up: stop uniformly
@@ -1147,6 +1123,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
       }
     }
     if (tid >= kChainThreads) {
+      CopyPlan cpy{};
       if (tid >= kRecThread) {
         bool late;
         const unsigned long long best = gather_keys(tpart, ns, epoch, err, limit, &late);
@@ -1155,9 +1132,11 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
           set_source<R>(s, usm, best, late || tl.err != 0);
         }
         __syncwarp();
+      } else {
+        cpy = plan_copy<R>(s, usm);
       }
       work_sync();
-      if (usm.ok) update_work<R>(s, usm, true, tcmode ? &tc->copied : nullptr, epoch + 1u);
+      if (usm.ok) update_work<R>(s, usm, cpy, true, tcmode || resident ? &tc->copied : nullptr, epoch + 1u);
     }
     __syncthreads();
     const bool ok = usm.ok != 0;
@@ -1189,8 +1168,6 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
       if (!stop) stage_next<R>(s, wk, wi, ny, usm);  // (the time budget is known to the publishing thread only)
     }
     ++epoch;
-    prev_px = px;
-    prev_py = py;
     __syncthreads();
     if (lane == 0) asm volatile("fence.proxy.async.global;" ::: "memory");
   };
@@ -1229,8 +1206,6 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
       tl.py = (int)((v >> 47) & 0x7fff);
     }
     ++epoch;
-    prev_px = px;
-    prev_py = py;
     __syncthreads();
     if (lane == 0) asm volatile("fence.proxy.async.global;" ::: "memory");
   }
@@ -1271,8 +1246,10 @@ __global__ void __launch_bounds__(kEngThreads) k_update_fast(ImgState s, cudaGra
   if (threadIdx.x < kChainThreads) {
     spec_chains<R>(s, usm);
   } else {
+    CopyPlan cpy{};
     if (threadIdx.x < kRecThread) {
       spec_rest<R>(s, usm);
+      cpy = plan_copy<R>(s, usm);
     } else {
       const int lane = threadIdx.x & 31;
       spec_record<R>(s, usm, false);
@@ -1289,7 +1266,7 @@ __global__ void __launch_bounds__(kEngThreads) k_update_fast(ImgState s, cudaGra
       __syncwarp();
     }
     work_sync();
-    if (usm.ok) update_work<R>(s, usm, false, nullptr, 0u);
+    if (usm.ok) update_work<R>(s, usm, cpy, false, nullptr, 0u);
   }
   __syncthreads();
   const bool ok = usm.ok != 0;

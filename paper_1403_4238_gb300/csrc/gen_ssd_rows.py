@@ -1,7 +1,7 @@
 """Writes ssd_rows.cuh: the inline-PTX row sequences of the engine's search.
 
-One target row of the masked SSD (Sec. 3, Eq. 4) for the 16 candidates a
-lane owns: for each known target column c and candidate k, the byte-SIMD
+One target row of the masked SSD (Sec. 3, Eq. 4) for the 4, 8 or 16 candidates
+a lane owns: for each known target column c and candidate k, the byte-SIMD
 absolute difference |t[c] - r[k + c]| (vabsdiff4) and its dot product with
 itself accumulated into acc[k] (dp4a), i.e. the squared RGB distance of one
 pixel pair.  A row whose known columns are [s, P) enters the ascending
@@ -13,11 +13,11 @@ The caller passes an index in [0, 2P) (it clamps it).
 The library build (paper_1403_4238_gb300/_lib.py) runs this script and
 writes its output to the build directory, which is on the include path.
 """
-NCL = 16           # candidates per lane
+NCLS = (4, 8, 16)  # candidates per lane (streaming: 4 or 8, resident: 4 or 16)
 RADII = range(1, 9)
 
 
-def row_macro(P: int) -> str:
+def row_macro(P: int, NCL: int) -> str:
     ns = (NCL + P - 1 + 3) & ~3   # strip words per lane
     tp = (P + 3) & ~3             # padded target row
     o_r, o_t = NCL, NCL + ns
@@ -46,8 +46,8 @@ def row_macro(P: int) -> str:
     body = "\\n\\t".join(lines)
     acc = ", ".join(f'"+r"(acc[{k}])' for k in range(NCL))
     ins = ", ".join([f'"r"(r[{i}])' for i in range(ns)] + [f'"r"(t[{i}])' for i in range(tp)] + ['"r"(idx)'])
-    return (f"// P = {P}: strip r[{ns}], target row t[{tp}], 16 accumulators\n"
-            f"#define INP_SSD_ROW16_P{P}(acc, r, t, idx) \\\n"
+    return (f"// P = {P}: strip r[{ns}], target row t[{tp}], {NCL} accumulators\n"
+            f"#define INP_SSD_ROW{NCL}_P{P}(acc, r, t, idx) \\\n"
             f"  asm volatile(\"{body}\" \\\n"
             f"               : {acc} \\\n"
             f"               : {ins})\n")
@@ -55,11 +55,12 @@ def row_macro(P: int) -> str:
 
 def main():
     print("// Generated by gen_ssd_rows.py: inline-PTX row sequences of the engine's")
-    print("// masked-SSD search, 16 candidates per lane (see that script).  Do not edit.")
+    print("// masked-SSD search, 4, 8 or 16 candidates per lane (see that script).  Do not edit.")
     print("#pragma once")
     print()
     for r in RADII:
-        print(row_macro(2 * r + 1))
+        for ncl in NCLS:
+            print(row_macro(2 * r + 1, ncl))
 
 
 if __name__ == "__main__":

@@ -173,33 +173,41 @@ __host__ __device__ inline uint32_t bf16_of_int(int v) {
   return u >> 16;
 }
 
-// The five plane values of pixel word w (R' G' B' hi lo) at offset o of
-// tile column tx, row y.
-__device__ inline void plane_store_at(const ImgState& s, int tx, int y, int o, uint32_t w) {
+// The five plane values of pixel word w (R' G' B' hi lo) at `row`, plane
+// pitch `len`.
+__device__ inline void plane_write(uint16_t* row, int len, uint32_t w) {
   const int d0 = (int)(w & 255u) - 128, d1 = (int)((w >> 8) & 255u) - 128, d2 = (int)((w >> 16) & 255u) - 128;
   const int sq = d0 * d0 + d1 * d1 + d2 * d2;
-  uint16_t* row = s.planes + ((size_t)tx * s.prows + y) * 5 * s.tc_len + o;
   row[0] = (uint16_t)bf16_of_int(d0);
-  row[s.tc_len] = (uint16_t)bf16_of_int(d1);
-  row[2 * s.tc_len] = (uint16_t)bf16_of_int(d2);
-  row[3 * s.tc_len] = (uint16_t)bf16_of_int(sq & ~255);  // 256 hi: hi < 256, exact in BF16
-  row[4 * s.tc_len] = (uint16_t)bf16_of_int(sq & 255);
+  row[len] = (uint16_t)bf16_of_int(d1);
+  row[2 * len] = (uint16_t)bf16_of_int(d2);
+  row[3 * len] = (uint16_t)bf16_of_int(sq & ~255);  // 256 hi: hi < 256, exact in BF16
+  row[4 * len] = (uint16_t)bf16_of_int(sq & 255);
 }
 
-// Pixel (x, y) changed to w: its copies in the (at most two) tile columns
-// whose segments hold column x, or in the (at most two) folds that hold row y.
-__device__ inline void plane_store(const ImgState& s, int x, int y, uint32_t w) {
-  const int xl = x - s.tc_xs0;
+// Where the planes hold pixel (x, y): the places (null: none) in the at most
+// two tile columns whose segments hold column x, or in the at most two folds
+// that hold row y.
+__device__ inline void plane_places(const ImgState& s, int x, int y, uint16_t*& a, uint16_t*& b) {
+  a = b = nullptr;
+  const int xl = x - s.tc_xs0, len = s.tc_len;
   if (xl < 0) return;  // left of every tile's source columns
   if (s.tc_f > 1) {
     if (xl >= 8 * s.tc_n1) return;
     for (int f = 0, yf = y; f < s.tc_f && yf >= 0; ++f, yf -= s.tc_h)
-      if (yf < s.prows) plane_store_at(s, 0, yf, xl + 8 * f * s.tc_n1, w);
+      if (yf < s.prows) {
+        b = a;
+        a = s.planes + (size_t)yf * 5 * len + xl + 8 * f * s.tc_n1;
+      }
     return;
   }
-  int tx = 0;  // (a few tile columns: cheaper than a division)
-  while (tx + 1 < s.tc_ntx && xl >= (tx + 1) * 8 * s.tc_n) ++tx;
-  for (; tx >= 0 && xl - tx * 8 * s.tc_n < s.tc_len; --tx) plane_store_at(s, tx, y, xl - tx * 8 * s.tc_n, w);
+  int tx = 0, xt = xl;  // (a few tile columns: cheaper than a division)
+  while (tx + 1 < s.tc_ntx && xt >= 8 * s.tc_n) {
+    xt -= 8 * s.tc_n;
+    ++tx;
+  }
+  if (xt < len) a = s.planes + ((size_t)tx * s.prows + y) * 5 * len + xt;
+  if (tx > 0 && xt + 8 * s.tc_n < len) b = s.planes + ((size_t)(tx - 1) * s.prows + y) * 5 * len + xt + 8 * s.tc_n;
 }
 
 // Candidate centre (x, y) of the search rectangle became valid: its bit.

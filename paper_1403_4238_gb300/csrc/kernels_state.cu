@@ -414,7 +414,6 @@ __global__ void __launch_bounds__(kUpdThreads) k_fill_big(ImgState s) {
         if (s.omega[t]) {
           const uint32_t w = s.img[(size_t)(qy + dy) * s.pitch + qx + dx];
           s.img[(size_t)ty * s.pitch + tx] = w;
-          if (s.planes) plane_store(s, tx, ty, w);
           s.gray[t] = (uint8_t)luma_word(w);
           s.conf[t] = cp;
           s.omega[t] = 0;

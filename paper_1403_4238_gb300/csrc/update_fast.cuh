@@ -750,6 +750,38 @@ __device__ inline void set_source(const ImgState& s, UpdSmem<R>& sm, unsigned lo
   sm.ok = ok;
 }
 
+// What a thread of warps 4-14 copies, worked out before the search's key is
+// there: one thread copies a pixel of Psi_p^ n Omega; when there are two
+// threads per pixel, the second one writes its planes (they take as long as
+// all the rest).
+struct CopyPlan {
+  bool mine, second;
+  int src;           // words from the source centre
+  int q, qi, l;      // the target pixel: linear index, word index, local index
+  uint16_t *p0, *p1; // its places in the planes
+};
+
+template <int R>
+__device__ inline CopyPlan plan_copy(const ImgState& s, const UpdSmem<R>& sm) {
+  using G = UpdGeom<R>;
+  constexpr int P = G::P;
+  constexpr bool kTwo = 2 * P * P <= kMidThreads;
+  const int t0 = (int)threadIdx.x - kChainThreads;
+  CopyPlan c;
+  c.second = kTwo && t0 >= P * P;
+  const int tp = c.second ? t0 - P * P : t0;
+  const bool planes = s.planes != nullptr;
+  c.mine = tp < P * P && (!c.second || planes) && sm.filled[tp < P * P ? tp : 0];
+  const int dy = tp / P - R, dx = tp % P - R, tx = sm.nx_px + dx, ty = sm.nx_py + dy;
+  c.src = dy * s.pitch + dx;
+  c.q = ty * s.W + tx;
+  c.qi = ty * s.pitch + tx;
+  c.l = (G::RB + dy) * G::NS + G::RB + dx;
+  c.p0 = c.p1 = nullptr;
+  if (c.mine && planes && (c.second || !kTwo)) plane_places(s, tx, ty, c.p0, c.p1);
+  return c;
+}
+
 // Applies the iteration whose source set_source has stored (warps 4-15, after
 // a barrier of theirs): the copy of the unknown in-image part of Psi_p^ from
 // Psi_q~, the validity counts of the candidates it touches, the isophotes of
@@ -761,8 +793,8 @@ __device__ inline void set_source(const ImgState& s, UpdSmem<R>& sm, unsigned lo
 // waits off the path, and the same fence makes its later publication of the
 // next round a release.
 template <int R>
-__device__ inline void update_work(const ImgState& s, UpdSmem<R>& sm, bool fence, unsigned* copied,
-                                   unsigned copied_val) {
+__device__ inline void update_work(const ImgState& s, UpdSmem<R>& sm, const CopyPlan& cpy, bool fence,
+                                   unsigned* copied, unsigned copied_val) {
   using G = UpdGeom<R>;
   constexpr int P = G::P, RB = G::RB, NS = G::NS, R2 = G::R2, NW = G::NW, NC = G::NC;
   static_assert(P * P <= kMidThreads, "one thread per patch pixel");
@@ -775,18 +807,10 @@ __device__ inline void update_work(const ImgState& s, UpdSmem<R>& sm, bool fence
     }
     return;
   }
-  const int px = sm.px, py = sm.py, W = s.W;
+  const int px = sm.px, py = sm.py;
   {
-    // one thread copies a pixel; the tensor-core search's planes of it are
-    // another thread's when there are two per pixel (the planes take as long
-    // as all the rest)
-    constexpr bool kTwo = 2 * P * P <= kMidThreads;
-    const bool second = kTwo && t0 >= P * P;
-    const int tp = second ? t0 - P * P : t0;
-    const bool mine = tp < P * P && (!second || s.planes) && sm.filled[tp < P * P ? tp : 0];
-    const int dy = tp / P - R, dx = tp % P - R;
     uint32_t w = 0u;
-    if (mine) w = __ldcg(&s.img[(sm.qy + dy) * s.pitch + sm.qx + dx]);  // in flight during the counts
+    if (cpy.mine) w = __ldcg(&s.img[sm.qy * s.pitch + sm.qx + cpy.src]);  // in flight during the counts
     int newly = 0;
 #pragma unroll 1
     for (int j = t0; j < NC * NC; j += kMidThreads) {
@@ -799,17 +823,17 @@ __device__ inline void update_work(const ImgState& s, UpdSmem<R>& sm, bool fence
         if (s.planes) vbit_set(s, x, y);
       }
     }
-    if (mine) {
-      const int tx = px + dx, ty = py + dy, q = ty * W + tx;
-      if (!second) {
+    if (cpy.mine) {
+      if (!cpy.second) {
         const uint8_t g = (uint8_t)luma_word(w);
-        s.img[ty * s.pitch + tx] = w;
-        s.gray[q] = g;
-        s.conf[q] = sm.cp;
-        s.omega[q] = 0;
-        sm.gr[(RB + dy) * NS + RB + dx] = g;
+        s.img[cpy.qi] = w;
+        s.gray[cpy.q] = g;
+        s.conf[cpy.q] = sm.cp;
+        s.omega[cpy.q] = 0;
+        sm.gr[cpy.l] = g;
       }
-      if (second || (!kTwo && s.planes)) plane_store(s, tx, ty, w);
+      if (cpy.p0) plane_write(cpy.p0, s.tc_len, w);
+      if (cpy.p1) plane_write(cpy.p1, s.tc_len, w);
     }
     if (newly) atomicAdd(&sm.newly, newly);
   }
