@@ -1164,8 +1164,9 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
       tl.stop = stop;
     }
     if (ok) {
-      update_store<R>(s, usm, wk, wi);
-      if (!stop) stage_next<R>(s, wk, wi, ny, usm);  // (the time budget is known to the publishing thread only)
+      auto store = [&]() { update_store<R>(s, usm, wk, wi); };
+      if (!stop) stage_next<R>(s, wk, wi, ny, usm, store);  // (the time budget is known to the publishing thread only)
+      else store();
     }
     ++epoch;
     __syncthreads();

@@ -77,10 +77,20 @@ constexpr int kMidThreads = 352;    // warps 4-14
 constexpr int kMidWarps = kMidThreads / 32;
 constexpr int kRecThread = kEngThreads - 32;  // first thread of warp 15
 
-// Named barriers: of warps 4-14, and of those with warp 15 (the chains join
-// neither).
+// Named barriers: of warps 4-14, of those with warp 15 (the chains join
+// neither), of those with the chain warps that had no chains and took
+// isophotes instead (which only arrive), and one that warp 15 only arrives at
+// when the integral image is there.
 __device__ __forceinline__ void mid_sync() { asm volatile("barrier.sync 1, 352;" ::: "memory"); }
 __device__ __forceinline__ void work_sync() { asm volatile("barrier.sync 2, 384;" ::: "memory"); }
+__device__ __forceinline__ void iso_arrive(int chain_threads) {
+  asm volatile("barrier.arrive 3, %0;" ::"r"(kMidThreads + kChainThreads - chain_threads) : "memory");
+}
+__device__ __forceinline__ void iso_sync(int chain_threads) {
+  asm volatile("barrier.sync 3, %0;" ::"r"(kMidThreads + kChainThreads - chain_threads) : "memory");
+}
+__device__ __forceinline__ void fsat_arrive() { asm volatile("barrier.arrive 4, 384;" ::: "memory"); }
+__device__ __forceinline__ void fsat_sync() { asm volatile("barrier.sync 4, 384;" ::: "memory"); }
 
 template <int R>
 struct __align__(16) UpdSmem {
@@ -97,7 +107,8 @@ struct __align__(16) UpdSmem {
   uint8_t gr[G::NS * G::NS];
   uint8_t filled[G::P * G::P];
   uint16_t list[2][G::NW * G::NW];  // (by parity) front pixels (window index)
-  int nlist[2], nfilled;
+  int nlist[2];
+  int iso_next;  // next chunk of the isophotes the fill cannot change
   // the staged target: centre, iteration, C(p^), priority key
   int nx_px, nx_py, nx_it;
   double nx_cp;
@@ -239,12 +250,18 @@ __device__ inline double data_term_direct(int dot, int nn) {
 
 // Stages the NS x NS neighbourhood of (cx, cy): mask (2 outside the image),
 // grey levels and confidences (+0.0 under Omega and outside).  NT threads;
-// each has up to U entries' loads in flight together.
-template <int R, int NT>
-__device__ inline void stage_nbhd(const ImgState& s, int cx, int cy, UpdSmem<R>& sm) {
+// each has up to U entries' loads in flight together, and `meanwhile` runs
+// before the first use of them.  FILL: the state after the fill of Psi at
+// (cx, cy), whose unknown pixels take the confidence *cp, and the filled
+// flags.
+template <int R, int NT, bool FILL, class F>
+__device__ inline void stage_nbhd(const ImgState& s, int cx, int cy, UpdSmem<R>& sm, const double* cp, F&& meanwhile) {
   using G = UpdGeom<R>;
-  constexpr int RB = G::RB, NS = G::NS;
+  constexpr int RB = G::RB, NS = G::NS, P = G::P;
   constexpr int U = (NS * NS + NT - 1) / NT < 6 ? (NS * NS + NT - 1) / NT : 6;
+  double cfill = 0.0;
+  if (FILL) cfill = __ldcg(cp);
+  if ((int)threadIdx.x >= NS * NS) meanwhile();  // (more threads than entries)
 #pragma unroll 1
   for (int i0 = threadIdx.x; i0 < NS * NS; i0 += U * NT) {
     uint8_t o[U], g[U];
@@ -263,13 +280,24 @@ __device__ inline void stage_nbhd(const ImgState& s, int cx, int cy, UpdSmem<R>&
         cf[u] = __ldcg(&s.conf[q]);  // read unconditionally, kept for known pixels
       }
     }
+    if (i0 == (int)threadIdx.x) meanwhile();
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int i = i0 + u * NT;
       if (i >= NS * NS) break;
+      const int dx = i % NS - RB, dy = i / NS - RB;
+      double c = o[u] ? 0.0 : cf[u];
+      if (FILL && abs(dx) <= R && abs(dy) <= R) {
+        const bool f = o[u] == 1;
+        sm.filled[(dy + R) * P + dx + R] = f;
+        if (f) {
+          o[u] = 0;
+          c = cfill;
+        }
+      }
       sm.om[i] = o[u];
       sm.gr[i] = g[u];
-      sm.cf[i] = o[u] ? 0.0 : cf[u];
+      sm.cf[i] = c;
     }
   }
 }
@@ -306,6 +334,28 @@ __device__ inline bool front_local(const uint8_t* om, int l, int NS) {
   return c == 1 && (a == 0 || b == 0 || u == 0 || d == 0);
 }
 
+// The isophotes the fill cannot change: it changes grey levels and the mask
+// only inside Psi_p^, so a candidate can change only in the box of Chebyshev
+// radius R + 1 around p^.  Handed out in chunks of 64 from sm.iso_next: the
+// chain warps without chains, then the others as they get to it.  Whole warps.
+template <int R>
+__device__ inline void static_isophotes(UpdSmem<R>& sm) {
+  constexpr int NS = UpdGeom<R>::NS, RB = UpdGeom<R>::RB, RR = R + 1;
+  const int lane = threadIdx.x & 31;
+  while (true) {
+    int base = 0;
+    if (lane == 0) base = atomicAdd(&sm.iso_next, 64);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (base >= NS * NS) break;
+#pragma unroll
+    for (int h = 0; h < 64; h += 32) {
+      const int i = base + h + lane, lx = i % NS, ly = i / NS;
+      if (i < NS * NS && (abs(lx - RB) > RR || abs(ly - RB) > RR)) sm.ikey[i] = isophote_key<R>(sm, lx, ly);
+    }
+    __syncwarp();
+  }
+}
+
 // Initial priorities, one CTA per NW x NW window of the image (direct
 // evaluation of every term).
 template <int R>
@@ -315,7 +365,7 @@ __global__ void __launch_bounds__(256, 2) k_prio_init_fast(ImgState s) {
   extern __shared__ __align__(128) uint8_t sm_raw[];
   UpdSmem<R>& sm = *reinterpret_cast<UpdSmem<R>*>(sm_raw);
   const int cx = R2 + blockIdx.x * NW, cy = R2 + blockIdx.y * NW;
-  stage_nbhd<R, 256>(s, cx, cy, sm);
+  stage_nbhd<R, 256, false>(s, cx, cy, sm, nullptr, [] {});
   __syncthreads();
 #pragma unroll 1
   for (int i = threadIdx.x; i < NS * NS; i += 256) sm.ikey[i] = isophote_key<R>(sm, i % NS, i / NS);
@@ -367,20 +417,23 @@ __device__ inline void stage_first(const ImgState& s, UpdSmem<R>& sm, bool overl
     sm.nlist[0] = sm.nlist[1] = 0;
     sm.rec_pending = 0;
     sm.tiles_pending = 0;
+    sm.iso_next = 0;
   }
-  stage_nbhd<R, kEngThreads>(s, px, py, sm);
+  stage_nbhd<R, kEngThreads, true>(s, px, py, sm, &c->conf, [] {});
 }
 
-// The next iteration's input, once the next target idx (in row npy) has been selected: its
-// neighbourhood, and in sm.nx_* its centre, iteration number and confidence.
-// Whole block; the caller's barrier makes it visible.
-template <int R>
-__device__ inline void stage_next(const ImgState& s, unsigned long long key, int idx, int npy, UpdSmem<R>& sm) {
+// The next iteration's input, once the next target idx (in row npy) has been
+// selected: its neighbourhood after its fill, and in sm.nx_* its centre,
+// iteration number and confidence.  `meanwhile` runs while the loads are in
+// flight.  Whole block; the caller's barrier makes it visible.
+template <int R, class F>
+__device__ inline void stage_next(const ImgState& s, unsigned long long key, int idx, int npy, UpdSmem<R>& sm,
+                                  F&& meanwhile) {
   const int npx = idx - npy * s.W;
   const bool mine = threadIdx.x == kEngThreads - 1;  // a thread with the fewest staging entries
   double ncp = 0.0;
   if (mine) ncp = __ldcg(&s.pconf[idx]);
-  stage_nbhd<R, kEngThreads>(s, npx, npy, sm);
+  stage_nbhd<R, kEngThreads, true>(s, npx, npy, sm, &s.pconf[idx], meanwhile);
   if (mine) {
     sm.nx_px = npx;
     sm.nx_py = npy;
@@ -388,29 +441,17 @@ __device__ inline void stage_next(const ImgState& s, unsigned long long key, int
     sm.nx_cp = ncp;
     sm.nx_key = key;
     sm.nlist[(sm.it + 1) & 1] = 0;
+    sm.iso_next = 0;
   }
 }
 
-// Post-fill mask and confidences of the staged neighbourhood, the filled set,
-// and the post-fill front of the window.  Whole block; ends with a
-// __syncthreads.
+// The post-fill front of the window from the staged neighbourhood.  Whole
+// block; ends with a __syncthreads.
 template <int R>
 __device__ inline void spec_front(UpdSmem<R>& sm) {
   using G = UpdGeom<R>;
-  constexpr int P = G::P, RB = G::RB, NS = G::NS, R2 = G::R2, NW = G::NW;
-  static_assert(P * P <= kEngThreads, "one thread per patch pixel");
+  constexpr int RB = G::RB, NS = G::NS, R2 = G::R2, NW = G::NW;
   const int tid = threadIdx.x, lane = tid & 31, par = sm.nx_it & 1;
-  bool f = false;
-  if (tid < P * P) {
-    const int l = (RB + tid / P - R) * NS + RB + tid % P - R;
-    f = sm.om[l] == 1;
-    if (f) {
-      sm.om[l] = 0;
-      sm.cf[l] = sm.nx_cp;
-    }
-    sm.filled[tid] = f;
-  }
-  const int filled = __syncthreads_count(f);
 #pragma unroll 1
   for (int i0 = 0; i0 < NW * NW; i0 += kEngThreads) {
     const int i = i0 + tid;
@@ -428,7 +469,6 @@ __device__ inline void spec_front(UpdSmem<R>& sm) {
       if (fr) sm.list[par][base + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)i;
     }
   }
-  if (tid == 0) sm.nfilled = filled;
   __syncthreads();
 }
 
@@ -444,7 +484,11 @@ __device__ inline void spec_chains(const ImgState& s, UpdSmem<R>& sm) {
   using G = UpdGeom<R>;
   constexpr int RB = G::RB, R2 = G::R2, NW = G::NW, P2 = G::P * G::P;
   const int par = sm.nx_it & 1, nfront = sm.nlist[par], nt = chain_threads(nfront);
-  if ((int)threadIdx.x >= nt) return;
+  if ((int)threadIdx.x >= nt) {
+    static_isophotes<R>(sm);
+    iso_arrive(nt);
+    return;
+  }
 #pragma unroll 1
   for (int k = threadIdx.x; k < nfront; k += nt) {
     const int i = sm.list[par][k];
@@ -576,20 +620,28 @@ __device__ inline void update_tiles(const ImgState& s, UpdSmem<R>& sm) {
     }
   }
   mid_sync();
-  if (wid == 0 && lane < g.nux * g.nuy) {
-    const int v = lane >= g.nux ? 1 : 0, ux = g.ux0 + lane - v * g.nux, uy = g.uy0 + v;
-    unsigned long long k = sm.seg[n0 + lane].key;
-    int idx = sm.seg[n0 + lane].idx, tx = g.tx0, ty = g.ty0;
+  if (wid == 0) {
+    // lane t: the new maximum of level-0 tile t, and the level-1 tile it is in
+    const int v = lane / g.ntx, tx = g.tx0 + lane - v * g.ntx, ty = g.ty0 + v;
+    const bool in = lane < n0;
+    const int mine = in ? ((ty >> 4) - g.uy0) * g.nux + (tx >> 4) - g.ux0 : -1;
+    const unsigned long long k0 = in ? sm.seg[lane].key : 0ull;
+    const int i0 = in ? sm.seg[lane].idx : 0x7fffffff;
 #pragma unroll 1
-    for (int t = 0; t < n0; ++t) {
-      if ((tx >> 4) == ux && (ty >> 4) == uy) prio_take(k, idx, sm.seg[t].key, sm.seg[t].idx);
-      if (++tx == g.tx0 + g.ntx) {
-        tx = g.tx0;
-        ++ty;
+    for (int u = 0; u < g.nux * g.nuy; ++u) {
+      unsigned long long k = mine == u ? k0 : 0ull;
+      int idx = mine == u ? i0 : 0x7fffffff;
+      if (lane == 31) {  // (n0 <= 16) the level-1 tile's other level-0 tiles
+        k = sm.seg[n0 + u].key;
+        idx = sm.seg[n0 + u].idx;
+      }
+      warp_best_prio(k, idx);
+      if (lane == 0) {
+        const int uy = g.uy0 + (u >= g.nux ? 1 : 0), ux = g.ux0 + u - (u >= g.nux ? g.nux : 0);
+        s.tiles1[uy * s.t1x + ux].key = k;
+        s.tiles1[uy * s.t1x + ux].idx = idx;
       }
     }
-    s.tiles1[uy * s.t1x + ux].key = k;
-    s.tiles1[uy * s.t1x + ux].idx = idx;
   }
   __syncwarp();
   mid_sync();
@@ -598,7 +650,10 @@ __device__ inline void update_tiles(const ImgState& s, UpdSmem<R>& sm) {
 // The best priority that the fill of (px, py) leaves alone, by segments: the
 // pixels outside the window of each level-0 tile it touches, the untouched
 // level-0 tiles of each level-1 tile it touches, and the untouched level-1
-// tiles; one warp per segment.  Warps 4-14.
+// tiles; one warp per segment.  Warps 4-14.  (A warp's lanes are brought
+// together after the predicated loads and at the end of each branch: left to
+// drift apart they took the keys one lane set after the other, 2.5k cycles
+// of the round.)
 template <int R>
 __device__ inline void scan_segments(const ImgState& s, UpdSmem<R>& sm, const TouchedTiles& g, int px, int py) {
   constexpr int R2 = UpdGeom<R>::R2;
@@ -617,8 +672,10 @@ __device__ inline void scan_segments(const ImgState& s, UpdSmem<R>& sm, const To
         const bool use = xt < W && y < H && (abs(xt - px) > R2 || abs(y - py) > R2);
         kk[j] = use ? __ldcg(&s.prio[y * W + xt]) : 0ull;
       }
+      __syncwarp();
 #pragma unroll
       for (int j = 0; j < 8; ++j) prio_take(k, idx, kk[j], (yt + 2 * j) * W + xt);
+      __syncwarp();
     } else if (e < nseg - 1) {
       const int u = e - n0, v = u >= g.nux ? 1 : 0;
       const int tx = (g.ux0 + u - v * g.nux) * kT1 + (lane & 15);
@@ -636,6 +693,7 @@ __device__ inline void scan_segments(const ImgState& s, UpdSmem<R>& sm, const To
 #pragma unroll
       for (int j = 0; j < 8; ++j)
         prio_take(k, idx, ((unsigned long long)b[j].y << 32) | b[j].x, (int)b[j].z);
+      __syncwarp();
     } else {
       const int n1 = s.t1x * s.t1y;
 #pragma unroll 1
@@ -658,7 +716,7 @@ __device__ inline void scan_segments(const ImgState& s, UpdSmem<R>& sm, const To
 template <int R>
 __device__ inline void spec_rest(const ImgState& s, UpdSmem<R>& sm) {
   using G = UpdGeom<R>;
-  constexpr int P = G::P, RB = G::RB, NS = G::NS, R2 = G::R2, NW = G::NW, NC = G::NC, RR = R + 1, P1 = P + 1;
+  constexpr int P = G::P, RB = G::RB, R2 = G::R2, NW = G::NW, NC = G::NC, P1 = P + 1;
   const int px = sm.nx_px, py = sm.nx_py, t0 = (int)threadIdx.x - kChainThreads, W = s.W, H = s.H;
 #pragma unroll 1
   for (int j = t0; j < NC * NC; j += kMidThreads) {
@@ -666,14 +724,11 @@ __device__ inline void spec_rest(const ImgState& s, UpdSmem<R>& sm) {
     const bool ok = x >= 0 && x < W && y >= 0 && y < H;
     cp_async4(&sm.cnt[j], ok ? &s.count[y * s.pitch + x] : s.count, ok);
   }
-  if (t0 >= kMidThreads - 32) warp_fsat<R>(sm);
   // (every thread reads the flag before update_tiles' barriers, which precede its reset)
   if (sm.tiles_pending) update_tiles<R>(s, sm);
   const TouchedTiles g = touched_tiles<R>(s, px, py);
   scan_segments<R>(s, sm, g, px, py);
-  // normals of the front pixels, and the isophotes the fill cannot change: it
-  // changes grey levels and the mask only inside Psi_p^, so a candidate can
-  // change only in the box of Chebyshev radius R + 1 around p^
+  // normals of the front pixels
   const int par = sm.nx_it & 1, nfront = sm.nlist[par];
 #pragma unroll 1
   for (int k = t0; k < nfront; k += kMidThreads) {
@@ -681,13 +736,11 @@ __device__ inline void spec_rest(const ImgState& s, UpdSmem<R>& sm) {
     const int wx = i % NW - R2, wy = i / NW - R2;
     sm.snrm[i] = normal_local<R>(sm, s, RB + wx, RB + wy, px + wx, py + wy);
   }
-#pragma unroll 1
-  for (int i = t0; i < NS * NS; i += kMidThreads) {
-    const int lx = i % NS, ly = i / NS;
-    if (abs(lx - RB) > RR || abs(ly - RB) > RR) sm.ikey[i] = isophote_key<R>(sm, lx, ly);
-  }
+  __syncwarp();
+  static_isophotes<R>(sm);
   cp_async_wait_all();
-  mid_sync();
+  __syncwarp();
+  iso_sync(chain_threads(nfront));
   if (t0 < 32) {
     const int nseg = g.ntx * g.nty + g.nux * g.nuy + 1;
     unsigned long long k = t0 < nseg ? sm.seg[t0].key : 0ull;
@@ -701,7 +754,9 @@ __device__ inline void spec_rest(const ImgState& s, UpdSmem<R>& sm) {
     }
   }
   // validity counts after the fill: the centre at (wx, wy) from p^ loses the
-  // filled pixels of its patch
+  // filled pixels of its patch (their integral image is warp 15's)
+  __syncwarp();
+  fsat_sync();
 #pragma unroll 1
   for (int j = t0; j < NC * NC; j += kMidThreads) {
     const int jy = j / NC, wy = jy - 2 * R, wx = j - jy * NC - 2 * R;
@@ -712,14 +767,19 @@ __device__ inline void spec_rest(const ImgState& s, UpdSmem<R>& sm) {
   }
 }
 
-// The scalars of the iteration on the staged target, after the last one's
-// record (thread kRecThread).
+// Warp 15 meanwhile: the integral image of the filled flags, then (one thread)
+// the last iteration's record and the scalars of the iteration on the staged
+// target.
 template <int R>
 __device__ inline void spec_record(const ImgState& s, UpdSmem<R>& sm, bool overlap_counts) {
+  constexpr int P = UpdGeom<R>::P;
+  warp_fsat<R>(sm);
+  __syncwarp();
+  fsat_arrive();
   if (threadIdx.x != kRecThread) return;
   update_times<R>(s, sm);
   if (sm.rec_pending) write_record<R>(s, sm, overlap_counts);
-  const int filled = sm.nfilled, W = s.W, H = s.H, px = sm.nx_px, py = sm.nx_py;
+  const int filled = sm.fsat[P * (P + 1) + P], W = s.W, H = s.H, px = sm.nx_px, py = sm.nx_py;
   sm.px = px;
   sm.py = py;
   sm.it = sm.nx_it;
