@@ -53,7 +53,6 @@ struct inpaint_ctx {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   ImgState st{};
-  int32_t* sat = nullptr;
   uint8_t* rgb_stage = nullptr;   // 3*W*H
   uint8_t* mask_stage = nullptr;  // W*H
   double* conf_stage = nullptr;   // W*H (import only)
@@ -444,7 +443,7 @@ int create_impl(const uint8_t* rgb, int W, int H, int rgb_stride, const uint8_t*
       !alloc_n(c, s.tiles1, (size_t)s.t1x * s.t1y) ||
       !alloc_n(c, s.ctrl, 1) || !alloc_n(c, s.trace, (size_t)s.trace_cap) ||
       !alloc_n(c, s.partial, (size_t)(s.n_partial > 0 ? s.n_partial : 1)) ||
-      !alloc_n(c, c->sat, (size_t)(W + 1) * (H + 1) + (size_t)sat_chunks(H) * W) || !alloc_n(c, c->rgb_stage, 3 * n) ||
+      !alloc_n(c, s.obits, (size_t)obits_pitch(W) * H) || !alloc_n(c, c->rgb_stage, 3 * n) ||
       !alloc_n(c, c->mask_stage, n)) {
     g_last_error = "device allocation failed";
     return fail(INPAINT_ERR_NOMEM);
@@ -508,7 +507,7 @@ int inpaint_reset(inpaint_ctx* c, const uint8_t* rgb, int rgb_stride, const uint
     rs = 3 * W;
     ms = W;
   }
-  CK(launch_init(c->st, drgb, rs, dmask, ms, c->sat, nullptr, c->stream));
+  CK(launch_init(c->st, drgb, rs, dmask, ms, c->stream));
   return finish_init(c);
 }
 
@@ -614,7 +613,7 @@ int inpaint_import_state(inpaint_ctx* c, const uint8_t* rgb, const uint8_t* omeg
   CK(cudaMemcpyAsync(c->rgb_stage, rgb, 3 * n, cudaMemcpyHostToDevice, c->stream));
   CK(cudaMemcpyAsync(c->mask_stage, omega, n, cudaMemcpyHostToDevice, c->stream));
   CK(cudaMemcpyAsync(c->conf_stage, conf, n * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  CK(launch_import(c->st, c->rgb_stage, c->mask_stage, c->conf_stage, c->sat, nullptr,
+  CK(launch_import(c->st, c->rgb_stage, c->mask_stage, c->conf_stage,
                    c->stream));
   return finish_init(c);
 }
@@ -1230,7 +1229,7 @@ void build_batch_graphs(inpaint_batch* b) {
       if (cudaStreamWaitEvent(b->aux[k], b->fork, 0) != cudaSuccess) return false;
     for (int i = 0; i < b->n; ++i) {
       inpaint_ctx* c = b->ctx[i];
-      if (launch_init(c->st, c->orig_rgb, 3 * c->W, c->orig_mask, c->W, c->sat, nullptr,
+      if (launch_init(c->st, c->orig_rgb, 3 * c->W, c->orig_mask, c->W,
                       b->aux[i % inpaint_batch::kBatchAux]) != cudaSuccess ||
           launch_planes(c->st, b->aux[i % inpaint_batch::kBatchAux]) != cudaSuccess)
         return false;
@@ -1322,7 +1321,7 @@ int inpaint_batch_reset(inpaint_batch* b) {
     return INPAINT_OK;
   }
   for (inpaint_ctx* c : b->ctx) {
-    CK(launch_init(c->st, c->orig_rgb, 3 * c->W, c->orig_mask, c->W, c->sat, nullptr, b->stream));
+    CK(launch_init(c->st, c->orig_rgb, 3 * c->W, c->orig_mask, c->W, b->stream));
     CK(launch_planes(c->st, b->stream));
   }
   CK(cudaStreamSynchronize(b->stream));

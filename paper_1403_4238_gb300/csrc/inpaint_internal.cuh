@@ -71,6 +71,7 @@ struct Ctrl {
   int tc_rounds;   // engine search rounds run in the tensor-core form
   int n_front;     // patch radius > 8: front pixels in ImgState::front whose priorities
                    // are to be evaluated; -1: the last update applied nothing
+  int tiles_done;  // initialisation: CTAs of k_tiles_all that are done
 };
 
 // Window codes of the speculative phase (update_fast.cuh): a pixel of the
@@ -147,6 +148,7 @@ struct ImgState {
   Ctrl* ctrl;
   inpaint_step_info* trace;
   unsigned long long* partial;  // per-CTA best search key of the iteration
+  uint32_t* obits;         // initialisation: Omega, one bit per pixel, rows of obits_pitch(W) words
   int* front;              // patch radius > 8: linear indices of the pixels to evaluate
   // tensor-core form (null otherwise): five BF16 planes of the image, R' G' B'
   // (byte - 128) and the square sum sq = sum_c (byte_c - 128)^2 as 256 hi and
@@ -163,6 +165,9 @@ struct ImgState {
   uint32_t* vbits;
   int tc_auto;  // 1: the engine chooses per launch between this form and the plain one
 };
+
+// Words per row of ImgState::obits.
+__host__ __device__ inline int obits_pitch(int W) { return (W + 31) / 32; }
 
 // BF16 bits of an integer with at most 8 significant bits (|v| <= 256, or
 // 256 times such a value: exact, the low half of the float is zero).
@@ -417,10 +422,9 @@ __device__ inline void warp_select(const ImgState& s) {
 // ---- host-side launchers (defined in the .cu files) ----
 void set_last_error(const char* msg);  // text returned by inpaint_last_error()
 cudaError_t launch_init(const ImgState& s, const uint8_t* rgb, int rgb_stride, const uint8_t* mask,
-                        int mask_stride, int32_t* sat, int* omega_count, cudaStream_t st);
+                        int mask_stride, cudaStream_t st);
 cudaError_t launch_import(const ImgState& s, const uint8_t* rgb, const uint8_t* omega,
-                          const double* conf, int32_t* sat, int* omega_count, cudaStream_t st);
-int sat_chunks(int H);  // the integral image needs (W+1)(H+1) + sat_chunks(H)*W ints
+                          const double* conf, cudaStream_t st);
 cudaError_t prepare_search_plain(int r);
 cudaError_t launch_prio_init_fast(const ImgState& s, cudaStream_t st);  // r <= 8
 cudaError_t launch_search_plain(const ImgState& s, cudaStream_t st);

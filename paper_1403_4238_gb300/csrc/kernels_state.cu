@@ -197,33 +197,35 @@ constexpr int kPrioCtas = 608;
 
 // ---------------------------------------------------------------- init
 
-__global__ void k_ctrl_init(Ctrl* c) {
-  c->iter = 0;
-  c->remaining = 0;
-  c->status = 0;
-  c->px = -1;
-  c->py = -1;
-  c->n_valid = 0;
-  c->iter_limit = 0x7fffffff;
-  c->n_adm = 0;
-  c->prio = 0.0;
-  c->conf = 0.0;
-  c->evals = 0ull;
-  c->t_search = 0ull;
-  c->t_update = 0ull;
-  c->t_last = 0ull;
-  c->timed_iters = 0;
-  c->tc_rounds = 0;
-  c->n_front = 0;
-}
-
-// RGB (or RGBA words) + mask -> packed state; counts |Omega|.
+// RGB + mask -> packed state, with key 0 everywhere, the bits of Omega
+// (ImgState::obits; columns past the image read as Omega) and the control
+// block of a fresh loop.
 __global__ void k_unpack(ImgState s, const uint8_t* rgb, int rgb_stride, const uint8_t* mask,
                          int mask_stride, const double* conf_in) {
-  __shared__ int scratch[32];
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y;
-  int om = 0;
+  if (x == 0 && y == 0) {
+    Ctrl* c = s.ctrl;
+    c->iter = 0;
+    c->remaining = 0;
+    c->status = 0;
+    c->px = -1;
+    c->py = -1;
+    c->n_valid = 0;
+    c->iter_limit = 0x7fffffff;
+    c->n_adm = 0;
+    c->prio = 0.0;
+    c->conf = 0.0;
+    c->evals = 0ull;
+    c->t_search = 0ull;
+    c->t_update = 0ull;
+    c->t_last = 0ull;
+    c->timed_iters = 0;
+    c->tc_rounds = 0;
+    c->n_front = 0;
+    c->tiles_done = 0;
+  }
+  int om = 1;
   if (x < s.W) {
     const uint8_t* p = rgb + (size_t)y * rgb_stride + 3 * (size_t)x;
     const uint32_t w = pack_rgb(p[0], p[1], p[2]);
@@ -233,129 +235,102 @@ __global__ void k_unpack(ImgState s, const uint8_t* rgb, int rgb_stride, const u
     s.omega[i] = (uint8_t)om;
     s.gray[i] = om ? 0 : (uint8_t)luma_word(w);
     s.conf[i] = om ? 0.0 : (conf_in ? conf_in[i] : 1.0);
+    s.prio[i] = 0ull;
+    s.pconf[i] = 0.0;
+  } else if (x < s.pitch) {
+    s.count[(size_t)y * s.pitch + x] = kCountInvalid;  // row padding
   }
-  const int tot = block_sum_int(om, scratch);
-  if (threadIdx.x == 0 && tot) atomicAdd(&s.ctrl->remaining, tot);
-}
-
-// Integral image of Omega: sat[y][x] = #Omega in [0,x) x [0,y), (W+1) x (H+1).
-// Pass 1: prefix along each row (one warp per row).  Pass 2: prefix down each
-// column within chunks of kSatChunk rows.  Pass 3: exclusive prefix of the
-// chunk totals per column.  Pass 4: add each chunk's offset.
-constexpr int kSatChunk = 64;
-
-__global__ void k_sat_rows(ImgState s, int32_t* sat) {
-  const int lane = threadIdx.x & 31;
-  const int y = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (y > s.H) return;
-  const int W1 = s.W + 1;
-  int32_t* row = sat + (size_t)y * W1;
-  if (y == 0) {
-    for (int x = lane; x < W1; x += 32) row[x] = 0;
-    return;
-  }
-  const uint8_t* om = s.omega + (size_t)(y - 1) * s.W;
-  if (lane == 0) row[0] = 0;
-  int carry = 0;
-  for (int base = 0; base < s.W; base += 32) {
-    const int x = base + lane;
-    int v = x < s.W ? (int)om[x] : 0;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, v, o);
-      if (lane >= o) v += t;
-    }
-    v += carry;
-    if (x < s.W) row[x + 1] = v;
-    carry = __shfl_sync(0xffffffffu, v, 31);
-  }
-}
-
-__global__ void k_sat_cols_chunk(ImgState s, int32_t* sat, int32_t* tot) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int ch = blockIdx.y;
-  if (x >= s.W) return;
-  const int W1 = s.W + 1;
-  const int y0 = 1 + ch * kSatChunk, y1 = min(s.H, ch * kSatChunk + kSatChunk);
-  int run = 0;
-  for (int y = y0; y <= y1; ++y) {
-    int32_t* p = sat + (size_t)y * W1 + x + 1;
-    run += *p;
-    *p = run;
-  }
-  tot[(size_t)ch * s.W + x] = run;
-}
-
-__global__ void k_sat_chunk_prefix(ImgState s, int32_t* tot, int nchunks) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= s.W) return;
-  int run = 0;
-  for (int ch = 0; ch < nchunks; ++ch) {
-    int32_t* p = tot + (size_t)ch * s.W + x;
-    const int v = *p;
-    *p = run;
-    run += v;
-  }
-}
-
-__global__ void k_sat_cols_apply(ImgState s, int32_t* sat, const int32_t* tot) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y + 1 + kSatChunk;  // the first chunk needs no offset
-  if (x >= s.W || y > s.H) return;
-  const int ch = (y - 1) / kSatChunk;
-  sat[(size_t)y * (s.W + 1) + x + 1] += tot[(size_t)ch * s.W + x];
+  const unsigned bal = __ballot_sync(0xffffffffu, om != 0);
+  if ((threadIdx.x & 31) == 0 && x < s.W) s.obits[(size_t)y * obits_pitch(s.W) + (x >> 5)] = bal;
 }
 
 __device__ inline bool in_rect(const ImgState& s, int x, int y) {
   return x >= s.cx0 && x <= s.cx1 && y >= s.cy0 && y <= s.cy1;
 }
 
-// Unknown count per candidate centre from the integral image; counts the
-// valid centres inside the search rectangle.
-__global__ void k_count(ImgState s, const int32_t* sat) {
+// Unknown pixels per candidate centre, |Omega| and the number of valid
+// centres: one CTA per kCountCols x kCountRows tile, one thread per column.
+// A patch row's count is the population of at most 65 bits of a row of
+// Omega bits; the thread slides the sum of 2 r + 1 rows down its column.  (An
+// integral image took four passes over 4 bytes a pixel, whose column pass
+// alone was 31 us at 512x384 and 33 us at 1920x1080: one thread walks 64
+// dependent rows.)
+constexpr int kCountCols = 128, kCountRows = 16;
+
+__global__ void __launch_bounds__(kCountCols) k_count(ImgState s) {
+  constexpr int WW = kCountCols / 32 + 3;  // a word of halo on either side, one for the funnel shifts
+  __shared__ uint32_t rows[(kCountRows + 2 * kMaxRadius) * WW];
   __shared__ int scratch[32];
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y;
-  const int r = s.r, W1 = s.W + 1;
-  int valid = 0;
-  if (x < s.W) {
-    int cnt = kCountInvalid;
-    if (x - r >= 0 && x + r < s.W && y - r >= 0 && y + r < s.H) {
-      const size_t a = (size_t)(y - r) * W1, b = (size_t)(y + r + 1) * W1;
-      cnt = sat[b + x + r + 1] - sat[a + x + r + 1] - sat[b + x - r] + sat[a + x - r];
-    }
-    s.count[(size_t)y * s.pitch + x] = cnt;
-    valid = (cnt == 0 && in_rect(s, x, y)) ? 1 : 0;
-  } else if (x < s.pitch) {
-    s.count[(size_t)y * s.pitch + x] = kCountInvalid;  // row padding
+  const int r = s.r, P = 2 * r + 1, tid = threadIdx.x;
+  const int x0 = blockIdx.x * kCountCols, y0 = blockIdx.y * kCountRows, ow = obits_pitch(s.W);
+  for (int e = tid; e < (kCountRows + 2 * r) * WW; e += kCountCols) {
+    const int v = e / WW, y = y0 - r + v, w = (x0 >> 5) - 1 + e - v * WW;
+    rows[e] = y >= 0 && y < s.H && w >= 0 && w < ow ? s.obits[(size_t)y * ow + w] : 0u;
   }
-  const int tot = block_sum_int(valid, scratch);
-  if (threadIdx.x == 0 && tot) atomicAdd(&s.ctrl->n_valid, tot);
+  __syncthreads();
+  const int x = x0 + tid, a = 32 + tid - r, w0 = a >> 5, sh = a & 31;
+  const uint32_t m0 = P >= 32 ? 0xffffffffu : (1u << P) - 1u;
+  const uint32_t m1 = P < 32 ? 0u : P >= 64 ? 0xffffffffu : (1u << (P - 32)) - 1u;
+  auto patch_row = [&](int v) {
+    const uint32_t* b = rows + v * WW + w0;
+    int n = __popc(__funnelshift_r(b[0], b[1], sh) & m0);
+    if (P > 32) n += __popc(__funnelshift_r(b[1], b[2], sh) & m1);
+    if (P > 64) n += (b[2] >> sh) & 1u;
+    return n;
+  };
+  int valid = 0, om = 0;
+  if (x < s.W) {
+    const bool xin = x - r >= 0 && x + r < s.W;
+    int cnt = 0;
+    for (int v = 0; v < 2 * r; ++v) cnt += patch_row(v);
+#pragma unroll 4
+    for (int v = 0; v < kCountRows; ++v) {
+      const int y = y0 + v;
+      if (y >= s.H) break;
+      cnt += patch_row(v + 2 * r);
+      const bool in = xin && y - r >= 0 && y + r < s.H;
+      s.count[(size_t)y * s.pitch + x] = in ? cnt : kCountInvalid;
+      valid += in && cnt == 0 && in_rect(s, x, y) ? 1 : 0;
+      om += (rows[(v + r) * WW + 1 + (tid >> 5)] >> (tid & 31)) & 1u;
+      cnt -= patch_row(v);
+    }
+  }
+  __syncwarp();
+  om = block_sum_int(om, scratch);
+  valid = block_sum_int(valid, scratch);
+  if (tid == 0) {
+    if (om) atomicAdd(&s.ctrl->remaining, om);
+    if (valid) atomicAdd(&s.ctrl->n_valid, valid);
+  }
 }
 
-// Key 0 everywhere and the list of the front pixels (patch radius > 8).
+// The list of the front pixels (patch radius > 8).
 __global__ void k_front_all(ImgState s) {
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y;
-  bool fr = false;
-  if (x < s.W) {
-    const size_t i = (size_t)y * s.W + x;
-    s.prio[i] = 0ull;
-    s.pconf[i] = 0.0;
-    fr = on_front(s, x, y);
+  append_front(s, x < s.W && on_front(s, x, y), y * s.W + x);
+}
+
+// All tiles and the first target: one CTA per level-1 tile, one warp per
+// level-0 tile in turn; the last CTA to finish selects.
+__global__ void __launch_bounds__(1024) k_tiles_all(ImgState s) {
+  __shared__ int last;
+  const int ux = blockIdx.x, uy = blockIdx.y, warp = threadIdx.x >> 5;
+  for (int t = warp; t < kT1 * kT1; t += 32) {
+    const int tx = ux * kT1 + t % kT1, ty = uy * kT1 + t / kT1;
+    if (tx < s.t0x && ty < s.t0y) warp_rescan_t0(s, tx, ty);
   }
-  append_front(s, fr, y * s.W + x);
-}
-
-// Level-0 tiles from the pixel keys, then level-1 tiles: one warp per tile.
-__global__ void k_tiles0_all(ImgState s) {
-  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (t < s.t0x * s.t0y) warp_rescan_t0(s, t % s.t0x, t / s.t0x);
-}
-
-__global__ void k_tiles1_all(ImgState s) {
-  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (t < s.t1x * s.t1y) warp_rescan_t1(s, t % s.t1x, t / s.t1x);
+  __syncthreads();
+  if (warp != 0) return;
+  warp_rescan_t1(s, ux, uy);
+  __syncwarp();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(&s.ctrl->tiles_done, 1) == (int)(gridDim.x * gridDim.y) - 1;
+    __threadfence();
+  }
+  __syncwarp();
+  if (last && loop_active(s.ctrl)) warp_select(s);
 }
 
 // ---------------------------------------------------------------- update
@@ -539,11 +514,6 @@ __global__ void __launch_bounds__(kUpdThreads) k_select_big(ImgState s, cudaGrap
   if (use_cond && tid == 0) cudaGraphSetConditional(cond, c->n_front >= 0 && loop_active(c) ? 1u : 0u);
 }
 
-// Selection of the first target (initialisation).  One warp.
-__global__ void k_select_first(ImgState s) {
-  if (loop_active(s.ctrl) && s.ctrl->remaining > 0) warp_select(s);
-}
-
 // Debug self-check: recount every candidate's unknown pixels and re-evaluate
 // every priority key from scratch; any difference sets INPAINT_ERR_INTERNAL.
 __global__ void k_verify(ImgState s) {
@@ -581,44 +551,30 @@ __global__ void k_export(ImgState s, uint8_t* rgb) {
 
 // ---------------------------------------------------------------- launchers
 
-int sat_chunks(int H) { return (H + kSatChunk - 1) / kSatChunk; }
-
-static cudaError_t init_tail(const ImgState& s, int32_t* sat, cudaStream_t st) {
+static cudaError_t init_state(const ImgState& s, const uint8_t* rgb, int rgb_stride, const uint8_t* mask,
+                              int mask_stride, const double* conf, cudaStream_t st) {
   const int W = s.W, H = s.H;
-  int32_t* tot = sat + (size_t)(W + 1) * (H + 1);
-  const int nch = sat_chunks(H);
-  k_sat_rows<<<(H + 1 + 7) / 8, 256, 0, st>>>(s, sat);
-  k_sat_cols_chunk<<<dim3((W + 127) / 128, nch), 128, 0, st>>>(s, sat, tot);
-  k_sat_chunk_prefix<<<(W + 127) / 128, 128, 0, st>>>(s, tot, nch);
-  if (H > kSatChunk) k_sat_cols_apply<<<dim3((W + 127) / 128, H - kSatChunk), 128, 0, st>>>(s, sat, tot);
-  const dim3 rows((W + 255) / 256, H);
-  k_count<<<dim3((s.pitch + 255) / 256, H), 256, 0, st>>>(s, sat);
+  k_unpack<<<dim3((s.pitch + 255) / 256, H), 256, 0, st>>>(s, rgb, rgb_stride, mask, mask_stride, conf);
+  k_count<<<dim3((W + kCountCols - 1) / kCountCols, (H + kCountRows - 1) / kCountRows), kCountCols, 0, st>>>(s);
   if (s.r <= 8) {
     const cudaError_t e = launch_prio_init_fast(s, st);
     if (e != cudaSuccess) return e;
   } else {
-    k_front_all<<<rows, 256, 0, st>>>(s);
+    k_front_all<<<dim3((W + 255) / 256, H), 256, 0, st>>>(s);
     k_prio_list<<<kPrioCtas, 64, 0, st>>>(s);
   }
-  k_tiles0_all<<<(s.t0x * s.t0y + 7) / 8, 256, 0, st>>>(s);
-  k_tiles1_all<<<(s.t1x * s.t1y + 7) / 8, 256, 0, st>>>(s);
-  k_select_first<<<1, 32, 0, st>>>(s);
+  k_tiles_all<<<dim3(s.t1x, s.t1y), 1024, 0, st>>>(s);
   return cudaGetLastError();
 }
 
 cudaError_t launch_init(const ImgState& s, const uint8_t* rgb, int rgb_stride, const uint8_t* mask,
-                        int mask_stride, int32_t* sat, int* /*omega_count*/, cudaStream_t st) {
-  k_ctrl_init<<<1, 1, 0, st>>>(s.ctrl);
-  k_unpack<<<dim3((s.W + 255) / 256, s.H), 256, 0, st>>>(s, rgb, rgb_stride, mask, mask_stride,
-                                                          nullptr);
-  return init_tail(s, sat, st);
+                        int mask_stride, cudaStream_t st) {
+  return init_state(s, rgb, rgb_stride, mask, mask_stride, nullptr, st);
 }
 
 cudaError_t launch_import(const ImgState& s, const uint8_t* rgb, const uint8_t* omega,
-                          const double* conf, int32_t* sat, int* /*omega_count*/, cudaStream_t st) {
-  k_ctrl_init<<<1, 1, 0, st>>>(s.ctrl);
-  k_unpack<<<dim3((s.W + 255) / 256, s.H), 256, 0, st>>>(s, rgb, 3 * s.W, omega, s.W, conf);
-  return init_tail(s, sat, st);
+                          const double* conf, cudaStream_t st) {
+  return init_state(s, rgb, 3 * s.W, omega, s.W, conf, st);
 }
 
 cudaError_t launch_update(const ImgState& s, unsigned long long cond_handle, int use_cond, cudaStream_t st) {

@@ -356,8 +356,12 @@ __device__ inline void static_isophotes(UpdSmem<R>& sm) {
   }
 }
 
-// Initial priorities, one CTA per NW x NW window of the image (direct
-// evaluation of every term).
+// Initial priorities of the front pixels (every key is 0 before), one CTA per
+// NW x NW window of the image; direct evaluation of every term.  Most windows
+// hold no front pixel, which a look at their Omega bits shows; in the others
+// the front pixels go to the threads one by one, so that their chains of
+// additions run side by side (evaluated where they lay, every window staged:
+// 23 us at 512x384 r 4, 93 us at 1920x1080 r 6).
 template <int R>
 __global__ void __launch_bounds__(256, 2) k_prio_init_fast(ImgState s) {
   using G = UpdGeom<R>;
@@ -365,33 +369,49 @@ __global__ void __launch_bounds__(256, 2) k_prio_init_fast(ImgState s) {
   extern __shared__ __align__(128) uint8_t sm_raw[];
   UpdSmem<R>& sm = *reinterpret_cast<UpdSmem<R>*>(sm_raw);
   const int cx = R2 + blockIdx.x * NW, cy = R2 + blockIdx.y * NW;
+  constexpr int NWD = (NW + 62) / 32;  // words that hold a window row, at most
+  bool any = false;
+  if ((int)threadIdx.x < NW * NWD) {
+    const int y = cy - R2 + (int)threadIdx.x / NWD, w = ((cx - R2) >> 5) + (int)threadIdx.x % NWD, ow = obits_pitch(s.W);
+    if (y < s.H && w < ow && 32 * w <= cx + R2) {
+      const uint32_t* row = s.obits + (size_t)y * ow + w;
+      const uint32_t o = row[0];
+      const uint32_t up = y > 0 ? row[-ow] : ~0u, down = y + 1 < s.H ? row[ow] : ~0u;
+      const uint32_t left = o << 1 | (w > 0 ? row[-1] >> 31 : 1u), right = o >> 1 | (w + 1 < ow ? row[1] << 31 : 1u << 31);
+      // the pixels of the window: columns [cx - R2, min(cx + R2, W - 1)]
+      const int lo = max(cx - R2 - 32 * w, 0), hi = min(min(cx + R2, s.W - 1) - 32 * w, 31);
+      const uint32_t in = (~0u << lo) & (~0u >> (31 - hi));
+      any = (o & ~(up & down & left & right) & in) != 0u;
+    }
+  }
+  if (threadIdx.x == 0) sm.nlist[0] = 0;
+  if (!__syncthreads_or(any)) return;
   stage_nbhd<R, 256, false>(s, cx, cy, sm, nullptr, [] {});
   __syncthreads();
 #pragma unroll 1
   for (int i = threadIdx.x; i < NS * NS; i += 256) sm.ikey[i] = isophote_key<R>(sm, i % NS, i / NS);
-  __syncthreads();
 #pragma unroll 1
   for (int i = threadIdx.x; i < NW * NW; i += 256) {
-    const int wx = i % NW - R2, wy = i / NW - R2;
-    const int lx = RB + wx, ly = RB + wy, l = ly * NS + lx;
-    if (sm.om[l] == 2) continue;
-    const int x = cx + wx, y = cy + wy;
-    unsigned long long key = 0ull;
-    double c = 0.0;
-    if (front_local(sm.om, l, NS)) {
-      c = __ddiv_rn(conf_local<R>(sm, lx, ly), (double)patch_area<R>(s, x, y));
-      const int nrm = normal_local<R>(sm, s, lx, ly, x, y);
-      uint32_t ik = 0u;
+    const int l = (RB + i / NW - R2) * NS + RB + i % NW - R2;
+    if (front_local(sm.om, l, NS)) sm.list[0][atomicAdd(&sm.nlist[0], 1)] = (uint16_t)i;
+  }
+  __syncthreads();
+  const int n = sm.nlist[0];
 #pragma unroll 1
-      for (int dy = -R; dy <= R; ++dy) {
+  for (int k = threadIdx.x; k < n; k += 256) {
+    const int i = sm.list[0][k], wx = i % NW - R2, wy = i / NW - R2;
+    const int lx = RB + wx, ly = RB + wy, l = ly * NS + lx, x = cx + wx, y = cy + wy;
+    const double c = __ddiv_rn(conf_local<R>(sm, lx, ly), (double)patch_area<R>(s, x, y));
+    const int nrm = normal_local<R>(sm, s, lx, ly, x, y);
+    uint32_t ik = 0u;
+#pragma unroll 1
+    for (int dy = -R; dy <= R; ++dy) {
 #pragma unroll
-        for (int dx = -R; dx <= R; ++dx) ik = max(ik, sm.ikey[l + dy * NS + dx]);
-      }
-      const double d = data_term_direct(isophote_dot<R>(sm, ik, nrm), nn_of(nrm));
-      key = (unsigned long long)__double_as_longlong(__dmul_rn(c, d)) + 1ull;
+      for (int dx = -R; dx <= R; ++dx) ik = max(ik, sm.ikey[l + dy * NS + dx]);
     }
+    const double d = data_term_direct(isophote_dot<R>(sm, ik, nrm), nn_of(nrm));
     const size_t p = (size_t)y * s.W + x;
-    s.prio[p] = key;
+    s.prio[p] = (unsigned long long)__double_as_longlong(__dmul_rn(c, d)) + 1ull;
     s.pconf[p] = c;
   }
 }
