@@ -7,6 +7,7 @@ allocator); every step of the method runs in the library's kernels.
 from __future__ import annotations
 
 import ctypes
+import threading
 
 import numpy as np
 
@@ -254,6 +255,57 @@ def probe_peaks() -> dict:
     return {f: getattr(pk, f) for f, _ in _lib.Peaks._fields_}
 
 
+class _ResultMemory:
+    """Result images whose pages are faulted in while the device works.
+
+    Fresh memory costs 0.3 ms a megabyte at its first write (its pages are
+    zeroed then): 54 ms of a 180 ms batch of 60 photos when the copies to the
+    host met it, and nothing beside the 125 ms that the device takes.  Every
+    array is handed out once; those not yet taken stay, at most one per image.
+    """
+
+    MIN_BYTES = 8 << 20  # 2.5 ms of faults; starting the thread costs 0.1 ms
+
+    def __init__(self):
+        self._lock = threading.Lock()
+        self._ready = {}
+        self._stop = None
+
+    def take(self, key, shape):
+        with self._lock:
+            a = self._ready.pop(key, None)
+        return a if a is not None else np.zeros(shape, np.uint8)
+
+    def put_back(self, key, a):
+        with self._lock:
+            self._ready[key] = a
+
+    def fill(self, shapes: dict, wanted):
+        """Starts faulting in the arrays of `shapes` that wanted(key) still holds for; until stop()."""
+        with self._lock:
+            todo = {k: v for k, v in shapes.items() if k not in self._ready}
+        if sum(int(np.prod(v)) for v in todo.values()) < self.MIN_BYTES:
+            return
+        stop = self._stop = threading.Event()
+
+        def work():
+            for key, shape in todo.items():
+                if stop.is_set():
+                    return
+                a = np.zeros(shape, np.uint8)
+                a.reshape(-1)[::4096] = 0  # a write to each page
+                with self._lock:
+                    if not stop.is_set() and wanted(key):
+                        self._ready.setdefault(key, a)
+
+        threading.Thread(target=work, daemon=True).start()
+
+    def stop(self):
+        stop, self._stop = self._stop, None
+        if stop is not None:
+            stop.set()
+
+
 class Batch:
     """Many independent removals in one persistent launch (inpaint_batch_*).
 
@@ -295,9 +347,11 @@ class Batch:
                "inpaint_batch_create")
         self.b = b
         self._keep = []  # inputs were copied
+        self._memory = _ResultMemory()
 
     def close(self):
         if getattr(self, "b", None):
+            self._memory = _ResultMemory()
             self.lib.inpaint_batch_destroy(self.b)
             self.b = None
 
@@ -318,12 +372,16 @@ class Batch:
 
     def run(self, max_iters: int = 0):
         st = (ctypes.c_int * self.n)()
-        _check(self.lib.inpaint_batch_run_ctx(self.b, int(max_iters), st), "inpaint_batch_run_ctx")
+        self._memory.fill({i: (H, W, 3) for i, (H, W) in enumerate(self.shapes)}, lambda i: True)
+        try:
+            _check(self.lib.inpaint_batch_run_ctx(self.b, int(max_iters), st), "inpaint_batch_run_ctx")
+        finally:
+            self._memory.stop()
         return list(st)
 
     def result(self, i: int):
         H, W = self.shapes[i]
-        out = np.zeros((H, W, 3), np.uint8)
+        out = self._memory.take(i, (H, W, 3))
         it, ev = ctypes.c_int(), ctypes.c_uint64()
         _check(self.lib.inpaint_batch_result(self.b, i, out.ctypes.data, 3 * W, ctypes.byref(it),
                                              ctypes.byref(ev)), "inpaint_batch_result")
@@ -393,9 +451,11 @@ class Server:
                                               ctypes.byref(opt), ctypes.byref(s)), "inpaint_server_create")
         self.s = s
         self.shapes = {}
+        self._memory = _ResultMemory()
 
     def close(self):
         if getattr(self, "s", None):
+            self._memory = _ResultMemory()
             self.lib.inpaint_server_destroy(self.s)
             self.s = None
 
@@ -424,17 +484,22 @@ class Server:
 
     def poll(self, rid: int):
         H, W = self.shapes[rid]
-        out = np.zeros((H, W, 3), np.uint8)
+        out = self._memory.take(rid, (H, W, 3))
         info = _lib.RequestInfo()
         rc = _check(self.lib.inpaint_server_poll(self.s, ctypes.c_uint64(rid), out.ctypes.data, 3 * W,
                                                  ctypes.byref(info)), "inpaint_server_poll")
         if rc == _lib.STATUS["PENDING"]:
+            self._memory.put_back(rid, out)
             return None
         del self.shapes[rid]
         return out, {f: getattr(info, f) for f, _ in _lib.RequestInfo._fields_}
 
     def wait_idle(self, timeout_s: float = 600.0):
-        return _check(self.lib.inpaint_server_wait_idle(self.s, float(timeout_s)), "inpaint_server_wait_idle")
+        self._memory.fill({k: (H, W, 3) for k, (H, W) in list(self.shapes.items())}, lambda k: k in self.shapes)
+        try:
+            return _check(self.lib.inpaint_server_wait_idle(self.s, float(timeout_s)), "inpaint_server_wait_idle")
+        finally:
+            self._memory.stop()
 
     def stats(self):
         st = _lib.ServerStats()
