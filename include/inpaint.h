@@ -115,7 +115,7 @@ typedef struct {
                             its SSD runs over the offsets whose target and source pixels
                             are both known and in the image, and it is admissible when a
                             known in-image source pixel lies under every unknown in-image
-                            target pixel.  Plain form, patch_radius <= 8, graph loop
+                            target pixel.  Plain form, patch_radius <= 8, loop auto or graph
                             (INPAINT_LOOP_AUTO picks it); not in batches or the server. */
 } inpaint_options;
 

@@ -66,8 +66,8 @@ class Inpainter:
     kernel) or "graph" (conditional CUDA graph).  tile_rows: engine search
     unit height (0 = library choice); tuning_file: autotuner table
     (paper_1403_4238_gb300.autotune) consulted when tile_rows is 0.  overlap:
-    the partial-overlap search variant of Algorithm 1 / Sec. 5.4 (graph loop,
-    r <= 8).  Inputs may be numpy arrays (host) or CUDA torch tensors (device,
+    the partial-overlap search variant of Algorithm 1 / Sec. 5.4 (loop auto or
+    graph, r <= 8).  Inputs may be numpy arrays (host) or CUDA torch tensors (device,
     uint8, contiguous).
     """
 

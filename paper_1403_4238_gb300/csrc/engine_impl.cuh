@@ -154,6 +154,123 @@ __device__ __forceinline__ void unit_ssd(const uint32_t* __restrict__ strip, int
   }
 }
 
+// The partial-overlap form (Algorithm 1, Sec. 5.4) of the same SSD for four
+// candidates: the sum runs over the known target pixels whose source pixel is
+// available, and a candidate with an unavailable source pixel under a pixel to
+// fill is inadmissible (kOvlBad added; the true sum is below it).  The tile's
+// words carry the availability in the alpha byte (0xff: unknown or outside the
+// image, RGB 0 then).
+// Where no lane that has a candidate meets an unavailable word, and where each
+// lane's words of the row are all available or all not (rows beyond the image,
+// a lane inside the object), a row takes the sequences above, and a lane
+// without any takes back what they summed for it (rowsq).  Only the rows at the
+// object's sides and the image's left and right border need a mask per word
+// (three instructions an evaluation and the masks: 1,200 cycles a row of four
+// warps a scheduler at 9x9, against 620; with masks in every row that meets an
+// unavailable word a round at 1024x550 took 16.5 us, now 14.2).  Unknown target pixels cost nothing:
+// a bit per word tells which candidates have an unavailable source pixel under
+// one.
+// `flags`: per target pixel 1 known, 2 unknown, 0 outside the image; `rowsq`:
+// per target row, the sum over its known pixels of the squared words (alpha
+// 0xff).
+constexpr uint32_t kOvlBad = 1u << 27;  // (at most P + 1 partial sums of a unit: no overflow)
+
+template <int R>
+__device__ __forceinline__ void unit_ssd_overlap(const uint32_t* __restrict__ strip, int pitch,
+                                                 const uint32_t* __restrict__ tgt, const uint32_t* __restrict__ rowd,
+                                                 const uint8_t* __restrict__ flags, const int* __restrict__ rowsq,
+                                                 int r0, int r1, bool live,
+                                                 uint32_t (&acc)[4]) {
+  constexpr int P = 2 * R + 1, NS = (4 + P - 1 + 3) & ~3, TP = (P + 3) & ~3;
+  uint32_t bad[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) acc[k] = bad[k] = 0u;
+#pragma unroll 1
+  for (int dy = r0; dy < r1; ++dy) {
+    uint32_t r[NS], t[TP];
+    lds_words(r, strip + dy * pitch);
+    uint32_t any = 0u, all = ~0u;
+#pragma unroll
+    for (int i = 0; i < P + 3; ++i) {
+      any |= r[i];
+      all &= r[i];
+    }
+    const uint32_t desc = rowd[dy];
+    const bool some = live && (any >> 31), none = all >> 31;
+    uint32_t unk = 0u;  // the row's pixels to fill
+    bool mixed = false;
+    if (__any_sync(0xffffffffu, some)) {
+      const int lane = threadIdx.x & 31;
+      unk = __ballot_sync(0xffffffffu, flags[dy * P + min(lane, P - 1)] == 2 && lane < P);
+      mixed = __any_sync(0xffffffffu, some && !none);
+    }
+    if (!mixed) {
+      if (none && unk) bad[0] = bad[1] = bad[2] = bad[3] = 1u;
+      if (desc == kRowSkip) continue;
+      lds_words(t, tgt + dy * TP);
+      const uint32_t kind = desc & (3u << 30);
+      if (kind != kRowMask) {
+        const uint32_t arg = desc & 0xffffu;
+        const uint32_t idx = min(kind == kRowFrom ? arg : (uint32_t)P + arg - 1u, (uint32_t)(2 * P - 1));
+#define INP_ROW(PP) \
+  if constexpr (P == PP) INP_SSD_ROW4_P##PP(acc, r, t, idx);
+        INP_ROW(3) INP_ROW(5) INP_ROW(7) INP_ROW(9) INP_ROW(11) INP_ROW(13) INP_ROW(15) INP_ROW(17)
+#undef INP_ROW
+      } else {
+#pragma unroll
+        for (int dx = 0; dx < P; ++dx) {
+          if (desc & (1u << dx)) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const uint32_t d = __vabsdiffu4(t[dx], r[k + dx]);
+              acc[k] = __dp4a(d, d, acc[k]);
+            }
+          }
+        }
+      }
+      if (none) {
+        const uint32_t sq = (uint32_t)rowsq[dy];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[k] -= sq;
+      }
+    } else {
+      // av: one bit per unavailable word; m: the RGB mask of an available one
+      uint32_t m[NS], av = 0u;
+#pragma unroll
+      for (int i = 0; i < NS; ++i) {
+        m[i] = (int)r[i] < 0 ? 0u : 0x00ffffffu;
+        if (i < P + 3) av |= (r[i] >> 31) << i;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) bad[k] |= (av >> k) & unk;
+      if (desc == kRowSkip) continue;
+      lds_words(t, tgt + dy * TP);
+      const uint32_t kind = desc & (3u << 30);
+      if (kind != kRowMask) {
+        const uint32_t arg = desc & 0xffffu;
+        const uint32_t idx = min(kind == kRowFrom ? arg : (uint32_t)P + arg - 1u, (uint32_t)(2 * P - 1));
+#define INP_ROW(PP) \
+  if constexpr (P == PP) INP_SSD_ROWM_P##PP(acc, r, m, t, idx);
+        INP_ROW(3) INP_ROW(5) INP_ROW(7) INP_ROW(9) INP_ROW(11) INP_ROW(13) INP_ROW(15) INP_ROW(17)
+#undef INP_ROW
+      } else {
+#pragma unroll
+        for (int dx = 0; dx < P; ++dx) {
+          if (desc & (1u << dx)) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const uint32_t d = __vabsdiffu4(t[dx], r[k + dx]) & m[k + dx];
+              acc[k] = __dp4a(d, d, acc[k]);
+            }
+          }
+        }
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) acc[k] += bad[k] ? kOvlBad : 0u;
+}
+
 // The compute of a streaming search round, outside the engine body so that its
 // registers hold only the row strips, the target row and the accumulators
 // (the engine body keeps the leader's state live across the search).  These
@@ -242,6 +359,25 @@ __host__ __device__ inline long long res_plan(ResPlan& pl, int kc, int ncu, int 
   return off;
 }
 
+// Shared memory that m units of kc columns need at most: two tiles (a range may
+// straddle a band boundary), the validity bits and, for kc < 16, the partial
+// SSDs.
+template <int R>
+__host__ __device__ inline int res_need(int kc, int m) {
+  return (kResRows + 2 * R) * 4 * (m * kc + 2 * (2 * R + 12)) + 640 + m * 64 + (kc < 16 ? m * kc * 128 : 0);
+}
+
+// Partial-overlap search: unit columns and the number of searchers among
+// ns_max; returns the most units of one share (0: no candidate).
+template <int R>
+__host__ __device__ inline int overlap_units(const ImgState& s, int ns_max, int* ncu, int* ns) {
+  const int xb = R + ((s.cx0 - R) & ~3);
+  const int nbands = s.cy1 >= s.cy0 ? (s.cy1 - s.cy0 + kResRows) / kResRows : 0;
+  *ncu = s.cx1 >= s.cx0 ? (s.cx1 - xb + 4) / 4 : 0;
+  *ns = ns_max < *ncu * nbands ? ns_max : *ncu * nbands;
+  return *ns > 0 ? (*ncu * nbands + *ns - 1) / *ns : 0;
+}
+
 // ---------------------------------------------------------------- kernel
 
 // The state of a CTA's tensor-core search that outlives a round: source rows
@@ -262,10 +398,11 @@ struct EngSmemTail {
   int stop;
   int px, py;
   int a2row[17];  // tensor-core search: per target row, sum of the known pixels' squared shifted values
+                  // (partial-overlap search: of their squared values with alpha 0xff)
   int tc_pref;    // tensor-core search: slots the producer prefetched for the next round
   TcRun tc_run;   // a searching leader's tensor-core search between its rounds
   int lim, status, err;  // leader: iteration limit, status and error word (the stop decision)
-  uint8_t known[17 * 17];     // known flags of the round's target
+  uint8_t known[17 * 17];     // round's target: 1 known, 2 (partial-overlap search) unknown in the image, else 0
   ResPlan plan;               // resident mode: this CTA's units and tiles
 };
 
@@ -407,6 +544,38 @@ __device__ inline unsigned long long gather_keys(const unsigned long long* slots
   if (late && lane == 0) atomicExch(err, INPAINT_ERR_TIMEOUT);
   *late_out = late;
   return best == ~0ull ? best : key_untag(best);
+}
+
+// Partial-overlap search: the number of admissible candidates of round
+// `epoch`, from the searchers' tagged counts (epoch << 32 | count) of that
+// round's parity, each polled, bounded; one warp.  Read a round later, beside
+// the next search, so that the counts need no fence before the keys.
+__device__ inline int gather_counts(const unsigned long long* slots, int n, unsigned epoch, int* err,
+                                    unsigned long long limit) {
+  constexpr int U = 5;
+  const int lane = threadIdx.x & 31;
+  const unsigned long long t0 = globaltimer();
+  int sum = 0;
+#pragma unroll 1
+  for (int b = lane; b < n; b += 32 * U) {
+    unsigned long long v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = b + 32 * u < n ? ld_relaxed64(&slots[b + 32 * u]) : (unsigned long long)epoch << 32;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+#pragma unroll 1
+      while ((unsigned)(v[u] >> 32) != epoch) {
+        if (globaltimer() - t0 > limit) {
+          atomicExch(err, INPAINT_ERR_TIMEOUT);
+          break;
+        }
+        v[u] = ld_relaxed64(&slots[b + 32 * u]);
+      }
+      sum += (int)(unsigned)v[u];
+    }
+  }
+  __syncwarp();
+  return __reduce_add_sync(0xffffffffu, sum);
 }
 
 __device__ inline bool ctrl_active(const Ctrl* c) {
@@ -703,8 +872,12 @@ __device__ __noinline__ unsigned long long tc_lead_share(const EngineArgs& ea, E
 // memory), compiled as a function of its own with everything inlined: the
 // registers a call saves come back from L2, since L1 is nearly all shared
 // memory (two nested calls per unit took 2,000 cycles a round).
-template <int R, int KC>
+// OVL: the partial-overlap form (KC 4): every centre of the rectangle is a
+// candidate, the tiles say which source pixels are available, and the number
+// of admissible candidates goes to the leader with the key.
+template <int R, int KC, bool OVL = false>
 __device__ __noinline__ void run_res_search(const EngineArgs& ea, EngCtx& x, int xb, int ncu, int acc_off) {
+  static_assert(!OVL || KC == 4, "the partial-overlap search has four candidates per lane");
   constexpr int P = 2 * R + 1, TP = (P + 3) & ~3, TH = kResRows + 2 * R;
   EngSmemTail& tl = *reinterpret_cast<EngSmemTail*>(eng_smem());
   const ImgState& s = tl.img;
@@ -730,6 +903,18 @@ __device__ __noinline__ void run_res_search(const EngineArgs& ea, EngCtx& x, int
     const int x0 = xb - R + sg.c_lo * KC, y0 = s.cy0 + sg.band * kResRows - R;
     const int nq = sg.pitch / 4;
     uint4* dst = reinterpret_cast<uint4*>(area + sg.off);
+    if constexpr (OVL) {
+      uint32_t* words = reinterpret_cast<uint32_t*>(area + sg.off);
+#pragma unroll 4
+      for (int i = tid; i < TH * sg.pitch; i += kEngThreads) {
+        const int row = i / sg.pitch, y = y0 + row, xw = x0 + i - row * sg.pitch;
+        const bool in = y >= 0 && y < s.H && xw >= 0 && xw < s.W;
+        const uint32_t w = in ? __ldcg(&s.img[(size_t)y * s.pitch + xw]) : 0u;
+        const uint8_t o = in ? __ldcg(&s.omega[(size_t)y * s.W + xw]) : 1;
+        words[i] = o ? 0xff000000u : w;
+      }
+      continue;
+    }
     for (int i = tid; i < TH * nq; i += kEngThreads) {
       const int row = i / nq, q = i - row * nq, y = y0 + row, xw = x0 + 4 * q;
       uint4 v = make_uint4(0u, 0u, 0u, 0u);
@@ -746,7 +931,7 @@ __device__ __noinline__ void run_res_search(const EngineArgs& ea, EngCtx& x, int
 #pragma unroll
       for (int k = 0; k < KC; ++k) {
         const int qx = qx0 + k;
-        if (qx >= s.cx0 && qx <= s.cx1 && __ldcg(&s.count[(size_t)qy * s.pitch + qx]) == 0) v |= 1u << k;
+        if (qx >= s.cx0 && qx <= s.cx1 && (OVL || __ldcg(&s.count[(size_t)qy * s.pitch + qx]) == 0)) v |= 1u << k;
       }
     }
     bits[j * 32 + lane] = (uint16_t)v;
@@ -759,7 +944,8 @@ __device__ __noinline__ void run_res_search(const EngineArgs& ea, EngCtx& x, int
       const int tx = px + lane - R, ty = py + dy - R;
       uint32_t w = 0;
       bool known = false;
-      if (lane < P && tx >= 0 && tx < s.W && ty >= 0 && ty < s.H) {
+      const bool in = lane < P && tx >= 0 && tx < s.W && ty >= 0 && ty < s.H;
+      if (in) {
         // both reads in flight together; the pixel is kept only if known
         const uint8_t o = __ldcg(&s.omega[(size_t)ty * s.W + tx]);
         const uint32_t v = __ldcg(&s.img[(size_t)ty * s.pitch + tx]);
@@ -769,14 +955,21 @@ __device__ __noinline__ void run_res_search(const EngineArgs& ea, EngCtx& x, int
       const unsigned bal = __ballot_sync(0xffffffffu, known);
       if (lane < P) {
         tgt[dy * TP + lane] = w;
-        tl.known[dy * P + lane] = (uint8_t)known;
+        tl.known[dy * P + lane] = (uint8_t)(known ? 1 : OVL && in ? 2 : 0);
       }
       if (lane == 0) rowd[dy] = row_desc(bal & ((1u << P) - 1u), P);
+      if constexpr (OVL) {
+        const uint32_t wa = known ? w | 0xff000000u : 0u;
+        const uint32_t sq = __reduce_add_sync(0xffffffffu, __dp4a(wa, wa, 0u));
+        if (lane == 0) tl.a2row[dy] = (int)sq;
+      }
     }
     if constexpr (KC < 16)
       for (int i = tid; i < n * KC * 32; i += kEngThreads) part[i] = 0u;
+    if (OVL && tid == 0) tl.red32[0] = 0;
     __syncthreads();
     unsigned long long best = ~0ull;
+    int n_adm = 0;
     auto take = [&](int j, const uint32_t (&acc)[KC]) {
       const int u = u0 + j, band = u / ncu, col = u - band * ncu;
       const uint32_t vb = bits[j * 32 + lane];
@@ -784,7 +977,9 @@ __device__ __noinline__ void run_res_search(const EngineArgs& ea, EngCtx& x, int
 #pragma unroll
       for (int k = 0; k < KC; ++k) {
         const unsigned long long key = ((unsigned long long)acc[k] << 32) | (idx0 + (unsigned)k);
-        if ((vb & (1u << k)) && key < best) best = key;
+        const bool adm = (vb & (1u << k)) && (!OVL || acc[k] < kOvlBad);
+        if (OVL) n_adm += adm;
+        if (adm && key < best) best = key;
       }
     };
     // (KC 16: whole units, warp w takes w, w + 16, ...; else the rows
@@ -798,7 +993,10 @@ __device__ __noinline__ void run_res_search(const EngineArgs& ea, EngCtx& x, int
       const ResSeg& sg = pl.seg[band - b0];
       const uint32_t* strip = reinterpret_cast<const uint32_t*>(area + sg.off) + lane * sg.pitch + (col - sg.c_lo) * KC;
       uint32_t acc[KC];
-      unit_ssd<R, KC>(strip, sg.pitch, tgt, rowd, r0, r1, acc);
+      if constexpr (OVL)
+        unit_ssd_overlap<R>(strip, sg.pitch, tgt, rowd, tl.known, tl.a2row, r0, r1, bits[j * 32 + lane] != 0, acc);
+      else
+        unit_ssd<R, KC>(strip, sg.pitch, tgt, rowd, r0, r1, acc);
       if constexpr (KC < 16) {
 #pragma unroll
         for (int k = 0; k < KC; ++k) atomicAdd(&part[(j * KC + k) * 32 + lane], acc[k]);
@@ -818,8 +1016,16 @@ __device__ __noinline__ void run_res_search(const EngineArgs& ea, EngCtx& x, int
         take(j, acc);
       }
     }
+    if constexpr (OVL) {
+      __syncwarp();
+      n_adm = __reduce_add_sync(0xffffffffu, n_adm);
+      if (lane == 0 && n_adm) atomicAdd(&tl.red32[0], n_adm);
+    }
     best = block_min_u64(best, tl.red64);
     if (tid == 0) {
+      if (OVL)
+        st_relaxed64(&tpart[x.tsize * (1 + (epoch & 1u)) + rank],
+                     (unsigned long long)epoch << 32 | (unsigned)tl.red32[0]);
       if (!withheld) st_relaxed64(&tpart[rank], key_tag(best, epoch));
       // the tiles are brought up to date as soon as the copy is done, while the
       // leader still works on the priorities (after the publication, this and
@@ -836,14 +1042,14 @@ __device__ __noinline__ void run_res_search(const EngineArgs& ea, EngCtx& x, int
       // it that became valid; every load in flight before the first use
       constexpr int NCW = 4 * R + 1, NV = (NCW * NCW + kEngThreads - 1) / kEngThreads;
       const int tx = px + tid % P - R, ty = py + tid / P - R;
-      const bool filled = tid < P * P && tx >= 0 && tx < s.W && ty >= 0 && ty < s.H && !tl.known[tid < P * P ? tid : 0];
+      const bool filled = tid < P * P && tx >= 0 && tx < s.W && ty >= 0 && ty < s.H && tl.known[tid < P * P ? tid : 0] != 1;
       uint32_t w = 0u;
       if (filled) w = __ldcg(&s.img[(size_t)ty * s.pitch + tx]);
       int cnt[NV];
 #pragma unroll
       for (int v = 0; v < NV; ++v) {
         const int jj = tid + v * kEngThreads, qx = px + jj % NCW - 2 * R, qy = py + jj / NCW - 2 * R;
-        const bool in = jj < NCW * NCW && qx >= s.cx0 && qx <= s.cx1 && qy >= s.cy0 && qy <= s.cy1;
+        const bool in = !OVL && jj < NCW * NCW && qx >= s.cx0 && qx <= s.cx1 && qy >= s.cy0 && qy <= s.cy1;
         cnt[v] = in ? __ldcg(&s.count[(size_t)qy * s.pitch + qx]) : 1;
       }
       if (filled) {
@@ -888,7 +1094,6 @@ __device__ __noinline__ void run_lead_only(const EngineArgs& ea, int j, EngCtx& 
 template <int R, int SRW, bool kLeadOnly>
 __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x) {
   using G = EngGeom<R, SRW>;
-  constexpr int TH = kResRows + 2 * R;  // rows of a resident tile
   constexpr int P = G::P, B = G::B;
   uint8_t* const smem = eng_smem();
   EngSmemTail& tl = *reinterpret_cast<EngSmemTail*>(smem);
@@ -950,25 +1155,27 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
              (!s.tc_auto || tc_round_cycles(s, tc_ns) < plain_round_cycles(s, tsize));
     tc_nb = min(kTcRing, ((int)x.smem_bytes - (tc_off - (int)kHeadBytes) - fixed) / tc_slot_b);
   }
-  const bool lead_searches = tcmode ? tc_lead : tsize == 1 || nbatch >= 8 * tsize;
+  const bool lead_searches = tcmode ? tc_lead : !s.overlap && (tsize == 1 || nbatch >= 8 * tsize);
   const int nsmax = lead_searches ? tsize : tsize - 1;  // CTAs that may search
   // Plain form, resident mode when the leader does not search and every
   // searching CTA's tiles fit (the same decision in every CTA of the team: it
-  // depends only on the image and the team): two tiles (a range may straddle a
-  // band boundary), the validity bits and the partial SSDs; more than one band
-  // of units per CTA streams instead.
+  // depends only on the image and the team); more than one band of units per
+  // CTA streams instead.  A partial-overlap search comes here only when it fits
+  // (overlap_fits).
   const int nbands = s.cy1 >= s.cy0 ? (s.cy1 - s.cy0 + kResRows) / kResRows : 0;
   int kc = 16, ncu = 0, ns = 0;
   bool resident = false;
   if (tcmode) {
     ns = min(nsmax, tc_ntiles);
+  } else if (s.overlap) {
+    kc = 4;
+    resident = overlap_units<R>(s, nsmax, &ncu, &ns) > 0;
   } else {
     for (; !lead_searches; kc = 4) {
       ncu = s.cx1 >= s.cx0 ? (s.cx1 - xb + kc) / kc : 0;
       ns = min(nsmax, ncu * nbands);
       const int m = ns > 0 ? (ncu * nbands + ns - 1) / ns : 0;  // most units of one CTA
-      const int need = TH * 4 * (m * kc + 2 * (2 * R + 12)) + 640 + m * 64 + (kc < 16 ? m * kc * 128 : 0);
-      resident = m > 0 && m <= ncu && need <= (int)x.smem_bytes - (int)kHeadBytes;
+      resident = m > 0 && m <= ncu && res_need<R>(kc, m) <= (int)x.smem_bytes - (int)kHeadBytes;
       if (m >= 3 * kEngWarps / 4 || kc == 4) break;
     }
     if (!resident) ns = min(nsmax, nbatch);
@@ -995,7 +1202,8 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     }
     if (resident && searcher) {
       const int acc_off = ((int)kHeadBytes + tl.plan.bits_off + (tl.plan.u1 - tl.plan.u0) * 64 + 127) & ~127;
-      if (kc == 16) run_res_search<R, 16>(ea, x, xb, ncu, acc_off);
+      if (s.overlap) run_res_search<R, 4, true>(ea, x, xb, ncu, acc_off);
+      else if (kc == 16) run_res_search<R, 16>(ea, x, xb, ncu, acc_off);
       else run_res_search<R, 4>(ea, x, xb, ncu, acc_off);
       return;
     }
@@ -1096,6 +1304,14 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     return block_min_u64(best, tl.red64);
   };
 
+  // Partial-overlap search: the last round's candidates, for its record (warp 15).
+  auto last_counts = [&]() {
+    if (!s.overlap || !usm.rec_pending) return;
+    const int n = gather_counts(&tpart[tsize * (1 + ((epoch - 1u) & 1u))], ns, epoch - 1u, err, limit);
+    if (lane == 0) usm.n_cand = n;
+    __syncwarp();
+  };
+
   // One iteration of the leader on the staged target (and its own search
   // share when it searches), up to the publication of the next round and the
   // staging of its target.  Whole block.
@@ -1112,7 +1328,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
         tl.status = __ldcg(&c->status);
         tl.err = __ldcg(err);
       }
-      spec_record<R>(s, usm, false);
+      spec_record<R>(s, usm, false, last_counts);
       __syncwarp();
     }
     if constexpr (!kLeadOnly) {
@@ -1182,6 +1398,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     if (!tl.stop) {
       do lead_round(false);
       while (!tl.stop);
+      if (tid >= kRecThread) last_counts();
       if (tid == kRecThread) update_times<R>(s, usm);
       update_drain<R>(s, usm, false);
     }
@@ -1253,7 +1470,7 @@ __global__ void __launch_bounds__(kEngThreads) k_update_fast(ImgState s, cudaGra
       cpy = plan_copy<R>(s, usm);
     } else {
       const int lane = threadIdx.x & 31;
-      spec_record<R>(s, usm, false);
+      spec_record<R>(s, usm, false, [] {});
       __syncwarp();
       unsigned long long best = ~0ull;
 #pragma unroll 4
@@ -1320,9 +1537,19 @@ template <int R>
 static size_t eng_smem_r(int srw) {
   return srw == 2 ? engine_smem_for<R, 2>() : engine_smem_for<R, 1>();
 }
+// Whether the engine runs the image's partial-overlap search with a team of
+// tsize CTAs: every searcher's tiles are resident (the streaming search has no
+// such form), and a target fits the publication word.
+template <int R>
+static bool overlap_fits_t(const ImgState& s, int tsize, size_t smem) {
+  int ncu, ns;
+  const int m = overlap_units<R>(s, tsize - 1, &ncu, &ns);
+  return m > 0 && m <= ncu && smem > kHeadBytes && res_need<R>(4, m) <= (int)(smem - kHeadBytes) && s.W <= 0x7fff &&
+         s.H <= 0x7fff;
+}
 template <int R>
 const EngineFns* engine_fns_for() {
-  static const EngineFns f = {eng_smem_r<R>, upd_fast_t<R>, prio_init_t<R>};
+  static const EngineFns f = {eng_smem_r<R>, upd_fast_t<R>, prio_init_t<R>, overlap_fits_t<R>};
   return &f;
 }
 

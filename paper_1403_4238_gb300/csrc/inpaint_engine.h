@@ -150,6 +150,8 @@ struct EngineArgs {
                                // of every team skip its arrival; 0 normally
   int tc_cols;                 // tensor-memory columns every CTA holds for the
                                // tensor-core search (0: no image uses it)
+  int overlap;                 // 1: partial-overlap search (one image): behind the keys,
+                               // two more slots per CTA with its counts of even and odd rounds
 };
 
 // The mbarriers of an engine CTA, at the start of its shared memory (the
@@ -201,6 +203,7 @@ struct EngineFns {
   cudaError_t (*update_fast)(const ImgState& s, unsigned long long cond, int use_cond,
                              cudaStream_t st);
   cudaError_t (*prio_init)(const ImgState& s, cudaStream_t st);
+  bool (*overlap_fits)(const ImgState& s, int tsize, size_t smem);
 };
 const EngineFns* engine_fns_r1();
 const EngineFns* engine_fns_r2();

@@ -789,13 +789,14 @@ __device__ inline void spec_rest(const ImgState& s, UpdSmem<R>& sm) {
 
 // Warp 15 meanwhile: the integral image of the filled flags, then (one thread)
 // the last iteration's record and the scalars of the iteration on the staged
-// target.
-template <int R>
-__device__ inline void spec_record(const ImgState& s, UpdSmem<R>& sm, bool overlap_counts) {
+// target.  `before` (whole warp) runs before the record.
+template <int R, class F>
+__device__ inline void spec_record(const ImgState& s, UpdSmem<R>& sm, bool overlap_counts, F&& before) {
   constexpr int P = UpdGeom<R>::P;
   warp_fsat<R>(sm);
   __syncwarp();
   fsat_arrive();
+  before();
   if (threadIdx.x != kRecThread) return;
   update_times<R>(s, sm);
   if (sm.rec_pending) write_record<R>(s, sm, overlap_counts);
