@@ -306,10 +306,10 @@ def measured_peaks():
         return {}
 
 
-def launches_init(H):
-    # ctrl init, unpack, SAT rows / column chunks / chunk prefix (/ apply),
-    # validity counts, priorities, two tile levels, first selection
-    return 10 + (1 if H > 64 else 0)
+def launches_per_removal(form):
+    # unpack, validity counts, priorities, tiles and first selection; begin,
+    # engine, end; tensor-core form: planes and validity bits
+    return 4 + 3 + (2 if form == "tc" else 0)
 
 
 def time_removals(ip, drgb, dmask, steps, warmup, flush):
@@ -791,9 +791,7 @@ def main():
             "ms_per_removal": total_ms / args.steps,
             "e2e": {"value": e2e_value, "unit": UNIT, "ms_per_removal": e2e_ms,
                     "h2d_bytes_per_step": 4 * W * H, "d2h_bytes_per_step": 3 * W * H},
-            # per removal: the initialisation kernels, (tensor-core form) the
-            # planes, and one persistent engine launch
-            "gpu_launches": (launches_init(H) + (2 if args.form == "tc" else 1)) * args.steps,
+            "gpu_launches": launches_per_removal(args.form) * args.steps,
             "roofline": roof,
             "clocks": clocks,
             "plain_engine": {"ms_per_removal": plain_ms, "value": evals_per_removal / (plain_ms / 1e3),

@@ -77,7 +77,8 @@ struct inpaint_ctx {
   bool overlap_engine = false;  // partial-overlap search: the engine runs it
   unsigned long long* d_epart = nullptr;
   int* d_err = nullptr;
-  int* h_err = nullptr;
+  bool ctrl_known = false;  // h_ctrl is the device's state (it changes only in calls that read it back)
+  bool no_limit = false;    // the device's iteration limit is INT_MAX
   unsigned long long* d_key = nullptr;  // key applied by inpaint_apply_key
 
   void* dalloc(size_t bytes) {
@@ -111,10 +112,8 @@ struct inpaint_ctx {
     if (stream) cudaStreamSynchronize(stream);
     if (h_ctrl) cudaFreeHost(h_ctrl);
     if (h_limit) cudaFreeHost(h_limit);
-    if (h_err) cudaFreeHost(h_err);
     h_ctrl = nullptr;
     h_limit = nullptr;
-    h_err = nullptr;
     if (own_stream && stream) cudaStreamDestroy(stream);
     stream = nullptr;
   }
@@ -168,6 +167,7 @@ int finish_init(inpaint_ctx* c) {
     return INPAINT_ERR_ARG;
   }
   if (c->h_ctrl->status != 0) return c->h_ctrl->status;
+  c->ctrl_known = c->no_limit = true;
   return INPAINT_OK;
 }
 
@@ -269,7 +269,6 @@ int setup_engine(inpaint_ctx* c) {
       !alloc_n(c, c->d_ints, (size_t)c->eng_grid + 5) || !alloc_n(c, c->d_team, 1) ||
       !alloc_n(c, c->d_epart, (size_t)c->eng_grid * slots) || !alloc_n(c, c->d_err, 1))
     return INPAINT_ERR_NOMEM;
-  if (!c->h_err && cudaMallocHost(&c->h_err, sizeof(int)) != cudaSuccess) return INPAINT_ERR_NOMEM;
   CUtensorMap tm[2];
   if (make_image_tmap(c->st, sr, tm) != 0) {
     g_last_error = "cuTensorMapEncodeTiled failed";
@@ -303,14 +302,15 @@ int setup_engine(inpaint_ctx* c) {
   return INPAINT_OK;
 }
 
-int run_engine(inpaint_ctx* c) {
+int run_engine(inpaint_ctx* c, int limit) {
   int rc = setup_engine(c);
   if (rc) return rc;
-  CK(cudaMemsetAsync(c->d_team, 0, sizeof(TeamCtl), c->stream));
-  CK(cudaMemsetAsync(c->d_err, 0, sizeof(int), c->stream));
+  c->no_limit = false;
+  CK(engine_begin(c->ea, 1, c->eng_grid, c->st.ctrl, limit, c->stream));
   CK(launch_planes(c->st, c->stream));  // the image may have changed since the last launch
   CK(engine_launch(c->eng_smem, c->ea, c->eng_grid, c->stream));
-  CK(cudaMemcpyAsync(c->h_err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+  CK(engine_end(c->ea, c->st.ctrl, c->stream));
+  c->no_limit = true;
   return INPAINT_OK;
 }
 
@@ -340,9 +340,12 @@ int build_run_graph(inpaint_ctx* c) {
 }
 
 int set_limit(inpaint_ctx* c, int limit) {
+  if (limit == INT_MAX && c->no_limit) return INPAINT_OK;
   *c->h_limit = limit;
+  c->no_limit = false;
   CK(cudaMemcpyAsync(&c->st.ctrl->iter_limit, c->h_limit, sizeof(int), cudaMemcpyHostToDevice,
                      c->stream));
+  c->no_limit = limit == INT_MAX;
   return INPAINT_OK;
 }
 
@@ -351,6 +354,11 @@ int read_ctrl(const inpaint_ctx* c) {
   CK(cudaStreamSynchronize(c->stream));
   return INPAINT_OK;
 }
+
+// The state in h_ctrl, read only if a call before this one may have left
+// it behind the device's: a step or a run reads it back when it ends (a read
+// is a copy and a synchronisation, 9 us of a 42 us step).
+int known_ctrl(const inpaint_ctx* c) { return c->ctrl_known ? INPAINT_OK : read_ctrl(c); }
 
 int create_impl(const uint8_t* rgb, int W, int H, int rgb_stride, const uint8_t* mask,
                 int mask_stride, int r, const inpaint_options* opt, inpaint_ctx** out, bool tc_auto = false) {
@@ -507,6 +515,7 @@ int inpaint_create(const uint8_t* rgb, int width, int height, int rgb_stride_byt
 int inpaint_reset(inpaint_ctx* c, const uint8_t* rgb, int rgb_stride, const uint8_t* mask,
                   int mask_stride, int input_on_device) {
   if (!c || !rgb || !mask || rgb_stride < 3 * c->W || mask_stride < c->W) return INPAINT_ERR_ARG;
+  c->ctrl_known = c->no_limit = false;
   const int W = c->W, H = c->H;
   const uint8_t* drgb = rgb;
   const uint8_t* dmask = mask;
@@ -527,14 +536,16 @@ int inpaint_reset(inpaint_ctx* c, const uint8_t* rgb, int rgb_stride, const uint
 
 int inpaint_step(inpaint_ctx* c, inpaint_step_info* info) {
   if (!c) return INPAINT_ERR_ARG;
-  int rc = read_ctrl(c);
+  int rc = known_ctrl(c);
   if (rc) return rc;
   if (c->h_ctrl->status != 0) return c->h_ctrl->status;
   if (c->h_ctrl->remaining == 0) return INPAINT_DONE;
+  c->ctrl_known = false;
   if ((rc = set_limit(c, INT_MAX))) return rc;
   CK(launch_planes(c->st, c->stream));  // the image may have changed since the last call
   if ((rc = launch_iteration(c, 0))) return rc;
   if ((rc = read_ctrl(c))) return rc;
+  c->ctrl_known = true;
   if (c->h_ctrl->status != 0) return c->h_ctrl->status;
   if (info) *info = c->h_ctrl->last;
   return INPAINT_OK;
@@ -544,8 +555,7 @@ int inpaint_run(inpaint_ctx* c, int max_iters, int* iters_done, inpaint_step_inf
                 int trace_cap) {
   if (iters_done) *iters_done = 0;
   if (!c || (trace && trace_cap < 0)) return INPAINT_ERR_ARG;
-  if (c->h_err) *c->h_err = 0;
-  int rc = read_ctrl(c);
+  int rc = known_ctrl(c);
   if (rc) return rc;
   if (c->h_ctrl->status != 0) return c->h_ctrl->status;
   if (c->h_ctrl->remaining == 0) return INPAINT_DONE;
@@ -554,26 +564,29 @@ int inpaint_run(inpaint_ctx* c, int max_iters, int* iters_done, inpaint_step_inf
   // suffice: the device loop is bounded even if a kernel misbehaved.
   long long lim = (long long)start + c->h_ctrl->remaining;
   if (max_iters > 0 && (long long)start + max_iters < lim) lim = (long long)start + max_iters;
-  if ((rc = set_limit(c, lim > INT_MAX ? INT_MAX : (int)lim))) return rc;
-  if (use_engine(c)) {
+  const int limit = lim > INT_MAX ? INT_MAX : (int)lim;
+  const bool engine = use_engine(c);
+  c->ctrl_known = false;
+  if (engine) {
     if (c->opt.debug_checks) {  // engine has no per-iteration hook: drive it one iteration at a time
       for (long long i = start; i < lim; ++i) {
-        if ((rc = set_limit(c, (int)(i + 1)))) return rc;
-        if ((rc = run_engine(c))) return rc;
+        if ((rc = run_engine(c, (int)(i + 1)))) return rc;
         CK(launch_verify_count(c->st, c->stream));
         if ((rc = read_ctrl(c))) return rc;
-        if (*c->h_err || c->h_ctrl->status != 0 || c->h_ctrl->remaining == 0) break;
+        if (c->h_ctrl->engine_err || c->h_ctrl->status != 0 || c->h_ctrl->remaining == 0) break;
       }
-    } else if ((rc = run_engine(c))) {
+    } else if ((rc = run_engine(c, limit))) {
       return rc;
     }
   } else {
     if ((rc = build_run_graph(c))) return rc;
+    if ((rc = set_limit(c, limit))) return rc;
     CK(launch_planes(c->st, c->stream));  // the image may have changed since the last call
     CK(cudaGraphLaunch(c->run_exec, c->stream));
   }
   if ((rc = set_limit(c, INT_MAX))) return rc;
   if ((rc = read_ctrl(c))) return rc;
+  c->ctrl_known = true;
   const int done = c->h_ctrl->iter - start;
   if (iters_done) *iters_done = done;
   if (trace && trace_cap > 0 && done > 0) {
@@ -585,7 +598,7 @@ int inpaint_run(inpaint_ctx* c, int max_iters, int* iters_done, inpaint_step_inf
       CK(cudaStreamSynchronize(c->stream));
     }
   }
-  if (c->h_err && *c->h_err) {
+  if (engine && c->h_ctrl->engine_err) {
     g_last_error = "a bounded device wait in the persistent engine gave up";
     return INPAINT_ERR_TIMEOUT;
   }
@@ -622,6 +635,7 @@ int inpaint_export_state(const inpaint_ctx* c, uint8_t* rgb, uint8_t* omega, dou
 int inpaint_import_state(inpaint_ctx* c, const uint8_t* rgb, const uint8_t* omega,
                          const double* conf) {
   if (!c || !rgb || !omega || !conf) return INPAINT_ERR_ARG;
+  c->ctrl_known = c->no_limit = false;
   const size_t n = (size_t)c->W * c->H;
   if (!c->conf_stage && !alloc_n(c, c->conf_stage, n)) return INPAINT_ERR_NOMEM;
   CK(cudaMemcpyAsync(c->rgb_stage, rgb, 3 * n, cudaMemcpyHostToDevice, c->stream));
@@ -776,6 +790,7 @@ int inpaint_apply_key(inpaint_ctx* c, unsigned long long key, inpaint_step_info*
   if ((rc = read_ctrl(c))) return rc;
   if (c->h_ctrl->status != 0) return c->h_ctrl->status;
   if (c->h_ctrl->remaining == 0) return INPAINT_DONE;
+  c->ctrl_known = false;
   if (!c->d_key && !alloc_n(c, c->d_key, 1)) return INPAINT_ERR_NOMEM;
   if ((rc = set_limit(c, INT_MAX))) return rc;
   CK(cudaMemcpyAsync(c->d_key, &key, sizeof(key), cudaMemcpyHostToDevice, c->stream));
@@ -1096,8 +1111,7 @@ int engine_set_run(EngineSet& es, const std::vector<inpaint_ctx*>& cs, int max_i
     CK(cudaMemcpyAsync(&cs[i]->st.ctrl->iter_limit, &es.h_pinned[1 + i], sizeof(int),
                        cudaMemcpyHostToDevice, st));
   }
-  CK(cudaMemsetAsync((void*)es.ea.teams, 0, sizeof(TeamCtl) * es.n_teams, st));
-  CK(cudaMemsetAsync(es.d_err, 0, sizeof(int), st));
+  CK(engine_begin(es.ea, es.n_teams, es.grid, nullptr, 0, st));
   es.ea.tick_ns = tick_ns;
   CK(engine_launch(es.smem, es.ea, es.grid, st));
   es.ea.tick_ns = 0ull;
@@ -1256,8 +1270,7 @@ void build_batch_graphs(inpaint_batch* b) {
   });
   EngineSet& es = b->es;
   capture_graph(b->stream, &b->run_exec, [&] {
-    if (cudaMemsetAsync((void*)es.ea.teams, 0, sizeof(TeamCtl) * es.n_teams, b->stream) != cudaSuccess ||
-        cudaMemsetAsync(es.d_err, 0, sizeof(int), b->stream) != cudaSuccess ||
+    if (engine_begin(es.ea, es.n_teams, es.grid, nullptr, 0, b->stream) != cudaSuccess ||
         engine_launch(es.smem, es.ea, es.grid, b->stream) != cudaSuccess ||
         cudaMemcpyAsync(es.h_pinned, es.d_err, sizeof(int), cudaMemcpyDeviceToHost, b->stream) != cudaSuccess)
       return false;

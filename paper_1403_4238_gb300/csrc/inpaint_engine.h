@@ -220,6 +220,8 @@ const EngineFns* engine_fns(int r);
 cudaError_t engine_occupancy(size_t smem, int* blocks_per_sm);
 // Dynamic shared memory of every engine launch: all an SM offers one CTA.
 size_t engine_launch_smem();
+cudaError_t engine_begin(const EngineArgs& ea, int n_teams, int grid, Ctrl* c, int limit, cudaStream_t st);
+cudaError_t engine_end(const EngineArgs& ea, Ctrl* c, cudaStream_t st);
 cudaError_t engine_launch(size_t smem, const EngineArgs& ea, int grid, cudaStream_t st);
 int make_image_tmap(const ImgState& s, int srw, CUtensorMap* out);  // writes out[0], out[1]
 int make_image_tmap_box(const ImgState& s, int box_w, int box_h, CUtensorMap* out);

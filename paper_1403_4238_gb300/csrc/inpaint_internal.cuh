@@ -71,6 +71,7 @@ struct Ctrl {
   int tc_rounds;   // engine search rounds run in the tensor-core form
   int n_front;     // patch radius > 8: front pixels in ImgState::front whose priorities
                    // are to be evaluated; -1: the last update applied nothing
+  int engine_err;  // error word of the last engine launch (single image)
   int tiles_done;  // initialisation: CTAs of k_tiles_all that are done
 };
 

@@ -224,6 +224,7 @@ __global__ void k_unpack(ImgState s, const uint8_t* rgb, int rgb_stride, const u
     c->tc_rounds = 0;
     c->n_front = 0;
     c->tiles_done = 0;
+    c->engine_err = 0;
   }
   int om = 1;
   if (x < s.W) {
