@@ -40,3 +40,20 @@ def test_whole_removal(api, r, W, H):
     for f in ("priority", "confidence"):
         assert [np.float64(t[f]).view(np.uint64) for t in tr] == [np.float64(t[f]).view(np.uint64) for t in ora.trace]
     assert (out == ora.rgb).all() and (left == ora.mask).all()
+
+
+@pytest.mark.parametrize("r,W,H", [(9, 75, 66), (17, 120, 101)])
+def test_steps_and_applied_keys(api, r, W, H):
+    """The same iterations outside the graph: search and speculative part on two streams, and applied alone."""
+    rgb = synth.image(W, H, 8, 35.0, 70 + r)
+    m = np.zeros((H, W), np.uint8)
+    m[0:4, 5:9] = m[H // 2:H // 2 + 9, W // 2:W // 2 + 5] = m[H - 3:, W - 6:] = 1
+    ora = oracle.run(rgb, m, r)
+    with api.Inpainter(rgb, m, r, debug=True) as a, api.Inpainter(rgb, m, r, debug=True) as b:
+        for i in range(ora.iters):
+            t = a.step()
+            u = b.apply_key(b.search_rows(0, H))
+            for f in ("px", "py", "qx", "qy", "ssd", "priority", "confidence", "filled", "n_cand"):
+                assert t[f] == ora.trace[i][f] and u[f] == ora.trace[i][f], (i, f)
+        assert a.step() is None
+        assert (a.result() == ora.rgb).all() and (b.result() == ora.rgb).all()
