@@ -359,7 +359,7 @@ int inpaint_batch_run(int n, const uint8_t* const* rgb, const uint8_t* const* ma
  * while slots are free and the estimated device memory of the admitted ones
  * stays within the budget (their state stays on the device until they
  * finish); each tick is one persistent engine launch over every active slot
- * that runs until about 20 ms of device time have passed (teams stop between
+ * that runs until about 8 ms of device time have passed (teams stop between
  * iterations and resume in the next tick) or each slot has done
  * iters_per_tick iterations, after which finished requests release their
  * memory and their result waits for inpaint_server_poll.

@@ -412,13 +412,11 @@ constexpr int kTgtOff = (int)((sizeof(EngSmemTail) + 15) & ~size_t(15));
 constexpr int kTgtWords = 17 * 20 + 17 + 3;  // padded target rows + row masks (R <= 8)
 constexpr size_t kHeadBytes = ((kTgtOff + kTgtWords * 4 + 127) / 128) * 128;
 
-// Shared memory of an engine CTA: head | (the leader only) update state and
-// update cache | two count tiles | tile slots.  The slots hold the source
-// tiles of the CTA's search batches: all of them, resident across the
-// iterations of a removal, when they fit, else two used as a double buffer.
-// A searching CTA that does not lead starts its count tiles right after the
-// head.  The kernel is launched with all the shared memory an SM offers and
-// takes as many slots as fit.
+// Shared memory of an engine CTA: head | (the leader only) update state | its
+// search's state: resident tiles, validity bits and partial SSDs; or the
+// tensor-core form's A strips, target table and ring; or two count tiles and
+// two tile slots of the streaming search, used as a double buffer.  The kernel
+// is launched with all the shared memory an SM offers.
 template <int R>
 __host__ __device__ constexpr size_t upd_smem_bytes() {
   return ((sizeof(UpdSmem<R>) + 127) / 128) * 128;

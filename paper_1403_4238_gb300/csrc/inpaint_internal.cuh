@@ -20,9 +20,10 @@
 //                        argmax over the front reads only these few entries
 //   ctrl   Ctrl          loop control block (selected p^, counters, status)
 //   trace  inpaint_step_info[trace_cap]   one record per iteration
-//   planes uint16[5][prows*ppitch]  tensor-core form in the engine only: BF16
-//                        R' G' B' (byte - 128) and the two halves of the
-//                        square sum, the operands of its correlations
+//   planes uint16[]      images that may be searched in the tensor-core form:
+//                        BF16 R' G' B' (byte - 128) and the two halves of the
+//                        square sum, the operands of its correlations, tiled
+//                        (ImgState), with the candidates' validity bits behind
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>

@@ -4,9 +4,9 @@
 // (Eq. 1-2), the copy of the best source patch into the unknown part of the
 // target patch, and the confidence update.  Table 2 lists these as the grey
 // conversion, border update, source marking, priority and confidence updates
-// and the RGB/grey update; here they are: one init pass per image, then one
-// single-CTA update kernel per iteration that touches only the neighbourhood
-// of the filled patch.
+// and the RGB/grey update; here they are: one init pass per image, then, for
+// patch radii above 8, three small kernels per iteration that touch only the
+// neighbourhood of the filled patch (radii to 8: update_fast.cuh).
 //
 // Bit-exactness of the FP64 priority: the library is compiled with
 // --fmad=false, the confidence sum runs in row-major patch order (dy outer,
