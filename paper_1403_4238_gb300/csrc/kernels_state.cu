@@ -19,21 +19,20 @@ namespace inp {
 
 // ---------------------------------------------------------------- priority
 
-__device__ inline bool known_px(const ImgState& s, int x, int y) {
-  return x >= 0 && x < s.W && y >= 0 && y < s.H && s.omega[(size_t)y * s.W + x] == 0;
-}
-
 __device__ inline int omega_clamped(const ImgState& s, int x, int y) {
   x = x < 0 ? 0 : (x >= s.W ? s.W - 1 : x);
   y = y < 0 ? 0 : (y >= s.H ? s.H - 1 : y);
   return s.omega[(size_t)y * s.W + x] ? 1 : 0;
 }
 
-// Fill front membership: p in Omega with an in-image 4-neighbour in Phi.
+// Fill front membership: p in Omega with an in-image 4-neighbour in Phi.  The
+// five reads are independent (a chain of them, one L2 round trip each, took half
+// of k_fill_big).
 __device__ inline bool on_front(const ImgState& s, int x, int y) {
-  if (s.omega[(size_t)y * s.W + x] == 0) return false;
-  return known_px(s, x - 1, y) || known_px(s, x + 1, y) || known_px(s, x, y - 1) ||
-         known_px(s, x, y + 1);
+  const uint8_t* o = s.omega + (size_t)y * s.W + x;
+  const uint8_t c = o[0], l = x > 0 ? o[-1] : 1, r = x + 1 < s.W ? o[1] : 1;
+  const uint8_t u = y > 0 ? o[-s.W] : 1, d = y + 1 < s.H ? o[s.W] : 1;
+  return (c != 0) & ((l == 0) | (r == 0) | (u == 0) | (d == 0));
 }
 
 // D(p) of Eq. 2 from the isophote's gradient; normal to the front: Sobel of
@@ -111,14 +110,18 @@ __device__ inline void append_front(const ImgState& s, bool mine, int i) {
 
 // Priorities of the listed front pixels for patch radii above the engine's:
 // one CTA of two warps per pixel.  Warp 0 sums the confidences: its lanes load
-// a patch row coalesced (the next row while this one is summed) and the known
-// entries are added one by one in row-major order; unknown ones are skipped,
-// which changes nothing (adding +0.0 to a non-negative sum) and halves the
-// chain of dependent FP64 additions (69 cycles each).  Warp 1 meanwhile finds
-// the strongest isophote.  (One thread per pixel reading the patch from global
-// memory, in the update's one CTA, took 390 us an iteration at 512x384, 25x25.)
+// four patch rows coalesced (the next four while these are summed), write the
+// known entries one after the other to shared memory, and add them one by one in
+// row-major order; unknown ones are skipped, which changes nothing (adding +0.0
+// to a non-negative sum) and halves the chain of dependent FP64 additions (69
+// cycles each; with a bit scan and a shuffle per entry in the chain 140).  Warp 1
+// meanwhile finds the strongest isophote.  (One thread per pixel reading the
+// patch from global memory, in the update's one CTA, took 390 us an iteration at
+// 512x384, 25x25.)
 __global__ void __launch_bounds__(64) k_prio_list(ImgState s) {
+  constexpr int kGroup = 4;
   __shared__ unsigned long long iso_s;
+  __shared__ __align__(16) double vals[kGroup * (2 * kMaxRadius + 1) + 4];
   const int n = s.ctrl->n_front;
   const int W = s.W, H = s.H, r = s.r, P = 2 * r + 1;
   const int lane = threadIdx.x & 31;
@@ -128,30 +131,40 @@ __global__ void __launch_bounds__(64) k_prio_list(ImgState s) {
     double sum = 0.0;
     if (threadIdx.x < 32) {
       constexpr int NB = (2 * kMaxRadius + 1 + 31) / 32;
-      double c[NB], nc[NB];
-      bool kn[NB], nkn[NB];
-      auto load_row = [&](int yy, double (&cv)[NB], bool (&kv)[NB]) {
+      double c[kGroup][NB];
+      bool kn[kGroup][NB];
+      auto load_rows = [&](int y0) {
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-          const int xx = x0 + 32 * b + lane;
-          const bool in = 32 * b < P && xx <= x1;
-          cv[b] = in ? s.conf[(size_t)yy * W + xx] : 0.0;
-          kv[b] = in && s.omega[(size_t)yy * W + xx] == 0;
+        for (int g = 0; g < kGroup; ++g) {
+#pragma unroll
+          for (int b = 0; b < NB; ++b) {
+            const int xx = x0 + 32 * b + lane;
+            const bool in = 32 * b < P && xx <= x1 && y0 + g <= y1;
+            c[g][b] = in ? s.conf[(size_t)(y0 + g) * W + xx] : 0.0;
+            kn[g][b] = in && s.omega[(size_t)(y0 + g) * W + xx] == 0;
+          }
         }
       };
-      load_row(y0, c, kn);
-      for (int yy = y0; yy <= y1; ++yy) {
-        if (yy < y1) load_row(yy + 1, nc, nkn);
+      load_rows(y0);
+      for (int yy = y0; yy <= y1; yy += kGroup) {
+        int n_val = 0;
+        __syncwarp();
 #pragma unroll
-        for (int b = 0; b < NB; ++b) {
-          if (32 * b >= P) break;
-          for (unsigned m = __ballot_sync(0xffffffffu, kn[b]); m; m &= m - 1)
-            sum = __dadd_rn(sum, __shfl_sync(0xffffffffu, c[b], __ffs(m) - 1));
+        for (int g = 0; g < kGroup; ++g) {
+#pragma unroll
+          for (int b = 0; b < NB; ++b) {
+            const unsigned m = __ballot_sync(0xffffffffu, kn[g][b]);
+            if (kn[g][b]) vals[n_val + __popc(m & ((1u << lane) - 1u))] = c[g][b];
+            n_val += __popc(m);
+          }
         }
-#pragma unroll
-        for (int b = 0; b < NB; ++b) {
-          c[b] = nc[b];
-          kn[b] = nkn[b];
+        if (lane < 4) vals[n_val + lane] = 0.0;  // (+0.0 changes no sum here)
+        __syncwarp();
+        if (yy + kGroup <= y1) load_rows(yy + kGroup);
+#pragma unroll 2
+        for (int q = 0; q < n_val; q += 4) {
+          const double2 v = *reinterpret_cast<const double2*>(&vals[q]), w = *reinterpret_cast<const double2*>(&vals[q + 2]);
+          sum = __dadd_rn(__dadd_rn(__dadd_rn(__dadd_rn(sum, v.x), v.y), w.x), w.y);
         }
       }
     } else {
@@ -341,6 +354,7 @@ struct UpdSmem {
   int32_t fsat[(2 * kMaxRadius + 2) * (2 * kMaxRadius + 2)];
   unsigned long long u64s[32];
   int ints[32];
+  int n_front;
 };
 
 // One iteration's copy and validity update for patch radii above the
@@ -419,51 +433,82 @@ __global__ void __launch_bounds__(kUpdThreads) k_fill_big(ImgState s) {
       }
     }
     __syncthreads();
-    for (int u = tid + 1; u <= P; u += nt)
-      for (int v = 2; v <= P; ++v) sm.fsat[v * P1 + u] += sm.fsat[(v - 1) * P1 + u];
+    for (int u = tid + 1; u <= P; u += nt) {
+      int run = 0;
+#pragma unroll 5
+      for (int v = 1; v <= P; ++v) {
+        run += sm.fsat[v * P1 + u];
+        sm.fsat[v * P1 + u] = run;
+      }
+    }
     __syncthreads();
 
     // Validity map: every centre within 2r of p^ loses the filled pixels of
     // its patch from its unknown count.
     const int side = 4 * r + 1;
     int newly = 0;
-    for (int j = tid; j < side * side; j += nt) {
-      const int wy = j / side - 2 * r, wx = j % side - 2 * r;
-      const int x = px + wx, y = py + wy;
-      if (x < 0 || x >= W || y < 0 || y >= H) continue;
-      const int u0 = max(0, wx), u1 = min(P - 1, wx + 2 * r);
-      const int v0 = max(0, wy), v1 = min(P - 1, wy + 2 * r);
-      if (u0 > u1 || v0 > v1) continue;
-      const int dec = sm.fsat[(v1 + 1) * P1 + u1 + 1] - sm.fsat[v0 * P1 + u1 + 1] -
-                      sm.fsat[(v1 + 1) * P1 + u0] + sm.fsat[v0 * P1 + u0];
-      if (dec) {
-        const size_t qi = (size_t)y * s.pitch + x;
-        const int nv = s.count[qi] - dec;
-        s.count[qi] = nv;
-        if (nv == 0 && in_rect(s, x, y)) ++newly;
+    constexpr int U = 5;  // counts of a thread in flight together
+    for (int j0 = tid; j0 < side * side; j0 += U * nt) {
+      int cnt[U], dec[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = j0 + u * nt, wy = j / side - 2 * r, wx = j % side - 2 * r;
+        const int x = px + wx, y = py + wy;
+        cnt[u] = dec[u] = 0;
+        if (j < side * side && x >= 0 && x < W && y >= 0 && y < H) {
+          // (a patch at most 2 r away overlaps the target's)
+          const int u0 = max(0, wx), u1 = min(P - 1, wx + 2 * r);
+          const int v0 = max(0, wy), v1 = min(P - 1, wy + 2 * r);
+          dec[u] = sm.fsat[(v1 + 1) * P1 + u1 + 1] - sm.fsat[v0 * P1 + u1 + 1] -
+                   sm.fsat[(v1 + 1) * P1 + u0] + sm.fsat[v0 * P1 + u0];
+          cnt[u] = s.count[(size_t)y * s.pitch + x];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (dec[u] == 0) continue;
+        const int j = j0 + u * nt, y = py + j / side - 2 * r, x = px + j % side - 2 * r;
+        s.count[(size_t)y * s.pitch + x] = cnt[u] - dec[u];
+        if (cnt[u] == dec[u] && in_rect(s, x, y)) ++newly;
       }
     }
     newly = block_sum_int(newly, sm.ints);  // also orders the global writes above
 
-    if (tid == 0) c->n_front = 0;
-    __syncthreads();
-    // Priorities that can change: front pixels within 2r+1 of p^.
+    // Priorities that can change: front pixels within 2r+1 of p^, listed with a
+    // counter in shared memory (every round trip here is a serial one: with a
+    // counter in global memory and a chain of reads per pixel this kernel took
+    // 14 us at 25x25).
     const int R2 = 2 * r + 1, side2 = 2 * R2 + 1;
-    for (int j0 = 0; j0 < side2 * side2; j0 += nt) {
-      const int j = j0 + tid;
-      const int x = px - R2 + j % side2, y = py - R2 + j / side2;
-      bool fr = false;
-      if (j < side2 * side2 && x >= 0 && x < W && y >= 0 && y < H) {
-        fr = on_front(s, x, y);
-        if (!fr) {
-          s.prio[(size_t)y * W + x] = 0ull;
-          s.pconf[(size_t)y * W + x] = 0.0;
+    if (tid == 0) sm.n_front = 0;
+    __syncthreads();
+    constexpr int V = 3;
+    for (int j0 = tid; j0 - tid < side2 * side2; j0 += V * nt) {
+      bool in[V], fr[V];
+#pragma unroll
+      for (int u = 0; u < V; ++u) {
+        const int j = j0 + u * nt, x = px - R2 + j % side2, y = py - R2 + j / side2;
+        in[u] = j < side2 * side2 && x >= 0 && x < W && y >= 0 && y < H;
+        fr[u] = in[u] && on_front(s, x, y);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int u = 0; u < V; ++u) {
+        const int j = j0 + u * nt, i = (py - R2 + j / side2) * W + px - R2 + j % side2, lane = tid & 31;
+        const unsigned bal = __ballot_sync(0xffffffffu, fr[u]);
+        int base = 0;
+        if (lane == 0 && bal) base = atomicAdd(&sm.n_front, __popc(bal));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (fr[u]) {
+          s.front[base + __popc(bal & ((1u << lane) - 1u))] = i;
+        } else if (in[u]) {
+          s.prio[i] = 0ull;
+          s.pconf[i] = 0.0;
         }
       }
-      append_front(s, fr, y * W + x);
     }
     __syncthreads();
     if (tid == 0) {
+      c->n_front = sm.n_front;
       if (filled == 0) {  // p^ must lie in Omega; stop rather than loop without progress
         c->status = INPAINT_ERR_INTERNAL;
         c->n_front = -1;
