@@ -187,7 +187,7 @@ int launch_iteration(inpaint_ctx* c, int use_cond) {
   if (c->opt.form == INPAINT_FORM_TC)
     CK(launch_search_tc(c->st, c->tc, c->stream));
   else
-    CK(launch_search_plain(c->st, c->stream));
+    CK(launch_search_plain(c->st, c->stream, true));
   if (c->r <= 8)
     CK(launch_update_fast(c->st, c->cond, use_cond, c->stream));
   else
@@ -461,7 +461,7 @@ int create_impl(const uint8_t* rgb, int W, int H, int rgb_stride, const uint8_t*
   const size_t n = (size_t)W * H;
   if (!alloc_n(c, s.img, (size_t)s.pitch * H) || !alloc_n(c, s.omega, n) || !alloc_n(c, s.gray, n) ||
       !alloc_n(c, s.conf, n) || !alloc_n(c, s.count, (size_t)s.pitch * H) || !alloc_n(c, s.prio, n) ||
-      !alloc_n(c, s.pconf, n) || (r > 8 && !alloc_n(c, s.front, n)) || !alloc_n(c, s.tiles0, (size_t)s.t0x * s.t0y) ||
+      !alloc_n(c, s.pconf, n) || (r > 8 && !alloc_n(c, s.front, n)) || (r > 8 && !alloc_n(c, s.fsum, (size_t)(4 * r + 3) * (4 * r + 3))) || !alloc_n(c, s.tiles0, (size_t)s.t0x * s.t0y) ||
       !alloc_n(c, s.tiles1, (size_t)s.t1x * s.t1y) ||
       !alloc_n(c, s.ctrl, 1) || !alloc_n(c, s.trace, (size_t)s.trace_cap) ||
       !alloc_n(c, s.partial, (size_t)(s.n_partial > 0 ? s.n_partial : 1)) ||
@@ -799,8 +799,10 @@ int inpaint_apply_key(inpaint_ctx* c, unsigned long long key, inpaint_step_info*
   s.n_partial = 1;
   if (c->r <= 8)
     CK(launch_update_fast(s, c->cond, 0, c->stream));
-  else
+  else {
+    CK(launch_sums(s, c->stream));
     CK(launch_update(s, c->cond, 0, c->stream));
+  }
   if (c->opt.debug_checks) CK(launch_verify_count(c->st, c->stream));
   if ((rc = read_ctrl(c))) return rc;
   if (c->h_ctrl->status != 0) return c->h_ctrl->status;

@@ -72,6 +72,7 @@ struct Ctrl {
   int tc_rounds;   // engine search rounds run in the tensor-core form
   int n_front;     // patch radius > 8: front pixels in ImgState::front whose priorities
                    // are to be evaluated; -1: the last update applied nothing
+  int n_spec;      // patch radius > 8: front pixels in ImgState::front after the coming fill
   int engine_err;  // error word of the last engine launch (single image)
   int tiles_done;  // initialisation: CTAs of k_tiles_all that are done
 };
@@ -152,6 +153,7 @@ struct ImgState {
   unsigned long long* partial;  // per-CTA best search key of the iteration
   uint32_t* obits;         // initialisation: Omega, one bit per pixel, rows of obits_pitch(W) words
   int* front;              // patch radius > 8: linear indices of the pixels to evaluate
+  double* fsum;            // patch radius > 8: their confidence sums after the coming fill
   // tensor-core form (null otherwise): five BF16 planes of the image, R' G' B'
   // (byte - 128) and the square sum sq = sum_c (byte_c - 128)^2 as 256 hi and
   // lo (sq = 256 hi + lo), stored per tile column tx of the search (columns
@@ -421,6 +423,74 @@ __device__ inline void warp_select(const ImgState& s) {
   }
 }
 
+// Patch radius > 8: sum in row-major order of the values of the entries of
+// [x0, x1] x [y0, y1] that count; value(x, y, q, c) loads entry q's value into c
+// and says whether it counts.  One warp: its lanes load four rows coalesced (the
+// next four while these are summed), write the entries that count one after the
+// other to `vals` (shared memory) and add them one by one in order; the others
+// are skipped, which changes nothing (adding +0.0 to a non-negative sum) and
+// halves the chain of dependent FP64 additions (69 cycles each; with a bit scan
+// and a shuffle per entry in the chain 140).
+constexpr int kSumRows = 4;
+constexpr int kSumVals = kSumRows * (2 * kMaxRadius + 1) + 4;
+template <class F>
+__device__ inline double warp_ordered_sum(const ImgState& s, double* vals, int x0, int x1, int y0, int y1, F&& value) {
+  constexpr int NB = (2 * kMaxRadius + 1 + 31) / 32;
+  const int lane = threadIdx.x & 31, W = s.W, P = 2 * s.r + 1;
+  double sum = 0.0, c[kSumRows][NB];
+  bool kn[kSumRows][NB];
+  auto load_rows = [&](int ya) {
+#pragma unroll
+    for (int g = 0; g < kSumRows; ++g) {
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        const int xx = x0 + 32 * b + lane, yy = ya + g;
+        c[g][b] = 0.0;
+        kn[g][b] = 32 * b < P && xx <= x1 && yy <= y1 && value(xx, yy, (size_t)yy * W + xx, c[g][b]);
+      }
+    }
+  };
+  load_rows(y0);
+  for (int yy = y0; yy <= y1; yy += kSumRows) {
+    int n = 0;
+    __syncwarp();
+#pragma unroll
+    for (int g = 0; g < kSumRows; ++g) {
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        const unsigned m = __ballot_sync(0xffffffffu, kn[g][b]);
+        if (kn[g][b]) vals[n + __popc(m & ((1u << lane) - 1u))] = c[g][b];
+        n += __popc(m);
+      }
+    }
+    if (lane < 4) vals[n + lane] = 0.0;  // (+0.0 changes no sum here)
+    __syncwarp();
+    if (yy + kSumRows <= y1) load_rows(yy + kSumRows);
+#pragma unroll 2
+    for (int q = 0; q < n; q += 4) {
+      const double2 v = *reinterpret_cast<const double2*>(&vals[q]), w = *reinterpret_cast<const double2*>(&vals[q + 2]);
+      sum = __dadd_rn(__dadd_rn(__dadd_rn(__dadd_rn(sum, v.x), v.y), w.x), w.y);
+    }
+  }
+  return sum;
+}
+
+// Patch radius > 8: the confidence sum of listed front pixel k after the coming
+// fill, whose pixels take the target's confidence.  One warp.
+__device__ inline void warp_fill_sum(const ImgState& s, double* vals, int k) {
+  const Ctrl* c = s.ctrl;
+  const int px = c->px, py = c->py, r = s.r, p = s.front[k], y = p / s.W, x = p - y * s.W;
+  const double cp = c->conf;
+  const double sum = warp_ordered_sum(s, vals, max(x - r, 0), min(x + r, s.W - 1), max(y - r, 0), min(y + r, s.H - 1),
+                                      [&](int xx, int yy, size_t q, double& v) {
+                                        const double cf = s.conf[q];
+                                        const bool om = s.omega[q] != 0;
+                                        v = om ? cp : cf;
+                                        return !om || (abs(xx - px) <= r && abs(yy - py) <= r);
+                                      });
+  if ((threadIdx.x & 31) == 0) s.fsum[k] = sum;
+}
+
 // ---- host-side launchers (defined in the .cu files) ----
 void set_last_error(const char* msg);  // text returned by inpaint_last_error()
 cudaError_t launch_init(const ImgState& s, const uint8_t* rgb, int rgb_stride, const uint8_t* mask,
@@ -429,7 +499,9 @@ cudaError_t launch_import(const ImgState& s, const uint8_t* rgb, const uint8_t* 
                           const double* conf, cudaStream_t st);
 cudaError_t prepare_search_plain(int r);
 cudaError_t launch_prio_init_fast(const ImgState& s, cudaStream_t st);  // r <= 8
-cudaError_t launch_search_plain(const ImgState& s, cudaStream_t st);
+// sums (patch radius > 8): also the confidence sums of the update that follows.
+cudaError_t launch_search_plain(const ImgState& s, cudaStream_t st, bool sums = false);
+cudaError_t launch_sums(const ImgState& s, cudaStream_t st);  // patch radius > 8: these alone
 dim3 search_plain_grid(const ImgState& s);
 // Tensor-core search (search_tc.cu), patch radius 1..8: a persistent grid over
 // tiles of 8 candidate rows; one partial key per CTA (grid partials).

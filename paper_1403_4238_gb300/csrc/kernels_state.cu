@@ -109,64 +109,26 @@ __device__ inline void append_front(const ImgState& s, bool mine, int i) {
 }
 
 // Priorities of the listed front pixels for patch radii above the engine's:
-// one CTA of two warps per pixel.  Warp 0 sums the confidences: its lanes load
-// four patch rows coalesced (the next four while these are summed), write the
-// known entries one after the other to shared memory, and add them one by one in
-// row-major order; unknown ones are skipped, which changes nothing (adding +0.0
-// to a non-negative sum) and halves the chain of dependent FP64 additions (69
-// cycles each; with a bit scan and a shuffle per entry in the chain 140).  Warp 1
-// meanwhile finds the strongest isophote.  (One thread per pixel reading the
-// patch from global memory, in the update's one CTA, took 390 us an iteration at
-// 512x384, 25x25.)
-__global__ void __launch_bounds__(64) k_prio_list(ImgState s) {
-  constexpr int kGroup = 4;
+// one CTA per pixel.  kSum (initialisation): warp 0 sums the confidences while
+// warp 1 finds the strongest isophote; else the sums are in fsum already.  (One
+// thread per pixel reading the patch from global memory, in the update's one
+// CTA, took 390 us an iteration at 512x384, 25x25.)
+template <bool kSum>
+__global__ void __launch_bounds__(kSum ? 64 : 32) k_prio_list(ImgState s) {
   __shared__ unsigned long long iso_s;
-  __shared__ __align__(16) double vals[kGroup * (2 * kMaxRadius + 1) + 4];
+  __shared__ __align__(16) double vals[kSum ? kSumVals : 2];
   const int n = s.ctrl->n_front;
   const int W = s.W, H = s.H, r = s.r, P = 2 * r + 1;
   const int lane = threadIdx.x & 31;
   for (int k = blockIdx.x; k < n; k += gridDim.x) {
     const int p = s.front[k], y = p / W, x = p - y * W;
     const int x0 = max(x - r, 0), x1 = min(x + r, W - 1), y0 = max(y - r, 0), y1 = min(y + r, H - 1);
-    double sum = 0.0;
-    if (threadIdx.x < 32) {
-      constexpr int NB = (2 * kMaxRadius + 1 + 31) / 32;
-      double c[kGroup][NB];
-      bool kn[kGroup][NB];
-      auto load_rows = [&](int y0) {
-#pragma unroll
-        for (int g = 0; g < kGroup; ++g) {
-#pragma unroll
-          for (int b = 0; b < NB; ++b) {
-            const int xx = x0 + 32 * b + lane;
-            const bool in = 32 * b < P && xx <= x1 && y0 + g <= y1;
-            c[g][b] = in ? s.conf[(size_t)(y0 + g) * W + xx] : 0.0;
-            kn[g][b] = in && s.omega[(size_t)(y0 + g) * W + xx] == 0;
-          }
-        }
-      };
-      load_rows(y0);
-      for (int yy = y0; yy <= y1; yy += kGroup) {
-        int n_val = 0;
-        __syncwarp();
-#pragma unroll
-        for (int g = 0; g < kGroup; ++g) {
-#pragma unroll
-          for (int b = 0; b < NB; ++b) {
-            const unsigned m = __ballot_sync(0xffffffffu, kn[g][b]);
-            if (kn[g][b]) vals[n_val + __popc(m & ((1u << lane) - 1u))] = c[g][b];
-            n_val += __popc(m);
-          }
-        }
-        if (lane < 4) vals[n_val + lane] = 0.0;  // (+0.0 changes no sum here)
-        __syncwarp();
-        if (yy + kGroup <= y1) load_rows(yy + kGroup);
-#pragma unroll 2
-        for (int q = 0; q < n_val; q += 4) {
-          const double2 v = *reinterpret_cast<const double2*>(&vals[q]), w = *reinterpret_cast<const double2*>(&vals[q + 2]);
-          sum = __dadd_rn(__dadd_rn(__dadd_rn(__dadd_rn(sum, v.x), v.y), w.x), w.y);
-        }
-      }
+    double sum = kSum ? 0.0 : s.fsum[k];
+    if (kSum && threadIdx.x < 32) {
+      sum = warp_ordered_sum(s, vals, x0, x1, y0, y1, [&](int, int, size_t q, double& c) {
+        c = s.conf[q];
+        return s.omega[q] == 0;
+      });
     } else {
       // key: (|grad|^2 + 1) << 32 | ~(row-major index in the patch), 0: none
       unsigned long long best = 0ull;
@@ -203,6 +165,53 @@ __global__ void __launch_bounds__(64) k_prio_list(ImgState s) {
     }
     __syncthreads();
   }
+}
+
+// The front of the window of the current target as it is after the coming fill
+// (the patch's unknown pixels known then), listed in front.  It does not depend
+// on the search's result, so its confidence sums run beside the search, as CTAs
+// of the same launch (search_plain.cu; 512x384, 25x25: 70 us an iteration with the
+// sums behind the fill, 64 so).  Whole block of kUpdThreads.
+__device__ inline void block_spec_list(const ImgState& s, int* n) {
+  const Ctrl* c = s.ctrl;
+  const int px = __ldcg(&c->px), py = __ldcg(&c->py), r = s.r, R2 = 2 * r + 1, side = 2 * R2 + 1, lane = threadIdx.x & 31;
+  auto known = [&](int x, int y) {
+    if (x < 0 || x >= s.W || y < 0 || y >= s.H) return false;
+    const bool k = s.omega[(size_t)y * s.W + x] == 0;
+    return k || (abs(x - px) <= r && abs(y - py) <= r);
+  };
+  if (threadIdx.x == 0) *n = 0;
+  __syncthreads();
+  constexpr int V = 3;
+  for (int j0 = threadIdx.x; j0 - (int)threadIdx.x < side * side; j0 += V * kUpdThreads) {
+    bool fr[V];
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+      const int j = j0 + u * kUpdThreads, x = px - R2 + j % side, y = py - R2 + j / side;
+      const bool in = j < side * side && x >= 0 && x < s.W && y >= 0 && y < s.H;
+      const bool k0 = known(x, y), kl = known(x - 1, y), kr = known(x + 1, y), ku = known(x, y - 1), kd = known(x, y + 1);
+      fr[u] = in & !k0 & (kl | kr | ku | kd);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+      const int j = j0 + u * kUpdThreads;
+      const unsigned bal = __ballot_sync(0xffffffffu, fr[u]);
+      int base = 0;
+      if (lane == 0 && bal) base = atomicAdd(n, __popc(bal));
+      base = __shfl_sync(0xffffffffu, base, 0);
+      if (fr[u])
+        s.front[base + __popc(bal & ((1u << lane) - 1u))] = (py - R2 + j / side) * s.W + px - R2 + j % side;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) s.ctrl->n_spec = *n;
+}
+
+// The first target's list (initialisation).  Single CTA.
+__global__ void __launch_bounds__(kUpdThreads) k_spec_first(ImgState s) {
+  __shared__ int n;
+  if (s.ctrl->px >= 0) block_spec_list(s, &n);
 }
 
 // CTAs of k_prio_list (a grid-stride loop): a window's front is 100-200 pixels.
@@ -354,12 +363,13 @@ struct UpdSmem {
   int32_t fsat[(2 * kMaxRadius + 2) * (2 * kMaxRadius + 2)];
   unsigned long long u64s[32];
   int ints[32];
-  int n_front;
 };
 
 // One iteration's copy and validity update for patch radii above the
-// engine's, up to the list of front pixels whose priorities it changes.
-// Single CTA; k_prio_list and k_select_big follow.
+// engine's.  Single CTA; k_prio_list (the front pixels listed before the search,
+// with the sums taken beside it) and k_select_big follow.  Every round trip here
+// is a serial one, so a thread's reads go out together (17 us cold with a chain
+// of reads per window pixel and the list counted in global memory, now 13).
 __global__ void __launch_bounds__(kUpdThreads) k_fill_big(ImgState s) {
   __shared__ UpdSmem sm;
   Ctrl* c = s.ctrl;
@@ -474,33 +484,22 @@ __global__ void __launch_bounds__(kUpdThreads) k_fill_big(ImgState s) {
     }
     newly = block_sum_int(newly, sm.ints);  // also orders the global writes above
 
-    // Priorities that can change: front pixels within 2r+1 of p^, listed with a
-    // counter in shared memory (every round trip here is a serial one: with a
-    // counter in global memory and a chain of reads per pixel this kernel took
-    // 14 us at 25x25).
+    // Priorities that can change are those of the front pixels within 2r+1 of
+    // p^ (listed before the search); the window's others have none.
     const int R2 = 2 * r + 1, side2 = 2 * R2 + 1;
-    if (tid == 0) sm.n_front = 0;
     __syncthreads();
     constexpr int V = 3;
-    for (int j0 = tid; j0 - tid < side2 * side2; j0 += V * nt) {
-      bool in[V], fr[V];
+    for (int j0 = tid; j0 < side2 * side2; j0 += V * nt) {
+      bool off[V];
 #pragma unroll
       for (int u = 0; u < V; ++u) {
         const int j = j0 + u * nt, x = px - R2 + j % side2, y = py - R2 + j / side2;
-        in[u] = j < side2 * side2 && x >= 0 && x < W && y >= 0 && y < H;
-        fr[u] = in[u] && on_front(s, x, y);
+        off[u] = j < side2 * side2 && x >= 0 && x < W && y >= 0 && y < H && !on_front(s, x, y);
       }
-      __syncwarp();
 #pragma unroll
       for (int u = 0; u < V; ++u) {
-        const int j = j0 + u * nt, i = (py - R2 + j / side2) * W + px - R2 + j % side2, lane = tid & 31;
-        const unsigned bal = __ballot_sync(0xffffffffu, fr[u]);
-        int base = 0;
-        if (lane == 0 && bal) base = atomicAdd(&sm.n_front, __popc(bal));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (fr[u]) {
-          s.front[base + __popc(bal & ((1u << lane) - 1u))] = i;
-        } else if (in[u]) {
+        const int j = j0 + u * nt, i = (py - R2 + j / side2) * W + px - R2 + j % side2;
+        if (off[u]) {
           s.prio[i] = 0ull;
           s.pconf[i] = 0.0;
         }
@@ -508,7 +507,7 @@ __global__ void __launch_bounds__(kUpdThreads) k_fill_big(ImgState s) {
     }
     __syncthreads();
     if (tid == 0) {
-      c->n_front = sm.n_front;
+      c->n_front = c->n_spec;
       if (filled == 0) {  // p^ must lie in Omega; stop rather than loop without progress
         c->status = INPAINT_ERR_INTERNAL;
         c->n_front = -1;
@@ -538,10 +537,11 @@ __global__ void __launch_bounds__(kUpdThreads) k_fill_big(ImgState s) {
   }
 }
 
-// After k_prio_list: the tiles over the window of the target just filled and
-// the selection of the next one.  Single CTA.
+// After k_prio_list: the tiles over the window of the target just filled, the
+// selection of the next one and its list.  Single CTA.
 __global__ void __launch_bounds__(kUpdThreads) k_select_big(ImgState s, cudaGraphConditionalHandle cond,
                                                             int use_cond) {
+  __shared__ int n_list;
   Ctrl* c = s.ctrl;
   const int tid = threadIdx.x;
   if (c->n_front >= 0) {
@@ -555,6 +555,9 @@ __global__ void __launch_bounds__(kUpdThreads) k_select_big(ImgState s, cudaGrap
         c->py = -1;
       }
     }
+    __syncthreads();
+    // (the next iteration's list; the selection above is visible after the barrier)
+    if (c->remaining > 0 && c->status == 0) block_spec_list(s, &n_list);
     __syncthreads();
   }
   if (use_cond && tid == 0) cudaGraphSetConditional(cond, c->n_front >= 0 && loop_active(c) ? 1u : 0u);
@@ -607,9 +610,10 @@ static cudaError_t init_state(const ImgState& s, const uint8_t* rgb, int rgb_str
     if (e != cudaSuccess) return e;
   } else {
     k_front_all<<<dim3((W + 255) / 256, H), 256, 0, st>>>(s);
-    k_prio_list<<<kPrioCtas, 64, 0, st>>>(s);
+    k_prio_list<true><<<kPrioCtas, 64, 0, st>>>(s);
   }
   k_tiles_all<<<dim3(s.t1x, s.t1y), 1024, 0, st>>>(s);
+  if (s.r > 8) k_spec_first<<<1, kUpdThreads, 0, st>>>(s);
   return cudaGetLastError();
 }
 
@@ -625,7 +629,7 @@ cudaError_t launch_import(const ImgState& s, const uint8_t* rgb, const uint8_t* 
 
 cudaError_t launch_update(const ImgState& s, unsigned long long cond_handle, int use_cond, cudaStream_t st) {
   k_fill_big<<<1, kUpdThreads, 0, st>>>(s);
-  k_prio_list<<<kPrioCtas, 64, 0, st>>>(s);
+  k_prio_list<false><<<kPrioCtas, 32, 0, st>>>(s);
   k_select_big<<<1, kUpdThreads, 0, st>>>(s, (cudaGraphConditionalHandle)cond_handle, use_cond);
   return cudaGetLastError();
 }

@@ -271,11 +271,21 @@ struct GenGeom {
   __host__ __device__ size_t bytes() const { return (size_t)(SH * SW + P * TP + 3 * P) * sizeof(uint32_t); }
 };
 
-__global__ void __launch_bounds__(kSearchThreads) k_search_generic(ImgState s) {
+__global__ void __launch_bounds__(kSearchThreads) k_search_generic(ImgState s, int n_sum, int gx) {
   extern __shared__ __align__(16) uint32_t dyn[];
   __shared__ unsigned long long red[32];
   const Ctrl* c = s.ctrl;
   if (!loop_active(c)) return;
+  if ((int)blockIdx.x < n_sum) {
+    // the first CTAs: confidence sums of the update that follows, one warp each
+    // (18 us of ordered additions an iteration at 512x384, 25x25, behind the
+    // search before)
+    __shared__ __align__(16) double vals[kSumVals];
+    if (threadIdx.x < 32)
+      for (int k = blockIdx.x; k < c->n_spec; k += n_sum) warp_fill_sum(s, vals, k);
+    return;
+  }
+  const int tile = blockIdx.x - n_sum, tx = tile % gx, ty = tile / gx;
   constexpr int S = kSearchS;
   const int R = s.r;
   const GenGeom g(R);
@@ -283,7 +293,7 @@ __global__ void __launch_bounds__(kSearchThreads) k_search_generic(ImgState s) {
   uint32_t* tgt = src + g.SH * g.SW;    // P x TP, 0 where unknown
   uint32_t* rmask = tgt + g.P * g.TP;   // P x 3: bits of the known columns
   const int px = c->px, py = c->py;
-  const int ox = s.cx0 + blockIdx.x * kSearchTW, oy = s.cy0 + blockIdx.y * kSearchTH;
+  const int ox = s.cx0 + tx * kSearchTW, oy = s.cy0 + ty * kSearchTH;
   const int tid = threadIdx.x, lane = tid & 31, wr = tid >> 5;
   int cnt[S];
   load_counts<S>(s, ox + lane * S, oy + wr, cnt);
@@ -348,7 +358,23 @@ __global__ void __launch_bounds__(kSearchThreads) k_search_generic(ImgState s) {
       }
     }
   }
-  write_partial(s, best_key<S>(s, acc, cnt, ox + lane * S, oy + wr), red);
+  const unsigned long long best = block_min_u64(best_key<S>(s, acc, cnt, ox + lane * S, oy + wr), red);
+  if (tid == 0) s.partial[tile] = best;
+}
+
+// The sums alone (an iteration whose search ran elsewhere).
+__global__ void __launch_bounds__(32) k_sums(ImgState s) {
+  __shared__ __align__(16) double vals[kSumVals];
+  if (!loop_active(s.ctrl)) return;
+  for (int k = blockIdx.x; k < s.ctrl->n_spec; k += gridDim.x) warp_fill_sum(s, vals, k);
+}
+
+// CTAs for the sums: a window's front is 100-200 pixels (k_prio_list's grid).
+constexpr int kSumCtas = 304;
+
+cudaError_t launch_sums(const ImgState& s, cudaStream_t st) {
+  k_sums<<<kSumCtas, 32, 0, st>>>(s);
+  return cudaGetLastError();
 }
 
 cudaError_t prepare_search_plain(int r) {
@@ -363,9 +389,9 @@ dim3 search_plain_grid(const ImgState& s) {
   return dim3((cw + kSearchTW - 1) / kSearchTW, (ch + kSearchTH - 1) / kSearchTH, 1);
 }
 
-cudaError_t launch_search_plain(const ImgState& s, cudaStream_t st) {
+cudaError_t launch_search_plain(const ImgState& s, cudaStream_t st, bool sums) {
   const dim3 g = search_plain_grid(s);
-  if (g.x == 0) return cudaSuccess;
+  if (g.x == 0) return sums && s.r > 8 ? launch_sums(s, st) : cudaSuccess;
   if (s.overlap) {
     switch (s.r) {
       case 1: k_search_overlap<1><<<g, kSearchThreads, 0, st>>>(s); break;
@@ -389,8 +415,10 @@ cudaError_t launch_search_plain(const ImgState& s, cudaStream_t st) {
     case 6: k_search_plain<6><<<g, kSearchThreads, 0, st>>>(s); break;
     case 7: k_search_plain<7><<<g, kSearchThreads, 0, st>>>(s); break;
     case 8: k_search_plain<8><<<g, kSearchThreads, 0, st>>>(s); break;
-    default:
-      k_search_generic<<<g, kSearchThreads, GenGeom(s.r).bytes(), st>>>(s);
+    default: {
+      const int n_sum = sums ? kSumCtas : 0;
+      k_search_generic<<<n_sum + (int)(g.x * g.y), kSearchThreads, GenGeom(s.r).bytes(), st>>>(s, n_sum, (int)g.x);
+    }
   }
   return cudaGetLastError();
 }
