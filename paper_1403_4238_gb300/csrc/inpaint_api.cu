@@ -565,6 +565,8 @@ int inpaint_run(inpaint_ctx* c, int max_iters, int* iters_done, inpaint_step_inf
   long long lim = (long long)start + c->h_ctrl->remaining;
   if (max_iters > 0 && (long long)start + max_iters < lim) lim = (long long)start + max_iters;
   const int limit = lim > INT_MAX ? INT_MAX : (int)lim;
+  // (the graph loop needs none of the engine's buffers and options)
+  if (c->overlap_engine && use_engine(c) && setup_engine(c) != INPAINT_OK) c->overlap_engine = false;
   const bool engine = use_engine(c);
   c->ctrl_known = false;
   if (engine) {

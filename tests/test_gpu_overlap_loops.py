@@ -56,3 +56,13 @@ def test_loops_agree(api, r, W, H, alpha):
             assert [np.float64(t[f]).view(np.uint64) for t in got] == \
                    [np.float64(t[f]).view(np.uint64) for t in ora.trace], f
         assert (out == ora.rgb).all() and evals == ora.evals
+
+
+def test_graph_loop_where_the_engine_cannot(api):
+    """Engine options that only the engine checks do not stop the variant: the graph loop runs it."""
+    rgb, m = synth.image(90, 60, 7, 30.0, 5), np.zeros((60, 90), np.uint8)
+    m[20:26, 30:44] = 1
+    ora = oracle.run(rgb, m, 3, overlap=True)
+    with api.Inpainter(rgb, m, 3, overlap=True, tile_rows=3) as ip:
+        rc, n, tr = ip.run(trace=True)
+        assert rc == 0 and n == ora.iters and (ip.result() == ora.rgb).all()
