@@ -83,12 +83,6 @@ struct Ctrl {
 constexpr int kSpecOutside = -2;   // window pixel outside the image
 constexpr int kSpecNotFront = -1;  // in the image, not on the post-fill front
 
-// Entry of a compact work list handled by thread t: consecutive entries go
-// to warps 0..3 in turn (one warp per SM sub-partition), so a short list of
-// long FP64 dependency chains uses all four sub-partitions with few active
-// lanes each.
-__device__ inline int list_entry(int t) { return ((t & 31) << 2) | ((t >> 5) & 3) | ((t >> 7) << 7); }
-
 // The squared lengths nn = |n|^2 a Sobel normal of a binary mask can take
 // (nx, ny in [-4, 4]) for the data term D = (dot / sqrt(nn)) / 510, dot in
 // [0, 2040], and their codes.
@@ -287,20 +281,6 @@ __device__ inline void warp_best_prio(unsigned long long& k, int& i) {
 // those itself (no lone warp between two barriers).  The leading barrier
 // keeps the previous call's readers ahead of this call's writers; scratch
 // holds one entry per warp; blockDim.x must be a multiple of 32.
-__device__ inline void block_best_prio(unsigned long long& k, int& i, PrioBest* scratch) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  warp_best_prio(k, i);
-  __syncthreads();
-  if (lane == 0) {
-    scratch[wid].key = k;
-    scratch[wid].idx = i;
-  }
-  __syncthreads();
-  k = lane < nw ? scratch[lane].key : 0ull;
-  i = lane < nw ? scratch[lane].idx : 0x7fffffff;
-  warp_best_prio(k, i);
-}
-
 __device__ inline unsigned long long block_min_u64(unsigned long long v, unsigned long long* scratch) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   v = warp_min_u64(v);
