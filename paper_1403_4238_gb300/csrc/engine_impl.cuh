@@ -1112,8 +1112,15 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
   unsigned epoch = x.epoch;
 
   // every role reads the image's fields from shared memory, which keeps
-  // about forty registers free for its phases
+  // about forty registers free for its phases.  The barrier before the write is
+  // the hand-over from the team's last image: its leader's warps 4-15 may still
+  // be in update_drain, with that image's fields and update state, when warps
+  // 0-3 come here (with more images than SMs a CTA does several in turn).  The
+  // fence orders the last image's accesses to shared memory before this one's
+  // bulk copies into it.  Once an image.
   if constexpr (!kLeadOnly) {
+    fence_proxy_async_smem();
+    __syncthreads();
     if (tid == 0) tl.img = ea.imgs[j];
     __syncthreads();
   }
