@@ -42,7 +42,7 @@ __global__ void k_planes(ImgState s) {
     const size_t ry = e / s.tc_len;
     const int y = (int)(ry % s.prows), tx = (int)(ry / s.prows);
     const int f = s.tc_f > 1 ? min((xl >> 3) / s.tc_n1, s.tc_f) : 0;
-    const int x = s.tc_xs0 + 8 * (tx * s.tc_n - f * s.tc_n1) + xl, yi = y + f * s.tc_h;
+    const int x = s.tc_xs0 + 8 * (tx * s.tc_n - f * s.tc_n1) + xl, yi = s.cy0 - s.r + y + f * s.tc_h;
     const bool in = x < s.W && yi < s.H && (f == 0 || f < s.tc_f);
     const uint32_t w = in ? __ldg(&s.img[(size_t)yi * s.pitch + x]) : 0x00808080u;
     plane_write(s.planes + ((size_t)tx * s.prows + y) * 5 * s.tc_len + xl, s.tc_len, w);  // outside the image: 128 - 128 = 0 everywhere

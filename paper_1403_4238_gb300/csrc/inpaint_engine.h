@@ -50,7 +50,10 @@ __host__ __device__ inline TcTiles tc_tiles(const ImgState& s) {
 __host__ __device__ inline float tc_mma_cycles(int N) { return 43.5f + 0.24f * (float)N; }
 
 // Tile and plane geometry of an image (the tc_* fields and prows of s); the
-// rows every tile reads (y0 - r .. y0 + 15 + r) all exist.  want > 0: the tiles
+// rows every tile reads (y0 - r .. y0 + 15 + r) all exist, and no others: a
+// fold's planes begin at the search rectangle's first source row, so that a
+// rectangle far down an image takes no more memory than one at the top, and a
+// pixel lies in at most two folds.  want > 0: the tiles
 // of one image spread over `want` CTAs, so the number of tile columns (narrower
 // tiles, cheaper MMAs) is what makes the round shortest; want 0: throughput of
 // small teams, so a narrow image is folded until its tiles are close to
@@ -93,8 +96,7 @@ inline size_t tc_plane_layout(ImgState& s, int want) {
   }
   s.tc_h = kTcRows * s.tc_nty;
   s.tc_len = 8 * (s.tc_n + nc - 1);
-  const int hr = s.cy0 + s.tc_h + s.r;
-  s.prows = folds == 1 && hr < s.H ? s.H : hr;
+  s.prows = s.tc_h + 2 * s.r;
   return (size_t)s.tc_ntx * s.prows * 5 * s.tc_len * 2 + (size_t)s.tc_ntx * s.tc_nty * kTcRows * s.tc_n;
 }
 // The planes and the bits in a buffer of that size.

@@ -151,10 +151,11 @@ struct ImgState {
   // tensor-core form (null otherwise): five BF16 planes of the image, R' G' B'
   // (byte - 128) and the square sum sq = sum_c (byte_c - 128)^2 as 256 hi and
   // lo (sq = 256 hi + lo), stored per tile column tx of the search (columns
-  // [tc_xs0 + tx * 8 tc_n, + tc_len)) as [tx][row y < prows][plane][tc_len],
+  // [tc_xs0 + tx * 8 tc_n, + tc_len)) as [tx][row < prows][plane][tc_len],
   // zero outside W x H, so that two source rows of a tile are one contiguous
-  // copy.  A narrow image can be folded: fold f < tc_f holds the rows from
-  // f * tc_h on, 8 tc_n1 columns to the right of fold f - 1 (tc_ntx is 1 then).
+  // copy.  Row 0 is image row cy0 - r, the first that the search reads.  A
+  // narrow image can be folded: fold f < tc_f holds the rows from f * tc_h on,
+  // 8 tc_n1 columns to the right of fold f - 1 (tc_ntx is 1 then).
   uint16_t* planes;
   int prows, tc_xs0, tc_len, tc_ntx, tc_nty, tc_n, tc_n1, tc_f, tc_h;
   // with the planes: one validity bit per candidate of every search tile,
@@ -190,27 +191,28 @@ __device__ inline void plane_write(uint16_t* row, int len, uint32_t w) {
 
 // Where the planes hold pixel (x, y): the places (null: none) in the at most
 // two tile columns whose segments hold column x, or in the at most two folds
-// that hold row y.
-__device__ inline void plane_places(const ImgState& s, int x, int y, uint16_t*& a, uint16_t*& b) {
+// that hold its row (a fold holds tc_h + 2r rows, and 2r <= 16 <= tc_h).
+__host__ __device__ inline void plane_places(const ImgState& s, int x, int y, uint16_t*& a, uint16_t*& b) {
   a = b = nullptr;
-  const int xl = x - s.tc_xs0, len = s.tc_len;
-  if (xl < 0) return;  // left of every tile's source columns
+  const int xl = x - s.tc_xs0, yl = y - (s.cy0 - s.r), len = s.tc_len;
+  if (xl < 0 || yl < 0) return;  // left of or above every tile's source pixels
   if (s.tc_f > 1) {
     if (xl >= 8 * s.tc_n1) return;
-    for (int f = 0, yf = y; f < s.tc_f && yf >= 0; ++f, yf -= s.tc_h)
+    for (int f = 0, yf = yl; f < s.tc_f && yf >= 0; ++f, yf -= s.tc_h)
       if (yf < s.prows) {
         b = a;
         a = s.planes + (size_t)yf * 5 * len + xl + 8 * f * s.tc_n1;
       }
     return;
   }
+  if (yl >= s.prows) return;
   int tx = 0, xt = xl;  // (a few tile columns: cheaper than a division)
   while (tx + 1 < s.tc_ntx && xt >= 8 * s.tc_n) {
     xt -= 8 * s.tc_n;
     ++tx;
   }
-  if (xt < len) a = s.planes + ((size_t)tx * s.prows + y) * 5 * len + xt;
-  if (tx > 0 && xt + 8 * s.tc_n < len) b = s.planes + ((size_t)(tx - 1) * s.prows + y) * 5 * len + xt + 8 * s.tc_n;
+  if (xt < len) a = s.planes + ((size_t)tx * s.prows + yl) * 5 * len + xt;
+  if (tx > 0 && xt + 8 * s.tc_n < len) b = s.planes + ((size_t)(tx - 1) * s.prows + yl) * 5 * len + xt + 8 * s.tc_n;
 }
 
 // Candidate centre (x, y) of the search rectangle became valid: its bit.

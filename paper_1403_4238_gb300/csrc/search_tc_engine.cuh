@@ -151,19 +151,20 @@ __device__ __forceinline__ void tc_build_a(uint8_t* A, const uint16_t* tpad, boo
 }
 
 // Producer: ring slots [h0, h1) of the tile in tile column tx whose source
-// rows start at y0 - R (ring sequence numbers g0 + h; slot h holds rows
+// rows start at image row y0 - R (ring sequence numbers g0 + h; slot h holds rows
 // 2h, 2h + 1, five plane segments of tc_len elements each).  One thread.
 // Returns false if a bounded wait gave up.
 template <int R>
 __device__ __forceinline__ bool tc_produce(const ImgState& s, const TcArea& ta, EngBars& bars, int tx, int y0,
                                            uint32_t g0, int h0, int h1, unsigned long long limit) {
   const uint32_t bytes = (uint32_t)(kTcRps * 5 * 2 * s.tc_len);
+  const int row0 = y0 - s.cy0;  // plane row of image row y0 - R
   for (int h = h0; h < h1; ++h) {
     const uint32_t g = g0 + (uint32_t)h;
     const int slot = (int)(g % (uint32_t)ta.nb);
     if (g >= (uint32_t)ta.nb && !mbar_wait(&bars.tc_empty[slot], ((g / ta.nb) - 1u) & 1u, limit)) return false;
     mbar_expect_tx(&bars.tc_full[slot], bytes);
-    const uint16_t* src = s.planes + ((size_t)tx * s.prows + (y0 - R + kTcRps * h)) * 5 * s.tc_len;
+    const uint16_t* src = s.planes + ((size_t)tx * s.prows + (row0 + kTcRps * h)) * 5 * s.tc_len;
     bulk_load(ta.ring + (size_t)slot * ta.slot, src, bytes, &bars.tc_full[slot]);
   }
   return true;
