@@ -1461,16 +1461,16 @@ struct SrvReq {
 
 // Upper estimate of a request's device memory (the buffers create_impl and
 // the batch member copy allocate: about 48 bytes per pixel, the tensor-core
-// search's planes, the trace).
-size_t est_bytes(int W, int H, int r, int n_omega) {
+// search's planes of its search rectangle, the trace).
+size_t est_bytes(const SrvReq& q, double alpha) {
   ImgState s{};
-  s.W = W;
-  s.H = H;
-  s.r = r;
-  s.cx0 = s.cy0 = r;
-  s.cx1 = W - 1 - r;
-  s.cy1 = H - 1 - r;
-  return (size_t)W * H * 48 + tc_plane_layout(s, 0) + (size_t)(n_omega + 1) * sizeof(inpaint_step_info) + (1u << 20);
+  s.W = q.W;
+  s.H = q.H;
+  s.r = q.r;
+  search_rect(q.mask.data(), q.W, q.W, q.H, q.r, alpha, false, &s.cx0, &s.cx1, &s.cy0, &s.cy1);
+  size_t n_omega = 0;
+  for (uint8_t m : q.mask) n_omega += m != 0;
+  return (size_t)q.W * q.H * 48 + tc_plane_layout(s, 0) + (n_omega + 1) * sizeof(inpaint_step_info) + (1u << 20);
 }
 
 }  // namespace
@@ -1526,9 +1526,7 @@ struct inpaint_server {
         if (stop) return;
         while (!queue.empty() && (int)(active.size() + admit.size()) < max_slots) {
           SrvReq* q = queue.front();
-          int n_omega = 0;
-          for (uint8_t m : q->mask) n_omega += m != 0;
-          const size_t b = est_bytes(q->W, q->H, q->r, n_omega);
+          const size_t b = est_bytes(*q, opt.search_alpha);
           if (used + b > budget && !(active.empty() && admit.empty())) break;
           queue.pop_front();
           q->bytes = b;
