@@ -59,7 +59,6 @@ struct inpaint_ctx {
   uint8_t* orig_rgb = nullptr;    // 3*W*H, batch members only: input kept for reset
   uint8_t* orig_mask = nullptr;   // W*H
   Ctrl* h_ctrl = nullptr;         // pinned mirror of the control block
-  int* h_limit = nullptr;         // pinned staging for iter_limit
   std::vector<std::pair<void*, size_t>> allocs;
   cudaGraph_t run_graph = nullptr;
   cudaGraphExec_t run_exec = nullptr;
@@ -111,9 +110,7 @@ struct inpaint_ctx {
     allocs.clear();
     if (stream) cudaStreamSynchronize(stream);
     if (h_ctrl) cudaFreeHost(h_ctrl);
-    if (h_limit) cudaFreeHost(h_limit);
     h_ctrl = nullptr;
-    h_limit = nullptr;
     if (own_stream && stream) cudaStreamDestroy(stream);
     stream = nullptr;
   }
@@ -339,12 +336,13 @@ int build_run_graph(inpaint_ctx* c) {
   return INPAINT_OK;
 }
 
+// The limit is an argument of the launch, not a word in host memory: with work
+// pending on the caller's stream the next call's limit could be written over
+// one that the device has yet to read.
 int set_limit(inpaint_ctx* c, int limit) {
   if (limit == INT_MAX && c->no_limit) return INPAINT_OK;
-  *c->h_limit = limit;
   c->no_limit = false;
-  CK(cudaMemcpyAsync(&c->st.ctrl->iter_limit, c->h_limit, sizeof(int), cudaMemcpyHostToDevice,
-                     c->stream));
+  CK(launch_set_limit(c->st, limit, c->stream));
   c->no_limit = limit == INT_MAX;
   return INPAINT_OK;
 }
@@ -414,7 +412,6 @@ int create_impl(const uint8_t* rgb, int W, int H, int rgb_stride, const uint8_t*
     c->own_stream = true;
   }
   if (cudaMallocHost(&c->h_ctrl, sizeof(Ctrl)) != cudaSuccess) return fail(INPAINT_ERR_NOMEM);
-  if (cudaMallocHost(&c->h_limit, sizeof(int)) != cudaSuccess) return fail(INPAINT_ERR_NOMEM);
 
   ImgState& s = c->st;
   s.W = W;

@@ -498,6 +498,7 @@ cudaError_t launch_search_tc(const ImgState& s, const TcPlan& plan, cudaStream_t
 cudaError_t launch_update(const ImgState& s, unsigned long long cond_handle, int use_cond,
                           cudaStream_t st);  // patch radius > 8
 cudaError_t launch_verify_count(const ImgState& s, cudaStream_t st);
+cudaError_t launch_set_limit(const ImgState& s, int limit, cudaStream_t st);  // Ctrl::iter_limit
 cudaError_t launch_export(const ImgState& s, uint8_t* rgb_dense, cudaStream_t st);
 
 }  // namespace inp

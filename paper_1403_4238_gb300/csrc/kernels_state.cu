@@ -598,6 +598,8 @@ __global__ void k_export(ImgState s, uint8_t* rgb) {
   rgb[3 * i + 2] = (uint8_t)((w >> 16) & 255u);
 }
 
+__global__ void k_set_limit(Ctrl* c, int limit) { c->iter_limit = limit; }
+
 // ---------------------------------------------------------------- launchers
 
 static cudaError_t init_state(const ImgState& s, const uint8_t* rgb, int rgb_stride, const uint8_t* mask,
@@ -631,6 +633,11 @@ cudaError_t launch_update(const ImgState& s, unsigned long long cond_handle, int
   k_fill_big<<<1, kUpdThreads, 0, st>>>(s);
   k_prio_list<false><<<kPrioCtas, 32, 0, st>>>(s);
   k_select_big<<<1, kUpdThreads, 0, st>>>(s, (cudaGraphConditionalHandle)cond_handle, use_cond);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_set_limit(const ImgState& s, int limit, cudaStream_t st) {
+  k_set_limit<<<1, 1, 0, st>>>(s.ctrl, limit);
   return cudaGetLastError();
 }
 
