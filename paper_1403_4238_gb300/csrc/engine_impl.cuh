@@ -434,12 +434,22 @@ __host__ __device__ constexpr size_t eng_smem_bytes() {
 static_assert(eng_smem_bytes<8, 2>() <= 227 * 1024, "engine CTA must fit in shared memory");
 static_assert(eng_smem_bytes<7, 2>() <= 227 * 1024, "engine CTA must fit in shared memory");
 
-// Team publication word: epoch (bits 0-31), next target px (32-46), py
-// (47-61), stop flag (62).  One acquire load gives a waiting CTA everything
-// it needs to start the next search round.
-__device__ inline unsigned long long pub_pack(unsigned epoch, int px, int py, bool stop) {
-  return (unsigned long long)epoch | ((unsigned long long)(px & 0x7fff) << 32) |
-         ((unsigned long long)(py & 0x7fff) << 47) | ((unsigned long long)(stop ? 1 : 0) << 62);
+// Team publication word: epoch (bits 0-31), next target px (from bit 32, as
+// many bits as a column of the image needs), py (the bits above) and the stop
+// flag (63).  One acquire load gives a waiting CTA everything it needs to start
+// the next search round.  px and py take at most 31 bits together: W H <= 2^30,
+// and the bits of two numbers are at most two more than those of their
+// product's logarithm.
+__device__ inline int pub_bits(int W) { return 32 - __clz(W - 1); }
+__device__ inline unsigned long long pub_pack(unsigned epoch, int px, int py, bool stop, int bits) {
+  const unsigned hi = (unsigned)px | (unsigned)py << bits | (stop ? 1u << 31 : 0u);
+  return (unsigned long long)hi << 32 | epoch;
+}
+__device__ inline void pub_unpack(unsigned long long v, int bits, int& px, int& py, int& stop) {
+  const unsigned hi = (unsigned)(v >> 32);
+  px = (int)(hi & ((1u << bits) - 1u));
+  py = (int)((hi & 0x7fffffffu) >> bits);
+  stop = (int)(hi >> 31);
 }
 
 __device__ inline unsigned long long ld_acquire64(const unsigned long long* p) {
@@ -479,7 +489,7 @@ __device__ inline unsigned long long wait_pub(TeamCtl* tc, unsigned epoch, int* 
     if ((unsigned)v != epoch) return v;
     if (globaltimer() - t0 > limit) {
       atomicExch(err, INPAINT_ERR_TIMEOUT);
-      return pub_pack(epoch + 1u, 0, 0, true);
+      return pub_pack(epoch + 1u, 0, 0, true, 0);
     }
   }
 }
@@ -811,10 +821,8 @@ __device__ __noinline__ void run_tc_search(const EngineArgs& ea, EngCtx& x, cons
     }
     // wait for the next round
     if (tid == 0) {
-      const unsigned long long v = wait_pub(tc, epoch, err, limit);
-      tl.stop = ((v >> 62) & 1ull) != 0;
-      tl.px = (int)((v >> 32) & 0x7fff);
-      tl.py = (int)((v >> 47) & 0x7fff);
+      const int bits = pub_bits(s.W);
+      pub_unpack(wait_pub(tc, epoch, err, limit), bits, tl.px, tl.py, tl.stop);
     }
     ++epoch;
     __syncthreads();
@@ -1070,10 +1078,8 @@ __device__ __noinline__ void run_res_search(const EngineArgs& ea, EngCtx& x, int
       }
     }
     if (tid == 0) {
-      const unsigned long long v = wait_pub(tc, epoch, err, limit);
-      tl.stop = ((v >> 62) & 1ull) != 0;
-      tl.px = (int)((v >> 32) & 0x7fff);
-      tl.py = (int)((v >> 47) & 0x7fff);
+      const int bits = pub_bits(s.W);
+      pub_unpack(wait_pub(tc, epoch, err, limit), bits, tl.px, tl.py, tl.stop);
     }
     ++epoch;
     __syncthreads();
@@ -1377,7 +1383,7 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
         stop = true;  // the launch's time budget is spent: resume in the next launch
         tc->expired = 1u;
       }
-      const unsigned long long v = pub_pack(epoch + 1u, stop ? 0 : wi - ny * s.W, stop ? 0 : ny, stop);
+      const unsigned long long v = pub_pack(epoch + 1u, stop ? 0 : wi - ny * s.W, stop ? 0 : ny, stop, pub_bits(s.W));
       if (ok && !spent)
         st_relaxed64(&tc->pub, v);
       else
@@ -1423,10 +1429,8 @@ __device__ __forceinline__ void run_image(const EngineArgs& ea, int j, EngCtx& x
     }
     // searchers and idle CTAs: wait for the next round
     if (tid == 0) {
-      const unsigned long long v = wait_pub(tc, epoch, err, limit);
-      tl.stop = ((v >> 62) & 1ull) != 0;
-      tl.px = (int)((v >> 32) & 0x7fff);
-      tl.py = (int)((v >> 47) & 0x7fff);
+      const int bits = pub_bits(s.W);
+      pub_unpack(wait_pub(tc, epoch, err, limit), bits, tl.px, tl.py, tl.stop);
     }
     ++epoch;
     __syncthreads();
@@ -1544,13 +1548,12 @@ static size_t eng_smem_r(int srw) {
 }
 // Whether the engine runs the image's partial-overlap search with a team of
 // tsize CTAs: every searcher's tiles are resident (the streaming search has no
-// such form), and a target fits the publication word.
+// such form).
 template <int R>
 static bool overlap_fits_t(const ImgState& s, int tsize, size_t smem) {
   int ncu, ns;
   const int m = overlap_units<R>(s, tsize - 1, &ncu, &ns);
-  return m > 0 && m <= ncu && smem > kHeadBytes && res_need<R>(4, m) <= (int)(smem - kHeadBytes) && s.W <= 0x7fff &&
-         s.H <= 0x7fff;
+  return m > 0 && m <= ncu && smem > kHeadBytes && res_need<R>(4, m) <= (int)(smem - kHeadBytes);
 }
 template <int R>
 const EngineFns* engine_fns_for() {
