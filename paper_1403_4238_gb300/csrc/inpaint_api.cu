@@ -90,6 +90,7 @@ struct inpaint_ctx {
         p = nullptr;
       }
     } else if (cudaMallocAsync(&p, bytes, stream) != cudaSuccess) {
+      cudaGetLastError();  // reported here: the next launch's status is its own
       p = nullptr;
     }
     if (p) allocs.emplace_back(p, bytes);
@@ -891,8 +892,10 @@ struct DevAlloc {
     void* p = nullptr;
     if (opt.dev_alloc)
       p = opt.dev_alloc(bytes, (void*)stream, opt.alloc_user);
-    else if (cudaMallocAsync(&p, bytes, stream) != cudaSuccess)
+    else if (cudaMallocAsync(&p, bytes, stream) != cudaSuccess) {
+      cudaGetLastError();  // reported here: the next launch's status is its own
       p = nullptr;
+    }
     if (p) allocs.emplace_back(p, bytes);
     return p;
   }
