@@ -470,11 +470,14 @@ int create_impl(const uint8_t* rgb, int W, int H, int rgb_stride, const uint8_t*
   }
   if (plane_bytes > 0) {
     uint8_t* planes = nullptr;
-    if (!alloc_n(c, planes, plane_bytes)) {
+    if (alloc_n(c, planes, plane_bytes)) {
+      tc_bind_planes(s, planes);
+    } else if (tc_auto) {  // the engine's choice is the plain form then
+      s.tc_auto = s.tc_ntx = s.tc_nty = 0;
+    } else {
       g_last_error = "device allocation failed";
       return fail(INPAINT_ERR_NOMEM);
     }
-    tc_bind_planes(s, planes);
   }
   if (prepare_search_plain(r) != cudaSuccess) return fail(INPAINT_ERR_CUDA);
   *out = c;
@@ -1144,8 +1147,9 @@ void engine_set_free(EngineSet& es) {
 }
 
 // Creates a context for one image on the given stream, with a device copy of
-// its input kept for resets.
-int make_member(const inpaint_image& im, const inpaint_options& base, cudaStream_t st, int index,
+// its input kept for resets.  tc_auto: with planes, if they fit, for the engine
+// to choose the form.
+int make_member(const inpaint_image& im, const inpaint_options& base, cudaStream_t st, int index, bool tc_auto,
                 inpaint_ctx** out) {
   *out = nullptr;
   if (im.patch_radius < 1 || im.patch_radius > 8) {
@@ -1159,7 +1163,7 @@ int make_member(const inpaint_image& im, const inpaint_options& base, cudaStream
   o.loop_mode = INPAINT_LOOP_ENGINE;
   inpaint_ctx* c = nullptr;
   int rc = create_impl(im.rgb, im.width, im.height, im.rgb_stride_bytes, im.mask, im.mask_stride_bytes,
-                       im.patch_radius, &o, &c, true);
+                       im.patch_radius, &o, &c, tc_auto);
   if (rc >= 0 && launch_planes(c->st, st) != cudaSuccess) {
     inpaint_destroy(c);
     return INPAINT_ERR_CUDA;
@@ -1286,7 +1290,7 @@ void build_batch_graphs(inpaint_batch* b) {
   });
 }
 
-int batch_create_impl(const inpaint_image* images, int n, const inpaint_options* opt, inpaint_batch** out) {
+int batch_create_impl(const inpaint_image* images, int n, const inpaint_options* opt, bool tc_auto, inpaint_batch** out) {
   if (!out || !images || n < 1) return INPAINT_ERR_ARG;
   *out = nullptr;
   inpaint_batch* b = new (std::nothrow) inpaint_batch();
@@ -1318,7 +1322,7 @@ int batch_create_impl(const inpaint_image* images, int n, const inpaint_options*
   std::vector<double> work(n);
   for (int i = 0; i < n; ++i) {
     inpaint_ctx* c = nullptr;
-    const int rc = make_member(images[i], b->opt, b->stream, i, &c);
+    const int rc = make_member(images[i], b->opt, b->stream, i, tc_auto, &c);
     if (rc < 0) return fail(rc);
     b->ctx.push_back(c);
     work[i] = left_of(*c->h_ctrl);
@@ -1338,7 +1342,9 @@ extern "C" {
 int inpaint_batch_create(const inpaint_image* images, int n, const inpaint_options* opt,
                          inpaint_batch** out) {
   try {
-    return batch_create_impl(images, n, opt, out);
+    const int rc = batch_create_impl(images, n, opt, true, out);
+    // (the planes of some members can leave too little for what the others need)
+    return rc == INPAINT_ERR_NOMEM ? batch_create_impl(images, n, opt, false, out) : rc;
   } catch (...) {
     return INPAINT_ERR_NOMEM;
   }
@@ -1540,7 +1546,8 @@ struct inpaint_server {
       for (SrvReq* q : admit) {
         inpaint_image im{q->rgb.data(), q->W, q->H, 3 * q->W, q->mask.data(), q->W, q->r};
         inpaint_ctx* c = nullptr;
-        const int rc = make_member(im, opt, stream, (int)q->id, &c);
+        int rc = make_member(im, opt, stream, (int)q->id, true, &c);
+        if (rc == INPAINT_ERR_NOMEM) rc = make_member(im, opt, stream, (int)q->id, false, &c);
         q->t_admit = now();
         if (rc < 0) {
           retire(q, rc);
