@@ -261,10 +261,12 @@ class _ResultMemory:
     Fresh memory costs 0.3 ms a megabyte at its first write (its pages are
     zeroed then): 54 ms of a 180 ms batch of 60 photos when the copies to the
     host met it, and nothing beside the 125 ms that the device takes.  Every
-    array is handed out once; those not yet taken stay, at most one per image.
+    array is handed out once; those not yet taken stay, at most one per image
+    and MAX_BYTES in all (a caller may fetch few of them, or one at a time).
     """
 
     MIN_BYTES = 8 << 20  # 2.5 ms of faults; starting the thread costs 0.1 ms
+    MAX_BYTES = 256 << 20
 
     def __init__(self):
         self._lock = threading.Lock()
@@ -282,8 +284,15 @@ class _ResultMemory:
 
     def fill(self, shapes: dict, wanted):
         """Starts faulting in the arrays of `shapes` that wanted(key) still holds for; until stop()."""
+        todo = {}
         with self._lock:
-            todo = {k: v for k, v in shapes.items() if k not in self._ready}
+            room = self.MAX_BYTES - sum(a.nbytes for a in self._ready.values())
+            for key, shape in shapes.items():
+                if key not in self._ready:
+                    room -= int(np.prod(shape))
+                    if room < 0:
+                        break
+                    todo[key] = shape
         if sum(int(np.prod(v)) for v in todo.values()) < self.MIN_BYTES:
             return
         stop = self._stop = threading.Event()
