@@ -274,9 +274,13 @@ class _ResultMemory:
         self._stop = None
 
     def take(self, key, shape):
-        with self._lock:
-            a = self._ready.pop(key, None)
+        a = self.pop(key)
         return a if a is not None else np.zeros(shape, np.uint8)
+
+    def pop(self, key):
+        """The array of `key` if there is one; it is not kept any more."""
+        with self._lock:
+            return self._ready.pop(key, None)
 
     def put_back(self, key, a):
         with self._lock:
@@ -493,14 +497,17 @@ class Server:
 
     def poll(self, rid: int):
         H, W = self.shapes[rid]
-        out = self._memory.take(rid, (H, W, 3))
+        ready = self._memory.pop(rid)
+        out = ready if ready is not None else np.zeros((H, W, 3), np.uint8)
         info = _lib.RequestInfo()
         rc = _check(self.lib.inpaint_server_poll(self.s, ctypes.c_uint64(rid), out.ctypes.data, 3 * W,
                                                  ctypes.byref(info)), "inpaint_server_poll")
         if rc == _lib.STATUS["PENDING"]:
-            self._memory.put_back(rid, out)
+            if ready is not None:  # (an array of its own costs nothing yet, and none is kept)
+                self._memory.put_back(rid, ready)
             return None
         del self.shapes[rid]
+        self._memory.pop(rid)  # one that came after this call had looked for it
         return out, {f: getattr(info, f) for f, _ in _lib.RequestInfo._fields_}
 
     def wait_idle(self, timeout_s: float = 600.0):

@@ -4,7 +4,8 @@ import time
 
 import pytest
 
-from paper_1403_4238_gb300.api import _ResultMemory
+from paper_1403_4238_gb300 import _lib
+from paper_1403_4238_gb300.api import Server, _ResultMemory
 
 
 def settle(before):
@@ -28,3 +29,44 @@ def test_total_is_bounded(monkeypatch, limit, kept):
         settle(before)
         assert sorted(m._ready) == [0, 2, 3, *range(4, kept + 1)] and a.shape == shapes[1]
     m.stop()
+
+
+class PolledLib:
+    """inpaint_server_poll of a fake library; `during` runs inside each call."""
+
+    def __init__(self, codes, during):
+        self.codes, self.during = list(codes), during
+
+    def inpaint_server_poll(self, *args):
+        self.during()
+        return self.codes.pop(0)
+
+
+def polled_server(codes, during=lambda: None):
+    srv = Server.__new__(Server)  # without a device
+    srv.lib, srv.s, srv.shapes, srv._memory = PolledLib(codes, during), None, {5: (2000, 1500), 6: (2000, 1500)}, _ResultMemory()
+    return srv
+
+
+def test_none_is_kept_for_a_request_that_was_polled():
+    before = threading.active_count()
+
+    def during():  # another thread's wait_idle finishes the array between the look for it and the end of the poll
+        srv._memory.fill({5: (2000, 1500, 3)}, lambda k: k in srv.shapes)
+        settle(before)
+
+    srv = polled_server([_lib.STATUS["OK"]], during)
+    out, _ = srv.poll(5)
+    assert out.shape == (2000, 1500, 3) and 5 not in srv.shapes
+    assert not srv._memory._ready
+
+
+def test_pending_polls_keep_only_what_was_faulted_in():
+    before = threading.active_count()
+    srv = polled_server([_lib.STATUS["PENDING"]] * 3 + [_lib.STATUS["OK"]])
+    assert srv.poll(5) is None and not srv._memory._ready
+    srv._memory.fill({k: (*v, 3) for k, v in srv.shapes.items()}, lambda k: k in srv.shapes)  # 5 is not left out
+    settle(before)
+    a = srv._memory._ready[5]
+    assert srv.poll(5) is None and srv.poll(5) is None and srv._memory._ready[5] is a
+    assert srv.poll(5)[0] is a and list(srv._memory._ready) == [6]
