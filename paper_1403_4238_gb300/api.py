@@ -267,11 +267,12 @@ class _ResultMemory:
 
     MIN_BYTES = 8 << 20  # 2.5 ms of faults; starting the thread costs 0.1 ms
     MAX_BYTES = 256 << 20
+    RANGE = 1 << 20  # bytes faulted in between two looks at the stop event
 
     def __init__(self):
         self._lock = threading.Lock()
         self._ready = {}
-        self._stop = None
+        self._jobs = []  # (stop event, thread) of every fill() that is not stopped yet
 
     def take(self, key, shape):
         a = self.pop(key)
@@ -287,7 +288,8 @@ class _ResultMemory:
             self._ready[key] = a
 
     def fill(self, shapes: dict, wanted):
-        """Starts faulting in the arrays of `shapes` that wanted(key) still holds for; until stop()."""
+        """Starts faulting in the arrays of `shapes` that wanted(key) still holds for; until stop()
+        of what this returns (None: too little to start for)."""
         todo = {}
         with self._lock:
             room = self.MAX_BYTES - sum(a.nbytes for a in self._ready.values())
@@ -298,25 +300,37 @@ class _ResultMemory:
                         break
                     todo[key] = shape
         if sum(int(np.prod(v)) for v in todo.values()) < self.MIN_BYTES:
-            return
-        stop = self._stop = threading.Event()
+            return None
+        stop = threading.Event()
 
         def work():
             for key, shape in todo.items():
-                if stop.is_set():
-                    return
                 a = np.zeros(shape, np.uint8)
-                a.reshape(-1)[::4096] = 0  # a write to each page
+                flat = a.reshape(-1)
+                for o in range(0, flat.size, self.RANGE):
+                    if stop.is_set():
+                        return
+                    flat[o:o + self.RANGE:4096] = 0  # a write to each page
                 with self._lock:
-                    if not stop.is_set() and wanted(key):
+                    held = sum(b.nbytes for b in self._ready.values())  # (other waits fill it too)
+                    if not stop.is_set() and wanted(key) and held + a.nbytes <= self.MAX_BYTES:
                         self._ready.setdefault(key, a)
 
-        threading.Thread(target=work, daemon=True).start()
+        job = stop, threading.Thread(target=work, daemon=True)
+        job[1].start()
+        with self._lock:
+            self._jobs.append(job)
+        return job
 
-    def stop(self):
-        stop, self._stop = self._stop, None
-        if stop is not None:
+    def stop(self, job=None):
+        """Ends the given fill(), by default every one; nothing of it runs on afterwards."""
+        with self._lock:
+            jobs = [j for j in self._jobs if job is None or j is job]
+            self._jobs = [j for j in self._jobs if j not in jobs]
+        for stop, _ in jobs:
             stop.set()
+        for _, thread in jobs:
+            thread.join()
 
 
 class Batch:
@@ -364,6 +378,7 @@ class Batch:
 
     def close(self):
         if getattr(self, "b", None):
+            self._memory.stop()
             self._memory = _ResultMemory()
             self.lib.inpaint_batch_destroy(self.b)
             self.b = None
@@ -385,11 +400,12 @@ class Batch:
 
     def run(self, max_iters: int = 0):
         st = (ctypes.c_int * self.n)()
-        self._memory.fill({i: (H, W, 3) for i, (H, W) in enumerate(self.shapes)}, lambda i: True)
+        job = self._memory.fill({i: (H, W, 3) for i, (H, W) in enumerate(self.shapes)}, lambda i: True)
         try:
             _check(self.lib.inpaint_batch_run_ctx(self.b, int(max_iters), st), "inpaint_batch_run_ctx")
         finally:
-            self._memory.stop()
+            if job is not None:
+                self._memory.stop(job)
         return list(st)
 
     def result(self, i: int):
@@ -468,6 +484,7 @@ class Server:
 
     def close(self):
         if getattr(self, "s", None):
+            self._memory.stop()
             self._memory = _ResultMemory()
             self.lib.inpaint_server_destroy(self.s)
             self.s = None
@@ -511,11 +528,13 @@ class Server:
         return out, {f: getattr(info, f) for f, _ in _lib.RequestInfo._fields_}
 
     def wait_idle(self, timeout_s: float = 600.0):
-        self._memory.fill({k: (H, W, 3) for k, (H, W) in list(self.shapes.items())}, lambda k: k in self.shapes)
+        shapes = {k: (H, W, 3) for k, (H, W) in list(self.shapes.items())}
+        job = self._memory.fill(shapes, lambda k: k in self.shapes)
         try:
             return _check(self.lib.inpaint_server_wait_idle(self.s, float(timeout_s)), "inpaint_server_wait_idle")
         finally:
-            self._memory.stop()
+            if job is not None:
+                self._memory.stop(job)
 
     def stats(self):
         st = _lib.ServerStats()

@@ -70,3 +70,26 @@ def test_pending_polls_keep_only_what_was_faulted_in():
     a = srv._memory._ready[5]
     assert srv.poll(5) is None and srv.poll(5) is None and srv._memory._ready[5] is a
     assert srv.poll(5)[0] is a and list(srv._memory._ready) == [6]
+
+
+def test_stop_ends_its_own_fill_and_waits_for_it():
+    m, before = _ResultMemory(), threading.active_count()
+    gate, started = threading.Event(), threading.Event()
+
+    def hold(i):
+        started.set()
+        gate.wait(10.0)
+        return True
+
+    m.fill({i: (4000, 2000, 3) for i in range(40)}, lambda i: True)  # a wait of one thread
+    m.stop()
+    assert threading.active_count() == before  # not even in the middle of an array
+    first = m.fill({i: (1000, 3000, 3) for i in range(3)}, hold)
+    assert started.wait(10.0)
+    gate.set()
+    second = m.fill({i: (1000, 3000, 3) for i in range(10, 13)}, lambda i: True)  # and of another
+    m.stop(first)
+    settle(before)
+    assert {10, 11, 12} <= set(m._ready)  # the other thread's wait had them made all the same
+    m.stop(second)
+    assert threading.active_count() == before
