@@ -317,9 +317,9 @@ class _ResultMemory:
                         self._ready.setdefault(key, a)
 
         job = stop, threading.Thread(target=work, daemon=True)
-        job[1].start()
         with self._lock:
             self._jobs.append(job)
+        job[1].start()
         return job
 
     def stop(self, job=None):
@@ -330,7 +330,8 @@ class _ResultMemory:
         for stop, _ in jobs:
             stop.set()
         for _, thread in jobs:
-            thread.join()
+            if thread.ident is not None:  # (it could not be started)
+                thread.join()
 
 
 class Batch:
