@@ -725,6 +725,10 @@ int inpaint_time_search(inpaint_ctx* c, int form, int reps, double* ms_per_searc
   if (e == cudaSuccess)
     e = cudaMemcpy2D(om.data(), P, s.omega + (size_t)y0 * c->W + x0, c->W, x1 - x0 + 1, y1 - y0 + 1,
                      cudaMemcpyDeviceToHost);
+  // the partial-overlap searches have counted their admissible candidates into
+  // the count of the next iteration
+  if (e == cudaSuccess && s.overlap)
+    e = cudaMemcpy(&s.ctrl->n_adm, &h.n_adm, sizeof(h.n_adm), cudaMemcpyHostToDevice);
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   cudaFree(part);
