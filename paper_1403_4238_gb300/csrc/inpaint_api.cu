@@ -676,6 +676,13 @@ int inpaint_time_search(inpaint_ctx* c, int form, int reps, double* ms_per_searc
   TcPlan plan{};
   uint16_t* tmp_planes = nullptr;  // a plain-form context has no planes: build them for the timing
   if (form == INPAINT_FORM_TC) {
+    // the full search's candidates, whose patches lie inside the image: the
+    // rectangle of a partial-overlap search begins at the border, and planes
+    // laid out for it would be filled from pixels before the image
+    s.cx0 = std::max(s.cx0, s.r);
+    s.cx1 = std::min(s.cx1, s.W - 1 - s.r);
+    s.cy0 = std::max(s.cy0, s.r);
+    s.cy1 = std::min(s.cy1, s.H - 1 - s.r);
     if (!s.planes) {
       int dev = 0, sms = 0;
       CK(cudaGetDevice(&dev));
