@@ -517,10 +517,13 @@ __device__ inline void spec_chains(const ImgState& s, UpdSmem<R>& sm) {
     const double sum = conf_local<R>(sm, RB + wx, RB + wy), q = div_known(sum, (double)P2, sm.dinvP);
     // a second correction by the same reciprocal: after the first the
     // quotient is within an ulp, so this one rounds it correctly (Markstein),
-    // unless the remainder underflows or is inf - inf: tiny and infinite sums (an
-    // imported state's) and clipped patches divide
+    // unless the remainder underflows or is inf - inf: sums outside
+    // [2^-830, inf) (an imported state's) and clipped patches divide.  (The range
+    // by the sum's high word: an FP64 compare is a turn of the busy unit.)
     const double c = __fma_rn(__fma_rn(-q, (double)P2, sum), sm.dinvP, q);
-    sm.sC[par][i] = n_in == P2 && sum > 1e-250 && sum <= 1.7976931348623157e308 ? c : __ddiv_rn(sum, (double)n_in);
+    constexpr unsigned kLo = (1023u - 830u) << 20, kInf = 2047u << 20;
+    const bool in_range = (unsigned)__double2hiint(sum) - kLo < kInf - kLo;
+    sm.sC[par][i] = n_in == P2 && in_range ? c : __ddiv_rn(sum, (double)n_in);
   }
 }
 
