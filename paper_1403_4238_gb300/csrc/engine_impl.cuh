@@ -57,11 +57,9 @@ struct EngGeom {
   static constexpr int B = kEngBatchRows;          // candidate rows per batch (one per lane)
   static constexpr int BW = eng_tile_width(R, SRW);  // staged width (words)
   static constexpr int BH = B + 2 * R;             // staged rows
-  static constexpr int PIX_BYTES = ((BW * BH * 4 + 127) / 128) * 128;
+  static constexpr int SLOT_BYTES = ((BW * BH * 4 + 127) / 128) * 128;
   static constexpr int CW = eng_count_width(SRW);  // count tile width (words), CW / 4 odd
   static constexpr int CNT_BYTES = ((CW * B * 4 + 127) / 128) * 128;
-  static constexpr int VB_BYTES = kEngWarps * 32;  // validity bits: one byte per (warp, lane)
-  static constexpr int SLOT_BYTES = PIX_BYTES + VB_BYTES;
   static constexpr int COFF = R & 3;  // first candidate column within the count tile
   static constexpr int NS = (NCL + P - 1 + 3) & ~3;  // strip words per lane
   static constexpr int TP = (P + 3) & ~3;            // padded target row (words)
@@ -310,7 +308,7 @@ __device__ __noinline__ unsigned long long unit_best(int strip, int pitch, int t
 // about 500 cycles a row, most of it latency.  Only CTAs that do not lead
 // search this way (a leader that searches too has a small team and streams).
 constexpr int kResRows = 32;   // candidate rows per unit (one per lane)
-constexpr int kResMaxSeg = 4;  // bands one CTA's tiles may span
+constexpr int kResMaxSeg = 2;  // bands one CTA's tiles span at most: it has no more units than a band
 
 struct ResSeg {
   int band;      // 32-row band of the search rectangle
@@ -327,11 +325,10 @@ struct ResPlan {
   ResSeg seg[kResMaxSeg];
 };
 
-// Plan of rank `rank`'s units: the tile of each band its range touches.
-// Returns the bytes of shared memory the plan needs (tiles + validity
-// bits), or -1 when the range spans more bands than kResMaxSeg.
+// Plan of rank `rank`'s units: the tile of each band its range touches.  A range
+// has at most ncu units (the condition of the resident mode), so two bands.
 template <int R>
-__host__ __device__ inline long long res_plan(ResPlan& pl, int kc, int ncu, int nbands, int rank, int ns) {
+__device__ inline void res_plan(ResPlan& pl, int kc, int ncu, int nbands, int rank, int ns) {
   const long long U = (long long)ncu * nbands;
   pl.u0 = (int)(U * rank / ns);
   pl.u1 = (int)(U * (rank + 1) / ns);
@@ -339,10 +336,9 @@ __host__ __device__ inline long long res_plan(ResPlan& pl, int kc, int ncu, int 
   pl.nseg = 0;
   if (pl.u1 <= pl.u0) {
     pl.bits_off = 0;
-    return 0;
+    return;
   }
   const int b_lo = pl.u0 / ncu, b_hi = (pl.u1 - 1) / ncu;
-  if (b_hi - b_lo + 1 > kResMaxSeg) return -1;
   long long off = 0;
   for (int b = b_lo; b <= b_hi; ++b) {
     const int c_lo = b == b_lo ? pl.u0 % ncu : 0;
@@ -355,8 +351,6 @@ __host__ __device__ inline long long res_plan(ResPlan& pl, int kc, int ncu, int 
     off += (((long long)sg.pitch * (kResRows + 2 * R) * 4) + 127) / 128 * 128;
   }
   pl.bits_off = (int)off;
-  off += (long long)(pl.u1 - pl.u0) * 32 * 2;
-  return off;
 }
 
 // Shared memory that m units of kc columns need at most: two tiles (a range may
@@ -1519,10 +1513,6 @@ static cudaError_t upd_fast_t(const ImgState& s, unsigned long long cond, int us
   return cudaGetLastError();
 }
 
-
-
-
-
 template <int R>
 static cudaError_t prio_init_t(const ImgState& s, cudaStream_t st) {
   using G = UpdGeom<R>;
@@ -1534,12 +1524,6 @@ static cudaError_t prio_init_t(const ImgState& s, cudaStream_t st) {
   k_prio_init_fast<R><<<grid, 256, smem, st>>>(s);
   return cudaGetLastError();
 }
-
-
-
-}  // namespace inp
-
-namespace inp {
 
 // Host entry points of one radius R, exported through EngineFns.
 template <int R>

@@ -67,7 +67,6 @@ __global__ void __launch_bounds__(kEngThreads, 1) k_engine(EngineArgs ea) {
   x.tc_rows = 0;
   x.tc_tiles = 0;
   x.tc_nb = 0;
-  x.tc_pref = 0;
   x.ph0 = 0;
   x.ph1 = 0;
   x.epoch = (unsigned)ld_acquire64_pub(&x.tc->pub);

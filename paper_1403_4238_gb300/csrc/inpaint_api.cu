@@ -66,7 +66,7 @@ struct inpaint_ctx {
   TcPlan tc{};  // tensor-core search plan (form INPAINT_FORM_TC)
   // persistent engine (one team of every CTA)
   bool eng_ready = false;
-  int eng_grid = 0, eng_sr = 0;
+  int eng_grid = 0;
   size_t eng_smem = 0;
   EngineArgs ea{};
   ImgState* d_img = nullptr;
@@ -260,7 +260,6 @@ int setup_engine(inpaint_ctx* c) {
   if (!sr) sr = pick_rows_per_warp(c->st, grid);
   c->eng_smem = smem;
   c->eng_grid = grid;
-  c->eng_sr = sr;
   c->st.srw = sr;
   const int slots = c->st.overlap ? 3 : 1;  // of each CTA among the partials
   if (!alloc_n(c, c->d_img, 1) || !alloc_n(c, c->d_tmap, 2) ||

@@ -179,7 +179,6 @@ struct EngCtx {
   unsigned long long t_start;   // global timer at the CTA's start (tick budget)
   uint32_t tmem;                // tensor-memory base address (tensor-core search)
   uint32_t tc_rows;             // ring slots filled so far (their phases)
-  int tc_pref;                  // slots of the next round's first tile already requested
   uint32_t tc_tiles;            // tiles whose MMAs completed so far (done barrier phases)
   int tc_nb;                    // ring slots tc_rows was counted with (0: none yet)
 };

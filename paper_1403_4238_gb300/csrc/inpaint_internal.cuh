@@ -67,7 +67,7 @@ struct Ctrl {
   inpaint_step_info last;    // record of the most recent iteration
   // persistent-engine phase clocks (global timer, ns): search round (from the
   // previous publish to the last arrival) and update phase, summed
-  unsigned long long t_search, t_update, t_last;
+  unsigned long long t_search, t_update;
   int timed_iters;
   int tc_rounds;   // engine search rounds run in the tensor-core form
   int n_front;     // patch radius > 8: front pixels in ImgState::front whose priorities

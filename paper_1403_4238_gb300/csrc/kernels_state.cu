@@ -241,7 +241,6 @@ __global__ void k_unpack(ImgState s, const uint8_t* rgb, int rgb_stride, const u
     c->evals = 0ull;
     c->t_search = 0ull;
     c->t_update = 0ull;
-    c->t_last = 0ull;
     c->timed_iters = 0;
     c->tc_rounds = 0;
     c->n_front = 0;

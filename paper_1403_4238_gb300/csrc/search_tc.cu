@@ -29,8 +29,7 @@ struct TcHead {
 constexpr int kTcHeadBytes = (int)((sizeof(TcHead) + 127) / 128 * 128);
 
 template <int R>
-__host__ __device__ inline int tc_fixed_bytes(int N) {
-  (void)N;
+__host__ __device__ inline int tc_fixed_bytes() {
   return kTcHeadBytes + TcEngGeom<R>::A_BYTES + TcEngGeom<R>::TPAD_BYTES;
 }
 
@@ -125,7 +124,7 @@ cudaError_t prepare_r(const ImgState& s, TcPlan* plan) {
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
-  const int slot = tc_slot(tt.N, R), fixed = tc_fixed_bytes<R>(tt.N) + 128;  // + base alignment
+  const int slot = tc_slot(tt.N, R), fixed = tc_fixed_bytes<R>() + 128;  // + base alignment
   const int nb = (optin - fixed) / slot < kTcRing ? (optin - fixed) / slot : kTcRing;
   if (nb < 4) return cudaErrorInvalidConfiguration;
   plan->nb = nb;
