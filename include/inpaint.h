@@ -56,13 +56,18 @@ typedef enum {
 #define INPAINT_FORM_PLAIN 0 /* CUDA-core integer SSD (byte-SIMD abs-diff + dot) */
 #define INPAINT_FORM_TC 1    /* exact tensor-core correlation form (tcgen05, BF16 operands
                                 holding small integers, FP32 accumulation exact below 2^24);
-                                patch_radius <= 8.  In the persistent engine (single image,
-                                teams of two or more CTAs) the image's candidates are cut
-                                into tiles of 16 rows x 512 or 1024 columns searched from
-                                five BF16 planes of the image (about 10 bytes per pixel of
-                                extra device memory); where those tiles do not fit a CTA
-                                the engine searches with the plain form.  inpaint_step
-                                always runs the graph-loop kernels. */
+                                patch_radius <= 8.  In the persistent engine the image's
+                                candidates are cut into tiles of 16 rows x a multiple of
+                                128 columns (1024 at most), searched from five BF16 planes
+                                of the search rectangle (about 10 bytes per pixel of it in
+                                extra device memory); where a ring of their rows does not
+                                fit a CTA the engine searches with the plain form.
+                                inpaint_step always runs the graph-loop kernels.
+                                Batches and servers take INPAINT_FORM_PLAIN and choose
+                                themselves: an image whose planes fit the device memory,
+                                narrow ones with several row blocks side by side in a tile,
+                                is searched in the form with the lower estimate for its
+                                team, with the same results. */
 
 /* Device allocator hooks: lets a host framework (e.g. PyTorch's caching
  * allocator) own device memory.  Both NULL: cudaMallocAsync/cudaFreeAsync on
@@ -95,13 +100,14 @@ typedef struct {
                             the whole loop (patch_radius <= 8 only);
                             INPAINT_LOOP_GRAPH: a CUDA graph with a conditional while
                             node around [search kernel, update kernel] */
-  int tile_rows;         /* engine search, streaming mode (small images or small
-                            teams): a search batch is 32 candidate rows (one per lane)
-                            x 16 warps x 4 * tile_rows candidate columns per lane,
-                            i.e. 64 (tile_rows = 1) or 128 (tile_rows = 2) columns;
-                            0 = chosen by the library.  Large images on large teams
-                            use the resident mode (units of 32 rows x 16 columns,
-                            source tiles kept in shared memory), whatever this is */
+  int tile_rows;         /* engine search, streaming mode (teams whose leader searches
+                            too, and images whose tiles do not fit shared memory): a
+                            search batch is 32 candidate rows (one per lane) x 16 warps
+                            x 4 * tile_rows candidate columns per lane, i.e. 64
+                            (tile_rows = 1) or 128 (tile_rows = 2) columns; 0 = chosen
+                            by the library.  Otherwise the resident mode runs (units of
+                            32 rows x 16 columns, or x 4 where a CTA has few; source
+                            tiles kept in shared memory), whatever this is */
   const char* tuning_file; /* NULL, or a text table written by the autotuner: one line
                             "radius max_pixels tile_rows" per bucket; the first line
                             with the image's radius and max_pixels >= the image's

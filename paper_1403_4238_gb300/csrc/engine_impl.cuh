@@ -4,14 +4,15 @@
 // CTAs form teams; a team runs the fill loop of one image at a time (a list
 // of images per team gives the batched form).  One iteration of a team:
 //   1. every member CTA searches its share of the candidate centres
-//      (findBestPatch, Eq. 3-4).  Resident mode (large images): the CTA
-//      owns a contiguous range of units of 32 candidate rows x 16 columns,
-//      keeps their source window in shared memory for the whole removal and
-//      only patches the pixels the previous iteration filled; streaming
-//      mode (small images, small teams): batches of 32 rows x 64 or 128
-//      columns whose source window and validity counts arrive by TMA,
-//      double-buffered.  Each lane owns the candidates of one row; the
-//      CTA reduces them to one (SSD << 32 | idx) key;
+//      (findBestPatch, Eq. 3-4).  Resident mode (the leader does not search
+//      and the tiles fit): the CTA owns a contiguous range of units of 32
+//      candidate rows x 16 columns, or x 4 where it has few, keeps their
+//      source window in shared memory for the whole removal and only patches
+//      the pixels the previous iteration filled; streaming mode (small teams,
+//      whose leader searches too): batches of 32 rows x 64 or 128 columns
+//      whose source window and validity counts arrive by TMA, double-buffered.
+//      Each lane owns the candidates of one row; the CTA reduces them to one
+//      (SSD << 32 | idx) key.  Tensor-core form: search_tc_engine.cuh;
 //   2. each member writes its key, tagged with the round, to its slot; the
 //      leader polls the slots, runs the copy/update phase and the selection
 //      of the next target (update_fast.cuh) and publishes the next epoch;
@@ -1445,13 +1446,8 @@ constexpr size_t engine_smem_for() {
   return eng_smem_bytes<R, SRW>();
 }
 
-}  // namespace inp
-
-
-namespace inp {
-
 // Single-CTA copy/update kernel of the graph-driven loop for R <= 8 (the same
-// update phase the engine runs in its last-arriving CTA).
+// update phase that the engine runs in a team's leader).
 template <int R>
 __global__ void __launch_bounds__(kEngThreads) k_update_fast(ImgState s, cudaGraphConditionalHandle cond,
                                                             int use_cond) {

@@ -3,9 +3,10 @@
 // The three stages of Sec. 4.2 (initialisation, iterative computation,
 // finalisation) map to inpaint_create/inpaint_reset, inpaint_step/inpaint_run
 // and inpaint_result.  inpaint_run drives the whole iterative stage from the
-// device: one CUDA graph whose conditional while-node repeats
+// device, with no host round trip per iteration: one launch of the persistent
+// engine, or one CUDA graph whose conditional while-node repeats
 // [findBestPatch search -> copy/update + next selection] until the update
-// kernel reports an empty Omega, so no host round trip happens per iteration.
+// kernel reports an empty Omega.
 #include <algorithm>
 #include <chrono>
 #include <climits>
@@ -948,7 +949,9 @@ namespace {
 // Estimated cycles that image s (n_omega pixels left) takes on a team of
 // `size` CTAs: about 2 |Omega| / P^2 iterations, each a search round of the
 // form the engine would choose and 16,000 cycles of leader work, which a
-// leader that also searches does before and after its share.
+// leader that also searches does before and after its share.  (A leader that
+// does not works beside the search for part of them: the estimate of a team
+// whose leader only leads is high by as much.)
 double image_cycles(const ImgState& s, double n_omega, int size) {
   const int P = 2 * s.r + 1;
   const double iters = 2.0 * n_omega / (P * P) + 1.0;
@@ -1107,13 +1110,11 @@ int engine_set_prepare(EngineSet& es, const std::vector<inpaint_ctx*>& cs, const
   return INPAINT_OK;
 }
 
-// One launch: every context runs until its Omega is empty, it fails, or it
-// has done max_iters more iterations (<= 0: no limit).  Control blocks are
-// read back into es.h_ctrls.  Returns INPAINT_ERR_TIMEOUT if a bounded
+// One launch: every context runs until its Omega is empty, it fails, it has
+// done max_iters (> 0) more iterations, or the launch has run tick_ns (> 0;
+// teams stop between iterations and resume in the next call).  Control blocks
+// are read back into es.h_ctrls.  Returns INPAINT_ERR_TIMEOUT if a bounded
 // device wait gave up.
-// Runs every member until it is done, or for at most max_iters (> 0) more
-// iterations, or until the launch has run tick_ns (> 0; teams stop between
-// iterations and resume in the next call).
 int engine_set_run(EngineSet& es, const std::vector<inpaint_ctx*>& cs, int max_iters, cudaStream_t st,
                    unsigned long long tick_ns = 0ull) {
   const int n = (int)cs.size();

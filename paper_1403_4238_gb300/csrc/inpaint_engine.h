@@ -110,7 +110,9 @@ inline void tc_bind_planes(ImgState& s, void* p) {
 // (rows) x (MMAs a row), after about 4,500 cycles of target staging, A strips
 // and read-back.  Plain form: about 0.6 of the patch known, 24 evaluations a
 // cycle and CTA (the streaming mode of one- and two-CTA teams measured 20-28 of
-// the 64 its two instructions allow), after 2,500 cycles.
+// the 64 its two instructions allow), after 2,500 cycles.  The same rate stands
+// for larger teams, which are resident and faster (about 40 at 1920x1080, r 6):
+// there the estimate leans towards the tensor cores and towards more CTAs.
 __host__ __device__ inline float tc_round_cycles(const ImgState& s, int ns) {
   const int P = 2 * s.r + 1, nc = tc_chunks(s.r), tiles = s.tc_ntx * s.tc_nty;
   const float tile = (float)((kTcRows + P - 1) * ((3 * nc + 1) / 2 + nc)) * tc_mma_cycles(s.tc_n) + 300.f;
@@ -121,17 +123,19 @@ __host__ __device__ inline float plain_round_cycles(const ImgState& s, int ns) {
   return 2500.f + (float)(s.cx1 - s.cx0 + 1) * (float)(s.cy1 - s.cy0 + 1) * 0.6f * P2 / (24.f * (float)ns);
 }
 
-// The five planes of the image's current pixels and the validity bits (run
-// before every engine launch of an image in the tensor-core form).
+// The five planes of the search rectangle's current source pixels and the
+// validity bits: before every launch of a single image in the tensor-core form
+// (the caller may have changed it), after a batch or server image's
+// initialisation (its launches keep them up to date).
 cudaError_t launch_planes(const ImgState& s, cudaStream_t st);
 
 // Per-team synchronisation words (global memory).
 struct TeamCtl {
-  unsigned long long pub;  // epoch | next px | next py | stop (release-published)
+  unsigned long long pub;  // epoch | next px | next py | stop (pub_pack; release-published)
   unsigned expired;        // the launch's time budget ended this team's work
   unsigned copied;         // e + 1 once round e's fill is in the image and its planes
-                           // (release-published; the tensor-core searchers then
-                           // prefetch the next round's source rows)
+                           // (release-published; the searchers then bring their
+                           // resident tiles up to date or prefetch source rows)
   unsigned pad[28];        // keep teams on separate 128-byte lines
 };
 

@@ -411,7 +411,7 @@ __device__ inline void warp_select(const ImgState& s) {
 // next four while these are summed), write the entries that count one after the
 // other to `vals` (shared memory) and add them one by one in order; the others
 // are skipped, which changes nothing (adding +0.0 to a non-negative sum) and
-// halves the chain of dependent FP64 additions (69 cycles each; with a bit scan
+// halves the chain of dependent FP64 additions (64 cycles each; with a bit scan
 // and a shuffle per entry in the chain 140).
 constexpr int kSumRows = 4;
 constexpr int kSumVals = kSumRows * (2 * kMaxRadius + 1) + 4;
@@ -485,10 +485,9 @@ cudaError_t launch_prio_init_fast(const ImgState& s, cudaStream_t st);  // r <= 
 cudaError_t launch_search_plain(const ImgState& s, cudaStream_t st, bool sums = false);
 cudaError_t launch_sums(const ImgState& s, cudaStream_t st);  // patch radius > 8: these alone
 dim3 search_plain_grid(const ImgState& s);
-// Tensor-core search (search_tc.cu), patch radius 1..8: a persistent grid over
-// tiles of 8 candidate rows; one partial key per CTA (grid partials).
-// Tensor-core search, one launch per iteration: one CTA per tile of the
-// engine's tensor-core form (reads the image's BF16 planes).
+// Tensor-core search of the graph loop (search_tc.cu), patch radius 1..8, one
+// launch per iteration: one CTA and one partial key per tile of the engine's
+// tensor-core form (16 candidate rows x 8 N columns; reads the BF16 planes).
 struct TcPlan {
   int grid = 0, ntiles = 0, smem = 0, nb = 0, slot = 0;
 };
